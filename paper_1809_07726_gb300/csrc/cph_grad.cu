@@ -22,6 +22,7 @@
 #include <cstdint>
 #include <mutex>
 #include <string>
+#include <type_traits>
 
 #include "../../include/cphremd.h"
 #include "cph_device.cuh"
@@ -79,6 +80,21 @@ int gfail(int code, const std::string& m) {
     return code;
 }
 
+// j-tiles per work item: the largest of 16, 8 and 2 that still gives every SM
+// eight items (two waves of four CTAs), else 2.  At 16 x 1203 items of 16 leave
+// 1.6 CTAs an SM (energy and gradient 622 us, 435 with items of 2); past that
+// line the staging and atomics of smaller items cost more than they fill.
+int pick_chunk(const SView& g) {
+    long long items[3] = {0, 0, 0};
+    const int chunk[3] = {16, 8, 2};
+    for (int c = 0; c < 3; ++c) {
+        for (int t = 0; t < g.n_itile; ++t) items[c] += (g.n_jtile - t * (kGI / kGJ) + chunk[c] - 1) / chunk[c];
+        items[c] *= g.n_rep;
+        if (items[c] >= 152 * 8) return chunk[c];
+    }
+    return 2;
+}
+
 int setup(SView& g, int n_rep, int n, const float* x, const float* q, const float* rho,
           const float* screen, const cph_gb_params* gb, void* ws, size_t wsb) {
     if (n_rep < 1 || n < 1 || !x || !q || !rho || !screen || !gb || !ws)
@@ -98,7 +114,8 @@ int setup(SView& g, int n_rep, int n, const float* x, const float* q, const floa
     g.n = n;
     g.n_itile = (n + kGI - 1) / kGI;
     g.n_jtile = (n + kGJ - 1) / kGJ;
-    g.n_chunk = (g.n_jtile + kGChunk - 1) / kGChunk;
+    g.chunk = pick_chunk(g);
+    g.n_chunk = (g.n_jtile + g.chunk - 1) / g.chunk;
     g.x = x;
     g.q = q;
     g.rho = rho;
@@ -127,6 +144,13 @@ int setup(SView& g, int n_rep, int n, const float* x, const float* q, const floa
     return CPH_OK;
 }
 
+// calls f with the kernels' staged group: 8 j-tiles, or 2 for items of 2
+template <class F>
+void by_group(const SView& g, F&& f) {
+    if (g.chunk < kGG) f(std::integral_constant<int, 2>{});
+    else f(std::integral_constant<int, kGG>{});
+}
+
 // bound and Born radii, shared by both directions
 int launch_radii(SView& g, cudaStream_t st) {
     const size_t na = (size_t)g.n_rep * g.n;
@@ -136,8 +160,11 @@ int launch_radii(SView& g, cudaStream_t st) {
     const int ba = (int)((na + 255) / 256);
     const int grid = g.n_rep * g.n_itile * g.n_chunk;
     k_gbound<<<ba, 256, 0, st>>>(g);
-    if (g.rgbmax < INFINITY) k_gborn_sym<true><<<grid, kGT, 0, st>>>(g);
-    else k_gborn_sym<false><<<grid, kGT, 0, st>>>(g);
+    by_group(g, [&](auto gg) {
+        constexpr int GG = decltype(gg)::value;
+        if (g.rgbmax < INFINITY) k_gborn_sym<true, GG><<<grid, kGT, 0, st>>>(g);
+        else k_gborn_sym<false, GG><<<grid, kGT, 0, st>>>(g);
+    });
     k_gfin_born<<<ba, 256, 0, st>>>(g);
     return CPH_OK;
 }
@@ -161,8 +188,11 @@ extern "C" int cph_gb_energy(int n_rep, int n, const float* x, const float* q, c
     if (rc != CPH_OK) return rc;
     const size_t na = (size_t)n_rep * n;
     const int ba = (int)((na + 255) / 256);
-    if (g.kappa > 0) k_gpair_sym<false, true><<<n_rep * g.n_itile * g.n_chunk, kGT, 0, st>>>(g);
-    else k_gpair_sym<false, false><<<n_rep * g.n_itile * g.n_chunk, kGT, 0, st>>>(g);
+    by_group(g, [&](auto gg) {
+        constexpr int GG = decltype(gg)::value;
+        if (g.kappa > 0) k_gpair_sym<false, true, GG><<<n_rep * g.n_itile * g.n_chunk, kGT, 0, st>>>(g);
+        else k_gpair_sym<false, false, GG><<<n_rep * g.n_itile * g.n_chunk, kGT, 0, st>>>(g);
+    });
     k_gfin_c<false><<<ba, 256, 0, st>>>(g);
     k_genergy_out<<<(n_rep + 127) / 128, 128, 0, st>>>(g);
     cudaError_t ce = cudaGetLastError();
@@ -188,11 +218,14 @@ extern "C" int cph_gb_energy_backward(int n_rep, int n, const float* x, const fl
     const size_t na = (size_t)n_rep * n;
     const int ba = (int)((na + 255) / 256);
     const int grid = n_rep * g.n_itile * g.n_chunk;
-    if (g.kappa > 0) k_gpair_sym<true, true><<<grid, kGT, 0, st>>>(g);
-    else k_gpair_sym<true, false><<<grid, kGT, 0, st>>>(g);
-    k_gfin_c<true><<<ba, 256, 0, st>>>(g);
-    if (g.rgbmax < INFINITY) k_gchain_sym<true><<<grid, kGT, 0, st>>>(g);
-    else k_gchain_sym<false><<<grid, kGT, 0, st>>>(g);
+    by_group(g, [&](auto gg) {
+        constexpr int GG = decltype(gg)::value;
+        if (g.kappa > 0) k_gpair_sym<true, true, GG><<<grid, kGT, 0, st>>>(g);
+        else k_gpair_sym<true, false, GG><<<grid, kGT, 0, st>>>(g);
+        k_gfin_c<true><<<ba, 256, 0, st>>>(g);
+        if (g.rgbmax < INFINITY) k_gchain_sym<true, GG><<<grid, kGT, 0, st>>>(g);
+        else k_gchain_sym<false, GG><<<grid, kGT, 0, st>>>(g);
+    });
     k_gfin_out<<<ba, 256, 0, st>>>(g);
     cudaError_t ce = cudaGetLastError();
     if (ce != cudaSuccess) return gfail(CPH_E_CUDA, std::string("cph_gb_energy_backward: ") + cudaGetErrorString(ce));

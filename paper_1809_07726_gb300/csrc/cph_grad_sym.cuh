@@ -28,11 +28,10 @@ constexpr int kGT = 128;     // threads per CTA
 constexpr int kGI = 256;     // atoms per i-tile
 constexpr int kGJ = kTileJ;   // atoms per j-tile
 constexpr int kGG = 8;       // j-tiles staged per barrier (four tile pairs)
-constexpr int kGChunk = 16;  // j-tiles per work item
 constexpr float kFar = 1.0e4f; // padding / invalid atoms sit this far away
 
 struct SView {
-    int n_rep, n, n_itile, n_jtile, n_chunk;
+    int n_rep, n, n_itile, n_jtile, n_chunk, chunk; // chunk: j-tiles per work item
     const float *x, *q, *rho, *screen;
     double tau, sqrt_k, alpha, beta, gamma, offset;
     // Debye-Hueckel salt screening: kappa (1/A), 1/eps_in, 1/eps_out; tau_pair is
@@ -85,8 +84,8 @@ __device__ __forceinline__ GItem gitem(const SView& g) {
     const int rem = blockIdx.x % per_rep;
     const int ti = rem / g.n_chunk, ch = rem % g.n_chunk;
     it.i0 = ti * kGI;
-    it.jt0 = (it.i0 / kGJ) + ch * kGChunk;
-    it.jt1 = min(g.n_jtile, it.jt0 + kGChunk);
+    it.jt0 = (it.i0 / kGJ) + ch * g.chunk;
+    it.jt1 = min(g.n_jtile, it.jt0 + g.chunk);
     it.ok = it.jt0 < g.n_jtile;
     return it;
 }
@@ -109,10 +108,13 @@ __device__ __forceinline__ bool gmasked(int jt, int i0, int n) {
 }
 
 // ------------------------------------------------------------ Born radii
-template <bool CUT>
-__global__ void __launch_bounds__(kGT, 6) k_gborn_sym(SView g) {
-    __shared__ BoJs sj[kGG / 2];
-    __shared__ float red[kGG][4][kGJ];
+template <bool CUT, int GG>
+__global__ void __launch_bounds__(kGT, 5) k_gborn_sym(SView g) {
+    __shared__ BoJs sj[GG / 2];
+    __shared__ float red[GG][4][kGJ];
+    __shared__ uint16_t nearq[kGT / 32][kNearCap];
+    __shared__ long long ihx[kGI];     // the near pairs' sums (2^40 fixed point), i side
+    __shared__ long long jhx[GG][kGJ]; // and partner side, of the staged group
     const GItem it = gitem(g);
     if (!it.ok) return;
     const int n = g.n, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -138,10 +140,13 @@ __global__ void __launch_bounds__(kGT, 6) k_gborn_sym(SView g) {
         I[u].s = si;
         I[u].rt = rt;
         I[u].irt = 1.f / rt;
+        ihx[warp * 64 + u * 32 + lane] = 0;
     }
+    for (int q = tid; q < GG * kGJ; q += kGT) jhx[q / kGJ][q % kGJ] = 0;
+    int nq = 0; // this warp's waiting near pairs
     long long hx[2] = {0, 0};
-    for (int g0 = it.jt0; g0 < it.jt1; g0 += kGG) {
-        const int ng = min(kGG, it.jt1 - g0), npair = (ng + 1) >> 1;
+    for (int g0 = it.jt0; g0 < it.jt1; g0 += GG) {
+        const int ng = min(GG, it.jt1 - g0), npair = (ng + 1) >> 1;
         __syncthreads();
         // stage the tile pairs: thread (pair, copy, entry) writes whole rows
         for (int q = tid; q < npair * 2 * kGJ; q += kGT) {
@@ -168,7 +173,14 @@ __global__ void __launch_bounds__(kGT, 6) k_gborn_sym(SView g) {
             S.n[r] = make_float4(v[0][4], v[1][4], v[0][5], v[1][5]);
         }
         __syncthreads();
+        const int pr0 = live_pair(it.i0, warp, n, g0);
         for (int pr = 0; pr < npair; ++pr) {
+            if (pr < pr0) {
+                red[2 * pr][warp][lane] = 0.f;
+                red[2 * pr + 1][warp][lane] = 0.f;
+                continue;
+            }
+            NearBits nb = {};
             float2 jh = make_float2(0.f, 0.f);
             float2 ah[2] = {{0.f, 0.f}, {0.f, 0.f}};
             uint32_t sk[2][2] = {{0u, 0u}, {0u, 0u}};
@@ -182,25 +194,49 @@ __global__ void __launch_bounds__(kGT, 6) k_gborn_sym(SView g) {
                     for (int u = 0; u < 2; ++u) sk[u][h] = gskip(ii[u], vi[u], jt * kGJ, n);
                 }
             }
-            if (masked) born_tile<true, CUT>(sj[pr], lane, I, ah, jh, sk, band);
-            else born_tile<false, CUT>(sj[pr], lane, I, ah, jh, sk, band);
+            if (masked) born_tile<true, CUT>(sj[pr], lane, I, ah, jh, sk, band, nb);
+            else born_tile<false, CUT>(sj[pr], lane, I, ah, jh, sk, band, nb);
 #pragma unroll
             for (int u = 0; u < 2; ++u)
                 hx[u] += to_fixed(ah[u].x, (float)kScaleH) + to_fixed(ah[u].y, (float)kScaleH);
             red[2 * pr][warp][lane] = jh.x;
             red[2 * pr + 1][warp][lane] = jh.y;
+            near_drain(nb, nearq[warp], nq, lane, pr, pr == npair - 1, [&](uint32_t e, bool valid) {
+                const int l = e & 31u, jj = (e >> 7) & 31u, p = e >> 12;
+                const bool u = (e >> 5) & 1u, h = (e >> 6) & 1u;
+                auto of_i = [&](float a, float b) {
+                    a = __shfl_sync(0xffffffffu, a, l);
+                    b = __shfl_sync(0xffffffffu, b, l);
+                    return u ? b : a;
+                };
+                const float xi = of_i(I[0].x.x, I[1].x.x), yi = of_i(I[0].y.x, I[1].y.x), zi = of_i(I[0].z.x, I[1].z.x);
+                const float si = of_i(I[0].s, I[1].s), rti = of_i(I[0].rt, I[1].rt), irti = of_i(I[0].irt, I[1].irt);
+                const BoJs& S = sj[p];
+                const float4 A = S.a[jj], B = S.b[jj], C = S.c[jj], Nj = S.n[jj];
+                const float dx = xi + (h ? A.y : A.x), dy = yi + (h ? A.w : A.z), dz = zi + (h ? B.y : B.x);
+                const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+                const float2 hv = born_near(r2, rsqrt_ftz(r2), rti, irti, si, h ? C.w : C.z, h ? Nj.y : Nj.x,
+                                            h ? Nj.w : Nj.z, band.rc);
+                if (valid) {
+                    atomicAdd((unsigned long long*)&ihx[warp * 64 + u * 32 + l], (unsigned long long)to_fixed(hv.x, (float)kScaleH));
+                    atomicAdd((unsigned long long*)&jhx[2 * p + h][jj], (unsigned long long)to_fixed(hv.y, (float)kScaleH));
+                }
+            });
         }
         __syncthreads();
         for (int q = tid; q < ng * kGJ; q += kGT) {
             const int gt = q / kGJ, j = q % kGJ;
             const float v = red[gt][0][j] + red[gt][1][j] + red[gt][2][j] + red[gt][3][j];
             const int jg = g0 * kGJ + q;
-            if (jg < n) atomicAdd((unsigned long long*)&g.Hfix[base + jg], (unsigned long long)to_fixed(v, (float)kScaleH));
+            if (jg < n)
+                atomicAdd((unsigned long long*)&g.Hfix[base + jg],
+                          (unsigned long long)(to_fixed(v, (float)kScaleH) + jhx[gt][j]));
+            jhx[gt][j] = 0;
         }
     }
 #pragma unroll
     for (int u = 0; u < 2; ++u)
-        if (vi[u]) atomicAdd((unsigned long long*)&g.Hfix[base + ii[u]], (unsigned long long)hx[u]);
+        if (vi[u]) atomicAdd((unsigned long long*)&g.Hfix[base + ii[u]], (unsigned long long)(hx[u] + ihx[warp * 64 + u * 32 + lane]));
 }
 
 // psi, R (FP64); resets the fixed-point accumulators of the pair passes.
@@ -345,10 +381,10 @@ __device__ __forceinline__ void gpair_tile(const GpJs& sj, int lane, const GpI2 
     }
 }
 
-template <bool BACKWARD, bool SALT>
+template <bool BACKWARD, bool SALT, int GG>
 __global__ void __launch_bounds__(kGT, 5) k_gpair_sym(SView g) {
-    __shared__ GpJs sj[kGG / 2];
-    __shared__ float red[kGG][4][kGJ][5];
+    __shared__ GpJs sj[GG / 2];
+    __shared__ float red[GG][4][kGJ][5];
     __shared__ long long sfx[5][kGI]; // i-side sums, component-major (conflict-free)
     __shared__ double ered[kGT / 32];
     const GItem it = gitem(g);
@@ -377,8 +413,8 @@ __global__ void __launch_bounds__(kGT, 5) k_gpair_sym(SView g) {
         for (int c = 0; c < 5; ++c) sfx[c][warp * 64 + u * 32 + lane] = 0;
     }
     KSum<float> egb;
-    for (int g0 = it.jt0; g0 < it.jt1; g0 += kGG) {
-        const int ng = min(kGG, it.jt1 - g0), npair = (ng + 1) >> 1;
+    for (int g0 = it.jt0; g0 < it.jt1; g0 += GG) {
+        const int ng = min(GG, it.jt1 - g0), npair = (ng + 1) >> 1;
         __syncthreads();
         // stage the tile pairs: thread (pair, copy, entry) writes whole rows
         for (int q = tid; q < npair * 2 * kGJ; q += kGT) {
@@ -405,11 +441,22 @@ __global__ void __launch_bounds__(kGT, 5) k_gpair_sym(SView g) {
         __syncthreads();
         // i-side partials of the staged group in FP32 (tile pairs in turn, halves
         // = even / odd tiles), one fixed-point conversion per group; groups are
-        // aligned runs of kGG j-tiles, whatever the item's chunk
+        // aligned runs of GG j-tiles, whatever the item's chunk
         float2 ai[2][5];
 #pragma unroll
         for (int c = 0; c < 5; ++c) ai[0][c] = ai[1][c] = make_float2(0.f, 0.f);
+        // passing dead pairs by spills in the adjoint: measured faster only where the
+        // diagonal is most of the work (items of 2 j-tiles: 452 -> 435 us at
+        // 16 x 1203), slower in the large batch (21.37 -> 21.67 ms at 128 x 8000)
+        const int pr0 = (BACKWARD && GG > 2) ? 0 : live_pair(it.i0, warp, n, g0);
         for (int pr = 0; pr < npair; ++pr) {
+            if (pr < pr0) {
+                if (BACKWARD) {
+#pragma unroll
+                    for (int c = 0; c < 5; ++c) red[2 * pr][warp][lane][c] = red[2 * pr + 1][warp][lane][c] = 0.f;
+                }
+                continue;
+            }
             float2 aj[5], ei[2] = {{0.f, 0.f}, {0.f, 0.f}};
 #pragma unroll
             for (int c = 0; c < 5; ++c) aj[c] = make_float2(0.f, 0.f);
@@ -553,8 +600,7 @@ struct GcNear {
 };
 
 // Closed forms of one pair inside r_far or in the cutoff band, out of line
-// (a warp only gets here when one of its lanes has such a pair): the gradient
-// factor t, dH/drt both ways, and the c-weighted dH/ds both ways.
+// (called where a warp's queued near pairs are evaluated): the gradient factor t, dH/drt both ways, and the c-weighted dH/ds both ways.
 static __device__ __noinline__ GcNear gchain_near(float r2, float rinv, float ci, float rti, float irti, float si,
                                                   float cj, float sj, float rtj, float irtj, float rc) {
     const float r = r2 * rinv;
@@ -568,17 +614,15 @@ static __device__ __noinline__ GcNear gchain_near(float r2, float rinv, float ci
 }
 
 template <bool MASKED, bool CUT>
-__device__ __forceinline__ void gchain_tile(const GcJs& sj, int lane, const GcI2 (&I)[2], float2 (&ai)[2][5],
-                                            float2 (&aj)[5], const uint32_t (&sk)[2][2], const PairBand& band,
-                                            float* __restrict__ hti, float2* __restrict__ htj) {
+__device__ __forceinline__ void gchain_tile(const GcJs& sj, int lane, const GcI2 (&I)[2], float2 (&ai)[2][4],
+                                            float2 (&aj)[4], const uint32_t (&sk)[2][2], const PairBand& band,
+                                            NearBits& nb) {
     const int src = (lane + 1) & 31;
-    const float skr2 = band.skr2;
-    const float2 mone = splat<float2>(-1.f);
 #pragma unroll 2
     for (int k = 0; k < kGJ; ++k) {
         const float4 A = sj.a[lane + k], B = sj.b[lane + k], C = sj.c[lane + k];
         const float2 cj = make_float2(B.z, B.w), s2j = make_float2(C.x, C.y), s3j = make_float2(C.z, C.w);
-        float2 dx[2], dy[2], dz[2], r2[2], t[2], asi[2], asj[2], wt[2];
+        float2 dx[2], dy[2], dz[2], r2[2];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             dx[u] = __fadd2_rn(I[u].x, make_float2(A.x, A.y));
@@ -587,98 +631,53 @@ __device__ __forceinline__ void gchain_tile(const GcJs& sj, int lane, const GcI2
             r2[u] = __ffma2_rn(dx[u], dx[u], __ffma2_rn(dy[u], dy[u], __fmul2_rn(dz[u], dz[u])));
             if (MASKED) {
                 const int jj = (lane + k) & (kGJ - 1);
-                r2[u].x = ((sk[u][0] >> jj) & 1u) ? skr2 : r2[u].x;
-                r2[u].y = ((sk[u][1] >> jj) & 1u) ? skr2 : r2[u].y;
-            }
-            const float2 rinv2 = make_float2(rcp_ftz(r2[u].x), rcp_ftz(r2[u].y));
-            const float2 rinv4 = __fmul2_rn(rinv2, rinv2);
-            const float2 yj = __fmul2_rn(s2j, rinv2), yi = __fmul2_rn(I[u].s2, rinv2);
-            const float2 qj = hct_series_dr(yj), qi = hct_series_dr(yi);
-            // t = (c_i dH_i/dr + c_j dH_j/dr) / r = -(c_i s_j^3 Q_j + c_j s_i^3 Q_i) / r^6
-            const float2 term = __ffma2_rn(__fmul2_rn(I[u].c, s3j), qj, __fmul2_rn(__fmul2_rn(cj, I[u].s3), qi));
-            t[u] = __fmul2_rn(term, __fmul2_rn(__fmul2_rn(rinv4, rinv2), mone));
-            // c_j dH(r; rt_j, s_i)/ds = c_j s_i^2 S_i / r^4, and i <-> j, with r^-4 the
-            // weight of their fused accumulate (1 for closed forms, 0 if not counted)
-            asi[u] = __fmul2_rn(__fmul2_rn(cj, I[u].s2), hct_series_ds(yi));
-            asj[u] = __fmul2_rn(__fmul2_rn(I[u].c, s2j), hct_series_ds(yj));
-            wt[u] = rinv4;
-            if (CUT) { // beyond rc + s_max nothing descreens
-                const bool o0 = r2[u].x >= band.rout2, o1 = r2[u].y >= band.rout2;
-                t[u].x = o0 ? 0.f : t[u].x;
-                t[u].y = o1 ? 0.f : t[u].y;
-                wt[u].x = o0 ? 0.f : wt[u].x;
-                wt[u].y = o1 ? 0.f : wt[u].y;
+                r2[u].x = ((sk[u][0] >> jj) & 1u) ? INFINITY : r2[u].x;
+                r2[u].y = ((sk[u][1] >> jj) & 1u) ? INFINITY : r2[u].y;
             }
         }
-        // closed forms only where some lane has such a pair (rare; skipped
-        // pairs never get here, and dH/drt is zero in the far regime, so only
-        // this branch adds to the rt sums)
-        const bool nr = band_near<CUT>(r2[0].x, band) || band_near<CUT>(r2[0].y, band) ||
-                        band_near<CUT>(r2[1].x, band) || band_near<CUT>(r2[1].y, band);
-        if (__any_sync(0xffffffffu, nr)) {
-            const float4 Nj = sj.n[lane + k];
-            const float2 Mj = sj.m[lane + k];
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                if (band_near<CUT>(r2[u].x, band)) {
-                    const GcNear o = gchain_near(r2[u].x, rsqrt_ftz(r2[u].x), I[u].c.x, I[u].rt, I[u].irt,
-                                                 I[u].s, B.z, Nj.x, Nj.z, Mj.x, band.rc);
-                    t[u].x = o.t;
-                    hti[u * 32] += o.hti;
-                    htj[(lane + k) & (kGJ - 1)].x += o.htj;
-                    asi[u].x = o.asi;
-                    asj[u].x = o.asj;
-                    wt[u].x = 1.f;
-                }
-                if (band_near<CUT>(r2[u].y, band)) {
-                    const GcNear o = gchain_near(r2[u].y, rsqrt_ftz(r2[u].y), I[u].c.x, I[u].rt, I[u].irt,
-                                                 I[u].s, B.w, Nj.y, Nj.w, Mj.y, band.rc);
-                    t[u].y = o.t;
-                    hti[u * 32] += o.hti;
-                    htj[(lane + k) & (kGJ - 1)].y += o.htj;
-                    asi[u].y = o.asi;
-                    asj[u].y = o.asj;
-                    wt[u].y = 1.f;
-                }
-            }
-        }
+        note_near<CUT>(r2, band, k, nb);
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-            if (MASKED) {
-                const int jj = (lane + k) & (kGJ - 1);
-                const bool s0 = (sk[u][0] >> jj) & 1u, s1 = (sk[u][1] >> jj) & 1u;
-                t[u].x = s0 ? 0.f : t[u].x;
-                t[u].y = s1 ? 0.f : t[u].y;
-                wt[u].x = s0 ? 0.f : wt[u].x;
-                wt[u].y = s1 ? 0.f : wt[u].y;
+            const float2 rinv2 = make_float2(rcp_ftz(r2[u].x), rcp_ftz(r2[u].y));
+            float2 wt = __fmul2_rn(rinv2, rinv2); // r^-4, the weight of every far term
+            if (CUT) { // beyond rc + s_max nothing descreens
+                wt.x = r2[u].x >= band.rout2 ? 0.f : wt.x;
+                wt.y = r2[u].y >= band.rout2 ? 0.f : wt.y;
             }
-            ai[u][0] = __ffma2_rn(t[u], dx[u], ai[u][0]);
-            ai[u][1] = __ffma2_rn(t[u], dy[u], ai[u][1]);
-            ai[u][2] = __ffma2_rn(t[u], dz[u], ai[u][2]);
-            aj[0] = __ffma2_rn(t[u], dx[u], aj[0]); // the partner's gradient is minus this sum
-            aj[1] = __ffma2_rn(t[u], dy[u], aj[1]);
-            aj[2] = __ffma2_rn(t[u], dz[u], aj[2]);
-            ai[u][4] = __ffma2_rn(asi[u], wt[u], ai[u][4]);
-            aj[4] = __ffma2_rn(asj[u], wt[u], aj[4]);
+            const float2 yj = __fmul2_rn(s2j, rinv2), yi = __fmul2_rn(I[u].s2, rinv2);
+            const float2 qj = hct_series_dr(yj), qi = hct_series_dr(yi);
+            // t = -(c_i dH_i/dr + c_j dH_j/dr) / r = (c_i s_j^3 Q_j + c_j s_i^3 Q_i) / r^6 (the
+            // sums below take its negative)
+            const float2 term = __ffma2_rn(__fmul2_rn(I[u].c, s3j), qj, __fmul2_rn(__fmul2_rn(cj, I[u].s3), qi));
+            const float2 t = __fmul2_rn(term, __fmul2_rn(wt, rinv2));
+            // c_j dH(r; rt_j, s_i)/ds = c_j s_i^2 S_i / r^4, and i <-> j
+            const float2 asi = __fmul2_rn(__fmul2_rn(cj, I[u].s2), hct_series_ds(yi));
+            const float2 asj = __fmul2_rn(__fmul2_rn(I[u].c, s2j), hct_series_ds(yj));
+            ai[u][0] = __ffma2_rn(t, dx[u], ai[u][0]); // minus the i atom's gradient, and the partner's
+            ai[u][1] = __ffma2_rn(t, dy[u], ai[u][1]);
+            ai[u][2] = __ffma2_rn(t, dz[u], ai[u][2]);
+            aj[0] = __ffma2_rn(t, dx[u], aj[0]);
+            aj[1] = __ffma2_rn(t, dy[u], aj[1]);
+            aj[2] = __ffma2_rn(t, dz[u], aj[2]);
+            ai[u][3] = __ffma2_rn(asi, wt, ai[u][3]);
+            aj[3] = __ffma2_rn(asj, wt, aj[3]);
         }
 #pragma unroll
-        for (int c = 0; c < 5; ++c) {
-            if (c == 3) continue; // dH/drt partials are kept in shared memory (closed forms only)
+        for (int c = 0; c < 4; ++c) {
             aj[c].x = __shfl_sync(0xffffffffu, aj[c].x, src);
             aj[c].y = __shfl_sync(0xffffffffu, aj[c].y, src);
         }
     }
 }
 
-template <bool CUT>
+template <bool CUT, int GG>
 __global__ void __launch_bounds__(kGT, 4) k_gchain_sym(SView g) {
-    __shared__ GcJs sj[kGG / 2];
-    __shared__ float red[kGG][4][kGJ][5];
+    __shared__ GcJs sj[GG / 2];
+    __shared__ float red[GG][4][kGJ][5];
     __shared__ long long sfx[5][kGI]; // i-side sums, component-major (conflict-free)
-    // dH/drt sums, which only the rare closed-form pairs feed: i side per
-    // thread and atom over a staged group, partner side per warp and tile pair
-    __shared__ float hti_s[kGI];
-    __shared__ float2 htj_s[kGT / 32][kGJ];
+    // near pairs: the warps' queues, and the i-side sums of the staged group
+    __shared__ uint16_t nearq[kGT / 32][kNearCap];
+    __shared__ float inear[5][kGI];
     const GItem it = gitem(g);
     if (!it.ok) return;
     const int n = g.n, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -708,8 +707,9 @@ __global__ void __launch_bounds__(kGT, 4) k_gchain_sym(SView g) {
 #pragma unroll
         for (int c = 0; c < 5; ++c) sfx[c][warp * 64 + u * 32 + lane] = 0;
     }
-    for (int g0 = it.jt0; g0 < it.jt1; g0 += kGG) {
-        const int ng = min(kGG, it.jt1 - g0), npair = (ng + 1) >> 1;
+    int nq = 0; // this warp's waiting near pairs
+    for (int g0 = it.jt0; g0 < it.jt1; g0 += GG) {
+        const int ng = min(GG, it.jt1 - g0), npair = (ng + 1) >> 1;
         __syncthreads();
         // stage the tile pairs: thread (pair, copy, entry) writes whole rows
         for (int q = tid; q < npair * 2 * kGJ; q += kGT) {
@@ -738,17 +738,22 @@ __global__ void __launch_bounds__(kGT, 4) k_gchain_sym(SView g) {
         }
         __syncthreads();
         // i-side partials of the staged group in FP32, one conversion per group
-        float2 ai[2][5];
+        float2 ai[2][4];
 #pragma unroll
-        for (int c = 0; c < 5; ++c) ai[0][c] = ai[1][c] = make_float2(0.f, 0.f);
-        hti_s[warp * 64 + lane] = 0.f;
-        hti_s[warp * 64 + 32 + lane] = 0.f;
+        for (int c = 0; c < 4; ++c) ai[0][c] = ai[1][c] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int c = 0; c < 5; ++c) inear[c][warp * 64 + lane] = inear[c][warp * 64 + 32 + lane] = 0.f;
+        const int pr0 = live_pair(it.i0, warp, n, g0);
         for (int pr = 0; pr < npair; ++pr) {
-            float2 aj[5];
+            if (pr < pr0) {
 #pragma unroll
-            for (int c = 0; c < 5; ++c) aj[c] = make_float2(0.f, 0.f);
-            htj_s[warp][lane] = make_float2(0.f, 0.f);
-            __syncwarp();
+                for (int c = 0; c < 5; ++c) red[2 * pr][warp][lane][c] = red[2 * pr + 1][warp][lane][c] = 0.f;
+                continue;
+            }
+            NearBits nb = {};
+            float2 aj[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) aj[c] = make_float2(0.f, 0.f);
             uint32_t sk[2][2] = {{0u, 0u}, {0u, 0u}};
             bool masked = false;
 #pragma unroll
@@ -760,23 +765,63 @@ __global__ void __launch_bounds__(kGT, 4) k_gchain_sym(SView g) {
                     for (int u = 0; u < 2; ++u) sk[u][h] = gskip(ii[u], vi[u], jt * kGJ, n);
                 }
             }
-            if (masked) gchain_tile<true, CUT>(sj[pr], lane, I, ai, aj, sk, band, &hti_s[warp * 64 + lane], htj_s[warp]);
-            else gchain_tile<false, CUT>(sj[pr], lane, I, ai, aj, sk, band, &hti_s[warp * 64 + lane], htj_s[warp]);
-            __syncwarp();
-            aj[3] = htj_s[warp][lane]; // lane l: partner l of both tiles
+            if (masked) gchain_tile<true, CUT>(sj[pr], lane, I, ai, aj, sk, band, nb);
+            else gchain_tile<false, CUT>(sj[pr], lane, I, ai, aj, sk, band, nb);
+            // component 3: dH/drt, which only near pairs have; 4: the weighted dH/ds
+            float(&ra)[5] = red[2 * pr][warp][lane];
+            float(&rb)[5] = red[2 * pr + 1][warp][lane];
 #pragma unroll
-            for (int c = 0; c < 5; ++c) {
-                const float sgn = c < 3 ? -1.f : 1.f;
-                red[2 * pr][warp][lane][c] = sgn * aj[c].x;
-                red[2 * pr + 1][warp][lane][c] = sgn * aj[c].y;
+            for (int c = 0; c < 3; ++c) {
+                ra[c] = aj[c].x;
+                rb[c] = aj[c].y;
             }
+            ra[3] = rb[3] = 0.f;
+            ra[4] = aj[3].x;
+            rb[4] = aj[3].y;
+            near_drain(nb, nearq[warp], nq, lane, pr, pr == npair - 1, [&](uint32_t e, bool valid) {
+                const int l = e & 31u, jj = (e >> 7) & 31u, p = e >> 12;
+                const bool u = (e >> 5) & 1u, h = (e >> 6) & 1u;
+                auto of_i = [&](float a, float b) {
+                    a = __shfl_sync(0xffffffffu, a, l);
+                    b = __shfl_sync(0xffffffffu, b, l);
+                    return u ? b : a;
+                };
+                const float xi = of_i(I[0].x.x, I[1].x.x), yi = of_i(I[0].y.x, I[1].y.x), zi = of_i(I[0].z.x, I[1].z.x);
+                const float ci = of_i(I[0].c.x, I[1].c.x), si = of_i(I[0].s, I[1].s), rti = of_i(I[0].rt, I[1].rt),
+                            irti = of_i(I[0].irt, I[1].irt);
+                const GcJs& S = sj[p];
+                const float4 A = S.a[jj], B = S.b[jj], Nj = S.n[jj];
+                const float2 Mj = S.m[jj];
+                const float dx = xi + (h ? A.y : A.x), dy = yi + (h ? A.w : A.z), dz = zi + (h ? B.y : B.x);
+                const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+                const GcNear o = gchain_near(r2, rsqrt_ftz(r2), ci, rti, irti, si, h ? B.w : B.z, h ? Nj.y : Nj.x,
+                                             h ? Nj.w : Nj.z, h ? Mj.y : Mj.x, band.rc);
+                const int row = warp * 64 + u * 32 + l;
+                in_turn(u * 32 + l, valid, lane, [&] {
+                    inear[0][row] += o.t * dx;
+                    inear[1][row] += o.t * dy;
+                    inear[2][row] += o.t * dz;
+                    inear[3][row] += o.hti;
+                    inear[4][row] += o.asi;
+                });
+                float(&r)[5] = red[2 * p + h][warp][jj];
+                in_turn(p * 64 + h * 32 + jj, valid, lane, [&] {
+                    r[0] -= o.t * dx;
+                    r[1] -= o.t * dy;
+                    r[2] -= o.t * dz;
+                    r[3] += o.htj;
+                    r[4] += o.asj;
+                });
+            });
         }
+        __syncwarp();
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             const int row = warp * 64 + u * 32 + lane;
-            ai[u][3] = make_float2(hti_s[row], 0.f);
 #pragma unroll
-            for (int c = 0; c < 5; ++c) sfx[c][row] += to_fixed(ai[u][c].x + ai[u][c].y, (float)kScaleE);
+            for (int c = 0; c < 3; ++c) sfx[c][row] += to_fixed(inear[c][row] - (ai[u][c].x + ai[u][c].y), (float)kScaleE);
+            sfx[3][row] += to_fixed(inear[3][row], (float)kScaleE);
+            sfx[4][row] += to_fixed(inear[4][row] + (ai[u][3].x + ai[u][3].y), (float)kScaleE);
         }
         __syncthreads();
         for (int v = tid; v < ng * kGJ * 5; v += kGT) {

@@ -9,6 +9,7 @@
 #include <numeric>
 #include <set>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -54,12 +55,6 @@ __device__ __forceinline__ Real mc_pair(Real dx, Real dy, Real dz, Real Rm, Real
     return (excluded ? Real(0) : iei * rinv) - tf * fi;
 }
 
-template <class Real>
-__device__ __forceinline__ Real mc_const(double d, float f) {
-    if constexpr (sizeof(Real) == 4) return f;
-    else return d;
-}
-
 __device__ inline bool mc_excluded(const View& V, int P, int at, int an) {
     for (int e = V.excl_off[P + at]; e < V.excl_off[P + at + 1]; ++e)
         if (V.excl_j[e] == an) return true;
@@ -87,9 +82,9 @@ __global__ void __launch_bounds__(kMcThreads) k_mc_site(View V, int kind, int s_
     __shared__ double redd[kMcThreads / 32];
     const double cx = V.x[3 * A], cy = V.x[3 * A + 1], cz = V.x[3 * A + 2];
     // FP32: the host-rounded copies (no double -> float conversion in the loops)
-    const Real sqk = mc_const<Real>(V.sqrt_k, V.sqk32), tau = mc_const<Real>(V.tau, V.tau32),
-               iei = mc_const<Real>(V.inv_eps_in, V.iei32);
-    const Real kap = mc_const<Real>(V.kappa, V.kappa32), ieo = mc_const<Real>(V.inv_eps_out, V.ieo32);
+    const Real sqk = host_const<Real>(V.sqrt_k, V.sqk32), tau = host_const<Real>(V.tau, V.tau32),
+               iei = host_const<Real>(V.inv_eps_in, V.iei32);
+    const Real kap = host_const<Real>(V.kappa, V.kappa32), ieo = host_const<Real>(V.inv_eps_out, V.ieo32);
     const bool salt = V.kappa > 0;
     const int nat = V.site_nat[g], nst = V.site_nst[g], ao = V.site_aoff[g], qo = V.site_qoff[g];
     if (tid == 0) {
@@ -128,12 +123,11 @@ __global__ void __launch_bounds__(kMcThreads) k_mc_site(View V, int kind, int s_
         }
         Pr::add(lin, part, Real(kScaleE));
     };
-    if (sizeof(Real) == 4 && !V.sys_ordered[s]) {
-        // FP32 on the symmetric tiles: the partners from the step's staged FP32
-        // operands (positions relative to the walker's first atom from the
-        // Born-radii pass; sqrt(k) q and R staged again just before this
-        // sweep), with no FP64 subtraction or conversion per partner (both
-        // issue to the narrow FP64 pipe)
+    if (sizeof(Real) == 4) {
+        // FP32: the partners from the step's staged FP32 operands (positions
+        // relative to the walker's first atom; sqrt(k) q and R at the charges of
+        // this sweep's start), with no FP64 subtraction or conversion per partner
+        // (both issue to the narrow FP64 pipe)
         for (int j = tid; j < N; j += kMcThreads) {
             const float4 p = V.xs[A + j], gj = V.gq[A + j];
             linear_j(j, Real(p.x), Real(p.y), Real(p.z), Real(gj.x), Real(gj.y));
@@ -150,26 +144,14 @@ __global__ void __launch_bounds__(kMcThreads) k_mc_site(View V, int kind, int s_
     // FP64 mode in FP64 from the master positions.
     double corr = 0.0;
     if (sizeof(Real) == 4) {
-        const bool staged = !V.sys_ordered[s];
         for (int idx = tid; idx < nat * nat + nat; idx += kMcThreads) {
             Real term = 0;
             if (idx >= nat * nat) {
                 const int m = idx - nat * nat, at = mat[m];
                 for (int e = V.excl_off[P + at]; e < V.excl_off[P + at + 1]; ++e) {
                     const int j = V.excl_j[e];
-                    Real xj, yj, zj, qj;
-                    if (staged) {
-                        const float4 p = V.xs[A + j];
-                        xj = Real(p.x);
-                        yj = Real(p.y);
-                        zj = Real(p.z);
-                        qj = Real(V.gq[A + j].x);
-                    } else {
-                        xj = Real(V.x[3 * (A + j)] - cx);
-                        yj = Real(V.x[3 * (A + j) + 1] - cy);
-                        zj = Real(V.x[3 * (A + j) + 2] - cz);
-                        qj = Real(V.q[A + j]) * sqk;
-                    }
+                    const float4 p = V.xs[A + j];
+                    const Real xj = Real(p.x), yj = Real(p.y), zj = Real(p.z), qj = Real(V.gq[A + j].x);
                     const Real d0 = mx[m] - xj, d1 = my[m] - yj, d2 = mz[m] - zj;
                     term -= mdq[m] * qj * iei * Pr::rsqrt(d0 * d0 + d1 * d1 + d2 * d2);
                 }
@@ -266,9 +248,9 @@ __global__ void __launch_bounds__(kMcThreads) k_mc_sweep(View V, int kind, int c
     __shared__ double redd[kMcThreads / 32];
     const double cx = V.x[3 * A], cy = V.x[3 * A + 1], cz = V.x[3 * A + 2];
     // FP32: the host-rounded copies (no double -> float conversion in the loops)
-    const Real sqk = mc_const<Real>(V.sqrt_k, V.sqk32), tau = mc_const<Real>(V.tau, V.tau32),
-               iei = mc_const<Real>(V.inv_eps_in, V.iei32);
-    const Real kap = mc_const<Real>(V.kappa, V.kappa32), ieo = mc_const<Real>(V.inv_eps_out, V.ieo32);
+    const Real sqk = host_const<Real>(V.sqrt_k, V.sqk32), tau = host_const<Real>(V.tau, V.tau32),
+               iei = host_const<Real>(V.inv_eps_in, V.iei32);
+    const Real kap = host_const<Real>(V.kappa, V.kappa32), ieo = host_const<Real>(V.inv_eps_out, V.ieo32);
     const bool salt = V.kappa > 0;
     int n_taken = 0; // sites of this sweep accepted so far (uniform across the CTA)
     for (int k = 0; k < ns; ++k) {
@@ -656,6 +638,12 @@ struct cph_engine {
     std::vector<int> h_sys_shape;  // CPH_SHAPE_* per system (FP32 mode)
     int* d_sys_ordered = nullptr;  // 1 where a system runs the ordered passes
     int ordered_wpa = 1;           // warps per atom of the ordered passes (1 or 4)
+    // FP32 ordered passes read the operands staged once per step.  Not with
+    // constraints: hydrogens at fixed lengths amplify a change of rounding (100
+    // steps of the 246-atom peptide turned 1e-7 in the forces into 5e-5 in the
+    // velocities), so constrained runs keep every rounding they had: operands
+    // from the master arrays, undivided work items, near pairs in line.
+    bool staged = true;
     std::vector<int> h_w_local;    // 1 for the walkers this engine advances
     int* d_w_local = nullptr;
     bool sharded = false;          // some walker is not local
@@ -664,6 +652,8 @@ struct cph_engine {
     SymItem* d_sym_by_w = nullptr;     // grouped by walker (per-replica mode)
     int n_sym = 0;
     int sym_chunk = kSymChunk;         // j-tiles per symmetric work item (autotuned)
+    int sym_split = 1;                 // CTAs that share a symmetric work item (1, or 4 on small grids)
+    bool queue_near = true;            // near pairs of the symmetric chain pass: queued, or in line
     int max_sites = 0;                 // largest site count of any system
     int max_terms = 0;                 // largest bonds + angles count of any system
     std::vector<int> sym_w_off, h_sys_sst_off, h_sys_st_off;
@@ -766,45 +756,50 @@ bool sys_ordered(const cph_engine* E, int s) {
 // The ordered passes run one warp per atom (four atoms per CTA), or, in FP64
 // mode with few atoms (E->ordered_wpa = 4), four warps per atom: even a single
 // small walker then spreads its FP64 work over one CTA per atom.
-template <class Real, int WPA>
-void born_t(const Item* items, int n, View V, int ze, cudaStream_t st) {
-    k_born<Real, WPA><<<n, kTile, 0, st>>>(items, V, ze);
-}
-template <class Real, int WPA>
-void gb_t(const Item* items, int n, View V, bool energy, cudaStream_t st) {
-    if (energy) k_gb<Real, true, WPA><<<n, kTile, 0, st>>>(items, V);
-    else k_gb<Real, false, WPA><<<n, kTile, 0, st>>>(items, V);
-}
-template <class Real, int WPA>
-void chain_t(const Item* items, int n, View V, bool energy, cudaStream_t st) {
-    if (energy) k_chain<Real, true, WPA><<<n, kTile, 0, st>>>(items, V);
-    else k_chain<Real, false, WPA><<<n, kTile, 0, st>>>(items, V);
+// f with the passes' precision, warps per atom and operand source: FP64 (one
+// or four warps), FP32 from the staged operands or from the master arrays (one)
+template <class F>
+void by_form(const cph_engine* E, F&& f) {
+    using One = std::integral_constant<int, 1>;
+    using Four = std::integral_constant<int, 4>;
+    if (E->precision == CPH_PREC_FP64) {
+        if (E->ordered_wpa == 4) f(double{}, Four{}, std::false_type{});
+        else f(double{}, One{}, std::false_type{});
+    } else if (E->staged) f(float{}, One{}, std::true_type{});
+    else f(float{}, One{}, std::false_type{});
 }
 
 int launch_born(cph_engine* E, const Item* items, int n, bool zero_energy, cudaStream_t st) {
     if (n <= 0) return CPH_OK;
-    const bool f32 = E->precision == CPH_PREC_FP32, w4 = E->ordered_wpa == 4;
-    const int ze = zero_energy ? 1 : 0;
-    if (f32) (w4 ? born_t<float, 4> : born_t<float, 1>)(items, n, E->V, ze, st);
-    else (w4 ? born_t<double, 4> : born_t<double, 1>)(items, n, E->V, ze, st);
+    by_form(E, [&](auto real, auto wpa, auto staged) {
+        k_born<decltype(real), decltype(wpa)::value, decltype(staged)::value><<<n, kTile, 0, st>>>(items, E->V, zero_energy ? 1 : 0);
+    });
     CK(cudaGetLastError());
     return CPH_OK;
 }
 
 int launch_gb(cph_engine* E, const Item* items, int n, bool energy, cudaStream_t st) {
     if (n <= 0) return CPH_OK;
-    const bool f32 = E->precision == CPH_PREC_FP32, w4 = E->ordered_wpa == 4;
-    if (f32) (w4 ? gb_t<float, 4> : gb_t<float, 1>)(items, n, E->V, energy, st);
-    else (w4 ? gb_t<double, 4> : gb_t<double, 1>)(items, n, E->V, energy, st);
+    by_form(E, [&](auto real, auto wpa, auto staged) {
+        using R = decltype(real);
+        constexpr int WPA = decltype(wpa)::value;
+        constexpr bool ST = decltype(staged)::value;
+        if (energy) k_gb<R, true, WPA, ST><<<n, kTile, 0, st>>>(items, E->V);
+        else k_gb<R, false, WPA, ST><<<n, kTile, 0, st>>>(items, E->V);
+    });
     CK(cudaGetLastError());
     return CPH_OK;
 }
 
 int launch_chain(cph_engine* E, const Item* items, int n, bool energy, cudaStream_t st) {
     if (n <= 0) return CPH_OK;
-    const bool f32 = E->precision == CPH_PREC_FP32, w4 = E->ordered_wpa == 4;
-    if (f32) (w4 ? chain_t<float, 4> : chain_t<float, 1>)(items, n, E->V, energy, st);
-    else (w4 ? chain_t<double, 4> : chain_t<double, 1>)(items, n, E->V, energy, st);
+    by_form(E, [&](auto real, auto wpa, auto staged) {
+        using R = decltype(real);
+        constexpr int WPA = decltype(wpa)::value;
+        constexpr bool ST = decltype(staged)::value;
+        if (energy) k_chain<R, true, WPA, ST><<<n, kTile, 0, st>>>(items, E->V);
+        else k_chain<R, false, WPA, ST><<<n, kTile, 0, st>>>(items, E->V);
+    });
     CK(cudaGetLastError());
     return CPH_OK;
 }
@@ -846,10 +841,13 @@ int launch_mc(cph_engine* E, int kinds, int s_off, cudaStream_t st) {
         if (!(kinds & bit)) continue;
         if (E->max_sites <= 0) break;
         const bool f32 = E->precision == CPH_PREC_FP32;
-        // the per-site kernel reads sqrt(k) q and R from the FP32 staging of the
-        // symmetric tiles: stage them at this sweep's charges
+        // the per-site kernel reads sqrt(k) q and R from the FP32 staging, which the
+        // Born-radii pass wrote: stage them again at a second sweep's charges
+        const bool again = f32 && !first;
+        const bool first_x = f32 && first && !(E->staged || E->n_sym > 0); // no pass staged the positions
         if (E->launch_mode == 0) {
-            if (f32 && E->n_sym > 0) TRY(launch_stage(E, 1, 0, E->V.total_atoms, st));
+            if (first_x) TRY(launch_stage(E, 0, 0, E->V.total_atoms, st));
+            if (again) TRY(launch_stage(E, 1, 0, E->V.total_atoms, st));
             const dim3 g1(E->max_sites, W);
             if (f32) k_mc_site<float><<<g1, kMcThreads, 0, st>>>(E->V, kind, s_off, 0);
             else k_mc_site<double><<<g1, kMcThreads, 0, st>>>(E->V, kind, s_off, 0);
@@ -860,8 +858,8 @@ int launch_mc(cph_engine* E, int kinds, int s_off, cudaStream_t st) {
             for (int w = 0; w < W; ++w) {
                 if (!E->h_w_local[w]) continue;
                 cudaStream_t s = lane_stream(E, w, st);
-                if (f32 && !sys_ordered(E, E->h_w_sys[w]))
-                    TRY(launch_stage(E, 1, E->h_w_off[w], E->h_w_off[w + 1] - E->h_w_off[w], s));
+                if (first_x) TRY(launch_stage(E, 0, E->h_w_off[w], E->h_w_off[w + 1] - E->h_w_off[w], s));
+                if (again) TRY(launch_stage(E, 1, E->h_w_off[w], E->h_w_off[w + 1] - E->h_w_off[w], s));
                 if (f32) k_mc_site<float><<<E->max_sites, kMcThreads, 0, s>>>(E->V, kind, s_off, w);
                 else k_mc_site<double><<<E->max_sites, kMcThreads, 0, s>>>(E->V, kind, s_off, w);
                 if (f32) k_mc_sweep<float><<<1, kMcThreads, 0, s>>>(E->V, kind, first, w);
@@ -881,29 +879,29 @@ int launch_mc(cph_engine* E, int kinds, int s_off, cudaStream_t st) {
 int launch_sym_pair(cph_engine* E, const SymItem* items, int n, bool energy, int pass,
                     cudaStream_t st) {
     if (n <= 0) return CPH_OK;
-    const bool cut = E->V.rgbmax < INFINITY;
-    if (pass == 0) {
-        if (cut) k_born_sym<true><<<n, kSymThreads, 0, st>>>(items, E->V);
-        else k_born_sym<false><<<n, kSymThreads, 0, st>>>(items, E->V);
-    } else if (pass == 2) {
-        if (cut) k_chain_sym<true><<<n, kSymThreads, 0, st>>>(items, E->V);
-        else k_chain_sym<false><<<n, kSymThreads, 0, st>>>(items, E->V);
-    }
-    else if (E->V.kappa > 0) {
-        if (energy) k_gb_sym<true, true><<<n, kSymThreads, 0, st>>>(items, E->V);
-        else k_gb_sym<false, true><<<n, kSymThreads, 0, st>>>(items, E->V);
-    } else if (energy) k_gb_sym<true, false><<<n, kSymThreads, 0, st>>>(items, E->V);
-    else k_gb_sym<false, false><<<n, kSymThreads, 0, st>>>(items, E->V);
+    const bool cut = E->V.rgbmax < INFINITY, salt = E->V.kappa > 0;
+    auto launch = [&](auto gg) {
+        constexpr int GG = decltype(gg)::value;
+        auto go = [&](auto kernel) { kernel<<<n, kSymThreads, 0, st>>>(items, E->V); };
+        if (pass == 0) go(cut ? k_born_sym<true, GG> : k_born_sym<false, GG>);
+        else if (pass == 2 && (GG < kSymG || E->queue_near)) go(cut ? k_chain_sym<true, GG, true> : k_chain_sym<false, GG, true>);
+        else if (pass == 2) go(cut ? k_chain_sym<true, kSymG, false> : k_chain_sym<false, kSymG, false>);
+        else if (salt) go(energy ? k_gb_sym<true, true, GG> : k_gb_sym<false, true, GG>);
+        else go(energy ? k_gb_sym<true, false, GG> : k_gb_sym<false, false, GG>);
+    };
+    if (E->sym_split == 1) launch(std::integral_constant<int, kSymG>{});
+    else launch(std::integral_constant<int, kSymG / 4>{});
     CK(cudaGetLastError());
     return CPH_OK;
 }
 
-// operand staging of the FP32 pair kernels: positions before the Born-radii
-// pass, charge and radius terms before the GB pass (after any MC sweep)
-int launch_stage(cph_engine* E, int pass, int a0, int n, cudaStream_t st) {
+// operand staging of the FP32 pair kernels: positions (which = 0) before the
+// Born-radii pass, charge and radius terms (1) after a sweep that changed charges
+// (the Born-radii pass itself writes them otherwise)
+int launch_stage(cph_engine* E, int which, int a0, int n, cudaStream_t st) {
     const int bs = 256, g = (n + bs - 1) / bs;
-    if (n <= 0 || pass == 2) return CPH_OK;
-    if (pass == 0) k_stage_x<<<g, bs, 0, st>>>(E->V, a0, n);
+    if (n <= 0) return CPH_OK;
+    if (which == 0) k_stage_x<<<g, bs, 0, st>>>(E->V, a0, n);
     else k_stage_gb<<<g, bs, 0, st>>>(E->V, a0, n);
     CK(cudaGetLastError());
     return CPH_OK;
@@ -944,8 +942,8 @@ int launch_pass(cph_engine* E, int pass, bool energy, cudaStream_t st) {
             return pass == 1 ? launch_gb(E, E->d_items, E->n_items, energy, st)
                              : launch_chain(E, E->d_items, E->n_items, energy, st);
         }
+        if (pass == 0 && (E->staged || E->n_sym > 0)) TRY(launch_stage(E, 0, 0, E->V.total_atoms, st));
         if (E->n_sym > 0) {
-            TRY(launch_stage(E, pass, 0, E->V.total_atoms, st));
             TRY(launch_sym_pair(E, E->d_sym, E->n_sym, energy, pass, st));
             if (pass == 2) TRY(launch_bonded(E, energy, 0, E->V.W, st));
             TRY(launch_atoms(E, fin, energy, 0, E->V.total_atoms, st));
@@ -963,11 +961,11 @@ int launch_pass(cph_engine* E, int pass, bool energy, cudaStream_t st) {
         const Item* it = E->d_items_by_w + E->item_w_off[w];
         const int ni = E->item_w_off[w + 1] - E->item_w_off[w];
         cudaStream_t s = lane_stream(E, w, st);
+        if (fp32 && pass == 0 && (E->staged || E->n_sym > 0)) TRY(launch_stage(E, 0, E->h_w_off[w], E->h_w_off[w + 1] - E->h_w_off[w], s));
         if (!fp32 || sys_ordered(E, E->h_w_sys[w])) {
             if (pass == 0) TRY(launch_born(E, it, ni, energy, s));
             else TRY(pass == 1 ? launch_gb(E, it, ni, energy, s) : launch_chain(E, it, ni, energy, s));
         } else {
-            TRY(launch_stage(E, pass, E->h_w_off[w], E->h_w_off[w + 1] - E->h_w_off[w], s));
             TRY(launch_sym_pair(E, E->d_sym_by_w + E->sym_w_off[w], E->sym_w_off[w + 1] - E->sym_w_off[w],
                                 energy, pass, s));
             if (pass == 2) TRY(launch_bonded(E, energy, w, 1, s));
@@ -980,7 +978,19 @@ int launch_pass(cph_engine* E, int pass, bool energy, cudaStream_t st) {
 int launch_forces(cph_engine* E, bool energy, cudaStream_t st, bool mc_between, int s_off,
                   int mc_kinds) {
     TRY(launch_pass(E, 0, energy, st));
-    if (mc_between && mc_kinds) TRY(launch_mc(E, mc_kinds, s_off, st));
+    if (mc_between && mc_kinds && E->max_sites > 0) {
+        TRY(launch_mc(E, mc_kinds, s_off, st));
+        if (E->precision == CPH_PREC_FP32) { // the sweeps changed charges
+            if (E->launch_mode == 0) TRY(launch_stage(E, 1, 0, E->V.total_atoms, st));
+            else {
+                TRY(fan_out(E, st));
+                for (int w = 0; w < E->V.W; ++w)
+                    if (E->h_w_local[w])
+                        TRY(launch_stage(E, 1, E->h_w_off[w], E->h_w_off[w + 1] - E->h_w_off[w], lane_stream(E, w, st)));
+                TRY(fan_in(E, st));
+            }
+        }
+    }
     TRY(launch_pass(E, 1, energy, st));
     TRY(launch_pass(E, 2, energy, st));
     return CPH_OK;
@@ -1111,10 +1121,12 @@ namespace {
 // per-system shape flags, and drops captured graphs (they hold the old item
 // pointers).
 int build_items(cph_engine* E, int chunk) {
-    // the pair passes sum i-side partials per aligned group of kSymG j-tiles:
-    // items must start and end on group boundaries (or at the row's end)
+    // the pair passes sum i-side partials per aligned group of kSymG j-tiles (2 of
+    // them where four CTAs share an item): items must start and end on group
+    // boundaries (or at the row's end)
     if (chunk < kSymG || chunk % kSymG != 0 || kSymI % (kSymG * kSymJ) != 0)
         return fail(E, CPH_E_INVALID, "work-item size %d is not a multiple of %d j-tiles", chunk, kSymG);
+    const int per = chunk / E->sym_split; // j-tiles per CTA
     const int W = E->V.W;
     std::vector<Item> oitems, o_by_w;
     std::vector<int> o_off(W + 1, 0);
@@ -1153,8 +1165,8 @@ int build_items(cph_engine* E, int chunk) {
         const int njt = (N + kSymJ - 1) / kSymJ;
         for (int it = 0; it * kSymI < N; ++it) {
             const int i0 = it * kSymI;
-            for (int jt = i0 / kSymJ; jt < njt; jt += chunk)
-                by_w.push_back(SymItem{w, i0, jt, std::min(njt, jt + chunk), E->h_sys_sst_off[s] + it, 0});
+            for (int jt = i0 / kSymJ; jt < njt; jt += per)
+                by_w.push_back(SymItem{w, i0, jt, std::min(njt, jt + per), E->h_sys_sst_off[s] + it, 0});
         }
         w_off[w + 1] = (int)by_w.size();
     }
@@ -1721,7 +1733,19 @@ int cph_init_system(const cph_system_desc* sys, int n_sys, const cph_grid_desc* 
         E->d_rows = drw;
         V.ex_rows = drw;
     }
-    TRY(build_items(E, kSymChunk));
+    {
+        // four CTAs share each item when the whole grid (local walkers or not,
+        // whatever its tile shapes) is too small for eight items of 8 j-tiles an SM
+        long long items = 0;
+        for (int w = 0; w < W; ++w) {
+            const int njt = (sys_n[w_sys[w]] + kSymJ - 1) / kSymJ;
+            for (int t = 0; t * (kSymI / kSymJ) < njt; ++t) items += (njt - t * (kSymI / kSymJ) + kSymG - 1) / kSymG;
+        }
+        E->staged = p->precision == CPH_PREC_FP32 && !p->shake;
+        E->sym_split = items < 152 * 8 && !p->shake ? 4 : 1;
+        E->queue_near = *std::max_element(sys_n.begin(), sys_n.end()) <= kQueueAtoms && !p->shake;
+    }
+    TRY(build_items(E, E->sym_split == 1 ? kSymChunk : kSymG));
 
     // reference energies of every (site, state)
     if (!site_np.empty()) {

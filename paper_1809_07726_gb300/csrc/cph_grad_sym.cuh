@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(kGT, 5) k_gborn_sym(SView g) {
             S.n[r] = make_float4(v[0][4], v[1][4], v[0][5], v[1][5]);
         }
         __syncthreads();
-        const int pr0 = live_pair(it.i0, warp, n, g0);
+        const int pr0 = live_pair(it.i0, warp, n, g0, npair);
         for (int pr = 0; pr < npair; ++pr) {
             if (pr < pr0) {
                 red[2 * pr][warp][lane] = 0.f;
@@ -448,7 +448,7 @@ __global__ void __launch_bounds__(kGT, 5) k_gpair_sym(SView g) {
         // passing dead pairs by spills in the adjoint: measured faster only where the
         // diagonal is most of the work (items of 2 j-tiles: 452 -> 435 us at
         // 16 x 1203), slower in the large batch (21.37 -> 21.67 ms at 128 x 8000)
-        const int pr0 = (BACKWARD && GG > 2) ? 0 : live_pair(it.i0, warp, n, g0);
+        const int pr0 = (BACKWARD && GG > 2) ? 0 : live_pair(it.i0, warp, n, g0, npair);
         for (int pr = 0; pr < npair; ++pr) {
             if (pr < pr0) {
                 if (BACKWARD) {
@@ -743,7 +743,7 @@ __global__ void __launch_bounds__(kGT, 4) k_gchain_sym(SView g) {
         for (int c = 0; c < 4; ++c) ai[0][c] = ai[1][c] = make_float2(0.f, 0.f);
 #pragma unroll
         for (int c = 0; c < 5; ++c) inear[c][warp * 64 + lane] = inear[c][warp * 64 + 32 + lane] = 0.f;
-        const int pr0 = live_pair(it.i0, warp, n, g0);
+        const int pr0 = live_pair(it.i0, warp, n, g0, npair);
         for (int pr = 0; pr < npair; ++pr) {
             if (pr < pr0) {
 #pragma unroll
@@ -798,17 +798,17 @@ __global__ void __launch_bounds__(kGT, 4) k_gchain_sym(SView g) {
                                              h ? Nj.w : Nj.z, h ? Mj.y : Mj.x, band.rc);
                 const int row = warp * 64 + u * 32 + l;
                 in_turn(u * 32 + l, valid, lane, [&] {
-                    inear[0][row] += o.t * dx;
-                    inear[1][row] += o.t * dy;
-                    inear[2][row] += o.t * dz;
+                    inear[0][row] = fmaf(o.t, dx, inear[0][row]);
+                    inear[1][row] = fmaf(o.t, dy, inear[1][row]);
+                    inear[2][row] = fmaf(o.t, dz, inear[2][row]);
                     inear[3][row] += o.hti;
                     inear[4][row] += o.asi;
                 });
                 float(&r)[5] = red[2 * p + h][warp][jj];
                 in_turn(p * 64 + h * 32 + jj, valid, lane, [&] {
-                    r[0] -= o.t * dx;
-                    r[1] -= o.t * dy;
-                    r[2] -= o.t * dz;
+                    r[0] = fmaf(-o.t, dx, r[0]);
+                    r[1] = fmaf(-o.t, dy, r[1]);
+                    r[2] = fmaf(-o.t, dz, r[2]);
                     r[3] += o.htj;
                     r[4] += o.asj;
                 });

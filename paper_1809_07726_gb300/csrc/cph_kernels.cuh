@@ -12,10 +12,10 @@
 // not depend on the launch shape (batched and per-replica launches agree bit
 // for bit) and no atomics are needed.  A warp per atom spreads even a
 // 160-atom walker over 40 CTAs (FP64 arithmetic is a small fraction of the
-// chip's, so it must run on every SM).  Positions are made relative to the
-// group's first atom in FP64 before any rounding.  With Real = float the
-// per-tile partials go into int64 fixed-point accumulators (scales 2^32 and
-// 2^40); with double everything is FP64.
+// chip's, so it must run on every SM).  With Real = float the operands come
+// staged in FP32 and the partials of eight tiles (32 pairs a lane, as many as a
+// tile pair of the symmetric passes sums) go into int64 fixed-point
+// accumulators (scales 2^32 and 2^40); with double everything is FP64.
 //
 // Tiles in which some atom i of the CTA meets itself or an excluded partner
 // are listed per (system, i-tile) at set-up; only those run the masked loop.
@@ -68,6 +68,79 @@ struct alignas(sizeof(Real) * 2) J2 {
     Real x, y;
 };
 
+// The (sqrt(k) q, R, 1/R, log2(e) / (4 R)) operand of the FP32 pair kernels.
+__device__ __forceinline__ float4 gb_operand(double q, double sqrt_k, double R) {
+    const float r = (float)R, ir = __frcp_rn(r);
+    return make_float4((float)(q * sqrt_k), r, ir, (0.25f * kLog2e) * ir);
+}
+
+// A constant of the engine in the kernel's precision: FP32 kernels take the
+// copy that the host rounded.
+template <class Real>
+__device__ __forceinline__ Real host_const(double d, float f) {
+    if constexpr (sizeof(Real) == 4) return f;
+    else return d;
+}
+
+// Where the ordered passes get an atom's operands from.  STAGED (FP32): the
+// arrays staged once per step (positions relative to the walker's first atom),
+// since every CTA reads every atom of its walker and each FP64 subtraction,
+// division or conversion holds a sub-partition's FP64 pipe for 64 clocks.
+// Else (FP64, and FP32 with constraints, see cph_engine::staged): the master
+// arrays, positions relative to the CTA's first atom.
+template <class Real, bool STAGED>
+struct Stage {
+    const View& V;
+    int A, P;
+    double cx, cy, cz;
+    __device__ __forceinline__ Stage(const View& v, int a, int p, int i0) : V(v), A(a), P(p) {
+        cx = V.x[3 * (A + i0)];
+        cy = V.x[3 * (A + i0) + 1];
+        cz = V.x[3 * (A + i0) + 2];
+    }
+    __device__ __forceinline__ J4<Real> position(int i) const {
+        return {Real(V.x[3 * (A + i)] - cx), Real(V.x[3 * (A + i) + 1] - cy), Real(V.x[3 * (A + i) + 2] - cz), Real(0)};
+    }
+    __device__ __forceinline__ J4<Real> gb(int i) const { // sqrt(k) q, R, 1/R
+        const double R = V.R[A + i];
+        return {Real(V.q[A + i]) * Real(V.sqrt_k), Real(R), Real(1.0 / R), Real(0)};
+    }
+    __device__ __forceinline__ J2<Real> lj(int i) const { // sigma / 2, sqrt(eps)
+        return {Real(V.sigh[P + i]), Real(V.sqe[P + i])};
+    }
+    __device__ __forceinline__ J2<Real> radii(int i) const { return {Real(V.sc[P + i]), Real(V.rt[P + i])}; } // s, rt
+    __device__ __forceinline__ Real weight(int i) const { return Real(V.c[A + i]); }
+    // whether tile jt ends a run of tiles whose partials are summed together
+    static __device__ __forceinline__ bool flush(int) { return true; }
+};
+
+template <>
+struct Stage<float, true> {
+    const View& V;
+    int A, P;
+    __device__ __forceinline__ Stage(const View& v, int a, int p, int) : V(v), A(a), P(p) {}
+    __device__ __forceinline__ J4<float> position(int i) const {
+        const float4 p = V.xs[A + i];
+        return {p.x, p.y, p.z, 0.f};
+    }
+    __device__ __forceinline__ J4<float> gb(int i) const {
+        const float4 g = V.gq[A + i];
+        return {g.x, g.y, g.z, 0.f};
+    }
+    __device__ __forceinline__ J2<float> lj(int i) const {
+        const float2 l = V.plj32[P + i];
+        return {l.x, l.y};
+    }
+    __device__ __forceinline__ J2<float> radii(int i) const {
+        const float4 r = V.pb32[P + i];
+        return {r.x, r.y};
+    }
+    __device__ __forceinline__ float weight(int i) const { return V.c32[A + i]; }
+    // eight tiles are summed in FP32 and converted once (a conversion issues to
+    // the narrow FP64 pipe too)
+    static __device__ __forceinline__ bool flush(int jt) { return (jt & 7) == 7; }
+};
+
 // Per-walker energy accumulators (fixed point 2^32): GB, Coulomb, LJ, bond, angle.
 constexpr int kEAcc = 5;
 
@@ -105,7 +178,7 @@ __device__ inline void tile_masks(const View& V, int P, int i, bool vi, int j0, 
 // ------------------------------------------------------------- pass 1: Born radii
 // psi_i = rt_i/2 sum_{j != i} H(r_ij, rt_i, s_j); R_i = 1/(1/rt_i - tanh(theta)/rho_i)
 // with theta = alpha psi - beta psi^2 + gamma psi^3, finalised in FP64.
-template <class Real, int WPA>
+template <class Real, int WPA, bool STAGED>
 __global__ void __launch_bounds__(kTile) k_born(const Item* __restrict__ items, View V,
                                                 int zero_energy) {
     using Pr = Prec<Real>;
@@ -122,18 +195,19 @@ __global__ void __launch_bounds__(kTile) k_born(const Item* __restrict__ items, 
         if (zero_energy && tid < kEAcc) V.eacc[w * kEAcc + tid] = 0;
         if (tid == kEAcc) V.vscale[w] = 1.0;
     }
-    const double cx = V.x[3 * (A + it.i0)], cy = V.x[3 * (A + it.i0) + 1],
-                 cz = V.x[3 * (A + it.i0) + 2];
+    const Stage<Real, STAGED> stage(V, A, P, it.i0);
     Real xi = Real(-kFarF), yi = Real(-kFarF), zi = Real(-kFarF), rti = Real(1);
     if (vi) {
-        xi = Real(V.x[3 * (A + i)] - cx);
-        yi = Real(V.x[3 * (A + i) + 1] - cy);
-        zi = Real(V.x[3 * (A + i) + 2] - cz);
-        rti = Real(V.rt[P + i]);
+        const J4<Real> p = stage.position(i);
+        xi = p.x;
+        yi = p.y;
+        zi = p.z;
+        rti = stage.radii(i).y;
     }
     const Real irti = Real(1) / rti;
     const Real rc = Real(V.rgbmax); // Born-radius cutoff (INFINITY = none)
     typename Pr::Acc acc = 0;
+    Real part = 0;
     int mp = V.mt_off[it.st];
     const int me = V.mt_off[it.st + 1];
     int next = mp < me ? V.mt_list[mp] : 0x7fffffff;
@@ -143,10 +217,8 @@ __global__ void __launch_bounds__(kTile) k_born(const Item* __restrict__ items, 
             const int j = j0 + tid;
             J4<Real> v;
             if (j < N) {
-                v.x = Real(V.x[3 * (A + j)] - cx);
-                v.y = Real(V.x[3 * (A + j) + 1] - cy);
-                v.z = Real(V.x[3 * (A + j) + 2] - cz);
-                v.w = Real(V.sc[P + j]);
+                v = stage.position(j);
+                v.w = stage.radii(j).x;
             } else {
                 v.x = v.y = v.z = Real(kFarF);
                 v.w = Real(0);
@@ -154,7 +226,6 @@ __global__ void __launch_bounds__(kTile) k_born(const Item* __restrict__ items, 
             sj[tid] = v;
         }
         __syncthreads();
-        Real part = 0;
         if (jt != next) {
 #pragma unroll
             for (int k = sub; k < kTile; k += 32 * WPA) {
@@ -180,8 +251,12 @@ __global__ void __launch_bounds__(kTile) k_born(const Item* __restrict__ items, 
                 part += self ? Real(0) : h;
             }
         }
-        Pr::add(acc, part, Real(kScaleH));
+        if (stage.flush(jt)) {
+            Pr::add(acc, part, Real(kScaleH));
+            part = 0;
+        }
     }
+    Pr::add(acc, part, Real(kScaleH));
     acc = group_total<WPA>(acc, gsh);
     if (vi && sub == 0) {
         const double sumH = Pr::value(acc, kScaleH);
@@ -191,6 +266,7 @@ __global__ void __launch_bounds__(kTile) k_born(const Item* __restrict__ items, 
         const double R = 1.0 / (V.irt[P + i] - th * irho);
         V.psi[A + i] = psi;
         V.R[A + i] = R;
+        if (sizeof(Real) == 4) V.gq[A + i] = gb_operand(V.q[A + i], V.sqrt_k, R);
         V.Ffix[3 * (A + i)] = 0;
         V.Ffix[3 * (A + i) + 1] = 0;
         V.Ffix[3 * (A + i) + 2] = 0;
@@ -202,7 +278,7 @@ __global__ void __launch_bounds__(kTile) k_born(const Item* __restrict__ items, 
 // ------------------------------------------- pass 2: GB + Coulomb + LJ pair pass
 // Owner i accumulates the direct force, dE_GB/dR_i and (optionally) its share
 // of the energies; the epilogue turns dE/dR_i into c_i = dE/dR_i dR_i/dpsi_i rt_i/2.
-template <class Real, bool ENERGY, int WPA>
+template <class Real, bool ENERGY, int WPA, bool STAGED>
 __global__ void __launch_bounds__(kTile) k_gb(const Item* __restrict__ items, View V) {
     using Pr = Prec<Real>;
     using Acc = typename Pr::Acc;
@@ -217,25 +293,28 @@ __global__ void __launch_bounds__(kTile) k_gb(const Item* __restrict__ items, Vi
     const int i = it.i0 + warp / WPA;
     __shared__ long long gsh[kTile / 32];
     const bool vi = i < N;
-    const Real sqk = Real(V.sqrt_k);
-    const double cx = V.x[3 * (A + it.i0)], cy = V.x[3 * (A + it.i0) + 1],
-                 cz = V.x[3 * (A + it.i0) + 2];
+    const Stage<Real, STAGED> stage(V, A, P, it.i0);
     Real xi = Real(-kFarF), yi = Real(-kFarF), zi = Real(-kFarF);
     Real qi = 0, Ri = 1, iRi = 1, sgi = 0, sei = 0;
     if (vi) {
-        xi = Real(V.x[3 * (A + i)] - cx);
-        yi = Real(V.x[3 * (A + i) + 1] - cy);
-        zi = Real(V.x[3 * (A + i) + 2] - cz);
-        qi = Real(V.q[A + i]) * sqk;
-        Ri = Real(V.R[A + i]);
-        iRi = Real(1.0 / V.R[A + i]);
-        sgi = Real(V.sigh[P + i]);
-        sei = Real(V.sqe[P + i]);
+        const J4<Real> p = stage.position(i), g = stage.gb(i);
+        const J2<Real> l = stage.lj(i);
+        xi = p.x;
+        yi = p.y;
+        zi = p.z;
+        qi = g.x;
+        Ri = g.y;
+        iRi = g.z;
+        sgi = l.x;
+        sei = l.y;
     }
-    const Real tau = Real(V.tau), iei = Real(V.inv_eps_in);
-    const Real kap = Real(V.kappa), ieo = Real(V.inv_eps_out);
+    // FP32: the host-rounded copies (no double -> float conversion in the loops)
+    const Real tau = host_const<Real>(V.tau, V.tau32), iei = host_const<Real>(V.inv_eps_in, V.iei32);
+    const Real kap = host_const<Real>(V.kappa, V.kappa32), ieo = host_const<Real>(V.inv_eps_out, V.ieo32);
     const bool salt = V.kappa > 0; // pair sums then carry tau(f) and taud(f) per pair
     Acc fx = 0, fy = 0, fz = 0, adr = 0, egb = 0, ec = 0, elj = 0;
+    Real px = 0, py = 0, pz = 0, pdr = 0;
+    KSum<Real> pgb, pc, plj;
     int mp = V.mt_off[it.st];
     const int me = V.mt_off[it.st + 1];
     int next = mp < me ? V.mt_list[mp] : 0x7fffffff;
@@ -245,14 +324,14 @@ __global__ void __launch_bounds__(kTile) k_gb(const Item* __restrict__ items, Vi
             const int j = j0 + tid;
             J4<Real> a, b;
             if (j < N) {
-                a.x = Real(V.x[3 * (A + j)] - cx);
-                a.y = Real(V.x[3 * (A + j) + 1] - cy);
-                a.z = Real(V.x[3 * (A + j) + 2] - cz);
-                a.w = Real(V.q[A + j]) * sqk;
-                b.x = Real(V.R[A + j]);
-                b.y = Real(1.0 / V.R[A + j]);
-                b.z = Real(V.sigh[P + j]);
-                b.w = Real(V.sqe[P + j]);
+                const J4<Real> g = stage.gb(j);
+                const J2<Real> l = stage.lj(j);
+                a = stage.position(j);
+                a.w = g.x;
+                b.x = g.y;
+                b.y = g.z;
+                b.z = l.x;
+                b.w = l.y;
             } else {
                 a.x = a.y = a.z = Real(kFarF);
                 a.w = 0;
@@ -263,8 +342,6 @@ __global__ void __launch_bounds__(kTile) k_gb(const Item* __restrict__ items, Vi
             sb[tid] = b;
         }
         __syncthreads();
-        Real px = 0, py = 0, pz = 0, pdr = 0;
-        KSum<Real> pgb, pc, plj;
         if (jt != next) {
 #pragma unroll
             for (int k = sub; k < kTile; k += 32 * WPA) {
@@ -351,14 +428,18 @@ __global__ void __launch_bounds__(kTile) k_gb(const Item* __restrict__ items, Vi
                 }
             }
         }
-        Pr::add(fx, px, Real(kScaleE));
-        Pr::add(fy, py, Real(kScaleE));
-        Pr::add(fz, pz, Real(kScaleE));
-        Pr::add(adr, pdr, Real(kScaleE));
-        if (ENERGY) {
-            Pr::add(egb, pgb.value(), Real(kScaleE));
-            Pr::add(ec, pc.value(), Real(kScaleE));
-            Pr::add(elj, plj.value(), Real(kScaleE));
+        if (stage.flush(jt) || j0 + kTile >= N) {
+            Pr::add(fx, px, Real(kScaleE));
+            Pr::add(fy, py, Real(kScaleE));
+            Pr::add(fz, pz, Real(kScaleE));
+            Pr::add(adr, pdr, Real(kScaleE));
+            px = py = pz = pdr = 0;
+            if (ENERGY) {
+                Pr::add(egb, pgb.value(), Real(kScaleE));
+                Pr::add(ec, pc.value(), Real(kScaleE));
+                Pr::add(elj, plj.value(), Real(kScaleE));
+                pgb = pc = plj = KSum<Real>();
+            }
         }
     }
     fx = group_total<WPA>(fx, gsh);
@@ -376,7 +457,9 @@ __global__ void __launch_bounds__(kTile) k_gb(const Item* __restrict__ items, Vi
         const double dEdR = 0.5 * (V.tau_pair * Pr::value(adr, kScaleE)
                                    + salt_taud(R, V.inv_eps_in, V.inv_eps_out, V.kappa) * q * q / (R * R))
                           - (V.sa_gamma != 0.0 ? 6.0 * sa_ace(V.sa_gamma, V.sa_probe, V.rho[P + i], R) / R : 0.0);
-        V.c[A + i] = dEdR * V.dRdpsi[A + i] * 0.5 * V.rt[P + i];
+        const double c = dEdR * V.dRdpsi[A + i] * 0.5 * V.rt[P + i];
+        V.c[A + i] = c;
+        if (sizeof(Real) == 4) V.c32[A + i] = (float)c;
         V.Fd[3 * (A + i)] = Pr::value(fx, kScaleE);
         V.Fd[3 * (A + i) + 1] = Pr::value(fy, kScaleE);
         V.Fd[3 * (A + i) + 2] = Pr::value(fz, kScaleE);
@@ -541,7 +624,7 @@ __device__ inline void bonded_atom32(const View& V, int A, int P, int li, int la
 // ------------------------------------------ pass 3: chain rule through Born radii
 // F_i -= sum_j (c_i dH(r; rt_i, s_j)/dr + c_j dH(r; rt_j, s_i)/dr) (x_i - x_j)/r,
 // then the direct pair force and the bonded terms are added: F is the total force.
-template <class Real, bool ENERGY, int WPA>
+template <class Real, bool ENERGY, int WPA, bool STAGED>
 __global__ void __launch_bounds__(kTile) k_chain(const Item* __restrict__ items, View V) {
     using Pr = Prec<Real>;
     using Acc = typename Pr::Acc;
@@ -556,19 +639,21 @@ __global__ void __launch_bounds__(kTile) k_chain(const Item* __restrict__ items,
     const int i = it.i0 + warp / WPA;
     __shared__ long long gsh[kTile / 32];
     const bool vi = i < N;
-    const double cx = V.x[3 * (A + it.i0)], cy = V.x[3 * (A + it.i0) + 1],
-                 cz = V.x[3 * (A + it.i0) + 2];
+    const Stage<Real, STAGED> stage(V, A, P, it.i0);
     Real xi = Real(-kFarF), yi = Real(-kFarF), zi = Real(-kFarF), ci = 0, si = 0, rti = 1;
     if (vi) {
-        xi = Real(V.x[3 * (A + i)] - cx);
-        yi = Real(V.x[3 * (A + i) + 1] - cy);
-        zi = Real(V.x[3 * (A + i) + 2] - cz);
-        ci = Real(V.c[A + i]);
-        si = Real(V.sc[P + i]);
-        rti = Real(V.rt[P + i]);
+        const J4<Real> p = stage.position(i);
+        const J2<Real> r = stage.radii(i);
+        xi = p.x;
+        yi = p.y;
+        zi = p.z;
+        ci = stage.weight(i);
+        si = r.x;
+        rti = r.y;
     }
     Acc fx = 0, fy = 0, fz = 0;
     const Real rc = Real(V.rgbmax); // Born-radius cutoff (INFINITY = none)
+    Real px = 0, py = 0, pz = 0;
     int mp = V.mt_off[it.st];
     const int me = V.mt_off[it.st + 1];
     int next = mp < me ? V.mt_list[mp] : 0x7fffffff;
@@ -579,12 +664,9 @@ __global__ void __launch_bounds__(kTile) k_chain(const Item* __restrict__ items,
             J4<Real> a;
             J2<Real> b;
             if (j < N) {
-                a.x = Real(V.x[3 * (A + j)] - cx);
-                a.y = Real(V.x[3 * (A + j) + 1] - cy);
-                a.z = Real(V.x[3 * (A + j) + 2] - cz);
-                a.w = Real(V.c[A + j]);
-                b.x = Real(V.sc[P + j]);
-                b.y = Real(V.rt[P + j]);
+                a = stage.position(j);
+                a.w = stage.weight(j);
+                b = stage.radii(j);
             } else {
                 a.x = a.y = a.z = Real(kFarF);
                 a.w = 0;
@@ -595,7 +677,6 @@ __global__ void __launch_bounds__(kTile) k_chain(const Item* __restrict__ items,
             sb[tid] = b;
         }
         __syncthreads();
-        Real px = 0, py = 0, pz = 0;
         if (jt != next) {
 #pragma unroll
             for (int k = sub; k < kTile; k += 32 * WPA) {
@@ -632,9 +713,12 @@ __global__ void __launch_bounds__(kTile) k_chain(const Item* __restrict__ items,
                 pz += t * dz;
             }
         }
-        Pr::add(fx, px, Real(kScaleE));
-        Pr::add(fy, py, Real(kScaleE));
-        Pr::add(fz, pz, Real(kScaleE));
+        if (stage.flush(jt) || j0 + kTile >= N) {
+            Pr::add(fx, px, Real(kScaleE));
+            Pr::add(fy, py, Real(kScaleE));
+            Pr::add(fz, pz, Real(kScaleE));
+            px = py = pz = 0;
+        }
     }
     fx = group_total<WPA>(fx, gsh);
     fy = group_total<WPA>(fy, gsh);

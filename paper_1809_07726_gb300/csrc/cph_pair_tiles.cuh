@@ -44,9 +44,9 @@ struct BoJs {
 // the band's lower edge r + s <= rc for every s, so the series still holds
 // there, and beyond its upper edge every integral and derivative of the pair
 // vanishes (L >= r - s_max >= rc >= U), which CUT tiles apply as a select.
-// Skipped pairs take r^2 = skr2, beyond r_far and the band (results zeroed).
+// Skipped pairs take r^2 = infinity, where every form is 0.
 struct PairBand {
-    float rfar2, rin2, rout2, rc, skr2;
+    float rfar2, rin2, rout2, rc;
 };
 
 // rfar2 and s_max over every atom; rc = INFINITY for no cutoff.  The band's
@@ -60,10 +60,8 @@ __host__ __device__ inline PairBand pair_band(float rfar2, float smax, float rc)
         const float rin = fmaxf(rc - smax, 0.f) * (1.f - 1e-5f), rout = (rc + smax) * (1.f + 1e-5f);
         b.rin2 = rin * rin;
         b.rout2 = rout * rout;
-        b.skr2 = 4.f * fmaxf(rfar2, b.rout2) + 1.f;
     } else {
         b.rin2 = b.rout2 = INFINITY;
-        b.skr2 = 4.f * rfar2 + 1.f;
     }
     return b;
 }
@@ -177,9 +175,9 @@ __device__ __forceinline__ void note_near(float2 (&r2)[2], const PairBand& band,
 // partners j <= i of the warp's 64 i atoms (i-tiles start at a multiple of 256
 // atoms), or, for a warp without atoms, all of them: nothing of them is
 // counted, and the warp passes them by.
-__device__ __forceinline__ int live_pair(int i0, int warp, int n, int g0) {
+__device__ __forceinline__ int live_pair(int i0, int warp, int n, int g0, int npair) {
     const int iw = i0 + warp * 2 * kTileJ;
-    return iw >= n ? 0x7fff : (iw / kTileJ - g0) / 2;
+    return iw >= n ? npair : min(npair, max(0, iw / kTileJ - g0) / 2);
 }
 
 template <bool MASKED, bool CUT>

@@ -46,17 +46,6 @@ struct SymItem {
     int w, i0, jt0, jt1, st, pad;
 };
 
-// Tile pairs of the staged group at g0 (npair of them) that a warp passes by:
-// the first pairs whose two j-tiles hold only partners j <= i of the warp's
-// 64 i atoms (an i-tile starts at a multiple of kSymI atoms), or all of them
-// when the warp has no atom.  Every pair there is skipped, so their partials
-// are exact zeros and the warp starts at the returned pair.
-__device__ __forceinline__ int first_live_pair(int i0, int warp, int N, int g0, int npair) {
-    if (i0 + warp * 64 >= N) return npair;
-    const int d = i0 / kSymJ + 2 * warp - g0; // tiles below g0 + d are passed by
-    return d <= 0 ? 0 : min(npair, d >> 1);
-}
-
 // Non-finite partials would saturate in the float -> int64 conversion and
 // vanish into a finite-looking sum, so they are flagged before converting.
 __device__ __forceinline__ void red_add(long long* p, float v, int* status) {
@@ -108,7 +97,8 @@ __device__ __forceinline__ float hct_dr_series(float rinv2, float rinv, float s)
 // The pair kernels read FP32 operands only.  Positions are taken relative to
 // the walker's first atom (|x| stays within the molecule's extent, so FP32
 // keeps ~4e-6 A at 40 A) and rounded once per step; the charge and Born-radius
-// terms are rounded once per step after the Born radii and any MC sweep.
+// terms are rounded where the Born radii are finished, and once more after a
+// sweep that changed charges.
 __global__ void k_stage_x(View V, int a0, int n) {
     const int l = blockIdx.x * blockDim.x + threadIdx.x;
     if (l >= n) return;
@@ -123,8 +113,7 @@ __global__ void k_stage_gb(View V, int a0, int n) {
     if (l >= n) return;
     const int a = a0 + l;
     if (!V.w_local[V.a_walker[a]]) return;
-    const float R = (float)V.R[a], iR = __frcp_rn(R);
-    V.gq[a] = make_float4((float)(V.q[a] * V.sqrt_k), R, iR, (0.25f * kLog2e) * iR);
+    V.gq[a] = gb_operand(V.q[a], V.sqrt_k, V.R[a]);
 }
 
 // ====================================================== GB + Coulomb + LJ
@@ -314,10 +303,10 @@ __device__ __forceinline__ void gb_tile(const GbJs& sj, int lane, const GbI2 (&I
     }
 }
 
-template <bool ENERGY, bool SALT>
-__global__ void __launch_bounds__(kSymThreads, 5) k_gb_sym(const SymItem* __restrict__ items, View V) {
-    __shared__ GbJs sj[kSymG / 2];
-    __shared__ __align__(16) float red[kSymG][4][kSymJ][4];
+template <bool ENERGY, bool SALT, int GG>
+__global__ void __launch_bounds__(kSymThreads, GG == 2 ? 4 : 5) k_gb_sym(const SymItem* __restrict__ items, View V) {
+    __shared__ GbJs sj[GG / 2];
+    __shared__ __align__(16) float red[GG][4][kSymJ][4];
     __shared__ long long sfx[4][kSymI]; // i-side fixed-point sums, component-major (conflict-free)
     __shared__ double ered[kSymThreads / 32][3];
     const SymItem it = items[blockIdx.x];
@@ -352,8 +341,8 @@ __global__ void __launch_bounds__(kSymThreads, 5) k_gb_sym(const SymItem* __rest
     const int me = V.smt_off[it.st + 1];
     while (mp < me && V.smt_list[mp] < it.jt0) ++mp;
     int next = mp < me ? V.smt_list[mp] : 0x7fffffff;
-    for (int g0 = it.jt0; g0 < it.jt1; g0 += kSymG) {
-        const int ng = min(kSymG, it.jt1 - g0), npair = (ng + 1) >> 1;
+    for (int g0 = it.jt0; g0 < it.jt1; g0 += GG) {
+        const int ng = min(GG, it.jt1 - g0), npair = (ng + 1) >> 1;
         __syncthreads();
         // stage the tile pairs: thread (pair, copy, entry) writes whole rows
         for (int q = tid; q < npair * 2 * kSymJ; q += kSymThreads) {
@@ -384,12 +373,21 @@ __global__ void __launch_bounds__(kSymThreads, 5) k_gb_sym(const SymItem* __rest
         __syncthreads();
         // i-side partials of the whole staged group, summed in FP32 in a fixed
         // order (tile pairs in turn, halves = even / odd tiles) and converted to
-        // fixed point once per group: groups are the aligned runs of kSymG
-        // j-tiles (items start at a multiple of kSymG tiles and span a multiple
+        // fixed point once per group: groups are the aligned runs of GG
+        // j-tiles (items start at a multiple of GG tiles and span a multiple
         // of it), so the sums do not depend on the item's chunking
         float2 acc[2][4] = {{{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}},
                             {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}}};
-        for (int pr = 0; pr < npair; ++pr) {
+        const int pr0 = GG > 2 ? 0 : live_pair(it.i0, warp, N, g0, npair);
+        for (int pr = 0; pr < pr0; ++pr)
+            *reinterpret_cast<float4*>(red[2 * pr][warp][lane]) = *reinterpret_cast<float4*>(red[2 * pr + 1][warp][lane]) =
+                make_float4(0.f, 0.f, 0.f, 0.f);
+        if (GG == 2)
+            while (next < min(g0 + 2 * pr0, it.jt1)) { // masked tiles passed by
+                ++mp;
+                next = mp < me ? V.smt_list[mp] : 0x7fffffff;
+            }
+        for (int pr = pr0; pr < npair; ++pr) {
             const int jtA = g0 + 2 * pr; // tile B (jtA + 1) may lie past the item: padding
             float2 ja[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
             GbMask m = {};
@@ -508,36 +506,55 @@ struct ChJs {
 };
 
 // Closed-form force weight t of one pair inside r_far (or in the cutoff
-// band).  Inlined: unlike born_near, this is measured faster in line (the
-// chain tile keeps fewer values live across the branch).
-__device__ __forceinline__ float chain_near(float r2, float rinv, float c_i, float rt_i, float s_i, float c_j,
+// band).  Evaluated from the warp's queue of near pairs, out of line (one copy,
+// so that the cutoff variant rounds as the plain one does); or, where few steps
+// meet a near pair, in line behind a warp vote in the tile loop, as measured
+// faster there (the tile keeps fewer values live across the branch).
+__device__ __forceinline__ float chain_near_inline(float r2, float rinv, float c_i, float rt_i, float s_i, float c_j,
                                          float s_j, float rt_j, float rc) {
     const float r = r2 * rinv;
     const float g = c_i * hct_dr_fastlog(r, rinv, rt_i, s_j, rc) + c_j * hct_dr_fastlog(r, rinv, rt_j, s_i, rc);
     return -g * rinv;
 }
 
-template <bool MASKED, bool CUT>
+static __device__ __noinline__ float chain_near(float r2, float rinv, float c_i, float rt_i, float s_i, float c_j,
+                                                float s_j, float rt_j, float rc) {
+    return chain_near_inline(r2, rinv, c_i, rt_i, s_i, c_j, s_j, rt_j, rc);
+}
+
+// Systems of at most this many atoms have their near pairs queued.  64 x 2400
+// atoms (20 % of the steps meet a near pair): chain pass 0.412 -> 0.355 ms with
+// the queue; the 500 / 2000 / 8000-atom grid (7 % at 8000): 5.51 -> 5.64 ms, so
+// that one keeps them in line.  The line is drawn where the two would meet
+// (9 % of the steps).
+constexpr int kQueueAtoms = 6000;
+
+template <bool MASKED, bool CUT, bool QUEUE>
 __device__ __forceinline__ void chain_tile(const ChJs& sj, int lane, const ChI2 (&I)[2], float2 (&a)[2][3],
-                                           float2 (&ja)[3], const uint32_t (&sk)[2][2], const PairBand& band) {
+                                           float2 (&ja)[3], const uint32_t (&sk)[2][2], const PairBand& band,
+                                           NearBits& nb) {
     const int src = (lane + 1) & 31;
-    const float skr2 = band.skr2;
 #pragma unroll 2
     for (int k = 0; k < kSymJ; ++k) {
         const float4 A = sj.a[lane + k], B = sj.b[lane + k], C = sj.c[lane + k];
         const float2 cj = make_float2(B.z, B.w), s2j = make_float2(C.x, C.y), s3j = make_float2(C.z, C.w);
-        float2 dx[2], dy[2], dz[2], r2[2], t[2];
+        float2 dx[2], dy[2], dz[2], r2[2];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             dx[u] = __fadd2_rn(I[u].x, make_float2(A.x, A.y));
             dy[u] = __fadd2_rn(I[u].y, make_float2(A.z, A.w));
             dz[u] = __fadd2_rn(I[u].z, make_float2(B.x, B.y));
             r2[u] = __ffma2_rn(dx[u], dx[u], __ffma2_rn(dy[u], dy[u], __fmul2_rn(dz[u], dz[u])));
-            if (MASKED) { // skipped pairs stay off the closed-form branch
+            if (MASKED) {
                 const int jj = (lane + k) & (kSymJ - 1);
-                r2[u].x = ((sk[u][0] >> jj) & 1u) ? skr2 : r2[u].x;
-                r2[u].y = ((sk[u][1] >> jj) & 1u) ? skr2 : r2[u].y;
+                r2[u].x = ((sk[u][0] >> jj) & 1u) ? INFINITY : r2[u].x;
+                r2[u].y = ((sk[u][1] >> jj) & 1u) ? INFINITY : r2[u].y;
             }
+        }
+        if (QUEUE) note_near<CUT>(r2, band, k, nb);
+        float2 t[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
             const float2 rinv2 = make_float2(rcp_ftz(r2[u].x), rcp_ftz(r2[u].y));
             const float2 qj = hct_series_dr(__fmul2_rn(s2j, rinv2));
             const float2 qi = hct_series_dr(__fmul2_rn(I[u].s2, rinv2));
@@ -549,28 +566,24 @@ __device__ __forceinline__ void chain_tile(const ChJs& sj, int lane, const ChI2 
                 t[u].y = r2[u].y >= band.rout2 ? 0.f : t[u].y;
             }
         }
-        // closed forms only where some lane has such a pair (rare)
-        const bool nr = band_near<CUT>(r2[0].x, band) || band_near<CUT>(r2[0].y, band) ||
-                        band_near<CUT>(r2[1].x, band) || band_near<CUT>(r2[1].y, band);
-        if (__any_sync(0xffffffffu, nr)) {
-            const float4 Nj = sj.n[lane + k];
+        if (!QUEUE) { // closed forms only where some lane has such a pair (rare)
+            const bool nr = band_near<CUT>(r2[0].x, band) || band_near<CUT>(r2[0].y, band) ||
+                            band_near<CUT>(r2[1].x, band) || band_near<CUT>(r2[1].y, band);
+            if (__any_sync(0xffffffffu, nr)) {
+                const float4 Nj = sj.n[lane + k];
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                if (band_near<CUT>(r2[u].x, band))
-                    t[u].x = chain_near(r2[u].x, rsqrt_ftz(r2[u].x), I[u].c.x, I[u].rt, I[u].s, B.z, Nj.x, Nj.z,
-                                        band.rc);
-                if (band_near<CUT>(r2[u].y, band))
-                    t[u].y = chain_near(r2[u].y, rsqrt_ftz(r2[u].y), I[u].c.x, I[u].rt, I[u].s, B.w, Nj.y, Nj.w,
-                                        band.rc);
+                for (int u = 0; u < 2; ++u) {
+                    if (band_near<CUT>(r2[u].x, band))
+                        t[u].x = chain_near_inline(r2[u].x, rsqrt_ftz(r2[u].x), I[u].c.x, I[u].rt, I[u].s, B.z, Nj.x,
+                                                   Nj.z, band.rc);
+                    if (band_near<CUT>(r2[u].y, band))
+                        t[u].y = chain_near_inline(r2[u].y, rsqrt_ftz(r2[u].y), I[u].c.x, I[u].rt, I[u].s, B.w, Nj.y,
+                                                   Nj.w, band.rc);
+                }
             }
         }
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-            if (MASKED) {
-                const int jj = (lane + k) & (kSymJ - 1);
-                t[u].x = ((sk[u][0] >> jj) & 1u) ? 0.f : t[u].x;
-                t[u].y = ((sk[u][1] >> jj) & 1u) ? 0.f : t[u].y;
-            }
             a[u][0] = __ffma2_rn(t[u], dx[u], a[u][0]);
             a[u][1] = __ffma2_rn(t[u], dy[u], a[u][1]);
             a[u][2] = __ffma2_rn(t[u], dz[u], a[u][2]);
@@ -586,11 +599,14 @@ __device__ __forceinline__ void chain_tile(const ChJs& sj, int lane, const ChI2 
     }
 }
 
-template <bool CUT>
+template <bool CUT, int GG, bool QUEUE>
 __global__ void __launch_bounds__(kSymThreads, 5) k_chain_sym(const SymItem* __restrict__ items, View V) {
-    __shared__ ChJs sj[kSymG / 2];
-    __shared__ __align__(16) float red[kSymG][4][kSymJ][4]; // component 3 unused (vector stores)
+    __shared__ ChJs sj[GG / 2];
+    __shared__ __align__(16) float red[GG][4][kSymJ][4]; // component 3 unused (vector stores)
     __shared__ long long sfx[3][kSymI]; // i-side fixed-point sums, component-major (conflict-free)
+    // near pairs: the warps' queues, and the i-side sums of the staged group
+    __shared__ uint16_t nearq[QUEUE ? kSymThreads / 32 : 1][QUEUE ? kNearCap : 1];
+    __shared__ float inear[3][QUEUE ? kSymI : 1];
     const SymItem it = items[blockIdx.x];
     const int w = it.w, s = V.w_sys[w], N = V.sys_n[s], A = V.w_off[w], P = V.sys_poff[s];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -618,12 +634,13 @@ __global__ void __launch_bounds__(kSymThreads, 5) k_chain_sym(const SymItem* __r
     for (int u = 0; u < 2; ++u)
 #pragma unroll
         for (int c = 0; c < 3; ++c) sfx[c][warp * 64 + u * 32 + lane] = 0;
+    int nq = 0; // this warp's waiting near pairs
     int mp = V.smt_off[it.st];
     const int me = V.smt_off[it.st + 1];
     while (mp < me && V.smt_list[mp] < it.jt0) ++mp;
     int next = mp < me ? V.smt_list[mp] : 0x7fffffff;
-    for (int g0 = it.jt0; g0 < it.jt1; g0 += kSymG) {
-        const int ng = min(kSymG, it.jt1 - g0), npair = (ng + 1) >> 1;
+    for (int g0 = it.jt0; g0 < it.jt1; g0 += GG) {
+        const int ng = min(GG, it.jt1 - g0), npair = (ng + 1) >> 1;
         __syncthreads();
         // stage the tile pairs: thread (pair, copy, entry) writes whole rows
         for (int q = tid; q < npair * 2 * kSymJ; q += kSymThreads) {
@@ -653,10 +670,22 @@ __global__ void __launch_bounds__(kSymThreads, 5) k_chain_sym(const SymItem* __r
         }
         __syncthreads();
         // i-side partials of the staged group in FP32, one conversion per group
-        // (aligned runs of kSymG j-tiles: independent of the item's chunking)
+        // (aligned runs of GG j-tiles: independent of the item's chunking)
         float2 acc[2][3] = {{{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}}, {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}}};
-        for (int pr = 0; pr < npair; ++pr) {
+        if (QUEUE)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) inear[c][warp * 64 + lane] = inear[c][warp * 64 + 32 + lane] = 0.f;
+        const int pr0 = QUEUE ? live_pair(it.i0, warp, N, g0, npair) : 0;
+        for (int pr = 0; pr < pr0; ++pr)
+            *reinterpret_cast<float4*>(red[2 * pr][warp][lane]) = *reinterpret_cast<float4*>(red[2 * pr + 1][warp][lane]) =
+                make_float4(0.f, 0.f, 0.f, 0.f);
+        while (next < min(g0 + 2 * pr0, it.jt1)) { // masked tiles passed by
+            ++mp;
+            next = mp < me ? V.smt_list[mp] : 0x7fffffff;
+        }
+        for (int pr = pr0; pr < npair; ++pr) {
             const int jtA = g0 + 2 * pr;
+            NearBits nb = {};
             float2 ja[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
             uint32_t sk[2][2] = {{0u, 0u}, {0u, 0u}};
             bool masked = false;
@@ -672,16 +701,48 @@ __global__ void __launch_bounds__(kSymThreads, 5) k_chain_sym(const SymItem* __r
                     for (int u = 0; u < 2; ++u) sym_masks(V, P, ii[u], vi[u], jt * kSymJ, N, sk[u][h], nbm);
                 }
             }
-            if (masked) chain_tile<true, CUT>(sj[pr], lane, I, acc, ja, sk, band);
-            else chain_tile<false, CUT>(sj[pr], lane, I, acc, ja, sk, band);
+            if (masked) chain_tile<true, CUT, QUEUE>(sj[pr], lane, I, acc, ja, sk, band, nb);
+            else chain_tile<false, CUT, QUEUE>(sj[pr], lane, I, acc, ja, sk, band, nb);
             *reinterpret_cast<float4*>(red[2 * pr][warp][lane]) = make_float4(-ja[0].x, -ja[1].x, -ja[2].x, 0.f);
             *reinterpret_cast<float4*>(red[2 * pr + 1][warp][lane]) = make_float4(-ja[0].y, -ja[1].y, -ja[2].y, 0.f);
+            if (QUEUE) near_drain(nb, nearq[warp], nq, lane, pr, pr == npair - 1, [&](uint32_t e, bool valid) {
+                const int l = e & 31u, jj = (e >> 7) & 31u, p = e >> 12;
+                const bool u = (e >> 5) & 1u, h = (e >> 6) & 1u;
+                auto of_i = [&](float v0, float v1) {
+                    v0 = __shfl_sync(0xffffffffu, v0, l);
+                    v1 = __shfl_sync(0xffffffffu, v1, l);
+                    return u ? v1 : v0;
+                };
+                const float xi = of_i(I[0].x.x, I[1].x.x), yi = of_i(I[0].y.x, I[1].y.x), zi = of_i(I[0].z.x, I[1].z.x);
+                const float ci = of_i(I[0].c.x, I[1].c.x), si = of_i(I[0].s, I[1].s), rti = of_i(I[0].rt, I[1].rt);
+                const ChJs& S = sj[p];
+                const float4 A = S.a[jj], B = S.b[jj], Nj = S.n[jj];
+                const float dx = xi + (h ? A.y : A.x), dy = yi + (h ? A.w : A.z), dz = zi + (h ? B.y : B.x);
+                const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+                const float t = chain_near(r2, rsqrt_ftz(r2), ci, rti, si, h ? B.w : B.z, h ? Nj.y : Nj.x,
+                                           h ? Nj.w : Nj.z, band.rc);
+                const int row = warp * 64 + u * 32 + l;
+                in_turn(u * 32 + l, valid, lane, [&] {
+                    inear[0][row] = fmaf(t, dx, inear[0][row]);
+                    inear[1][row] = fmaf(t, dy, inear[1][row]);
+                    inear[2][row] = fmaf(t, dz, inear[2][row]);
+                });
+                float(&r)[4] = red[2 * p + h][warp][jj];
+                in_turn(p * 64 + h * 32 + jj, valid, lane, [&] {
+                    r[0] = fmaf(-t, dx, r[0]);
+                    r[1] = fmaf(-t, dy, r[1]);
+                    r[2] = fmaf(-t, dz, r[2]);
+                });
+            });
         }
+        __syncwarp();
 #pragma unroll
         for (int u = 0; u < 2; ++u)
 #pragma unroll
             for (int c = 0; c < 3; ++c)
-                sfx[c][warp * 64 + u * 32 + lane] += to_fixed(acc[u][c].x + acc[u][c].y, (float)kScaleE);
+                sfx[c][warp * 64 + u * 32 + lane] +=
+                    to_fixed(acc[u][c].x + acc[u][c].y + (QUEUE ? inear[c][warp * 64 + u * 32 + lane] : 0.f),
+                             (float)kScaleE);
         __syncthreads();
         for (int v = tid; v < ng * kSymJ * 3; v += kSymThreads) {
             const int g = v / (kSymJ * 3), rem = v % (kSymJ * 3), j = rem / 3, c = rem % 3;
@@ -818,15 +879,17 @@ __global__ void k_final_forces(View V, int a0, int n) {
 // tile's own arithmetic, so the near/far decision is the same.
 constexpr int kNearQ = 192; // queue entries per warp: flushed at >= 64; a step adds <= 128
 
+template <int GG>
 struct BoNear {
     uint32_t q[kSymThreads / 32][kNearQ]; // lane | u << 5 | partner << 6 | half << 11 | pair << 12
     float4 ix[kSymThreads / 32][64];      // the warp's i atoms (x, y, z, s), slot u * 32 + lane
     float2 it[kSymThreads / 32][64];      // (rt, 1/rt)
     long long ihx[kSymThreads / 32][64];  // i-side sums of queued pairs (2^40 fixed point)
-    long long jhx[kSymG][kSymJ];          // partner-side sums of the staged group
+    long long jhx[GG][kSymJ];          // partner-side sums of the staged group
 };
 
-__device__ __noinline__ void born_flush(const BoJs* sj, BoNear& nb, int warp, int lane, int n, PairBand band,
+template <int GG>
+__device__ __noinline__ void born_flush(const BoJs* sj, BoNear<GG>& nb, int warp, int lane, int n, PairBand band,
                                         int* status) {
     for (int e = lane; e < n; e += 32) {
         const uint32_t q = nb.q[warp][e];
@@ -848,13 +911,12 @@ __device__ __noinline__ void born_flush(const BoJs* sj, BoNear& nb, int warp, in
 }
 
 // born_tile with the closed forms queued (weight 0 in the loop)
-template <bool MASKED, bool CUT>
+template <bool MASKED, bool CUT, int GG>
 __device__ __forceinline__ void born_tile_q(const BoJs* sjg, int pr, int lane, int warp, const BoI2 (&I)[2],
                                             float2 (&ah)[2], float2& jh, const uint32_t (&sk)[2][2],
-                                            const PairBand& band, BoNear& nb, int& nq, int* status) {
+                                            const PairBand& band, BoNear<GG>& nb, int& nq, int* status) {
     const BoJs& sj = sjg[pr];
     const int src = (lane + 1) & 31;
-    const float skr2 = band.skr2;
     const uint32_t lt = (1u << lane) - 1u;
 #pragma unroll 2
     for (int k = 0; k < kTileJ; ++k) {
@@ -869,8 +931,8 @@ __device__ __forceinline__ void born_tile_q(const BoJs* sjg, int pr, int lane, i
             r2[u] = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
             if (MASKED) { // skipped pairs stay off the closed-form queue
                 const int jj = (lane + k) & (kTileJ - 1);
-                r2[u].x = ((sk[u][0] >> jj) & 1u) ? skr2 : r2[u].x;
-                r2[u].y = ((sk[u][1] >> jj) & 1u) ? skr2 : r2[u].y;
+                r2[u].x = ((sk[u][0] >> jj) & 1u) ? INFINITY : r2[u].x;
+                r2[u].y = ((sk[u][1] >> jj) & 1u) ? INFINITY : r2[u].y;
             }
             const float2 rinv2 = make_float2(rcp_ftz(r2[u].x), rcp_ftz(r2[u].y));
             wt[u] = __fmul2_rn(rinv2, rinv2); // r^-4, the weight of both far terms
@@ -929,11 +991,11 @@ __device__ __forceinline__ void born_tile_q(const BoJs* sjg, int pr, int lane, i
         jh.y = __shfl_sync(0xffffffffu, jh.y, src);
     }
 }
-template <bool CUT>
+template <bool CUT, int GG>
 __global__ void __launch_bounds__(kSymThreads, 5) k_born_sym(const SymItem* __restrict__ items, View V) {
-    __shared__ BoJs sj[kSymG / 2];
-    __shared__ float red[kSymG][4][kSymJ];
-    __shared__ BoNear nb;
+    __shared__ BoJs sj[GG / 2];
+    __shared__ float red[GG][4][kSymJ];
+    __shared__ BoNear<GG> nb;
     const SymItem it = items[blockIdx.x];
     const int w = it.w, s = V.w_sys[w], N = V.sys_n[s], A = V.w_off[w], P = V.sys_poff[s];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -960,15 +1022,15 @@ __global__ void __launch_bounds__(kSymThreads, 5) k_born_sym(const SymItem* __re
         nb.it[warp][u * 32 + lane] = make_float2(I[u].rt, I[u].irt);
         nb.ihx[warp][u * 32 + lane] = 0;
     }
-    for (int q = tid; q < kSymG * kSymJ; q += kSymThreads) nb.jhx[q / kSymJ][q % kSymJ] = 0;
+    for (int q = tid; q < GG * kSymJ; q += kSymThreads) nb.jhx[q / kSymJ][q % kSymJ] = 0;
     int nq = 0; // this warp's queued pairs (warp-uniform)
     long long hx[2] = {0, 0}; // i-side fixed-point sums
     int mp = V.smt_off[it.st];
     const int me = V.smt_off[it.st + 1];
     while (mp < me && V.smt_list[mp] < it.jt0) ++mp;
     int next = mp < me ? V.smt_list[mp] : 0x7fffffff;
-    for (int g0 = it.jt0; g0 < it.jt1; g0 += kSymG) {
-        const int ng = min(kSymG, it.jt1 - g0), npair = (ng + 1) >> 1;
+    for (int g0 = it.jt0; g0 < it.jt1; g0 += GG) {
+        const int ng = min(GG, it.jt1 - g0), npair = (ng + 1) >> 1;
         __syncthreads();
         // stage the tile pairs: thread (pair, copy, entry) writes whole rows
         for (int q = tid; q < npair * 2 * kSymJ; q += kSymThreads) {
@@ -997,7 +1059,7 @@ __global__ void __launch_bounds__(kSymThreads, 5) k_born_sym(const SymItem* __re
             }
         }
         __syncthreads();
-        const int pr0 = first_live_pair(it.i0, warp, N, g0, npair);
+        const int pr0 = live_pair(it.i0, warp, N, g0, npair);
         for (int pr = 0; pr < pr0; ++pr) {
             red[2 * pr][warp][lane] = 0.f;
             red[2 * pr + 1][warp][lane] = 0.f;
@@ -1075,6 +1137,7 @@ __global__ void k_fin_born(View V, int a0, int n, int zero_energy) {
     const double R = 1.0 / (V.irt[P] - th * irho);
     V.psi[a] = psi;
     V.R[a] = R;
+    V.gq[a] = gb_operand(V.q[a], V.sqrt_k, R);
     V.dRdpsi[a] = R * R * (1.0 - th * th) * (V.alpha + psi * (-2.0 * V.beta + 3.0 * V.gamma * psi)) * irho;
     V.Ffix[3 * a] = 0;
     V.Ffix[3 * a + 1] = 0;

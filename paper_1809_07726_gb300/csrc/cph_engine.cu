@@ -16,6 +16,7 @@
 
 #include "cph_kernels.cuh"
 #include "cph_sym.cuh"
+#include "cph_small.cuh"
 
 namespace cph {
 
@@ -644,6 +645,11 @@ struct cph_engine {
     // velocities), so constrained runs keep every rounding they had: operands
     // from the master arrays, undivided work items, near pairs in line.
     bool staged = true;
+    // whole steps of small walkers in one launch (cph_small.cuh)
+    bool small_fits = false;       // every system can run that way
+    bool small = false;            // and every system's tile shape is CPH_SHAPE_WARP_PER_ATOM
+    SmallTab small_tab{};
+    int small_ga = 0, small_warps = 0, small_smem = 0; // atoms per warp, pair warps per CTA, bytes
     std::vector<int> h_w_local;    // 1 for the walkers this engine advances
     int* d_w_local = nullptr;
     bool sharded = false;          // some walker is not local
@@ -831,7 +837,43 @@ cudaStream_t lane_stream(const cph_engine* E, int w, cudaStream_t st) {
     return E->n_rs > 1 ? E->rs[w % E->n_rs] : st;
 }
 
-int launch_stage(cph_engine* E, int pass, int a0, int n, cudaStream_t st);
+int launch_stage(cph_engine* E, int which, int a0, int n, cudaStream_t st);
+
+template <class F>
+void by_small(const cph_engine* E, bool energy, F&& f) {
+    if (E->small_ga == 1) f(energy ? k_small<1, true> : k_small<1, false>);
+    else if (E->small_ga == 2) f(energy ? k_small<2, true> : k_small<2, false>);
+    else f(energy ? k_small<4, true> : k_small<4, false>);
+}
+
+// Steps s_off .. s_off + steps - 1 (relative to the device's step counter) of
+// every walker from phase `start` of the first to phase `end` of the last.
+int launch_small(cph_engine* E, bool energy, int s_off, int steps, int start, int end, bool zero_energy,
+                 cudaStream_t st) {
+    auto go = [&](int w0, int n, cudaStream_t s) -> int {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(n * kSmallRanks);
+        cfg.blockDim = dim3(32 * (E->small_warps + kSmallAux));
+        cfg.dynamicSmemBytes = E->small_smem;
+        cfg.stream = s;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = kSmallRanks;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        const SmallRun run{w0, E->small_warps, s_off, steps, start, end, zero_energy ? 1 : 0};
+        cudaError_t ce = cudaSuccess;
+        by_small(E, energy, [&](auto kernel) { ce = cudaLaunchKernelEx(&cfg, kernel, E->V, E->small_tab, run); });
+        CK(ce);
+        return CPH_OK;
+    };
+    if (E->launch_mode == 0) return go(0, E->V.W, st);
+    TRY(fan_out(E, st));
+    for (int w = 0; w < E->V.W; ++w)
+        if (E->h_w_local[w]) TRY(go(w, 1, lane_stream(E, w, st)));
+    return fan_in(E, st);
+}
 
 int launch_mc(cph_engine* E, int kinds, int s_off, cudaStream_t st) {
     const int W = E->V.W;
@@ -844,7 +886,8 @@ int launch_mc(cph_engine* E, int kinds, int s_off, cudaStream_t st) {
         // the per-site kernel reads sqrt(k) q and R from the FP32 staging, which the
         // Born-radii pass wrote: stage them again at a second sweep's charges
         const bool again = f32 && !first;
-        const bool first_x = f32 && first && !(E->staged || E->n_sym > 0); // no pass staged the positions
+        // no pass staged the positions
+        const bool first_x = f32 && first && !E->small && !(E->staged || E->n_sym > 0);
         if (E->launch_mode == 0) {
             if (first_x) TRY(launch_stage(E, 0, 0, E->V.total_atoms, st));
             if (again) TRY(launch_stage(E, 1, 0, E->V.total_atoms, st));
@@ -977,6 +1020,7 @@ int launch_pass(cph_engine* E, int pass, bool energy, cudaStream_t st) {
 
 int launch_forces(cph_engine* E, bool energy, cudaStream_t st, bool mc_between, int s_off,
                   int mc_kinds) {
+    if (E->small && !mc_between) return launch_small(E, energy, 0, 1, kSmallBorn, kSmallForces, energy, st);
     TRY(launch_pass(E, 0, energy, st));
     if (mc_between && mc_kinds && E->max_sites > 0) {
         TRY(launch_mc(E, mc_kinds, s_off, st));
@@ -1071,6 +1115,42 @@ int enqueue_step(cph_engine* E, long long t, int s_off, bool full_schedule, cuda
     return CPH_OK;
 }
 
+// n steps from global step t; s_off: the first one's offset from the device's
+// step counter.
+int enqueue_steps(cph_engine* E, long long t, long long n, int s_off, bool full_schedule, cudaStream_t st) {
+    if (!E->small) {
+        for (long long k = 0; k < n; ++k) TRY(enqueue_step(E, t + k, s_off + (int)k, full_schedule, st));
+        return CPH_OK;
+    }
+    // small walkers: launches from one event of the schedule to the next.  Open:
+    // step `open` from phase `from` on.
+    long long open = 0;
+    int from = kSmallBorn;
+    for (long long k = 0; full_schedule && k < n; ++k) {
+        const long long tk = t + k;
+        int kinds = 0;
+        if (tk > 0 && E->mc_ph > 0 && tk % E->mc_ph == 0) kinds |= CPH_MC_PH;
+        if (tk > 0 && E->mc_redox > 0 && tk % E->mc_redox == 0) kinds |= CPH_MC_REDOX;
+        const bool exch = tk > 0 && E->ex_every > 0 && tk % E->ex_every == 0;
+        if (kinds && E->max_sites > 0) {
+            TRY(launch_small(E, false, s_off + (int)open, (int)(k - open + 1), from, kSmallBorn, exch, st));
+            TRY(launch_mc(E, kinds, s_off + (int)k, st));
+            open = k;
+            from = kSmallForces;
+        }
+        if (exch) {
+            if (open < k) TRY(launch_small(E, false, s_off + (int)open, (int)(k - open), from, kSmallMove, false, st));
+            if (open < k) from = kSmallBorn;
+            TRY(launch_small(E, true, s_off + (int)k, 1, from, kSmallForces, from == kSmallBorn, st));
+            TRY(launch_exchange(E, CPH_DIM_NEXT, s_off + (int)k, st));
+            open = k;
+            from = kSmallMove;
+        }
+    }
+    if (open < n) TRY(launch_small(E, false, s_off + (int)open, (int)(n - open), from, kSmallMove, false, st));
+    return CPH_OK;
+}
+
 long long gcdll(long long a, long long b) { return b ? gcdll(b, a % b) : a; }
 
 int schedule_period(const cph_engine* E) {
@@ -1092,7 +1172,7 @@ int get_graph(cph_engine* E, cudaGraphExec_t* out) {
     CK(cudaStreamBeginCapture(E->cap_stream, cudaStreamCaptureModeThreadLocal));
     int rc = CPH_OK;
     // the captured period starts at a step t with t % P == 1 (t > 0 throughout)
-    for (int s = 0; s < P && rc == CPH_OK; ++s) rc = enqueue_step(E, 1 + s, s, true, E->cap_stream);
+    rc = enqueue_steps(E, 1, P, 0, true, E->cap_stream);
     if (rc == CPH_OK) rc = launch_tick(E, P, E->cap_stream);
     cudaError_t ce = cudaStreamEndCapture(E->cap_stream, &g);
     if (rc != CPH_OK) {
@@ -1113,6 +1193,100 @@ int get_graph(cph_engine* E, cudaGraphExec_t* out) {
 
 namespace {
 
+// Tables and launch shape of the small-walker kernel, if every system fits it:
+// FP32 mode, at most kSmallAtoms atoms and kSmallTerms bonded terms in a CTA, and
+// a device that can hold the cluster.
+int small_setup(cph_engine* E, const std::vector<int>& bond_off, const std::vector<int>& bond_idx,
+                const std::vector<int>& bond_ij, const std::vector<int>& ang_off, const std::vector<int>& ang_idx,
+                const std::vector<int>& ang_ijk, const std::vector<int>& sys_poff, const std::vector<int>& shk_sys_off,
+                const std::vector<float4>& shk_fac) {
+    const int nmax = *std::max_element(E->h_sys_n.begin(), E->h_sys_n.end());
+    if (E->precision != CPH_PREC_FP32 || nmax > kSmallAtoms) return CPH_OK;
+    const int ranks = kSmallRanks, ga = nmax <= 160 ? 1 : (nmax <= 256 ? 2 : 4); // atoms per warp
+    E->small_ga = ga;
+    {
+        std::vector<int> term_off, term, ref_off(1, 0), ref, ref_mid;
+        int max_terms = 0, max_bytes = 0;
+        const int warps = 4 * (((nmax + 3) / 4 + ranks - 1) / ranks) / ga;
+        for (int s = 0; s < E->n_sys; ++s) {
+            const int N = E->h_sys_n[s], P = sys_poff[s], own = 4 * (((N + 3) / 4 + ranks - 1) / ranks);
+            for (int r = 0; r < ranks; ++r) {
+                const int a0 = std::min(N, own * r), a1 = std::min(N, own * (r + 1));
+                std::vector<int> tb, ta; // the terms that touch atoms a0 .. a1 - 1
+                for (int a = a0; a < a1; ++a) {
+                    tb.insert(tb.end(), bond_idx.begin() + bond_off[P + a], bond_idx.begin() + bond_off[P + a + 1]);
+                    ta.insert(ta.end(), ang_idx.begin() + ang_off[P + a], ang_idx.begin() + ang_off[P + a + 1]);
+                }
+                for (auto* v : {&tb, &ta}) {
+                    std::sort(v->begin(), v->end());
+                    v->erase(std::unique(v->begin(), v->end()), v->end());
+                }
+                const int nb = (int)tb.size(), nt = nb + (int)ta.size();
+                term_off.push_back((int)term.size());
+                term_off.push_back((int)term.size() + nb);
+                term_off.push_back((int)term.size() + nt);
+                term.insert(term.end(), tb.begin(), tb.end());
+                term.insert(term.end(), ta.begin(), ta.end());
+                max_terms = std::max(max_terms, nt);
+                max_bytes = std::max(max_bytes, (int)small_bytes(N, own, nt));
+                for (int a = a0; a < a1; ++a) {
+                    for (int e = bond_off[P + a]; e < bond_off[P + a + 1]; ++e) {
+                        const int b = bond_idx[e];
+                        const int at = (int)(std::lower_bound(tb.begin(), tb.end(), b) - tb.begin());
+                        ref.push_back(at << 2 | (bond_ij[2 * b] == a ? 0 : 1));
+                    }
+                    ref_mid.push_back((int)ref.size());
+                    for (int e = ang_off[P + a]; e < ang_off[P + a + 1]; ++e) {
+                        const int g = ang_idx[e];
+                        const int at = nb + (int)(std::lower_bound(ta.begin(), ta.end(), g) - ta.begin());
+                        ref.push_back(at << 2 | (ang_ijk[3 * g] == a ? 0 : (ang_ijk[3 * g + 1] == a ? 1 : 2)));
+                    }
+                    ref_off.push_back((int)ref.size());
+                }
+            }
+        }
+        if (max_terms > kSmallTerms || max_bytes > 200 * 1024) return CPH_OK;
+        // can the device hold such a cluster?
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(ranks);
+        cfg.blockDim = dim3(32 * (warps + kSmallAux));
+        cfg.dynamicSmemBytes = max_bytes;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = ranks;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        bool ok = true;
+        for (bool energy : {false, true})
+            by_small(E, energy, [&](auto kernel) {
+                int n = 0;
+                ok = ok && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) == cudaSuccess;
+                ok = ok && cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n > 0;
+            });
+        if (!ok) {
+            (void)cudaGetLastError();
+            return CPH_OK;
+        }
+        int* d;
+        SmallTab& T = E->small_tab;
+        TRY(upload(E, term_off, &d)); T.term_off = d;
+        TRY(upload(E, term, &d)); T.term = d;
+        TRY(upload(E, ref_off, &d)); T.ref_off = d;
+        TRY(upload(E, ref, &d)); T.ref = d;
+        TRY(upload(E, ref_mid, &d)); T.ref_mid = d;
+        TRY(upload(E, shk_sys_off, &d)); T.shk_sys_off = d;
+        float4* d4;
+        TRY(upload(E, shk_fac, &d4)); T.shk_fac = d4;
+        float2* d2;
+        TRY(alloc0(E, (size_t)E->V.total_atoms, &d2)); T.rad = d2;
+        E->small_warps = warps;
+        E->small_smem = max_bytes;
+        E->small_fits = true;
+        return CPH_OK;
+    }
+}
+
 // Work items of the pair passes.  Ordered items: groups of kWarpAtoms atoms i
 // (one warp each) of the walkers whose system runs the ordered passes.
 // Symmetric items (FP32), for the other walkers: j-tile chunks of `chunk`
@@ -1132,6 +1306,9 @@ int build_items(cph_engine* E, int chunk) {
     std::vector<int> o_off(W + 1, 0);
     std::vector<int> ordered(E->n_sys);
     for (int s = 0; s < E->n_sys; ++s) ordered[s] = sys_ordered(E, s) ? 1 : 0;
+    // (by system, not by walker: every engine of a sharded grid decides alike)
+    E->small = E->small_fits;
+    for (int s = 0; s < E->n_sys; ++s) E->small = E->small && ordered[s];
     // FP64 arithmetic on few atoms (a small walker or two): four warps per atom,
     // one atom per CTA, so that the scarce FP64 units of every SM share the
     // work.  Counted over the whole grid, local or not, so that every engine of
@@ -1745,6 +1922,17 @@ int cph_init_system(const cph_system_desc* sys, int n_sys, const cph_grid_desc* 
         E->sym_split = items < 152 * 8 && !p->shake ? 4 : 1;
         E->queue_near = *std::max_element(sys_n.begin(), sys_n.end()) <= kQueueAtoms && !p->shake;
     }
+    {
+        std::vector<float4> fac(shk_h.size());
+        for (int sy = 0; sy < n_sys; ++sy)
+            for (int c = shk_sys_off[sy]; c < shk_sys_off[sy + 1]; ++c)
+                for (int h = shk_off[c]; h < shk_off[c + 1]; ++h) {
+                    const double i0 = 1.0 / sys[sy].mass[shk_heavy[c]], ih = 1.0 / sys[sy].mass[shk_h[h]];
+                    const double f0 = 0.5 * i0 / (i0 + ih), fh = 0.5 * ih / (i0 + ih);
+                    fac[h] = make_float4((float)f0, (float)(f0 - (double)(float)f0), (float)fh, (float)(fh - (double)(float)fh));
+                }
+        TRY(small_setup(E, bond_off, bond_idx, bond_ij, ang_off, ang_idx, ang_ijk, sys_poff, shk_sys_off, fac));
+    }
     TRY(build_items(E, E->sym_split == 1 ? kSymChunk : kSymG));
 
     // reference energies of every (site, state)
@@ -1978,7 +2166,7 @@ int cph_get_tile_shapes(const cph_engine* e, int* shapes) {
 int cph_step_replicas(cph_engine* e, int64_t n_steps, void* stream) {
     if (!e || n_steps < 0) return fail(e, CPH_E_INVALID, "bad arguments");
     cudaStream_t st = (cudaStream_t)stream;
-    for (int64_t s = 0; s < n_steps; ++s) TRY(enqueue_step(e, e->h_step + s, (int)s, false, st));
+    TRY(enqueue_steps(e, e->h_step, n_steps, 0, false, st));
     if (n_steps) TRY(launch_tick(e, n_steps, st));
     e->h_step += n_steps;
     return CPH_OK;
@@ -1987,7 +2175,8 @@ int cph_step_replicas(cph_engine* e, int64_t n_steps, void* stream) {
 int cph_mc_titrate(cph_engine* e, int kind, void* stream) {
     if (!e || kind < 1 || kind > 3) return fail(e, CPH_E_INVALID, "bad arguments");
     cudaStream_t st = (cudaStream_t)stream;
-    TRY(launch_pass(e, 0, false, st));
+    if (e->small) TRY(launch_small(e, false, 0, 1, kSmallBorn, kSmallBorn, false, st));
+    else TRY(launch_pass(e, 0, false, st));
     TRY(launch_mc(e, kind, 0, st));
     return CPH_OK;
 }
@@ -2037,10 +2226,14 @@ int cph_run(cph_engine* e, int64_t n_steps, void* stream) {
             done += P;
             e->mc_kinds_last = (e->mc_ph > 0 ? CPH_MC_PH : 0) | (e->mc_redox > 0 ? CPH_MC_REDOX : 0);
         } else {
-            TRY(enqueue_step(e, t, (int)direct, true, st));
-            ++direct;
-            ++e->h_step;
-            ++done;
+            // directly launched steps: up to where a whole period can be replayed
+            int64_t k = 1;
+            if (e->small)
+                while (done + k < n_steps && !(P > 1 && (t + k) % P == 1 && n_steps - done - k >= P)) ++k;
+            TRY(enqueue_steps(e, t, k, (int)direct, true, st));
+            direct += k;
+            e->h_step += k;
+            done += k;
         }
     }
     if (direct) TRY(launch_tick(e, direct, st));

@@ -27,6 +27,7 @@
 #include "../../include/cphremd.h"
 #include "cph_device.cuh"
 #include "cph_grad_sym.cuh"
+#include "cph_grad_small.cuh"
 
 namespace cph {
 namespace grad {
@@ -151,6 +152,14 @@ void by_group(const SView& g, F&& f) {
     else f(std::integral_constant<int, kGG>{});
 }
 
+// Whether a call goes to the one-launch cluster kernel: replicas it can hold, and
+// not so many that its twofold pair arithmetic outweighs the launches and the
+// near-empty tiles it saves.  Energy / backward in us, cluster kernel against
+// symmetric kernels: 1 x 237 12 / 25 against 60 / 118, 128 x 237 48 / 116 against
+// 74 / 149, 128 x 400 88 / 223 against 133 / 305, 128 x 512 110 / 286 against
+// 121 / 267, 512 x 237 168 / 409 against 158 / 362.
+bool gsmall(int n_rep, int n) { return n <= kGsAtoms && (long long)n_rep * n * n <= 24000000; }
+
 // bound and Born radii, shared by both directions
 int launch_radii(SView& g, cudaStream_t st) {
     const size_t na = (size_t)g.n_rep * g.n;
@@ -184,6 +193,12 @@ extern "C" int cph_gb_energy(int n_rep, int n, const float* x, const float* q, c
     if (!E) return gfail(CPH_E_INVALID, "cph_gb_energy: E is NULL");
     g.E = E;
     cudaStream_t st = (cudaStream_t)stream;
+    if (gsmall(n_rep, n)) {
+        k_gsmall<false><<<n_rep * kGsRanks, kGsThreads, 0, st>>>(g);
+        const cudaError_t ce = cudaGetLastError();
+        if (ce != cudaSuccess) return gfail(CPH_E_CUDA, std::string("cph_gb_energy: ") + cudaGetErrorString(ce));
+        return CPH_OK;
+    }
     rc = launch_radii(g, st);
     if (rc != CPH_OK) return rc;
     const size_t na = (size_t)n_rep * n;
@@ -213,6 +228,12 @@ extern "C" int cph_gb_energy_backward(int n_rep, int n, const float* x, const fl
     g.dqo = dq;
     g.drho = drho;
     cudaStream_t st = (cudaStream_t)stream;
+    if (gsmall(n_rep, n)) {
+        k_gsmall<true><<<n_rep * kGsRanks, kGsThreads, 0, st>>>(g);
+        const cudaError_t ce = cudaGetLastError();
+        if (ce != cudaSuccess) return gfail(CPH_E_CUDA, std::string("cph_gb_energy_backward: ") + cudaGetErrorString(ce));
+        return CPH_OK;
+    }
     rc = launch_radii(g, st);
     if (rc != CPH_OK) return rc;
     const size_t na = (size_t)n_rep * n;

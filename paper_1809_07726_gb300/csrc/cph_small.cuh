@@ -69,17 +69,6 @@ struct SmallRun {
     int zero_energy;
 };
 
-// __float2ll_rn(v * 2^32) through 32-bit conversions (exact: the integer part,
-// then the fraction's 32 bits, rounded half to even as a whole would be)
-__device__ __forceinline__ long long fix32(float v) {
-    const float a = fabsf(v);
-    if (!(a < 1073741824.f)) return to_fixed(v, (float)kScaleE);
-    const unsigned hi = __float2uint_rz(a);
-    const unsigned lo = __float2uint_rn((a - (float)hi) * 4294967296.f);
-    const long long m = (long long)(((unsigned long long)hi << 32) | lo);
-    return v < 0.f ? -m : m;
-}
-
 // a - b for a, b given as sums h + l of floats (48 bits), rounded to FP32
 __device__ __forceinline__ float diff2(const float2& a, const float2& b) {
     const float s = __fsub_rn(a.x, b.x), t = __fsub_rn(s, a.x);
@@ -90,45 +79,6 @@ __device__ __forceinline__ float diff2(const float2& a, const float2& b) {
 __device__ __forceinline__ float2 split2(double x) {
     const float h = (float)x;
     return make_float2(h, (float)(x - (double)h));
-}
-
-// sum over the warp, in every lane (exact integers: any order)
-__device__ __forceinline__ long long warp_sum(long long v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// 1 / x for normal x: the PTX approximation (20 bits) and two Newton steps
-__device__ __forceinline__ double rcp64(double x) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    y = fma(fma(-x, y, 1.0), y, y);
-    return fma(fma(-x, y, 1.0), y, y);
-}
-
-// 2^(j/16)
-static __constant__ double kExp2Tab[16] = {1.0, 1.0442737824274138, 1.0905077326652577, 1.1387886347566916, 1.189207115002721, 1.241857812073484, 1.2968395546510096, 1.3542555469368927, 1.4142135623730951, 1.4768261459394993, 1.5422108254079407, 1.6104903319492543, 1.681792830507429, 1.7562521603732995, 1.8340080864093424, 1.9152065613971474};
-
-// e^x for -700 < x <= 0 (smaller x: e^-700): x = k ln2/16 + r, a Taylor series in
-// r (|r| <= 0.022, remainder 1e-18) and the table
-__device__ __forceinline__ double exp64(double x) {
-    x = fmax(x, -700.0);
-    const double big = 6755399441055744.0; // 1.5 2^52: the sum's low word is the integer
-    const double t = fma(x, 23.083120654223414, big);
-    const double k = t - big;
-    double r = fma(k, -0.04332169878499658, x);
-    r = fma(k, -1.4494042586539372e-18, r);
-    double p = fma(r, 1.0 / 5040, 1.0 / 720);
-    p = fma(p, r, 1.0 / 120);
-    p = fma(p, r, 1.0 / 24);
-    p = fma(p, r, 1.0 / 6);
-    p = fma(p, r, 0.5);
-    p = fma(p, r, 1.0);
-    const int n = __double2loint(t);
-    const double T = kExp2Tab[n & 15];
-    const double v = fma(T * r, p, T);
-    return __hiloint2double(__double2hiint(v) + ((n >> 4) << 20), __double2loint(v));
 }
 
 // An atom's per-step FP64 state

@@ -1,6 +1,7 @@
-"""The GB energy's pair kernels at the edges of their tiles: near pairs (half
-of the warp steps of these small chains meet one) evaluated apart from the tile
-loop, with work items of 2 j-tiles (one replica) and of 16 (1300 replicas)."""
+"""The GB energy and its gradient at the edges of their kernels: the cluster
+kernel for small replicas, and the symmetric pair kernels, whose near pairs (half
+of the warp steps of small chains meet one) are evaluated apart from the tile
+loop, with work items of 2 to 16 j-tiles."""
 import numpy as np
 import pytest
 
@@ -22,9 +23,10 @@ def _rel(a, b):
 @pytest.mark.parametrize("rgbmax", [0.0, 9.0])
 @pytest.mark.parametrize("n", [2, 31, 33, 64, 65, 255, 257, 300])
 def test_energy_and_gradient_at_tile_edges(n, rgbmax):
-    """Both item sizes against the oracle, at the repository's bars (energy
-    1e-6, gradients 1e-5 RMS relative); the two sum the same FP32 pair terms in
-    another order, so they agree to a few roundings (2e-6)."""
+    """One replica and 1300 against the oracle, at the repository's bars (energy
+    1e-6, gradients 1e-5 RMS relative); where the two run different kernels they
+    sum the same FP32 pair terms in another order, so they agree to a few
+    roundings (2e-6)."""
     import torch
     s, x, q, rho = synth.config_c5(n_rep=1300, n=n, seed=90 + n)
     gb = cphremd.default_gb()
@@ -45,3 +47,22 @@ def test_energy_and_gradient_at_tile_edges(n, rgbmax):
         for a, b, o in zip(g, g1, go):
             assert _rel(a[r], o) <= 1e-5 and _rel(b, o) <= 1e-5
             assert _rel(a[r], b) <= 2e-6
+
+
+@pytest.mark.parametrize("n,n_rep", [(512, 1), (513, 1), (544, 2), (577, 1), (801, 3), (33, 24000), (65, 6000)])
+def test_symmetric_kernels_at_tile_edges(n, n_rep):
+    """Past the cluster kernel's sizes: work items of 2 j-tiles (a few replicas
+    of over 512 atoms) and of 8 or 16 (many small ones); 512 is its largest."""
+    import torch
+    s, x, q, rho = synth.config_c5(n_rep=n_rep, n=n, seed=70 + n)
+    t = [torch.tensor(a, dtype=torch.float32, device="cuda:0") for a in (x, q, rho)]
+    scr = torch.tensor(s.screen, dtype=torch.float32, device="cuda:0")
+    up = torch.ones(n_rep, dtype=torch.float64, device="cuda:0")
+    E = cphremd.gb_energy(*t, scr).cpu().numpy()
+    g = [a.cpu().numpy().astype(np.float64) for a in cphremd.gb_energy_backward(*t, scr, up)]
+    for r in {0, n_rep - 1}:
+        Eo, *go = oracle.gb_grad(*(a[r].astype(np.float32).astype(np.float64) for a in (x, q, rho)),
+                                 s.screen.astype(np.float32).astype(np.float64))
+        assert abs(E[r] - Eo) <= 1e-6 * abs(Eo), (r, E[r], Eo)
+        for a, o in zip(g, go):
+            assert _rel(a[r], o) <= 1e-5

@@ -136,21 +136,118 @@ __device__ __forceinline__ long long warp_sum(long long v) {
 // ------------------------------------------------ FP64 in few instructions
 // A warp instruction of FP64 holds a sub-partition of GB300 for 64 clocks, with
 // one active lane or with 32.
-// 1 / x for normal x: the PTX approximation (20 bits) and two Newton steps
+// 1 / x for normal x: the PTX approximation (20 bits) and one step of third
+// order, y (1 + e + e^2) with e = 1 - x y
 __device__ __forceinline__ double rcp64(double x) {
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    y = fma(fma(-x, y, 1.0), y, y);
-    return fma(fma(-x, y, 1.0), y, y);
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
 }
 
-// 2^(j/16)
-static __constant__ double kExp2Tab[16] = {1.0, 1.0442737824274138, 1.0905077326652577, 1.1387886347566916, 1.189207115002721, 1.241857812073484, 1.2968395546510096, 1.3542555469368927, 1.4142135623730951, 1.4768261459394993, 1.5422108254079407, 1.6104903319492543, 1.681792830507429, 1.7562521603732995, 1.8340080864093424, 1.9152065613971474};
+// 1 / sqrt(x) for normal x > 0: the same with y (1 + e/2 + 3 e^2/8), e = 1 - x y^2
+__device__ __forceinline__ double rsqrt64(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x * y, y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
+}
 
-// e^x for -700 < x <= 0 (smaller x: e^-700): x = k ln2/16 + r, a Taylor series in
-// r (|r| <= 0.022, remainder 1e-18) and the table
-__device__ __forceinline__ double exp64(double x) {
-    x = fmax(x, -700.0);
+// Tables of log64 and exp64, to be copied to shared memory (divergent indices):
+// for the j-th of 128 intervals of m in [0.6875, 1.375) an approximate 1/c of its
+// middle c and -log of that number; then 2^(j/16), two to an entry.
+constexpr int kTab64 = 136;
+static __device__ const double2 kTab64Values[kTab64] = {
+    {1.4504249291784703, -0.37185656810621104}, {1.4422535211267606, -0.36620683556409206},
+    {1.4341736694677871, -0.36058884325986873}, {1.426183844011142, -0.3550022365512289},
+    {1.4182825484764543, -0.3494466667066269}, {1.4104683195592287, -0.343921790774657},
+    {1.4027397260273973, -0.3384272714570163}, {1.3950953678474114, -0.3329627769849375},
+    {1.3875338753387534, -0.3275279809989806}, {1.3800539083557952, -0.3221225624320727},
+    {1.3726541554959786, -0.31674620539569226}, {1.3653333333333333, -0.31139859906909695},
+    {1.3580901856763925, -0.306079437591497}, {1.3509234828496042, -0.3007884199570814},
+    {1.3438320209973753, -0.2955252499128068}, {1.3368146214099217, -0.2902896358588618},
+    {1.3298701298701299, -0.28508129075172356}, {1.322997416020672, -0.279899932009726},
+    {1.3161953727506426, -0.2747452814210614}, {1.3094629156010231, -0.26961706505414207},
+    {1.3027989821882953, -0.2645150131702466}, {1.2962025316455696, -0.2594388601383859},
+    {1.2896725440806045, -0.25438834435231733}, {1.2832080200501252, -0.24936320814964427},
+    {1.2768079800498753, -0.24436319773293858}, {1.2704714640198511, -0.23938806309282482},
+    {1.2641975308641975, -0.23443755793296864}, {1.257985257985258, -0.22951143959691278},
+    {1.2518337408312958, -0.22460946899670603}, {1.245742092457421, -0.2197314105432732},
+    {1.2397094430992737, -0.21487703207847508}, {1.2337349397590363, -0.21004610480880959},
+    {1.2278177458033572, -0.20523840324070627}, {1.2219570405727924, -0.2004537051173701},
+    {1.2161520190023754, -0.19569179135712642}, {1.210401891252955, -0.1909524459932298},
+    {1.204705882352941, -0.18623545611509087}, {1.199063231850117, -0.18154061181088324},
+    {1.1934731934731935, -0.1768677061114908}, {1.1879350348027842, -0.17221653493575995},
+    {1.1824480369515011, -0.16758689703701793}, {1.1770114942528735, -0.16297859395082367},
+    {1.17162471395881, -0.15839142994391764}, {1.1662870159453302, -0.15382521196433638},
+    {1.1609977324263039, -0.14927974959266183}, {1.1557562076749435, -0.14475485499437207},
+    {1.150561797752809, -0.14025034287326765}, {1.145413870246085, -0.13576603042593893},
+    {1.1403118040089086, -0.13130173729725345}, {1.1352549889135255, -0.12685728553682943},
+    {1.130242825607064, -0.12243249955647377}, {1.1252747252747253, -0.11802720608855737},
+    {1.1203501094091903, -0.11364123414530306}, {1.1154684095860568, -0.10927441497896273},
+    {1.1106290672451193, -0.10492658204285929}, {1.1058315334773219, -0.10059757095327378},
+    {1.1010752688172043, -0.09628721945215148}, {1.0963597430406853, -0.09199536737061052},
+    {1.091684434968017, -0.0877218565932284}, {1.0870488322717622, -0.08346653102309001},
+    {1.0824524312896406, -0.07922923654757486}, {1.0778947368421052, -0.07500982100486656},
+    {1.0733752620545074, -0.07080813415116662}, {1.068893528183716, -0.06662402762859244},
+    {1.0644490644490645, -0.06245735493374666}, {1.060041407867495, -0.05830797138693517},
+    {1.0556701030927835, -0.054175734102024614}, {1.051334702258727, -0.05006050195691803},
+    {1.047034764826176, -0.04596213556463585}, {1.0427698574338085, -0.04188049724498711},
+    {1.0385395537525355, -0.037815450996817664}, {1.0343434343434343, -0.033766862470817484},
+    {1.0301810865191148, -0.029734598942879144}, {1.0260521042084167, -0.025718529287989036},
+    {1.0219560878243512, -0.021718523954642903}, {1.0178926441351888, -0.017734454939768475},
+    {1.0138613861386139, -0.01376619576414797}, {1.009861932938856, -0.00981362144832467},
+    {1.005893909626719, -0.005876608488984971}, {1.0019569471624266, -0.001955034835803295},
+    {0.9961089494163424, 0.003898640415657309}, {0.9884169884169884, 0.01165061721997525},
+    {0.9808429118773946, 0.019342962843130987}, {0.973384030418251, 0.026976587698202083},
+    {0.9660377358490566, 0.03455238150665973}, {0.9588014981273408, 0.042071213920687044},
+    {0.9516728624535316, 0.049533935122276676}, {0.9446494464944649, 0.05694137640013845},
+    {0.9377289377289377, 0.06429435070539725}, {0.9309090909090909, 0.07159365318700882},
+    {0.924187725631769, 0.078840061707776}, {0.9175627240143369, 0.08603433734180316},
+    {0.9110320284697508, 0.09317722485418334}, {0.9045936395759717, 0.10026945316367517},
+    {0.8982456140350877, 0.10731173578908804}, {0.89198606271777, 0.11430477128005863},
+    {0.8858131487889274, 0.12124924363286965}, {0.8797250859106529, 0.12814582269193006},
+    {0.8737201365187713, 0.13499516453750482}, {0.8677966101694915, 0.1417979118602574},
+    {0.8619528619528619, 0.1485546943231372}, {0.8561872909698997, 0.15526612891112396},
+    {0.8504983388704319, 0.16193282026931324}, {0.8448844884488449, 0.16855536102980664},
+    {0.839344262295082, 0.17513433212784915}, {0.8338762214983714, 0.18167030310763463},
+    {0.8284789644012945, 0.18816383241818294}, {0.8231511254019293, 0.19461546769967167},
+    {0.8178913738019169, 0.2010257460605908}, {0.8126984126984127, 0.2073951943460706},
+    {0.807570977917981, 0.21372432939771818}, {0.8025078369905956, 0.22001365830528213},
+    {0.7975077881619937, 0.2262636786504534}, {0.7925696594427245, 0.232474878743094},
+    {0.7876923076923077, 0.238647737850175}, {0.7828746177370031, 0.24478272641769092},
+    {0.7781155015197568, 0.25088030628580943}, {0.7734138972809668, 0.2569409308975004},
+    {0.7687687687687688, 0.26296504550088134}, {0.764179104477612, 0.26895308734550394},
+    {0.7596439169139466, 0.2749054858727992}, {0.7551622418879056, 0.2808226629008878},
+    {0.750733137829912, 0.2867050328039543}, {0.7463556851311953, 0.29255300268637746},
+    {0.7420289855072464, 0.2983669725517973}, {0.7377521613832853, 0.3041473354672968},
+    {0.7335243553008596, 0.3098944777228647}, {0.7293447293447294, 0.3156087789863033},
+    {1.0, 1.0442737824274138}, {1.0905077326652577, 1.1387886347566916}, {1.189207115002721, 1.241857812073484}, {1.2968395546510096, 1.3542555469368927}, {1.4142135623730951, 1.4768261459394993}, {1.5422108254079407, 1.6104903319492543}, {1.681792830507429, 1.7562521603732995}, {1.8340080864093424, 1.9152065613971474}};
+
+__device__ __forceinline__ void load_tab64(double2* tab, int tid, int n) {
+    for (int k = tid; k < kTab64; k += n) tab[k] = kTab64Values[k];
+}
+
+// log(x), x normal and positive (Tang, 1990): x = 2^e m, r = m/c - 1 (|r| < 0.006),
+// log x = e ln2 + log c + log1p(r); the series stops at r^7/7 < 1e-16 |r|.
+__device__ __forceinline__ double log64(double x, const double2* tab) {
+    const int i = __double2hiint(x) - 0x3fe60000;
+    const double2 c = tab[(i >> 13) & 127];
+    const double m = __hiloint2double(__double2hiint(x) - (i & 0xfff00000), __double2loint(x));
+    const double r = fma(m, c.x, -1.0);
+    const double e = __hiloint2double(0x43300000, (i >> 20) + 1024) - 4503599627371520.0; // 2^52 + 1024
+    double p = fma(r, 1.0 / 7, -1.0 / 6);
+    p = fma(p, r, 1.0 / 5);
+    p = fma(p, r, -0.25);
+    p = fma(p, r, 1.0 / 3);
+    p = fma(p, r, -0.5);
+    return fma(e, 0.6931471805599453, c.y + fma(r * r, p, r));
+}
+
+// e^x for x <= 0 (0 below -700): x = k ln2/16 + r, a Taylor series in r (|r| <=
+// 0.022, remainder 1e-18) and the table.  T(j) = 2^(j/16).
+template <class T>
+__device__ __forceinline__ double exp64_with(double x, T&& table) {
     const double big = 6755399441055744.0; // 1.5 2^52: the sum's low word is the integer
     const double t = fma(x, 23.083120654223414, big);
     const double k = t - big;
@@ -163,9 +260,20 @@ __device__ __forceinline__ double exp64(double x) {
     p = fma(p, r, 0.5);
     p = fma(p, r, 1.0);
     const int n = __double2loint(t);
-    const double T = kExp2Tab[n & 15];
-    const double v = fma(T * r, p, T);
-    return __hiloint2double(__double2hiint(v) + ((n >> 4) << 20), __double2loint(v));
+    const double b = table(n & 15);
+    const double v = fma(b * r, p, b);
+    const bool zero = (unsigned)__double2hiint(x) > 0xc085e000u; // x < -700
+    return zero ? 0.0 : __hiloint2double(__double2hiint(v) + ((n >> 4) << 20), __double2loint(v));
+}
+
+__device__ __forceinline__ double exp64(double x, const double2* tab) {
+    return exp64_with(x, [&](int j) { return reinterpret_cast<const double*>(tab + 128)[j]; });
+}
+
+// 2^(j/16), for the few evaluations that do not load the tables
+static __constant__ double kExp2Tab[16] = {1.0, 1.0442737824274138, 1.0905077326652577, 1.1387886347566916, 1.189207115002721, 1.241857812073484, 1.2968395546510096, 1.3542555469368927, 1.4142135623730951, 1.4768261459394993, 1.5422108254079407, 1.6104903319492543, 1.681792830507429, 1.7562521603732995, 1.8340080864093424, 1.9152065613971474};
+__device__ __forceinline__ double exp64(double x) {
+    return exp64_with(x, [&](int j) { return kExp2Tab[j]; });
 }
 
 // ---------------------------------------------- MUFU approximations (FP32)
@@ -351,6 +459,31 @@ __device__ __forceinline__ float hct_drt(float r, float rt, float irt, float s, 
         d = (a * a - s * s) * 0.5f * __fdividef(1.f, r) * irt * irt * irt;
     }
     return d;
+}
+
+// --------------------------------------- HCT, FP64, of the pair kernels
+// The closed forms below with one reciprocal and the short logarithm.  r2 = r^2.
+__device__ __forceinline__ double hct64(double r, double r2, double rinv, double rt, double irt, double s, double rc,
+                                        const double2* tab) {
+    const double U = fmin(r + s, rc), L = fmax(rt, fabs(r - s));
+    double h = 0.0;
+    if (L < U) {
+        const double iLU = rcp64(L * U), iL = U * iLU, iU = L * iLU, q = 0.25 * rinv;
+        h = fma(iL - iU, fma((iL + iU) * q, fma(s, s, -r2), 1.0), 0.5 * rinv * log64(L * iU, tab));
+    }
+    if (rt < s - r) {
+        const double top = fmin(s - r, rc);
+        if (rt < top) h += 2.0 * (irt - rcp64(top));
+    }
+    return h;
+}
+
+// - dH/dr
+__device__ __forceinline__ double hct_mdr64(double r, double rinv2, double rt, double s, double rc, const double2* tab) {
+    const double U = fmin(r + s, rc), L = fmax(rt, fabs(r - s));
+    if (!(L < U)) return 0.0;
+    const double iLU = rcp64(L * U), iL = U * iLU, iU = L * iLU;
+    return fma(0.25 * ((iL - iU) * (iL + iU)), fma(s * s, rinv2, 1.0), 0.5 * rinv2 * log64(L * iU, tab));
 }
 
 // ------------------------------------------------------------- HCT, FP64

@@ -16,6 +16,7 @@
 
 #include "cph_kernels.cuh"
 #include "cph_sym.cuh"
+#include "cph_f64.cuh"
 #include "cph_small.cuh"
 
 namespace cph {
@@ -762,50 +763,42 @@ bool sys_ordered(const cph_engine* E, int s) {
 // The ordered passes run one warp per atom (four atoms per CTA), or, in FP64
 // mode with few atoms (E->ordered_wpa = 4), four warps per atom: even a single
 // small walker then spreads its FP64 work over one CTA per atom.
-// f with the passes' precision, warps per atom and operand source: FP64 (one
-// or four warps), FP32 from the staged operands or from the master arrays (one)
-template <class F>
-void by_form(const cph_engine* E, F&& f) {
-    using One = std::integral_constant<int, 1>;
-    using Four = std::integral_constant<int, 4>;
+// f with the warps per atom (FP64 mode) or the operand source (FP32 mode) as a constant
+template <class F, class G>
+void by_form(const cph_engine* E, F&& f64, G&& f32) {
     if (E->precision == CPH_PREC_FP64) {
-        if (E->ordered_wpa == 4) f(double{}, Four{}, std::false_type{});
-        else f(double{}, One{}, std::false_type{});
-    } else if (E->staged) f(float{}, One{}, std::true_type{});
-    else f(float{}, One{}, std::false_type{});
+        if (E->ordered_wpa == 4) f64(std::integral_constant<int, 4>{});
+        else f64(std::integral_constant<int, 1>{});
+    } else if (E->staged) f32(std::true_type{});
+    else f32(std::false_type{});
 }
 
 int launch_born(cph_engine* E, const Item* items, int n, bool zero_energy, cudaStream_t st) {
     if (n <= 0) return CPH_OK;
-    by_form(E, [&](auto real, auto wpa, auto staged) {
-        k_born<decltype(real), decltype(wpa)::value, decltype(staged)::value><<<n, kTile, 0, st>>>(items, E->V, zero_energy ? 1 : 0);
-    });
+    const int ze = zero_energy ? 1 : 0;
+    by_form(
+        E, [&](auto wpa) { k_born64<decltype(wpa)::value><<<n, kTile, 0, st>>>(items, E->V, ze); },
+        [&](auto staged) { k_born<decltype(staged)::value><<<n, kTile, 0, st>>>(items, E->V, ze); });
     CK(cudaGetLastError());
     return CPH_OK;
 }
 
 int launch_gb(cph_engine* E, const Item* items, int n, bool energy, cudaStream_t st) {
     if (n <= 0) return CPH_OK;
-    by_form(E, [&](auto real, auto wpa, auto staged) {
-        using R = decltype(real);
-        constexpr int WPA = decltype(wpa)::value;
-        constexpr bool ST = decltype(staged)::value;
-        if (energy) k_gb<R, true, WPA, ST><<<n, kTile, 0, st>>>(items, E->V);
-        else k_gb<R, false, WPA, ST><<<n, kTile, 0, st>>>(items, E->V);
-    });
+    auto go = [&](auto kernel) { kernel<<<n, kTile, 0, st>>>(items, E->V); };
+    by_form(
+        E, [&](auto wpa) { energy ? go(k_gb64<true, decltype(wpa)::value>) : go(k_gb64<false, decltype(wpa)::value>); },
+        [&](auto staged) { energy ? go(k_gb<true, decltype(staged)::value>) : go(k_gb<false, decltype(staged)::value>); });
     CK(cudaGetLastError());
     return CPH_OK;
 }
 
 int launch_chain(cph_engine* E, const Item* items, int n, bool energy, cudaStream_t st) {
     if (n <= 0) return CPH_OK;
-    by_form(E, [&](auto real, auto wpa, auto staged) {
-        using R = decltype(real);
-        constexpr int WPA = decltype(wpa)::value;
-        constexpr bool ST = decltype(staged)::value;
-        if (energy) k_chain<R, true, WPA, ST><<<n, kTile, 0, st>>>(items, E->V);
-        else k_chain<R, false, WPA, ST><<<n, kTile, 0, st>>>(items, E->V);
-    });
+    auto go = [&](auto kernel) { kernel<<<n, kTile, 0, st>>>(items, E->V); };
+    by_form(
+        E, [&](auto wpa) { energy ? go(k_chain64<true, decltype(wpa)::value>) : go(k_chain64<false, decltype(wpa)::value>); },
+        [&](auto staged) { energy ? go(k_chain<true, decltype(staged)::value>) : go(k_chain<false, decltype(staged)::value>); });
     CK(cudaGetLastError());
     return CPH_OK;
 }

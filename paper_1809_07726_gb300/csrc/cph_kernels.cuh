@@ -178,9 +178,11 @@ __device__ inline void tile_masks(const View& V, int P, int i, bool vi, int j0, 
 // ------------------------------------------------------------- pass 1: Born radii
 // psi_i = rt_i/2 sum_{j != i} H(r_ij, rt_i, s_j); R_i = 1/(1/rt_i - tanh(theta)/rho_i)
 // with theta = alpha psi - beta psi^2 + gamma psi^3, finalised in FP64.
-template <class Real, int WPA, bool STAGED>
+template <bool STAGED>
 __global__ void __launch_bounds__(kTile) k_born(const Item* __restrict__ items, View V,
                                                 int zero_energy) {
+    using Real = float;
+    constexpr int WPA = 1;
     using Pr = Prec<Real>;
     __shared__ J4<Real> sj[kTile];
     const Item it = items[blockIdx.x];
@@ -278,8 +280,10 @@ __global__ void __launch_bounds__(kTile) k_born(const Item* __restrict__ items, 
 // ------------------------------------------- pass 2: GB + Coulomb + LJ pair pass
 // Owner i accumulates the direct force, dE_GB/dR_i and (optionally) its share
 // of the energies; the epilogue turns dE/dR_i into c_i = dE/dR_i dR_i/dpsi_i rt_i/2.
-template <class Real, bool ENERGY, int WPA, bool STAGED>
+template <bool ENERGY, bool STAGED>
 __global__ void __launch_bounds__(kTile) k_gb(const Item* __restrict__ items, View V) {
+    using Real = float;
+    constexpr int WPA = 1;
     using Pr = Prec<Real>;
     using Acc = typename Pr::Acc;
     __shared__ J4<Real> sa[kTile];
@@ -499,9 +503,9 @@ __device__ inline void bonded_atom(const View& V, int A, int P, int li, int lane
         const int o = (ia == li) ? ib : ia;
         double d[3];
         for (int c = 0; c < 3; ++c) d[c] = x[3 * (A + li) + c] - x[3 * (A + o) + c];
-        const double r = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-        const double dr = r - V.bond_r0[b];
-        const double g = 2.0 * V.bond_k[b] * dr / r; // one FP64 division per bond
+        const double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2], ir = rsqrt64(r2);
+        const double dr = r2 * ir - V.bond_r0[b];
+        const double g = 2.0 * V.bond_k[b] * dr * ir;
         for (int c = 0; c < 3; ++c) F[c] -= g * d[c];
         if (ia == li) eb += V.bond_k[b] * dr * dr;
     }
@@ -515,13 +519,12 @@ __device__ inline void bonded_atom(const View& V, int A, int P, int li, int lane
         }
         const double ru2 = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
         const double rv2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
-        // three FP64 divisions per angle (FP64 arithmetic is scarce on GB300)
-        const double iuv = 1.0 / sqrt(ru2 * rv2), iru2 = 1.0 / ru2, irv2 = 1.0 / rv2;
+        const double iuv = rsqrt64(ru2 * rv2), iru2 = rcp64(ru2), irv2 = rcp64(rv2);
         double cs = (u[0] * v[0] + u[1] * v[1] + u[2] * v[2]) * iuv;
         cs = fmin(1.0, fmax(-1.0, cs));
         const double th = acos(cs);
         const double dth = th - V.ang_t0[a];
-        const double k = -2.0 * V.ang_k[a] * dth / sqrt(fmax(1e-300, 1.0 - cs * cs)); // dE/dcos
+        const double k = -2.0 * V.ang_k[a] * dth * rsqrt64(fmax(1e-300, 1.0 - cs * cs)); // dE/dcos
         double gi[3], gk[3];
         for (int c = 0; c < 3; ++c) {
             gi[c] = k * (v[c] * iuv - cs * u[c] * iru2);
@@ -624,8 +627,10 @@ __device__ inline void bonded_atom32(const View& V, int A, int P, int li, int la
 // ------------------------------------------ pass 3: chain rule through Born radii
 // F_i -= sum_j (c_i dH(r; rt_i, s_j)/dr + c_j dH(r; rt_j, s_i)/dr) (x_i - x_j)/r,
 // then the direct pair force and the bonded terms are added: F is the total force.
-template <class Real, bool ENERGY, int WPA, bool STAGED>
+template <bool ENERGY, bool STAGED>
 __global__ void __launch_bounds__(kTile) k_chain(const Item* __restrict__ items, View V) {
+    using Real = float;
+    constexpr int WPA = 1;
     using Pr = Prec<Real>;
     using Acc = typename Pr::Acc;
     __shared__ J4<Real> sa[kTile];
@@ -726,20 +731,12 @@ __global__ void __launch_bounds__(kTile) k_chain(const Item* __restrict__ items,
     double eb = 0.0, ea = 0.0;
     double Fb[3] = {0.0, 0.0, 0.0};
     // bonded terms of atom i over the group's threads, summed in a fixed order
-    if constexpr (sizeof(Real) == 4) {
-        float fb[3] = {0.f, 0.f, 0.f}, ebf = 0.f, eaf = 0.f;
-        if (vi) bonded_atom32(V, A, P, i, sub, 32 * WPA, fb, ebf, eaf);
+    float fb[3] = {0.f, 0.f, 0.f}, ebf = 0.f, eaf = 0.f;
+    if (vi) bonded_atom32(V, A, P, i, sub, 32 * WPA, fb, ebf, eaf);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) Fb[c] = (double)group_total<WPA>(fb[c], gsh);
-        eb = (double)group_total<WPA>(ebf, gsh);
-        ea = (double)group_total<WPA>(eaf, gsh);
-    } else {
-        if (vi) bonded_atom(V, A, P, i, sub, 32 * WPA, Fb, eb, ea);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) Fb[c] = group_total<WPA>(Fb[c], gsh);
-        eb = group_total<WPA>(eb, gsh);
-        ea = group_total<WPA>(ea, gsh);
-    }
+    for (int c = 0; c < 3; ++c) Fb[c] = (double)group_total<WPA>(fb[c], gsh);
+    eb = (double)group_total<WPA>(ebf, gsh);
+    ea = (double)group_total<WPA>(eaf, gsh);
     if (sub != 0) eb = ea = 0.0; // the group's totals, counted once
     if (vi && sub == 0) {
         double F[3] = {V.Fd[3 * (A + i)] + Pr::value(fx, kScaleE) + Fb[0],

@@ -65,6 +65,7 @@ __device__ inline bool mc_excluded(const View& V, int P, int at, int an) {
 
 template <class Real>
 __global__ void __launch_bounds__(kMcThreads) k_mc_site(View V, int kind, int s_off, int w_begin) {
+    pdl_sync();
     using Pr = Prec<Real>;
     using Acc = typename Pr::Acc;
     const int w = w_begin + blockIdx.y, k = blockIdx.x;
@@ -231,6 +232,7 @@ __global__ void __launch_bounds__(kMcThreads) k_mc_site(View V, int kind, int s_
 
 template <class Real>
 __global__ void __launch_bounds__(kMcThreads) k_mc_sweep(View V, int kind, int clear_others, int w_begin) {
+    pdl_sync();
     using Pr = Prec<Real>;
     using Acc = typename Pr::Acc;
     const int w = w_begin + blockIdx.x;
@@ -362,19 +364,8 @@ constexpr int kObsThreads = 64;
 
 // one CTA per walker, threads over its sites
 __global__ void __launch_bounds__(kObsThreads) k_observe(View V) {
-    const int w = blockIdx.x;
-    if (!V.w_local[w]) return; // a sharded grid's counts are summed over its engines
-    const int s = V.slot_of[w];
-    if (threadIdx.x == 0) {
-        V.visits[(long long)w * V.W + s] += 1;
-        if (w == V.first_local) *V.n_obs += 1;
-    }
-    // the walker at slot s belongs to the system of the walker that started
-    // there, so slot s's rows are laid out like walker s's sites
-    const int ws0 = V.w_site_off[w], n = V.w_site_off[w + 1] - ws0;
-    const long long row0 = V.w_site_off[s];
-    for (int k = threadIdx.x; k < n; k += kObsThreads)
-        V.occ[(row0 + k) * CPH_MAX_STATES + V.site_state[ws0 + k]] += 1;
+    pdl_sync();
+    observe_walker(V, blockIdx.x, threadIdx.x, kObsThreads);
 }
 
 // =====================================================================
@@ -401,6 +392,7 @@ __device__ inline int walker_nelec(const View& V, int w) {
 // N_H and N_e of its site states, and the two sums the semi-grand T-exchange
 // energy needs: sum_k U_ref,k(s_k) and sum over redox sites of N_e,k(s_k) E0_ref,k.
 __global__ void k_exchange_rows(View V) {
+    pdl_sync();
     const int w = blockIdx.x * blockDim.x + threadIdx.x;
     if (w >= V.W || !V.w_local[w]) return;
     long long u = 0;
@@ -437,6 +429,7 @@ __device__ inline double row_energy(const View& V, const cph_exchange_row& r, do
 constexpr int kExThreads = 256;
 
 __global__ void __launch_bounds__(kExThreads) k_exchange(View V, int dim_req, int s_off) {
+    pdl_sync();
     __shared__ int sdim, spar;
     const int tid = threadIdx.x;
     const uint64_t t = (uint64_t)(*V.step + s_off);
@@ -753,6 +746,25 @@ bool finite_all(const double* p, size_t n) {
 // At most this many atoms on the FP64 ordered passes: four warps per atom.
 constexpr long long kOrderedFewAtoms = 2048;
 
+// A launch that may be set up while the one before it on the stream still runs
+// (every kernel launched so begins with pdl_sync).  A step is a chain of launches
+// of a few microseconds: 100 steps of the 160-atom FP64 walker 6.23 -> 5.35 ms, 20
+// steps of one 2003-atom walker 2.13 -> 1.88 ms, 10 steps of 64 x 2400 atoms 10.45
+// -> 10.21 ms.
+template <class... P, class... A>
+void launch_next(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, P(args)...); // the caller checks cudaGetLastError
+}
+
 // Whether walkers of system s run the ordered passes (one warp per atom i):
 // always in FP64 mode, by the system's tile shape in FP32 mode.
 bool sys_ordered(const cph_engine* E, int s) {
@@ -777,15 +789,15 @@ int launch_born(cph_engine* E, const Item* items, int n, bool zero_energy, cudaS
     if (n <= 0) return CPH_OK;
     const int ze = zero_energy ? 1 : 0;
     by_form(
-        E, [&](auto wpa) { k_born64<decltype(wpa)::value><<<n, kTile, 0, st>>>(items, E->V, ze); },
-        [&](auto staged) { k_born<decltype(staged)::value><<<n, kTile, 0, st>>>(items, E->V, ze); });
+        E, [&](auto wpa) { launch_next(k_born64<decltype(wpa)::value>, n, kTile, st, items, E->V, ze); },
+        [&](auto staged) { launch_next(k_born<decltype(staged)::value>, n, kTile, st, items, E->V, ze); });
     CK(cudaGetLastError());
     return CPH_OK;
 }
 
 int launch_gb(cph_engine* E, const Item* items, int n, bool energy, cudaStream_t st) {
     if (n <= 0) return CPH_OK;
-    auto go = [&](auto kernel) { kernel<<<n, kTile, 0, st>>>(items, E->V); };
+    auto go = [&](auto kernel) { launch_next(kernel, n, kTile, st, items, E->V); };
     by_form(
         E, [&](auto wpa) { energy ? go(k_gb64<true, decltype(wpa)::value>) : go(k_gb64<false, decltype(wpa)::value>); },
         [&](auto staged) { energy ? go(k_gb<true, decltype(staged)::value>) : go(k_gb<false, decltype(staged)::value>); });
@@ -795,7 +807,7 @@ int launch_gb(cph_engine* E, const Item* items, int n, bool energy, cudaStream_t
 
 int launch_chain(cph_engine* E, const Item* items, int n, bool energy, cudaStream_t st) {
     if (n <= 0) return CPH_OK;
-    auto go = [&](auto kernel) { kernel<<<n, kTile, 0, st>>>(items, E->V); };
+    auto go = [&](auto kernel) { launch_next(kernel, n, kTile, st, items, E->V); };
     by_form(
         E, [&](auto wpa) { energy ? go(k_chain64<true, decltype(wpa)::value>) : go(k_chain64<false, decltype(wpa)::value>); },
         [&](auto staged) { energy ? go(k_chain<true, decltype(staged)::value>) : go(k_chain<false, decltype(staged)::value>); });
@@ -849,12 +861,14 @@ int launch_small(cph_engine* E, bool energy, int s_off, int steps, int start, in
         cfg.blockDim = dim3(32 * (E->small_warps + kSmallAux));
         cfg.dynamicSmemBytes = E->small_smem;
         cfg.stream = s;
-        cudaLaunchAttribute at[1];
+        cudaLaunchAttribute at[2];
         at[0].id = cudaLaunchAttributeClusterDimension;
         at[0].val.clusterDim.x = kSmallRanks;
         at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[1].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = at;
-        cfg.numAttrs = 1;
+        cfg.numAttrs = 2;
         const SmallRun run{w0, E->small_warps, s_off, steps, start, end, zero_energy ? 1 : 0};
         cudaError_t ce = cudaSuccess;
         by_small(E, energy, [&](auto kernel) { ce = cudaLaunchKernelEx(&cfg, kernel, E->V, E->small_tab, run); });
@@ -885,10 +899,10 @@ int launch_mc(cph_engine* E, int kinds, int s_off, cudaStream_t st) {
             if (first_x) TRY(launch_stage(E, 0, 0, E->V.total_atoms, st));
             if (again) TRY(launch_stage(E, 1, 0, E->V.total_atoms, st));
             const dim3 g1(E->max_sites, W);
-            if (f32) k_mc_site<float><<<g1, kMcThreads, 0, st>>>(E->V, kind, s_off, 0);
-            else k_mc_site<double><<<g1, kMcThreads, 0, st>>>(E->V, kind, s_off, 0);
-            if (f32) k_mc_sweep<float><<<W, kMcThreads, 0, st>>>(E->V, kind, first, 0);
-            else k_mc_sweep<double><<<W, kMcThreads, 0, st>>>(E->V, kind, first, 0);
+            if (f32) launch_next(k_mc_site<float>, g1, kMcThreads, st, E->V, kind, s_off, 0);
+            else launch_next(k_mc_site<double>, g1, kMcThreads, st, E->V, kind, s_off, 0);
+            if (f32) launch_next(k_mc_sweep<float>, W, kMcThreads, st, E->V, kind, first, 0);
+            else launch_next(k_mc_sweep<double>, W, kMcThreads, st, E->V, kind, first, 0);
         } else {
             TRY(fan_out(E, st));
             for (int w = 0; w < W; ++w) {
@@ -896,10 +910,10 @@ int launch_mc(cph_engine* E, int kinds, int s_off, cudaStream_t st) {
                 cudaStream_t s = lane_stream(E, w, st);
                 if (first_x) TRY(launch_stage(E, 0, E->h_w_off[w], E->h_w_off[w + 1] - E->h_w_off[w], s));
                 if (again) TRY(launch_stage(E, 1, E->h_w_off[w], E->h_w_off[w + 1] - E->h_w_off[w], s));
-                if (f32) k_mc_site<float><<<E->max_sites, kMcThreads, 0, s>>>(E->V, kind, s_off, w);
-                else k_mc_site<double><<<E->max_sites, kMcThreads, 0, s>>>(E->V, kind, s_off, w);
-                if (f32) k_mc_sweep<float><<<1, kMcThreads, 0, s>>>(E->V, kind, first, w);
-                else k_mc_sweep<double><<<1, kMcThreads, 0, s>>>(E->V, kind, first, w);
+                if (f32) launch_next(k_mc_site<float>, E->max_sites, kMcThreads, s, E->V, kind, s_off, w);
+                else launch_next(k_mc_site<double>, E->max_sites, kMcThreads, s, E->V, kind, s_off, w);
+                if (f32) launch_next(k_mc_sweep<float>, 1, kMcThreads, s, E->V, kind, first, w);
+                else launch_next(k_mc_sweep<double>, 1, kMcThreads, s, E->V, kind, first, w);
             }
             TRY(fan_in(E, st));
         }
@@ -918,7 +932,7 @@ int launch_sym_pair(cph_engine* E, const SymItem* items, int n, bool energy, int
     const bool cut = E->V.rgbmax < INFINITY, salt = E->V.kappa > 0;
     auto launch = [&](auto gg) {
         constexpr int GG = decltype(gg)::value;
-        auto go = [&](auto kernel) { kernel<<<n, kSymThreads, 0, st>>>(items, E->V); };
+        auto go = [&](auto kernel) { launch_next(kernel, n, kSymThreads, st, items, E->V); };
         if (pass == 0) go(cut ? k_born_sym<true, GG> : k_born_sym<false, GG>);
         else if (pass == 2 && (GG < kSymG || E->queue_near)) go(cut ? k_chain_sym<true, GG, true> : k_chain_sym<false, GG, true>);
         else if (pass == 2) go(cut ? k_chain_sym<true, kSymG, false> : k_chain_sym<false, kSymG, false>);
@@ -937,8 +951,8 @@ int launch_sym_pair(cph_engine* E, const SymItem* items, int n, bool energy, int
 int launch_stage(cph_engine* E, int which, int a0, int n, cudaStream_t st) {
     const int bs = 256, g = (n + bs - 1) / bs;
     if (n <= 0) return CPH_OK;
-    if (which == 0) k_stage_x<<<g, bs, 0, st>>>(E->V, a0, n);
-    else k_stage_gb<<<g, bs, 0, st>>>(E->V, a0, n);
+    if (which == 0) launch_next(k_stage_x, g, bs, st, E->V, a0, n);
+    else launch_next(k_stage_gb, g, bs, st, E->V, a0, n);
     CK(cudaGetLastError());
     return CPH_OK;
 }
@@ -947,12 +961,12 @@ int launch_atoms(cph_engine* E, int which, bool energy, int a0, int n, cudaStrea
     const int bs = 256, g = (n + bs - 1) / bs;
     if (n <= 0) return CPH_OK;
     if (which == 2) {
-        k_fin_born<<<g, bs, 0, st>>>(E->V, a0, n, energy ? 1 : 0);
+        launch_next(k_fin_born, g, bs, st, E->V, a0, n, energy ? 1 : 0);
     } else if (which == 0) {
-        if (energy) k_fin_c<true><<<g, bs, 0, st>>>(E->V, a0, n);
-        else k_fin_c<false><<<g, bs, 0, st>>>(E->V, a0, n);
+        if (energy) launch_next(k_fin_c<true>, g, bs, st, E->V, a0, n);
+        else launch_next(k_fin_c<false>, g, bs, st, E->V, a0, n);
     } else {
-        k_final_forces<<<g, bs, 0, st>>>(E->V, a0, n);
+        launch_next(k_final_forces, g, bs, st, E->V, a0, n);
     }
     CK(cudaGetLastError());
     return CPH_OK;
@@ -961,8 +975,8 @@ int launch_atoms(cph_engine* E, int which, bool energy, int a0, int n, cudaStrea
 int launch_bonded(cph_engine* E, bool energy, int w0, int nw, cudaStream_t st) {
     if (E->max_terms <= 0 || nw <= 0) return CPH_OK;
     dim3 grid((E->max_terms + kBondedThreads - 1) / kBondedThreads, nw);
-    if (energy) k_bonded_terms<true><<<grid, kBondedThreads, 0, st>>>(E->V, w0);
-    else k_bonded_terms<false><<<grid, kBondedThreads, 0, st>>>(E->V, w0);
+    if (energy) launch_next(k_bonded_terms<true>, grid, kBondedThreads, st, E->V, w0);
+    else launch_next(k_bonded_terms<false>, grid, kBondedThreads, st, E->V, w0);
     CK(cudaGetLastError());
     return CPH_OK;
 }
@@ -1033,16 +1047,17 @@ int launch_forces(cph_engine* E, bool energy, cudaStream_t st, bool mc_between, 
     return CPH_OK;
 }
 
+// one sample of the observables and the Langevin step (and SHAKE)
 int launch_langevin(cph_engine* E, int s_off, cudaStream_t st) {
-    const int bs = 256;
+    const int batched = E->launch_mode == 0;
     auto one = [&](int a0, int n, cudaStream_t s) {
-        if (E->precision == CPH_PREC_FP32)
-            k_langevin<float><<<(n + bs - 1) / bs, bs, 0, s>>>(E->V, s_off, a0, n);
-        else
-            k_langevin<double><<<(n + bs - 1) / bs, bs, 0, s>>>(E->V, s_off, a0, n);
+        // few atoms: a warp to a block, so that each has a sub-partition's FP64 to itself
+        const int bs = n <= 32 * 152 ? 32 : 256, grid = (n + bs - 1) / bs, obs = batched ? E->V.W : 0;
+        if (E->precision == CPH_PREC_FP32) launch_next(k_langevin<float>, grid + obs, bs, s, E->V, s_off, a0, n, obs);
+        else launch_next(k_langevin<double>, grid + obs, bs, s, E->V, s_off, a0, n, obs);
     };
     auto shk = [&](int i0, int n, cudaStream_t s) {
-        if (n > 0) k_shake<<<(n + 127) / 128, 128, 0, s>>>(E->V, i0, n);
+        if (n > 0) launch_next(k_shake, (n + 127) / 128, 128, s, E->V, i0, n);
     };
     if (E->launch_mode == 0) {
         one(0, E->V.total_atoms, st);
@@ -1063,14 +1078,14 @@ int launch_langevin(cph_engine* E, int s_off, cudaStream_t st) {
 
 int launch_exchange_rows(cph_engine* E, cudaStream_t st) {
     const int bs = 128;
-    k_exchange_rows<<<(E->V.W + bs - 1) / bs, bs, 0, st>>>(E->V);
+    launch_next(k_exchange_rows, (E->V.W + bs - 1) / bs, bs, st, E->V);
     CK(cudaGetLastError());
     return CPH_OK;
 }
 
 // one exchange attempt from the rows in V.ex_rows (every walker's)
 int launch_exchange_only(cph_engine* E, int dim, int s_off, cudaStream_t st) {
-    k_exchange<<<1, kExThreads, 0, st>>>(E->V, dim, s_off);
+    launch_next(k_exchange, 1, kExThreads, st, E->V, dim, s_off);
     CK(cudaGetLastError());
     return CPH_OK;
 }
@@ -1081,13 +1096,13 @@ int launch_exchange(cph_engine* E, int dim, int s_off, cudaStream_t st) {
 }
 
 int launch_observe(cph_engine* E, cudaStream_t st) {
-    k_observe<<<E->V.W, kObsThreads, 0, st>>>(E->V);
+    launch_next(k_observe, E->V.W, kObsThreads, st, E->V);
     CK(cudaGetLastError());
     return CPH_OK;
 }
 
 int launch_tick(cph_engine* E, long long n, cudaStream_t st) {
-    k_tick<<<1, 1, 0, st>>>(E->V.step, n);
+    launch_next(k_tick, 1, 1, st, E->V.step, n);
     CK(cudaGetLastError());
     return CPH_OK;
 }
@@ -1103,7 +1118,7 @@ int enqueue_step(cph_engine* E, long long t, int s_off, bool full_schedule, cuda
     }
     TRY(launch_forces(E, exch, st, true, s_off, kinds));
     if (exch) TRY(launch_exchange(E, CPH_DIM_NEXT, s_off, st));
-    TRY(launch_observe(E, st));
+    if (E->launch_mode != 0) TRY(launch_observe(E, st));
     TRY(launch_langevin(E, s_off, st));
     return CPH_OK;
 }

@@ -65,6 +65,7 @@ __device__ __forceinline__ int place64() {
 
 template <int WPA>
 __global__ void __launch_bounds__(kTile) k_born64(const Item* __restrict__ items, View V, int zero_energy) {
+    pdl_sync();
     __shared__ J4<double> sj[kTile];
     __shared__ double2 tab[kTab64];
     __shared__ double red[16];
@@ -123,6 +124,7 @@ __global__ void __launch_bounds__(kTile) k_born64(const Item* __restrict__ items
 
 template <bool ENERGY, int WPA>
 __global__ void __launch_bounds__(kTile) k_gb64(const Item* __restrict__ items, View V) {
+    pdl_sync();
     constexpr int K = ENERGY ? 8 : 4;
     __shared__ J4<double> sa[kTile], sb[kTile];
     __shared__ double2 tab[kTab64];
@@ -245,6 +247,7 @@ __global__ void __launch_bounds__(kTile) k_gb64(const Item* __restrict__ items, 
 
 template <bool ENERGY, int WPA>
 __global__ void __launch_bounds__(kTile) k_chain64(const Item* __restrict__ items, View V) {
+    pdl_sync();
     constexpr int K = ENERGY ? 8 : 4;
     __shared__ J4<double> sa[kTile];
     __shared__ J2<double> sb[kTile];

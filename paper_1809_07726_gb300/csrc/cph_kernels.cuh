@@ -181,6 +181,7 @@ __device__ inline void tile_masks(const View& V, int P, int i, bool vi, int j0, 
 template <bool STAGED>
 __global__ void __launch_bounds__(kTile) k_born(const Item* __restrict__ items, View V,
                                                 int zero_energy) {
+    pdl_sync();
     using Real = float;
     constexpr int WPA = 1;
     using Pr = Prec<Real>;
@@ -282,6 +283,7 @@ __global__ void __launch_bounds__(kTile) k_born(const Item* __restrict__ items, 
 // of the energies; the epilogue turns dE/dR_i into c_i = dE/dR_i dR_i/dpsi_i rt_i/2.
 template <bool ENERGY, bool STAGED>
 __global__ void __launch_bounds__(kTile) k_gb(const Item* __restrict__ items, View V) {
+    pdl_sync();
     using Real = float;
     constexpr int WPA = 1;
     using Pr = Prec<Real>;
@@ -629,6 +631,7 @@ __device__ inline void bonded_atom32(const View& V, int A, int P, int li, int la
 // then the direct pair force and the bonded terms are added: F is the total force.
 template <bool ENERGY, bool STAGED>
 __global__ void __launch_bounds__(kTile) k_chain(const Item* __restrict__ items, View V) {
+    pdl_sync();
     using Real = float;
     constexpr int WPA = 1;
     using Pr = Prec<Real>;
@@ -761,25 +764,47 @@ __global__ void __launch_bounds__(kTile) k_chain(const Item* __restrict__ items,
 // v' = [(1 - g dt/2) v + dt A F/m + sqrt(2 g kB T A dt/m) z] / (1 + g dt/2),
 // x' = x + dt v', with T the temperature of the walker's current slot and z
 // three normals from one Philox draw (Box-Muller on words (0,1) and (2,3)).
-template <class Real>
-__device__ inline void normals3(uint64_t seed, uint32_t idx, uint32_t stream, uint64_t step,
-                                Real z[3]);
-
-template <>
-__device__ inline void normals3<double>(uint64_t seed, uint32_t idx, uint32_t stream,
-                                        uint64_t step, double z[3]) {
-    U4 u = draw(seed, idx, stream, step, kRngLangevin);
-    const double r0 = sqrt(-2.0 * log(unit_open(u.a)));
-    const double r1 = sqrt(-2.0 * log(unit_open(u.c)));
-    double sn, cs;
-    sincospi(2.0 * unit_open(u.b), &sn, &cs);
-    z[0] = r0 * cs;
-    z[1] = r0 * sn;
-    z[2] = r1 * cospi(2.0 * unit_open(u.d));
+// sin and cos of 2 pi (w + 1/2) / 2^32: the nearest quarter turn from the integer,
+// Taylor series on the rest (|t| <= pi/4; remainders 5e-17 and 2e-18).
+__device__ __forceinline__ void sincos64(uint32_t w, double& sn, double& cs) {
+    const uint32_t k = (w + 0x20000000u) >> 30;
+    const double t = fma((double)(int)(w - (k << 30)), 1.4629180792671596e-09, 7.314590396335798e-10);
+    const double t2 = t * t;
+    double p = fma(t2, -7.647163731819816e-13, 1.6059043836821613e-10);
+    p = fma(p, t2, -2.505210838544172e-08);
+    p = fma(p, t2, 2.7557319223985893e-06);
+    p = fma(p, t2, -0.0001984126984126984);
+    p = fma(p, t2, 0.008333333333333333);
+    p = fma(p, t2, -0.16666666666666666);
+    const double s = fma(p * t2, t, t);
+    double q = fma(t2, 4.779477332387385e-14, -1.1470745597729725e-11);
+    q = fma(q, t2, 2.08767569878681e-09);
+    q = fma(q, t2, -2.755731922398589e-07);
+    q = fma(q, t2, 2.48015873015873e-05);
+    q = fma(q, t2, -0.001388888888888889);
+    q = fma(q, t2, 0.041666666666666664);
+    q = fma(q, t2, -0.5);
+    const double c = fma(q, t2, 1.0);
+    const double a = (k & 1u) ? c : s, b = (k & 1u) ? s : c; // quarter turns
+    sn = (k & 2u) ? -a : a;
+    cs = ((k + 1u) & 2u) ? -b : b;
 }
 
-template <>
-__device__ inline void normals3<float>(uint64_t seed, uint32_t idx, uint32_t stream,
+// The library's sincospi, log and sqrt took ~190 FP64 instructions, this ~85.
+__device__ __forceinline__ void normals64(uint64_t seed, uint32_t idx, uint32_t stream, uint64_t step, double z[3],
+                                          const double2* tab) {
+    const U4 u = draw(seed, idx, stream, step, kRngLangevin);
+    const double l0 = -2.0 * log64(unit_open(u.a), tab), l1 = -2.0 * log64(unit_open(u.c), tab);
+    const double r0 = l0 * rsqrt64(l0), r1 = l1 * rsqrt64(l1);
+    double sn, cs, s1, c1;
+    sincos64(u.b, sn, cs);
+    sincos64(u.d, s1, c1);
+    z[0] = r0 * cs;
+    z[1] = r0 * sn;
+    z[2] = r1 * c1;
+}
+
+__device__ inline void normals3(uint64_t seed, uint32_t idx, uint32_t stream,
                                        uint64_t step, float z[3]) {
     U4 u = draw(seed, idx, stream, step, kRngLangevin);
     const float r0 = sqrtf(-2.0f * logf((float)unit_open(u.a)));
@@ -791,8 +816,37 @@ __device__ inline void normals3<float>(uint64_t seed, uint32_t idx, uint32_t str
     z[2] = r1 * cospif(2.0f * (float)unit_open(u.d));
 }
 
+// One sample of the observables for walker w (a warp or more; n threads).
+__device__ inline void observe_walker(const View& V, int w, int tid, int n) {
+    if (!V.w_local[w]) return; // a sharded grid's counts are summed over its engines
+    const int s = V.slot_of[w];
+    if (tid == 0) {
+        V.visits[(long long)w * V.W + s] += 1;
+        if (w == V.first_local) *V.n_obs += 1;
+    }
+    // the walker at slot s belongs to the system of the walker that started
+    // there, so slot s's rows are laid out like walker s's sites
+    const int ws0 = V.w_site_off[w], ns = V.w_site_off[w + 1] - ws0;
+    const long long row0 = V.w_site_off[s];
+    for (int k = tid; k < ns; k += n) V.occ[(row0 + k) * CPH_MAX_STATES + V.site_state[ws0 + k]] += 1;
+}
+
+// Blocks past the atoms' own (obs of them, one per walker) take the step's sample
+// of the observables, which depends on nothing the step moves: a launch of 5 us
+// less a step.
 template <class Real>
-__global__ void k_langevin(View V, int s_off, int a0, int n) {
+__global__ void k_langevin(View V, int s_off, int a0, int n, int obs) {
+    pdl_sync();
+    const int nb = gridDim.x - obs;
+    if ((int)blockIdx.x >= nb) {
+        observe_walker(V, (int)blockIdx.x - nb, threadIdx.x, blockDim.x);
+        return;
+    }
+    __shared__ double2 tab[sizeof(Real) == 8 ? kTab64 : 1];
+    if constexpr (sizeof(Real) == 8) {
+        load_tab64(tab, threadIdx.x, blockDim.x);
+        __syncthreads();
+    }
     const int l = blockIdx.x * blockDim.x + threadIdx.x;
     if (l >= n) return;
     const int a = a0 + l;
@@ -803,7 +857,8 @@ __global__ void k_langevin(View V, int s_off, int a0, int n) {
     const uint64_t t = (uint64_t)(*V.step + s_off);
     const int slot = V.slot_of[w];
     Real z[3];
-    normals3<Real>(V.seed, (uint32_t)li, (uint32_t)w, t, z);
+    if constexpr (sizeof(Real) == 8) normals64(V.seed, (uint32_t)li, (uint32_t)w, t, z, tab);
+    else normals3(V.seed, (uint32_t)li, (uint32_t)w, t, z);
     // per-atom factors dt A / m and sqrt(2 g kB A dt / m), and sqrt(T) per
     // slot, are set up once: no FP64 division or square root per step
     const double sd = V.lg_sqT[slot / (V.nE * V.npH)] * V.lg_sf[P + li];
@@ -832,6 +887,7 @@ __global__ void k_langevin(View V, int s_off, int a0, int n) {
 constexpr int kShakeMaxH = 8, kShakeMaxIter = 1000;
 
 __global__ void k_shake(View V, int i0, int n) {
+    pdl_sync();
     const int l = blockIdx.x * blockDim.x + threadIdx.x;
     if (l >= n) return;
     const int it = i0 + l;
@@ -898,6 +954,6 @@ __global__ void k_vscale_reset(View V) {
     if (w < V.W) V.vscale[w] = 1.0;
 }
 
-__global__ void k_tick(long long* step, long long n) { *step += n; }
+__global__ void k_tick(long long* step, long long n) { pdl_sync(); *step += n; }
 
 } // namespace cph

@@ -231,6 +231,7 @@ __device__ __noinline__ void small_shake(const View& V, const float4* fac, int c
 // GA: atoms per warp (1, 2 or 4 for up to 160, 256 or 512 atoms).
 template <int GA, bool ENERGY>
 __global__ void __launch_bounds__(GA == 1 ? 704 : 576, 1) k_small(View V, SmallTab T, SmallRun run) {
+    pdl_sync();
     namespace cg = cooperative_groups;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cg::cluster_group cl = cg::this_cluster();
@@ -620,7 +621,7 @@ __global__ void __launch_bounds__(GA == 1 ? 704 : 576, 1) k_small(View V, SmallT
         if (aux) {
             for (int a = atid; a < nown; a += 32 * kSmallAux) {
                 float z[3];
-                normals3<float>(V.seed, (uint32_t)(a0 + a), (uint32_t)w, t0 + (uint64_t)st, z);
+                normals3(V.seed, (uint32_t)(a0 + a), (uint32_t)w, t0 + (uint64_t)st, z);
                 for (int c = 0; c < 3; ++c) S.z[3 * a + c] = z[c];
             }
         }

@@ -100,6 +100,7 @@ __device__ __forceinline__ float hct_dr_series(float rinv2, float rinv, float s)
 // terms are rounded where the Born radii are finished, and once more after a
 // sweep that changed charges.
 __global__ void k_stage_x(View V, int a0, int n) {
+    pdl_sync();
     const int l = blockIdx.x * blockDim.x + threadIdx.x;
     if (l >= n) return;
     const int a = a0 + l, o = V.w_off[V.a_walker[a]];
@@ -109,6 +110,7 @@ __global__ void k_stage_x(View V, int a0, int n) {
 }
 
 __global__ void k_stage_gb(View V, int a0, int n) {
+    pdl_sync();
     const int l = blockIdx.x * blockDim.x + threadIdx.x;
     if (l >= n) return;
     const int a = a0 + l;
@@ -305,6 +307,7 @@ __device__ __forceinline__ void gb_tile(const GbJs& sj, int lane, const GbI2 (&I
 
 template <bool ENERGY, bool SALT, int GG>
 __global__ void __launch_bounds__(kSymThreads, GG == 2 ? 4 : 5) k_gb_sym(const SymItem* __restrict__ items, View V) {
+    pdl_sync();
     __shared__ GbJs sj[GG / 2];
     __shared__ __align__(16) float red[GG][4][kSymJ][4];
     __shared__ long long sfx[4][kSymI]; // i-side fixed-point sums, component-major (conflict-free)
@@ -467,6 +470,7 @@ __global__ void __launch_bounds__(kSymThreads, GG == 2 ? 4 : 5) k_gb_sym(const S
 // dE/dR (fixed point) -> chain weights c_i; GB self energy
 template <bool ENERGY>
 __global__ void k_fin_c(View V, int a0, int n) {
+    pdl_sync();
     const int l = blockIdx.x * blockDim.x + threadIdx.x;
     if (l >= n) return;
     const int a = a0 + l;
@@ -601,6 +605,7 @@ __device__ __forceinline__ void chain_tile(const ChJs& sj, int lane, const ChI2 
 
 template <bool CUT, int GG, bool QUEUE>
 __global__ void __launch_bounds__(kSymThreads, 5) k_chain_sym(const SymItem* __restrict__ items, View V) {
+    pdl_sync();
     __shared__ ChJs sj[GG / 2];
     __shared__ __align__(16) float red[GG][4][kSymJ][4]; // component 3 unused (vector stores)
     __shared__ long long sfx[3][kSymI]; // i-side fixed-point sums, component-major (conflict-free)
@@ -770,6 +775,7 @@ constexpr int kBondedThreads = 256;
 
 template <bool ENERGY>
 __global__ void __launch_bounds__(kBondedThreads) k_bonded_terms(View V, int w0) {
+    pdl_sync();
     __shared__ double re[kBondedThreads / 32][2];
     const int w = w0 + blockIdx.y;
     const int s = V.w_sys[w], A = V.w_off[w];
@@ -836,6 +842,7 @@ __global__ void __launch_bounds__(kBondedThreads) k_bonded_terms(View V, int w0)
 
 // total force: fixed-point pair forces + the atom's bonded-term forces
 __global__ void k_final_forces(View V, int a0, int n) {
+    pdl_sync();
     const int l = blockIdx.x * blockDim.x + threadIdx.x;
     if (l >= n) return;
     const int a = a0 + l;
@@ -993,6 +1000,7 @@ __device__ __forceinline__ void born_tile_q(const BoJs* sjg, int pr, int lane, i
 }
 template <bool CUT, int GG>
 __global__ void __launch_bounds__(kSymThreads, 5) k_born_sym(const SymItem* __restrict__ items, View V) {
+    pdl_sync();
     __shared__ BoJs sj[GG / 2];
     __shared__ float red[GG][4][kSymJ];
     __shared__ BoNear<GG> nb;
@@ -1121,6 +1129,7 @@ __global__ void __launch_bounds__(kSymThreads, 5) k_born_sym(const SymItem* __re
 // for this step's pair passes and, at a walker's first atom, the walker's
 // energy sums and velocity scale.
 __global__ void k_fin_born(View V, int a0, int n, int zero_energy) {
+    pdl_sync();
     const int l = blockIdx.x * blockDim.x + threadIdx.x;
     if (l >= n) return;
     const int a = a0 + l;

@@ -192,14 +192,25 @@ def _p(a):
     return C.c_void_p(a.ctypes.data) if a is not None else None
 
 
+_raw_stream = None  # the current device's current stream, once torch has a GPU
+
+
 def _stream(stream):
+    global _raw_stream
     if stream is not None:
-        return C.c_void_p(int(stream))
+        return int(stream)
+    if _raw_stream is not None:
+        return _raw_stream()
     try:
         import torch
         if torch.cuda.is_available():
-            return C.c_void_p(torch.cuda.current_stream().cuda_stream)
-    except ImportError:  # pragma: no cover
+            now = torch.cuda.current_stream().cuda_stream  # sets CUDA up
+            # the same two reads without the Python layers around them (a small
+            # call's host time is mostly these: 5 us of 18)
+            current, device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+            _raw_stream = lambda: current(device())  # noqa: E731
+            return now
+    except (ImportError, AttributeError):  # pragma: no cover
         pass
     return None
 
@@ -534,8 +545,7 @@ def gb_workspace_bytes(n_rep, n):
     return int(lib().cph_gb_workspace_bytes(n_rep, n))
 
 
-def _dptr(t):
-    return C.c_void_p(t.data_ptr())
+_GB0 = default_gb()  # passed by reference where the caller gives none; never written
 
 
 def gb_energy(x, q, rho, screen, gb=None, workspace=None, stream=None):
@@ -546,9 +556,9 @@ def gb_energy(x, q, rho, screen, gb=None, workspace=None, stream=None):
     x, q, rho, screen = (t.contiguous() for t in (x, q, rho, screen))
     E = torch.empty(n_rep, dtype=torch.float64, device=q.device)
     ws = workspace if workspace is not None else _workspace(n_rep, n, q.device)
-    g = gb or default_gb()
-    _check(lib().cph_gb_energy(n_rep, n, _dptr(x), _dptr(q), _dptr(rho), _dptr(screen),
-                               C.byref(g), _dptr(E), _dptr(ws), ws.numel(), _stream(stream)))
+    g = gb or _GB0
+    _check(lib().cph_gb_energy(n_rep, n, x.data_ptr(), q.data_ptr(), rho.data_ptr(), screen.data_ptr(),
+                               C.byref(g), E.data_ptr(), ws.data_ptr(), ws.numel(), _stream(stream)))
     return E
 
 
@@ -561,10 +571,10 @@ def gb_energy_backward(x, q, rho, screen, dE, gb=None, workspace=None, stream=No
     dq = torch.empty_like(q)
     drho = torch.empty_like(rho)
     ws = workspace if workspace is not None else _workspace(n_rep, n, q.device)
-    g = gb or default_gb()
-    _check(lib().cph_gb_energy_backward(n_rep, n, _dptr(x), _dptr(q), _dptr(rho), _dptr(screen),
-                                        C.byref(g), _dptr(dE), _dptr(dx), _dptr(dq),
-                                        _dptr(drho), _dptr(ws), ws.numel(), _stream(stream)))
+    g = gb or _GB0
+    _check(lib().cph_gb_energy_backward(n_rep, n, x.data_ptr(), q.data_ptr(), rho.data_ptr(), screen.data_ptr(),
+                                        C.byref(g), dE.data_ptr(), dx.data_ptr(), dq.data_ptr(),
+                                        drho.data_ptr(), ws.data_ptr(), ws.numel(), _stream(stream)))
     return dx, dq, drho
 
 
@@ -576,9 +586,9 @@ def gb_energy_noalloc(x, q, rho, screen, gb=None, stream=None):
     n_rep, n = q.shape
     x, q, rho, screen = (t.contiguous() for t in (x, q, rho, screen))
     E = torch.empty(n_rep, dtype=torch.float64, device=q.device)
-    g = gb or default_gb()
-    _check(lib().cph_gb_energy_noalloc(n_rep, n, _dptr(x), _dptr(q), _dptr(rho), _dptr(screen),
-                                       C.byref(g), _dptr(E), _stream(stream)))
+    g = gb or _GB0
+    _check(lib().cph_gb_energy_noalloc(n_rep, n, x.data_ptr(), q.data_ptr(), rho.data_ptr(), screen.data_ptr(),
+                                       C.byref(g), E.data_ptr(), _stream(stream)))
     return E
 
 
@@ -609,6 +619,6 @@ def _gb_function():
 
 
 def __getattr__(name):
-    if name == "GBEnergy":
-        return _gb_function()
+    if name == "GBEnergy":  # made on first use (torch stays optional), then an ordinary attribute
+        return globals().setdefault(name, _gb_function())
     raise AttributeError(name)

@@ -135,6 +135,16 @@ __device__ __forceinline__ long long fix32(float v) {
     return v < 0.f ? -m : m;
 }
 
+// 64-bit addition to shared memory as two 32-bit ones (a 64-bit atomic there is a
+// loop of compare-and-swap)
+__device__ __forceinline__ void shared_add(long long* p, long long v) {
+    unsigned* w = reinterpret_cast<unsigned*>(p);
+    const unsigned lo = (unsigned)v, hi = (unsigned)((unsigned long long)v >> 32);
+    const unsigned old = atomicAdd(w, lo);
+    const unsigned up = hi + (old > ~lo ? 1u : 0u);
+    if (up) atomicAdd(w + 1, up);
+}
+
 // sum over the warp, in every lane (exact integers: any order)
 __device__ __forceinline__ long long warp_sum(long long v) {
 #pragma unroll
@@ -283,6 +293,13 @@ __device__ __forceinline__ double exp64(double x, const double2* tab) {
 static __constant__ double kExp2Tab[16] = {1.0, 1.0442737824274138, 1.0905077326652577, 1.1387886347566916, 1.189207115002721, 1.241857812073484, 1.2968395546510096, 1.3542555469368927, 1.4142135623730951, 1.4768261459394993, 1.5422108254079407, 1.6104903319492543, 1.681792830507429, 1.7562521603732995, 1.8340080864093424, 1.9152065613971474};
 __device__ __forceinline__ double exp64(double x) {
     return exp64_with(x, [&](int j) { return kExp2Tab[j]; });
+}
+
+// tanh(x) = (1 - e) / (1 + e), e = e^(-2|x|): absolute error ~1e-16, which is what
+// the Born radius 1 / (1/rt - tanh / rho) asks for
+__device__ __forceinline__ double tanh64(double x) {
+    const double e = exp64(-2.0 * fabs(x));
+    return copysign(fma(-2.0 * e, rcp64(1.0 + e), 1.0), x);
 }
 
 // ---------------------------------------------- MUFU approximations (FP32)

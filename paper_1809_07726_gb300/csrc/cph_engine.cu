@@ -15,6 +15,7 @@
 #include <cuda_runtime.h>
 
 #include "cph_kernels.cuh"
+#include "cph_launch.h"
 #include "cph_sym.cuh"
 #include "cph_f64.cuh"
 #include "cph_small.cuh"
@@ -745,25 +746,6 @@ bool finite_all(const double* p, size_t n) {
 
 // At most this many atoms on the FP64 ordered passes: four warps per atom.
 constexpr long long kOrderedFewAtoms = 2048;
-
-// A launch that may be set up while the one before it on the stream still runs
-// (every kernel launched so begins with pdl_sync).  A step is a chain of launches
-// of a few microseconds: 100 steps of the 160-atom FP64 walker 6.23 -> 5.35 ms, 20
-// steps of one 2003-atom walker 2.13 -> 1.88 ms, 10 steps of 64 x 2400 atoms 10.45
-// -> 10.21 ms.
-template <class... P, class... A>
-void launch_next(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A&&... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kernel, P(args)...); // the caller checks cudaGetLastError
-}
 
 // Whether walkers of system s run the ordered passes (one warp per atom i):
 // always in FP64 mode, by the system's tile shape in FP32 mode.

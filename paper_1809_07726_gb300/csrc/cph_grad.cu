@@ -18,6 +18,7 @@
 // with g_i = dE/dR_i dR_i/dpsi_i and c_i = g_i rt_i / 2.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <mutex>
@@ -28,6 +29,7 @@
 #include "cph_device.cuh"
 #include "cph_grad_sym.cuh"
 #include "cph_grad_small.cuh"
+#include "cph_launch.h"
 
 namespace cph {
 namespace grad {
@@ -164,17 +166,16 @@ bool gsmall(int n_rep, int n) { return n <= kGsAtoms && (long long)n_rep * n * n
 int launch_radii(SView& g, cudaStream_t st) {
     const size_t na = (size_t)g.n_rep * g.n;
     cudaError_t ce = cudaMemsetAsync(g.bound, 0, 2 * sizeof(unsigned int), st);
-    if (ce == cudaSuccess) ce = cudaMemsetAsync(g.Hfix, 0, na * sizeof(long long), st);
     if (ce != cudaSuccess) return gfail(CPH_E_CUDA, std::string("cph_gb_energy: memset: ") + cudaGetErrorString(ce));
     const int ba = (int)((na + 255) / 256);
     const int grid = g.n_rep * g.n_itile * g.n_chunk;
-    k_gbound<<<ba, 256, 0, st>>>(g);
+    launch_next(k_gbound, std::min(ba, kGBoundBlocks), 256, st, g);
     by_group(g, [&](auto gg) {
         constexpr int GG = decltype(gg)::value;
-        if (g.rgbmax < INFINITY) k_gborn_sym<true, GG><<<grid, kGT, 0, st>>>(g);
-        else k_gborn_sym<false, GG><<<grid, kGT, 0, st>>>(g);
+        if (g.rgbmax < INFINITY) launch_next(k_gborn_sym<true, GG>, grid, kGT, st, g);
+        else launch_next(k_gborn_sym<false, GG>, grid, kGT, st, g);
     });
-    k_gfin_born<<<ba, 256, 0, st>>>(g);
+    launch_next(k_gfin_born, ba, 256, st, g);
     return CPH_OK;
 }
 } // namespace
@@ -205,11 +206,11 @@ extern "C" int cph_gb_energy(int n_rep, int n, const float* x, const float* q, c
     const int ba = (int)((na + 255) / 256);
     by_group(g, [&](auto gg) {
         constexpr int GG = decltype(gg)::value;
-        if (g.kappa > 0) k_gpair_sym<false, true, GG><<<n_rep * g.n_itile * g.n_chunk, kGT, 0, st>>>(g);
-        else k_gpair_sym<false, false, GG><<<n_rep * g.n_itile * g.n_chunk, kGT, 0, st>>>(g);
+        if (g.kappa > 0) launch_next(k_gpair_sym<false, true, GG>, n_rep * g.n_itile * g.n_chunk, kGT, st, g);
+        else launch_next(k_gpair_sym<false, false, GG>, n_rep * g.n_itile * g.n_chunk, kGT, st, g);
     });
-    k_gfin_c<false><<<ba, 256, 0, st>>>(g);
-    k_genergy_out<<<(n_rep + 127) / 128, 128, 0, st>>>(g);
+    launch_next(k_gfin_c<false>, ba, 256, st, g);
+    launch_next(k_genergy_out, (n_rep + 127) / 128, 128, st, g);
     cudaError_t ce = cudaGetLastError();
     if (ce != cudaSuccess) return gfail(CPH_E_CUDA, std::string("cph_gb_energy: ") + cudaGetErrorString(ce));
     return CPH_OK;
@@ -241,13 +242,13 @@ extern "C" int cph_gb_energy_backward(int n_rep, int n, const float* x, const fl
     const int grid = n_rep * g.n_itile * g.n_chunk;
     by_group(g, [&](auto gg) {
         constexpr int GG = decltype(gg)::value;
-        if (g.kappa > 0) k_gpair_sym<true, true, GG><<<grid, kGT, 0, st>>>(g);
-        else k_gpair_sym<true, false, GG><<<grid, kGT, 0, st>>>(g);
-        k_gfin_c<true><<<ba, 256, 0, st>>>(g);
-        if (g.rgbmax < INFINITY) k_gchain_sym<true, GG><<<grid, kGT, 0, st>>>(g);
-        else k_gchain_sym<false, GG><<<grid, kGT, 0, st>>>(g);
+        if (g.kappa > 0) launch_next(k_gpair_sym<true, true, GG>, grid, kGT, st, g);
+        else launch_next(k_gpair_sym<true, false, GG>, grid, kGT, st, g);
+        launch_next(k_gfin_c<true>, ba, 256, st, g);
+        if (g.rgbmax < INFINITY) launch_next(k_gchain_sym<true, GG>, grid, kGT, st, g);
+        else launch_next(k_gchain_sym<false, GG>, grid, kGT, st, g);
     });
-    k_gfin_out<<<ba, 256, 0, st>>>(g);
+    launch_next(k_gfin_out, ba, 256, st, g);
     cudaError_t ce = cudaGetLastError();
     if (ce != cudaSuccess) return gfail(CPH_E_CUDA, std::string("cph_gb_energy_backward: ") + cudaGetErrorString(ce));
     return CPH_OK;

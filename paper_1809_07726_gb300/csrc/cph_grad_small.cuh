@@ -72,9 +72,7 @@ __global__ void __launch_bounds__(kGsThreads) __cluster_dims__(kGsRanks, 1, 1) k
     for (int a = tid; a < nown; a += kGsThreads) {
         const double rho = g.rho[base + a0 + a], rt = rho - g.offset, irho = rcp64(rho);
         const double psi = rt * ((double)sum[a][0] * (0.5 / kScaleH));
-        const double th0 = psi * (g.alpha + psi * (-g.beta + psi * g.gamma));
-        const double e = exp64(-2.0 * fabs(th0)); // tanh = (1 - e) / (1 + e)
-        const double th = copysign(fma(-2.0 * e, rcp64(1.0 + e), 1.0), th0);
+        const double th = tanh64(psi * (g.alpha + psi * (-g.beta + psi * g.gamma)));
         const double iR = rcp64(rt) - th * irho, R = rcp64(iR);
         aR[a] = R;
         aiR[a] = iR;

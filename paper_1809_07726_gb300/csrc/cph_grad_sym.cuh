@@ -55,15 +55,34 @@ struct SView {
     float *dx, *dqo, *drho;
 };
 
-// max over every replica's atoms of s = screen (rho - offset) and rt = rho - offset
-__global__ void k_gbound(SView g) {
-    const size_t a = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (a >= (size_t)g.n_rep * g.n) return;
-    const float rt = g.rho[a] - g.off32;
-    const float s = g.screen[a % g.n] * rt;
-    // positive floats order like their bit patterns
-    atomicMax(&g.bound[0], __float_as_uint(fmaxf(s, 0.f)));
-    atomicMax(&g.bound[1], __float_as_uint(fmaxf(rt, 0.f)));
+// max over every replica's atoms of s = screen (rho - offset) and rt = rho - offset;
+// clears the descreening sums.  One atomic per block: a pair of atomics per atom on
+// two words took 45 us at 128 x 8000.
+constexpr int kGBoundBlocks = 608;
+
+__global__ void __launch_bounds__(256) k_gbound(SView g) {
+    pdl_sync();
+    __shared__ unsigned m[2][8];
+    const unsigned na = (unsigned)((size_t)g.n_rep * g.n), n = (unsigned)g.n, step = gridDim.x * 256;
+    unsigned s = 0u, r = 0u; // positive floats order like their bit patterns
+    for (size_t a = blockIdx.x * 256 + threadIdx.x; a < na; a += step) {
+        const float rt = g.rho[a] - g.off32;
+        s = max(s, __float_as_uint(fmaxf(g.screen[(unsigned)a % n] * rt, 0.f)));
+        r = max(r, __float_as_uint(fmaxf(rt, 0.f)));
+        g.Hfix[a] = 0;
+    }
+    s = __reduce_max_sync(0xffffffffu, s);
+    r = __reduce_max_sync(0xffffffffu, r);
+    if ((threadIdx.x & 31) == 0) {
+        m[0][threadIdx.x >> 5] = s;
+        m[1][threadIdx.x >> 5] = r;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        unsigned v = 0u;
+        for (int k = 0; k < 8; ++k) v = max(v, m[threadIdx.x][k]);
+        atomicMax(&g.bound[threadIdx.x], v);
+    }
 }
 
 __device__ __forceinline__ PairBand gband(const SView& g) {
@@ -110,6 +129,7 @@ __device__ __forceinline__ bool gmasked(int jt, int i0, int n) {
 // ------------------------------------------------------------ Born radii
 template <bool CUT, int GG>
 __global__ void __launch_bounds__(kGT, 5) k_gborn_sym(SView g) {
+    pdl_sync();
     __shared__ BoJs sj[GG / 2];
     __shared__ float red[GG][4][kGJ];
     __shared__ uint16_t nearq[kGT / 32][kNearCap];
@@ -218,8 +238,8 @@ __global__ void __launch_bounds__(kGT, 5) k_gborn_sym(SView g) {
                 const float2 hv = born_near(r2, rsqrt_ftz(r2), rti, irti, si, h ? C.w : C.z, h ? Nj.y : Nj.x,
                                             h ? Nj.w : Nj.z, band.rc);
                 if (valid) {
-                    atomicAdd((unsigned long long*)&ihx[warp * 64 + u * 32 + l], (unsigned long long)to_fixed(hv.x, (float)kScaleH));
-                    atomicAdd((unsigned long long*)&jhx[2 * p + h][jj], (unsigned long long)to_fixed(hv.y, (float)kScaleH));
+                    shared_add(&ihx[warp * 64 + u * 32 + l], fix32(hv.x * 256.f)); // 2^40
+                    shared_add(&jhx[2 * p + h][jj], fix32(hv.y * 256.f));
                 }
             });
         }
@@ -242,12 +262,13 @@ __global__ void __launch_bounds__(kGT, 5) k_gborn_sym(SView g) {
 // psi, R (FP64); resets the fixed-point accumulators of the pair passes.
 // Hfix and dRfix share a slot: H is read, then the slot starts dE/dR at zero.
 __global__ void k_gfin_born(SView g) {
+    pdl_sync();
     const size_t a = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (a >= (size_t)g.n_rep * g.n) return;
-    const double rho = g.rho[a], rt = rho - g.offset, irho = 1.0 / rho;
+    const double rho = g.rho[a], rt = rho - g.offset, irho = rcp64(rho);
     const double psi = 0.5 * rt * ((double)g.Hfix[a] / kScaleH);
-    const double th = tanh(psi * (g.alpha + psi * (-g.beta + psi * g.gamma)));
-    const double R = 1.0 / (1.0 / rt - th * irho);
+    const double th = tanh64(psi * (g.alpha + psi * (-g.beta + psi * g.gamma)));
+    const double R = rcp64(rcp64(rt) - th * irho);
     g.psi[a] = psi;
     g.R[a] = R;
     g.gpsi[a] = R * R * (1.0 - th * th) * (g.alpha + psi * (-2.0 * g.beta + 3.0 * g.gamma * psi)) * irho; // dR/dpsi for now
@@ -383,6 +404,7 @@ __device__ __forceinline__ void gpair_tile(const GpJs& sj, int lane, const GpI2 
 
 template <bool BACKWARD, bool SALT, int GG>
 __global__ void __launch_bounds__(kGT, 5) k_gpair_sym(SView g) {
+    pdl_sync();
     __shared__ GpJs sj[GG / 2];
     __shared__ float red[GG][4][kGJ][5];
     __shared__ long long sfx[5][kGI]; // i-side sums, component-major (conflict-free)
@@ -536,12 +558,14 @@ __global__ void __launch_bounds__(kGT, 5) k_gpair_sym(SView g) {
 // self energy; for the backward also dE/dR, c = dE/dR dR/dpsi rt/2, dE/dq
 template <bool BACKWARD>
 __global__ void k_gfin_c(SView g) {
+    pdl_sync();
     const size_t a = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (a >= (size_t)g.n_rep * g.n) return;
     const double q = (double)g.q[a] * g.sqrt_k, R = g.R[a];
     const double esa = sa_ace(g.sa_gamma, g.sa_probe, (double)g.rho[a], R);
     const double ts = salt_tau(R, g.inv_eps_in, g.inv_eps_out, g.kappa); // tau of the self term
-    const long long e = __double2ll_rn((-0.5 * ts * q * q / R + esa) * kScaleE);
+    const double iR = rcp64(R);
+    const long long e = __double2ll_rn((-0.5 * ts * q * q * iR + esa) * kScaleE);
     // one atomic per warp when the warp's atoms share a replica (exact integer
     // sums, so the total is the same whichever way they are grouped)
     const unsigned mask = __activemask();
@@ -557,11 +581,11 @@ __global__ void k_gfin_c(SView g) {
     }
     if (!BACKWARD) return;
     const double dEdR = 0.5 * (g.tau_pair * ((double)g.dRfix[a] / kScaleE)
-                               + salt_taud(R, g.inv_eps_in, g.inv_eps_out, g.kappa) * q * q / (R * R))
-                      - (g.sa_gamma != 0.0 ? 6.0 * esa / R : 0.0); // no FP64 division without the term
+                               + salt_taud(R, g.inv_eps_in, g.inv_eps_out, g.kappa) * q * q * iR * iR)
+                      - (g.sa_gamma != 0.0 ? 6.0 * esa * iR : 0.0);
     const double rt = (double)g.rho[a] - g.offset;
     const double gpsi = dEdR * g.gpsi[a]; // gpsi slot held dR/dpsi
-    const double dq = -g.sqrt_k * (g.tau_pair * ((double)g.dqfix[a] / kScaleE) + ts * q / R);
+    const double dq = -g.sqrt_k * (g.tau_pair * ((double)g.dqfix[a] / kScaleE) + ts * q * iR);
     g.dEdR[a] = dEdR; // same slot as dRfix
     g.gpsi[a] = gpsi;
     g.c[a] = gpsi * 0.5 * rt;
@@ -571,6 +595,7 @@ __global__ void k_gfin_c(SView g) {
 }
 
 __global__ void k_genergy_out(SView g) {
+    pdl_sync();
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r < g.n_rep) g.E[r] = (double)g.eacc[r] / kScaleE;
 }
@@ -672,6 +697,7 @@ __device__ __forceinline__ void gchain_tile(const GcJs& sj, int lane, const GcI2
 
 template <bool CUT, int GG>
 __global__ void __launch_bounds__(kGT, 4) k_gchain_sym(SView g) {
+    pdl_sync();
     __shared__ GcJs sj[GG / 2];
     __shared__ float red[GG][4][kGJ][5];
     __shared__ long long sfx[5][kGI]; // i-side sums, component-major (conflict-free)
@@ -849,17 +875,19 @@ __global__ void __launch_bounds__(kGT, 4) k_gchain_sym(SView g) {
 
 // outputs: dx, dq, drho scaled by the upstream gradient of the replica
 __global__ void k_gfin_out(SView g) {
+    pdl_sync();
     const size_t a = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (a >= (size_t)g.n_rep * g.n) return;
     const int r = (int)(a / g.n);
     const double up = g.dE[r];
     const double rho = g.rho[a], rt = rho - g.offset, R = g.R[a], psi = g.psi[a];
-    const double th = tanh(psi * (g.alpha + psi * (-g.beta + psi * g.gamma)));
+    const double irt = rcp64(rt), irho = rcp64(rho);
+    const double th = (irt - rcp64(R)) * rho; // from 1/R = 1/rt - th/rho
     const double esa = sa_ace(g.sa_gamma, g.sa_probe, rho, R); // explicit rho dependence at fixed R
-    const double dr = g.dEdR[a] * R * R * (1.0 / (rt * rt) - th / (rho * rho)) + g.gpsi[a] * psi / rt +
+    const double dr = g.dEdR[a] * R * R * (irt * irt - th * irho * irho) + g.gpsi[a] * psi * irt +
                       g.c[a] * ((double)g.artfix[a] / kScaleE) +
                       (double)g.screen[a % g.n] * ((double)g.asfix[a] / kScaleE) +
-                      (esa != 0.0 ? esa * (2.0 / (rho + g.sa_probe) + 6.0 / rho) : 0.0);
+                      (esa != 0.0 ? esa * (2.0 / (rho + g.sa_probe) + 6.0 * irho) : 0.0);
     g.dx[3 * a] = (float)(up * ((double)g.gfix[3 * a] / kScaleE));
     g.dx[3 * a + 1] = (float)(up * ((double)g.gfix[3 * a + 1] / kScaleE));
     g.dx[3 * a + 2] = (float)(up * ((double)g.gfix[3 * a + 2] / kScaleE));

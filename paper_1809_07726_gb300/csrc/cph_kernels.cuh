@@ -265,8 +265,8 @@ __global__ void __launch_bounds__(kTile) k_born(const Item* __restrict__ items, 
         const double sumH = Pr::value(acc, kScaleH);
         const double rt = V.rt[P + i], irho = V.irho[P + i]; // 1/rt, 1/rho from set-up
         const double psi = 0.5 * rt * sumH;
-        const double th = tanh(psi * (V.alpha + psi * (-V.beta + psi * V.gamma)));
-        const double R = 1.0 / (V.irt[P + i] - th * irho);
+        const double th = tanh64(psi * (V.alpha + psi * (-V.beta + psi * V.gamma)));
+        const double R = rcp64(V.irt[P + i] - th * irho);
         V.psi[A + i] = psi;
         V.R[A + i] = R;
         if (sizeof(Real) == 4) V.gq[A + i] = gb_operand(V.q[A + i], V.sqrt_k, R);

@@ -386,9 +386,7 @@ __global__ void __launch_bounds__(GA == 1 ? 704 : 576, 1) k_small(View V, SmallT
                 for (int a = tid; a < nown; a += nthr) { // R and dR/dpsi, to every CTA
                     SmallAtom& at = S.at[a];
                     const double psi = at.rt * ((double)S.sum[8 * a] * (0.5 / kScaleH));
-                    const double th0 = psi * (V.alpha + psi * (-V.beta + psi * V.gamma));
-                    const double e = exp64(-2.0 * fabs(th0)); // tanh = (1 - e) / (1 + e)
-                    const double th = copysign(fma(-2.0 * e, rcp64(1.0 + e), 1.0), th0);
+                    const double th = tanh64(psi * (V.alpha + psi * (-V.beta + psi * V.gamma)));
                     const double iR = at.irt - th * at.irho, R = rcp64(iR);
                     at.psi = psi;
                     at.R = R;

@@ -477,18 +477,18 @@ __global__ void k_fin_c(View V, int a0, int n) {
     const int w = V.a_walker[a];
     if (V.sys_ordered[V.w_sys[w]] || !V.w_local[w]) return; // ordered passes finish their atoms themselves
     const int P = V.sys_poff[V.w_sys[w]] + (a - V.w_off[w]);
-    const double q = V.q[a] * V.sqrt_k, R = V.R[a];
+    const double q = V.q[a] * V.sqrt_k, R = V.R[a], iR = rcp64(R);
     const double esa = sa_ace(V.sa_gamma, V.sa_probe, V.rho[P], R);
     const double dEdR = 0.5 * (V.tau_pair * ((double)V.dRfix[a] / kScaleE)
-                               + salt_taud(R, V.inv_eps_in, V.inv_eps_out, V.kappa) * q * q / (R * R))
-                      - (V.sa_gamma != 0.0 ? 6.0 * esa / R : 0.0); // no FP64 division without the term
+                               + salt_taud(R, V.inv_eps_in, V.inv_eps_out, V.kappa) * q * q * iR * iR)
+                      - (V.sa_gamma != 0.0 ? 6.0 * esa * iR : 0.0);
     const double c = dEdR * V.dRdpsi[a] * 0.5 * V.rt[P];
     V.c[a] = c;
     V.c32[a] = (float)c;
     if (ENERGY)
         atomicAdd((unsigned long long*)&V.eacc[w * kEAcc + 0],
                   (unsigned long long)__double2ll_rn((-0.5 * salt_tau(R, V.inv_eps_in, V.inv_eps_out, V.kappa)
-                                                      * q * q / R + esa) * kScaleE));
+                                                      * q * q * iR + esa) * kScaleE));
 }
 
 // ========================================================= chain rule
@@ -1142,8 +1142,8 @@ __global__ void k_fin_born(View V, int a0, int n, int zero_energy) {
     const double rt = V.rt[P], irho = V.irho[P];
     const double psi = 0.5 * rt * ((double)V.Hfix[a] / kScaleH);
     V.Hfix[a] = 0;
-    const double th = tanh(psi * (V.alpha + psi * (-V.beta + psi * V.gamma)));
-    const double R = 1.0 / (V.irt[P] - th * irho);
+    const double th = tanh64(psi * (V.alpha + psi * (-V.beta + psi * V.gamma)));
+    const double R = rcp64(V.irt[P] - th * irho);
     V.psi[a] = psi;
     V.R[a] = R;
     V.gq[a] = gb_operand(V.q[a], V.sqrt_k, R);

@@ -128,7 +128,7 @@ __device__ __forceinline__ bool gmasked(int jt, int i0, int n) {
 
 // ------------------------------------------------------------ Born radii
 template <bool CUT, int GG>
-__global__ void __launch_bounds__(kGT, 5) k_gborn_sym(SView g) {
+__global__ void __launch_bounds__(kGT, 6) k_gborn_sym(SView g) {
     pdl_sync();
     __shared__ BoJs sj[GG / 2];
     __shared__ float red[GG][4][kGJ];
@@ -403,7 +403,7 @@ __device__ __forceinline__ void gpair_tile(const GpJs& sj, int lane, const GpI2 
 }
 
 template <bool BACKWARD, bool SALT, int GG>
-__global__ void __launch_bounds__(kGT, 5) k_gpair_sym(SView g) {
+__global__ void __launch_bounds__(kGT, BACKWARD ? 5 : 8) k_gpair_sym(SView g) {
     pdl_sync();
     __shared__ GpJs sj[GG / 2];
     __shared__ float red[GG][4][kGJ][5];

@@ -45,23 +45,52 @@ namespace cph {
 constexpr int kMcThreads = 256;
 constexpr int kMaxSiteAtoms = 64;
 
-// A_mn * k (both i != j), without the Coulomb part when `excluded`
+// A_mn * k (both i != j), without the Coulomb part when `excluded`; iRm, iRn = 1/R.
+// FP32: approximate reciprocal square roots and exponential as in the GB pass.
 template <class Real>
-__device__ __forceinline__ Real mc_pair(Real dx, Real dy, Real dz, Real Rm, Real Rn, bool excluded, Real iei,
-                                        Real tau, Real kap, Real ieo, bool salt) {
-    using Pr = Prec<Real>;
+__device__ __forceinline__ Real mc_pair(Real dx, Real dy, Real dz, Real Rm, Real iRm, Real Rn, Real iRn, bool excluded,
+                                        Real iei, Real tau, Real kap, Real ieo, bool salt) {
     const Real r2 = dx * dx + dy * dy + dz * dz;
-    const Real rinv = Pr::rsqrt(r2);
-    const Real D = Real(0.25) * r2 / (Rm * Rn);
-    const Real fi = Pr::rsqrt(r2 + Rm * Rn * Pr::expm(D));
-    const Real tf = salt ? iei - ieo * Pr::expm(kap / fi) : tau;
-    return (excluded ? Real(0) : iei * rinv) - tf * fi;
+    if constexpr (sizeof(Real) == 4) {
+        const float rinv = rsqrt_ftz(r2);
+        const float fa = fmaf(Rm * Rn, exp2_ftz(-0.25f * kLog2e * r2 * (iRm * iRn)), r2), fi = rsqrt_ftz(fa);
+        const float tf = salt ? iei - ieo * exp2_ftz(-kLog2e * kap * (fa * fi)) : tau;
+        return (excluded ? 0.f : iei * rinv) - tf * fi;
+    } else {
+        const double rinv = rsqrt64(r2);
+        const double fa = fma(Rm * Rn, exp64(-0.25 * r2 * (iRm * iRn)), r2), fi = rsqrt64(fa);
+        const double tf = salt ? iei - ieo * exp64(-kap * (fa * fi)) : tau;
+        return (excluded ? 0.0 : iei * rinv) - tf * fi;
+    }
 }
+
+// The accumulators of the MC sums: int64 fixed point (2^32) in FP32 mode.
+__device__ __forceinline__ void mc_add(long long& a, float v) { a += fix32(v); }
+__device__ __forceinline__ void mc_add(double& a, double v) { a += v; }
 
 __device__ inline bool mc_excluded(const View& V, int P, int at, int an) {
     for (int e = V.excl_off[P + at]; e < V.excl_off[P + at + 1]; ++e)
         if (V.excl_j[e] == an) return true;
     return false;
+}
+
+// Sum over the CTA in a fixed order, for thread 0.
+__device__ __forceinline__ double mc_total(long long v, long long* red, double*) {
+    v = warp_sum(v);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    long long t = 0;
+    for (int q = 0; q < kMcThreads / 32; ++q) t += red[q];
+    return (double)t * (1.0 / kScaleE);
+}
+__device__ __forceinline__ double mc_total(double v, long long*, double* red) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double t = 0.0;
+    for (int q = 0; q < kMcThreads / 32; ++q) t += red[q];
+    return t;
 }
 
 template <class Real>
@@ -78,164 +107,112 @@ __global__ void __launch_bounds__(kMcThreads) k_mc_site(View V, int kind, int s_
     const uint64_t t = (uint64_t)(*V.step + s_off);
     const int tid = threadIdx.x;
     const uint32_t purpose = (kind == CPH_SITE_PH) ? kRngMcPh : kRngMcRedox;
-    __shared__ Real mx[kMaxSiteAtoms], my[kMaxSiteAtoms], mz[kMaxSiteAtoms], mR[kMaxSiteAtoms],
-        mdq[kMaxSiteAtoms];
+    // the site's atoms: (x, y, z, dq), (R, 1/R, the self term A_mm, -)
+    __shared__ J4<Real> ma[kMaxSiteAtoms], mb[kMaxSiteAtoms];
     __shared__ int mat[kMaxSiteAtoms];
     __shared__ int sh_b;
     __shared__ long long redl[kMcThreads / 32];
     __shared__ double redd[kMcThreads / 32];
-    const double cx = V.x[3 * A], cy = V.x[3 * A + 1], cz = V.x[3 * A + 2];
     // FP32: the host-rounded copies (no double -> float conversion in the loops)
     const Real sqk = host_const<Real>(V.sqrt_k, V.sqk32), tau = host_const<Real>(V.tau, V.tau32),
                iei = host_const<Real>(V.inv_eps_in, V.iei32);
     const Real kap = host_const<Real>(V.kappa, V.kappa32), ieo = host_const<Real>(V.inv_eps_out, V.ieo32);
     const bool salt = V.kappa > 0;
     const int nat = V.site_nat[g], nst = V.site_nst[g], ao = V.site_aoff[g], qo = V.site_qoff[g];
-    if (tid == 0) {
+    if (tid == 0 || tid == 32) {
         const U4 u = draw(V.seed, (uint32_t)k, (uint32_t)w, t, purpose);
-        const int a = V.site_state[so + k];
-        const int jj = (int)floor(unit_open(u.a) * (double)(nst - 1));
-        const int b = jj < a ? jj : jj + 1;
-        sh_b = b;
-        V.mc_from[so + k] = a;
-        V.mc_to[so + k] = b;
-        V.mc_lnu[so + k] = log(unit_open(u.b));
+        if (tid == 32) V.mc_lnu[so + k] = log(unit_open(u.b)); // (an FP64 log: nothing waits for it)
+        else {
+            const int a = V.site_state[so + k];
+            const int jj = (int)floor(unit_open(u.a) * (double)(nst - 1));
+            const int b = jj < a ? jj : jj + 1;
+            sh_b = b;
+            V.mc_from[so + k] = a;
+            V.mc_to[so + k] = b;
+        }
     }
     __syncthreads();
     const int b = sh_b;
+    // partners: in FP32 the step's staged operands (positions relative to the
+    // walker's first atom; sqrt(k) q and R at the charges of this sweep's start),
+    // with no FP64 subtraction or conversion per partner
+    auto partner = [&](int j, J4<Real>& p, J4<Real>& r) {
+        if constexpr (sizeof(Real) == 4) {
+            const float4 x = V.xs[A + j], q = V.gq[A + j];
+            p = {x.x, x.y, x.z, q.x};
+            r = {q.y, q.z, 0.f, 0.f};
+        } else {
+            const double R = V.R[A + j];
+            p = {V.x[3 * (A + j)], V.x[3 * (A + j) + 1], V.x[3 * (A + j) + 2], V.q[A + j] * V.sqrt_k};
+            r = {R, rcp64(R), 0.0, 0.0};
+        }
+    };
     for (int m = tid; m < nat; m += kMcThreads) {
         const int at = V.site_atoms[ao + m];
+        J4<Real> p, r;
+        partner(at, p, r);
+        p.w = Real((V.site_q[qo + b * nat + m] - V.q[A + at]) * V.sqrt_k);
+        Real ts = tau;
+        if (salt) {
+            if constexpr (sizeof(Real) == 4) ts = iei - ieo * __expf(-kap * r.x);
+            else ts = iei - ieo * exp64(-kap * r.x);
+        }
+        r.z = -ts * r.y;
         mat[m] = at;
-        mx[m] = Real(V.x[3 * (A + at)] - cx);
-        my[m] = Real(V.x[3 * (A + at) + 1] - cy);
-        mz[m] = Real(V.x[3 * (A + at) + 2] - cz);
-        mR[m] = Real(V.R[A + at]);
-        mdq[m] = Real((V.site_q[qo + b * nat + m] - V.q[A + at]) * V.sqrt_k);
+        ma[m] = p;
+        mb[m] = r;
     }
     __syncthreads();
     Acc lin = 0;
-    auto linear_j = [&](int j, Real xj, Real yj, Real zj, Real qj, Real Rj) {
+    for (int j = tid; j < N; j += kMcThreads) {
+        J4<Real> p, r;
+        partner(j, p, r);
         Real part = 0;
         for (int m = 0; m < nat; ++m) {
-            if (mat[m] == j) {
-                const Real ts = salt ? iei - ieo * Pr::expm(kap * mR[m]) : tau;
-                part += mdq[m] * qj * (-ts / mR[m]);
-            } else {
-                part += mdq[m] * qj * mc_pair<Real>(mx[m] - xj, my[m] - yj, mz[m] - zj, mR[m], Rj, false, iei, tau,
-                                                    kap, ieo, salt);
-            }
+            const J4<Real> a = ma[m], c = mb[m];
+            const bool same = mat[m] == j;
+            const Real v = mc_pair<Real>(same ? Real(1) : a.x - p.x, a.y - p.y, a.z - p.z, c.x, c.y, r.x, r.y, false, iei,
+                                         tau, kap, ieo, salt);
+            part += a.w * (same ? c.z : v);
         }
-        Pr::add(lin, part, Real(kScaleE));
-    };
-    if (sizeof(Real) == 4) {
-        // FP32: the partners from the step's staged FP32 operands (positions
-        // relative to the walker's first atom; sqrt(k) q and R at the charges of
-        // this sweep's start), with no FP64 subtraction or conversion per partner
-        // (both issue to the narrow FP64 pipe)
-        for (int j = tid; j < N; j += kMcThreads) {
-            const float4 p = V.xs[A + j], gj = V.gq[A + j];
-            linear_j(j, Real(p.x), Real(p.y), Real(p.z), Real(gj.x), Real(gj.y));
-        }
-    } else {
-        for (int j = tid; j < N; j += kMcThreads)
-            linear_j(j, Real(V.x[3 * (A + j)] - cx), Real(V.x[3 * (A + j) + 1] - cy),
-                     Real(V.x[3 * (A + j) + 2] - cz), Real(V.q[A + j]) * sqk, Real(V.R[A + j]));
+        mc_add(lin, part * p.w);
     }
     // The Coulomb part of excluded pairs (index nat * nat + m) and the
-    // quadratic term's pairs (index m * nat + n): in the pass's precision from
-    // the site atoms' staged values (FP32: no FP64 arithmetic per pair on the
-    // narrow FP64 pipe; the FP32 terms are at the linear term's accuracy), the
-    // FP64 mode in FP64 from the master positions.
-    double corr = 0.0;
-    if (sizeof(Real) == 4) {
-        for (int idx = tid; idx < nat * nat + nat; idx += kMcThreads) {
-            Real term = 0;
-            if (idx >= nat * nat) {
-                const int m = idx - nat * nat, at = mat[m];
-                for (int e = V.excl_off[P + at]; e < V.excl_off[P + at + 1]; ++e) {
-                    const int j = V.excl_j[e];
-                    const float4 p = V.xs[A + j];
-                    const Real xj = Real(p.x), yj = Real(p.y), zj = Real(p.z), qj = Real(V.gq[A + j].x);
-                    const Real d0 = mx[m] - xj, d1 = my[m] - yj, d2 = mz[m] - zj;
-                    term -= mdq[m] * qj * iei * Pr::rsqrt(d0 * d0 + d1 * d1 + d2 * d2);
-                }
-            } else {
-                const int m = idx / nat, n = idx % nat;
-                if (n == m) {
-                    const Real ts = salt ? iei - ieo * Pr::expm(kap * mR[m]) : tau;
-                    term = Real(0.5) * mdq[m] * mdq[m] * (-ts / mR[m]);
-                } else {
-                    term = Real(0.5) * mdq[m] * mdq[n] *
-                           mc_pair<Real>(mx[m] - mx[n], my[m] - my[n], mz[m] - mz[n], mR[m], mR[n],
-                                         mc_excluded(V, P, mat[m], mat[n]), iei, tau, kap, ieo, salt);
-                }
+    // quadratic term's pairs (index m * nat + n)
+    for (int idx = tid; idx < nat * nat + nat; idx += kMcThreads) {
+        Real term = 0;
+        if (idx >= nat * nat) {
+            const int m = idx - nat * nat, at = mat[m];
+            const J4<Real> a = ma[m];
+            for (int e = V.excl_off[P + at]; e < V.excl_off[P + at + 1]; ++e) {
+                J4<Real> p, r;
+                partner(V.excl_j[e], p, r);
+                const Real d0 = a.x - p.x, d1 = a.y - p.y, d2 = a.z - p.z, r2 = d0 * d0 + d1 * d1 + d2 * d2;
+                if constexpr (sizeof(Real) == 4) term -= a.w * p.w * iei * rsqrt_ftz(r2);
+                else term -= a.w * p.w * iei * rsqrt64(r2);
             }
-            corr += (double)term;
+        } else {
+            const int m = idx / nat, n = idx % nat;
+            const J4<Real> a = ma[m], c = mb[m], a2 = ma[n], c2 = mb[n];
+            const Real v = n == m ? c.z
+                                  : mc_pair<Real>(a.x - a2.x, a.y - a2.y, a.z - a2.z, c.x, c.y, c2.x, c2.y,
+                                                  mc_excluded(V, P, mat[m], mat[n]), iei, tau, kap, ieo, salt);
+            term = Real(0.5) * a.w * a2.w * v;
         }
-    } else {
-        for (int idx = tid; idx < nat * nat + nat; idx += kMcThreads) {
-            if (idx >= nat * nat) {
-                const int m = idx - nat * nat, at = mat[m];
-                const double dqm = (V.site_q[qo + b * nat + m] - V.q[A + at]);
-                const double xm0 = V.x[3 * (A + at)], xm1 = V.x[3 * (A + at) + 1], xm2 = V.x[3 * (A + at) + 2];
-                for (int e = V.excl_off[P + at]; e < V.excl_off[P + at + 1]; ++e) {
-                    const int j = V.excl_j[e];
-                    const double d0 = xm0 - V.x[3 * (A + j)], d1 = xm1 - V.x[3 * (A + j) + 1],
-                                 d2 = xm2 - V.x[3 * (A + j) + 2];
-                    const double r = sqrt(d0 * d0 + d1 * d1 + d2 * d2);
-                    corr -= dqm * V.q[A + j] * kCoulomb * V.inv_eps_in / r;
-                }
-                continue;
-            }
-            const int m = idx / nat, n = idx % nat, at = mat[m], an = mat[n];
-            const double dqm = (V.site_q[qo + b * nat + m] - V.q[A + at]);
-            const double dqn = (V.site_q[qo + b * nat + n] - V.q[A + an]);
-            const double Rm = V.R[A + at];
-            if (n == m) {
-                corr += 0.5 * dqm * dqn * (-salt_tau(Rm, V.inv_eps_in, V.inv_eps_out, V.kappa) * kCoulomb / Rm);
-                continue;
-            }
-            const double d0 = V.x[3 * (A + at)] - V.x[3 * (A + an)], d1 = V.x[3 * (A + at) + 1] - V.x[3 * (A + an) + 1],
-                         d2 = V.x[3 * (A + at) + 2] - V.x[3 * (A + an) + 2];
-            const double r2 = d0 * d0 + d1 * d1 + d2 * d2;
-            const double RR = Rm * V.R[A + an];
-            const double f = sqrt(r2 + RR * exp(-0.25 * r2 / RR));
-            double amn = -salt_tau(f, V.inv_eps_in, V.inv_eps_out, V.kappa) * kCoulomb / f;
-            if (!mc_excluded(V, P, at, an)) amn += kCoulomb * V.inv_eps_in / sqrt(r2);
-            corr += 0.5 * dqm * dqn * amn;
-        }
+        mc_add(lin, term);
     }
-    // block reduction (fixed order)
-    long long lv = 0;
-    double tot_d = corr;
-    if (sizeof(Real) == 4) lv = (long long)lin;
-    else tot_d += (double)lin;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        lv += __shfl_down_sync(0xffffffffu, lv, o);
-        tot_d += __shfl_down_sync(0xffffffffu, tot_d, o);
-    }
-    if ((tid & 31) == 0) {
-        redl[tid >> 5] = lv;
-        redd[tid >> 5] = tot_d;
-    }
-    __syncthreads();
-    if (tid == 0) {
-        long long L = 0;
-        double D = 0.0;
-        for (int q = 0; q < kMcThreads / 32; ++q) {
-            L += redl[q];
-            D += redd[q];
-        }
-        V.mc_du0[so + k] = (double)L / kScaleE + D;
-    }
+    const double du0 = mc_total(lin, redl, redd);
+    if (tid == 0) V.mc_du0[so + k] = du0;
 }
+
+// Atoms of accepted sites that a sweep keeps in shared memory; sites accepted
+// past that are read from the site tables again.
+constexpr int kMcKept = 768;
 
 template <class Real>
 __global__ void __launch_bounds__(kMcThreads) k_mc_sweep(View V, int kind, int clear_others, int w_begin) {
     pdl_sync();
-    using Pr = Prec<Real>;
-    using Acc = typename Pr::Acc;
+    using Acc = typename Prec<Real>::Acc;
     const int w = w_begin + blockIdx.x;
     if (!V.w_local[w]) return;
     const int s = V.w_sys[w], A = V.w_off[w], P = V.sys_poff[s];
@@ -244,95 +221,95 @@ __global__ void __launch_bounds__(kMcThreads) k_mc_sweep(View V, int kind, int c
     const int slot = V.slot_of[w];
     const int iE = slot % V.nE, ipH = (slot / V.nE) % V.npH, iT = slot / (V.nE * V.npH);
     const double E = V.gE[iE], pH = V.gpH[ipH], T = V.gT[iT];
-    const double kT = kBoltzmann * T;
-    __shared__ Real mx[kMaxSiteAtoms], my[kMaxSiteAtoms], mz[kMaxSiteAtoms], mR[kMaxSiteAtoms],
-        mdq[kMaxSiteAtoms];
-    __shared__ int mat[kMaxSiteAtoms];
-    __shared__ int sh_acc;
+    const double kT = kBoltzmann * T, ikT = 1.0 / kT;
+    __shared__ J4<Real> ma[kMaxSiteAtoms], ka[kMcKept]; // (x, y, z, sqrt(k) dq) of the site's and the kept atoms
+    __shared__ J2<Real> mb[kMaxSiteAtoms], kb[kMcKept]; // (R, 1/R)
+    __shared__ int mat[kMaxSiteAtoms], kat[kMcKept];
+    __shared__ int sh_acc[2]; // in turn: a site's is read while the next one's may be written
     __shared__ long long redl[kMcThreads / 32];
     __shared__ double redd[kMcThreads / 32];
-    const double cx = V.x[3 * A], cy = V.x[3 * A + 1], cz = V.x[3 * A + 2];
+    __shared__ double base[kMcThreads], lnus[kMcThreads];
     // FP32: the host-rounded copies (no double -> float conversion in the loops)
-    const Real sqk = host_const<Real>(V.sqrt_k, V.sqk32), tau = host_const<Real>(V.tau, V.tau32),
-               iei = host_const<Real>(V.inv_eps_in, V.iei32);
+    const Real tau = host_const<Real>(V.tau, V.tau32), iei = host_const<Real>(V.inv_eps_in, V.iei32);
     const Real kap = host_const<Real>(V.kappa, V.kappa32), ieo = host_const<Real>(V.inv_eps_out, V.ieo32);
     const bool salt = V.kappa > 0;
-    int n_taken = 0; // sites of this sweep accepted so far (uniform across the CTA)
+    auto stage = [&](int k, int m, J4<Real>& p, J2<Real>& r) { // atom m of site k and its change of charge
+        const int g = g0 + k, nat = V.site_nat[g], at = V.site_atoms[V.site_aoff[g] + m];
+        const double* q = V.site_q + V.site_qoff[g] + m;
+        const Real dq = Real((q[V.mc_to[so + k] * nat] - q[V.mc_from[so + k] * nat]) * V.sqrt_k);
+        if constexpr (sizeof(Real) == 4) {
+            const float4 x = V.xs[A + at], c = V.gq[A + at];
+            p = {x.x, x.y, x.z, dq};
+            r = {c.y, c.z};
+        } else {
+            const double R = V.R[A + at];
+            p = {V.x[3 * (A + at)], V.x[3 * (A + at) + 1], V.x[3 * (A + at) + 2], dq};
+            r = {R, rcp64(R)};
+        }
+        return at;
+    };
+    int n_taken = 0;       // sites of this sweep accepted so far (uniform across the CTA)
+    int n_kept = 0;        // their atoms in shared memory
+    int first_out = ns;    // the first accepted site whose atoms are not
+    int turn = 0;
     for (int k = 0; k < ns; ++k) {
-        const int g = g0 + k;
-        if (V.site_kind[g] != kind) {
-            if (clear_others && tid == 0) V.mc_rec[so + k].walker = -1;
-            continue;
-        }
-        const int nat = V.site_nat[g], ao = V.site_aoff[g], qo = V.site_qoff[g], no = V.site_noff[g];
-        const int a = V.mc_from[so + k], b = V.mc_to[so + k];
-        Acc cross = 0;
-        if (n_taken > 0) {
-            __syncthreads(); // the previous site's staging is no longer read
-            for (int m = tid; m < nat; m += kMcThreads) {
-                const int at = V.site_atoms[ao + m];
-                mat[m] = at;
-                mx[m] = Real(V.x[3 * (A + at)] - cx);
-                my[m] = Real(V.x[3 * (A + at) + 1] - cy);
-                mz[m] = Real(V.x[3 * (A + at) + 2] - cz);
-                mR[m] = Real(V.R[A + at]);
-                mdq[m] = Real((V.site_q[qo + b * nat + m] - V.site_q[qo + a * nat + m]) * V.sqrt_k);
-            }
+        if (k % kMcThreads == 0) { // what a site's decision needs besides the other sites', a thread per site
             __syncthreads();
-            // dq^T A dq' over the accepted earlier sites k2, pairs (m, n) split over threads
-            for (int k2 = 0; k2 < k; ++k2) {
-                const int g2 = g0 + k2;
-                if (V.site_kind[g2] != kind || !V.mc_take[so + k2]) continue;
-                const int nat2 = V.site_nat[g2], ao2 = V.site_aoff[g2], qo2 = V.site_qoff[g2];
-                const int a2 = V.mc_from[so + k2], b2 = V.mc_to[so + k2];
-                Real part = 0;
+            const int k1 = k + tid, g = g0 + k1;
+            if (k1 < ns && V.site_kind[g] == kind) {
+                const int a = V.mc_from[so + k1], b = V.mc_to[so + k1], no = V.site_noff[g];
+                double dG = -(V.site_uref[no + b] - V.site_uref[no + a]);
+                if (kind == CPH_SITE_PH)
+                    dG += kT * kLn10 * (double)(V.site_np[no + b] - V.site_np[no + a]) * (pH - V.site_ref[g]);
+                else
+                    dG += kFaraday * (double)(V.site_ne[no + b] - V.site_ne[no + a]) * (E - V.site_ref[g]);
+                base[tid] = dG;
+                lnus[tid] = V.mc_lnu[so + k1];
+            } else if (k1 < ns && clear_others) V.mc_rec[so + k1].walker = -1;
+            __syncthreads();
+        }
+        const int g = g0 + k;
+        if (V.site_kind[g] != kind) continue;
+        const int nat = V.site_nat[g];
+        double cross = 0.0;
+        if (n_taken > 0) {
+            // dq^T A dq' over the atoms of the accepted earlier sites
+            for (int m = tid; m < nat; m += kMcThreads) mat[m] = stage(k, m, ma[m], mb[m]);
+            __syncthreads();
+            Acc sum = 0;
+            for (int idx = tid; idx < nat * n_kept; idx += kMcThreads) {
+                const int m = idx % nat, n = idx / nat;
+                const J4<Real> a = ma[m], c = ka[n];
+                const J2<Real> r = mb[m], q = kb[n];
+                mc_add(sum, a.w * c.w * mc_pair<Real>(a.x - c.x, a.y - c.y, a.z - c.z, r.x, r.y, q.x, q.y,
+                                                      mc_excluded(V, P, mat[m], kat[n]), iei, tau, kap, ieo, salt));
+            }
+            for (int k2 = first_out; k2 < k; ++k2) { // accepted sites that are not kept
+                if (V.site_kind[g0 + k2] != kind || !V.mc_take[so + k2]) continue;
+                const int nat2 = V.site_nat[g0 + k2];
                 for (int idx = tid; idx < nat * nat2; idx += kMcThreads) {
-                    const int m = idx / nat2, n = idx % nat2;
-                    const int an = V.site_atoms[ao2 + n];
-                    const Real dqn = Real(V.site_q[qo2 + b2 * nat2 + n] - V.site_q[qo2 + a2 * nat2 + n]) * sqk;
-                    const Real xn = Real(V.x[3 * (A + an)] - cx), yn = Real(V.x[3 * (A + an) + 1] - cy),
-                               zn = Real(V.x[3 * (A + an) + 2] - cz);
-                    part += mdq[m] * dqn * mc_pair<Real>(mx[m] - xn, my[m] - yn, mz[m] - zn, mR[m], Real(V.R[A + an]),
-                                                         mc_excluded(V, P, mat[m], an), iei, tau, kap, ieo, salt);
+                    const int m = idx % nat;
+                    J4<Real> c;
+                    J2<Real> q;
+                    const int an = stage(k2, idx / nat, c, q);
+                    const J4<Real> a = ma[m];
+                    const J2<Real> r = mb[m];
+                    mc_add(sum, a.w * c.w * mc_pair<Real>(a.x - c.x, a.y - c.y, a.z - c.z, r.x, r.y, q.x, q.y,
+                                                          mc_excluded(V, P, mat[m], an), iei, tau, kap, ieo, salt));
                 }
-                Pr::add(cross, part, Real(kScaleE));
             }
+            cross = mc_total(sum, redl, redd);
         }
-        long long lv = 0;
-        double dv = 0.0;
-        if (sizeof(Real) == 4) lv = (long long)cross;
-        else dv = (double)cross;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            lv += __shfl_down_sync(0xffffffffu, lv, o);
-            dv += __shfl_down_sync(0xffffffffu, dv, o);
-        }
-        if ((tid & 31) == 0) {
-            redl[tid >> 5] = lv;
-            redd[tid >> 5] = dv;
-        }
-        __syncthreads();
         if (tid == 0) {
-            long long L = 0;
-            double D = 0.0;
-            for (int q = 0; q < kMcThreads / 32; ++q) {
-                L += redl[q];
-                D += redd[q];
-            }
-            const double lnu = V.mc_lnu[so + k];
-            const double dU = V.mc_du0[so + k] + ((double)L / kScaleE + D);
-            double dG = dU - (V.site_uref[no + b] - V.site_uref[no + a]);
-            if (kind == CPH_SITE_PH)
-                dG += kT * kLn10 * (double)(V.site_np[no + b] - V.site_np[no + a]) * (pH - V.site_ref[g]);
-            else
-                dG += kFaraday * (double)(V.site_ne[no + b] - V.site_ne[no + a]) * (E - V.site_ref[g]);
-            const double x = -dG / kT;
+            const double lnu = lnus[k % kMcThreads];
+            const double dU = V.mc_du0[so + k] + cross;
+            const double x = -(dU + base[k % kMcThreads]) * ikT;
             const int acc = lnu < x ? 1 : 0;
             cph_mc_record rec;
             rec.walker = w;
             rec.site = k;
-            rec.from = a;
-            rec.to = b;
+            rec.from = V.mc_from[so + k];
+            rec.to = V.mc_to[so + k];
             rec.accepted = acc;
             rec.pad_ = 0;
             rec.dU = dU;
@@ -340,18 +317,28 @@ __global__ void __launch_bounds__(kMcThreads) k_mc_sweep(View V, int kind, int c
             rec.lnu = lnu;
             V.mc_rec[so + k] = rec;
             V.mc_take[so + k] = acc;
-            if (acc) V.site_state[so + k] = b;
-            sh_acc = acc;
-            const int base = (kind == CPH_SITE_PH) ? 6 : 8;
-            atomicAdd((unsigned long long*)&V.stats[base], 1ull);
-            if (acc) atomicAdd((unsigned long long*)&V.stats[base + 1], 1ull);
+            if (acc) V.site_state[so + k] = rec.to;
+            sh_acc[turn] = acc;
+            const int st = (kind == CPH_SITE_PH) ? 6 : 8;
+            atomicAdd((unsigned long long*)&V.stats[st], 1ull);
+            if (acc) atomicAdd((unsigned long long*)&V.stats[st + 1], 1ull);
         }
         __syncthreads();
-        if (sh_acc) {
-            for (int m = tid; m < nat; m += kMcThreads)
-                V.q[A + V.site_atoms[ao + m]] = V.site_q[qo + b * nat + m];
+        const bool taken = sh_acc[turn];
+        turn ^= 1;
+        if (taken) {
+            const double* q = V.site_q + V.site_qoff[g] + V.mc_to[so + k] * nat;
+            const bool keep = first_out == ns && n_kept + nat <= kMcKept;
+            for (int m = tid; m < nat; m += kMcThreads) {
+                V.q[A + V.site_atoms[V.site_aoff[g] + m]] = q[m];
+                if (keep) kat[n_kept + m] = stage(k, m, ka[n_kept + m], kb[n_kept + m]);
+            }
+            if (keep) n_kept += nat;
+            else if (first_out == ns) first_out = k;
             ++n_taken;
         }
+        // (the next site's barrier after staging, or the one after its decision,
+        // comes before anything here is read)
     }
 }
 

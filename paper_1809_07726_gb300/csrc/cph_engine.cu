@@ -895,16 +895,23 @@ int launch_mc(cph_engine* E, int kinds, int s_off, cudaStream_t st) {
 
 // FP32: symmetric GB and chain passes (each unordered pair once), then the
 // per-atom finishing kernels; FP64: ordered passes (bonded terms in k_chain).
-int launch_sym_pair(cph_engine* E, const SymItem* items, int n, bool energy, int pass,
+// walkers w0 .. w0 + nw - 1: those of the items (their bonded terms are blocks of
+// the chain-rule launch).
+int launch_sym_pair(cph_engine* E, const SymItem* items, int n, bool energy, int pass, int w0, int nw,
                     cudaStream_t st) {
     if (n <= 0) return CPH_OK;
+    const int per = (E->max_terms + kSymThreads - 1) / kSymThreads;
+    const BondedBlocks bb{pass == 2 ? per * nw : 0, per, w0, energy ? 1 : 0};
     const bool cut = E->V.rgbmax < INFINITY, salt = E->V.kappa > 0;
     auto launch = [&](auto gg) {
         constexpr int GG = decltype(gg)::value;
         auto go = [&](auto kernel) { launch_next(kernel, n, kSymThreads, st, items, E->V); };
         if (pass == 0) go(cut ? k_born_sym<true, GG> : k_born_sym<false, GG>);
-        else if (pass == 2 && (GG < kSymG || E->queue_near)) go(cut ? k_chain_sym<true, GG, true> : k_chain_sym<false, GG, true>);
-        else if (pass == 2) go(cut ? k_chain_sym<true, kSymG, false> : k_chain_sym<false, kSymG, false>);
+        else if (pass == 2) {
+            auto chain = [&](auto kernel) { launch_next(kernel, n + bb.n, kSymThreads, st, items, E->V, bb); };
+            if (GG < kSymG || E->queue_near) chain(cut ? k_chain_sym<true, GG, true> : k_chain_sym<false, GG, true>);
+            else chain(cut ? k_chain_sym<true, kSymG, false> : k_chain_sym<false, kSymG, false>);
+        }
         else if (salt) go(energy ? k_gb_sym<true, true, GG> : k_gb_sym<false, true, GG>);
         else go(energy ? k_gb_sym<true, false, GG> : k_gb_sym<false, false, GG>);
     };
@@ -941,15 +948,6 @@ int launch_atoms(cph_engine* E, int which, bool energy, int a0, int n, cudaStrea
     return CPH_OK;
 }
 
-int launch_bonded(cph_engine* E, bool energy, int w0, int nw, cudaStream_t st) {
-    if (E->max_terms <= 0 || nw <= 0) return CPH_OK;
-    dim3 grid((E->max_terms + kBondedThreads - 1) / kBondedThreads, nw);
-    if (energy) launch_next(k_bonded_terms<true>, grid, kBondedThreads, st, E->V, w0);
-    else launch_next(k_bonded_terms<false>, grid, kBondedThreads, st, E->V, w0);
-    CK(cudaGetLastError());
-    return CPH_OK;
-}
-
 // pass: 0 born, 1 GB (+ finish), 2 chain (+ bonded terms, finish)
 int launch_pass(cph_engine* E, int pass, bool energy, cudaStream_t st) {
     const bool fp32 = E->precision == CPH_PREC_FP32;
@@ -963,8 +961,7 @@ int launch_pass(cph_engine* E, int pass, bool energy, cudaStream_t st) {
         }
         if (pass == 0 && (E->staged || E->n_sym > 0)) TRY(launch_stage(E, 0, 0, E->V.total_atoms, st));
         if (E->n_sym > 0) {
-            TRY(launch_sym_pair(E, E->d_sym, E->n_sym, energy, pass, st));
-            if (pass == 2) TRY(launch_bonded(E, energy, 0, E->V.W, st));
+            TRY(launch_sym_pair(E, E->d_sym, E->n_sym, energy, pass, 0, W, st));
             TRY(launch_atoms(E, fin, energy, 0, E->V.total_atoms, st));
         }
         if (E->n_items > 0) { // systems on the ordered passes (bonded terms in k_chain)
@@ -986,8 +983,7 @@ int launch_pass(cph_engine* E, int pass, bool energy, cudaStream_t st) {
             else TRY(pass == 1 ? launch_gb(E, it, ni, energy, s) : launch_chain(E, it, ni, energy, s));
         } else {
             TRY(launch_sym_pair(E, E->d_sym_by_w + E->sym_w_off[w], E->sym_w_off[w + 1] - E->sym_w_off[w],
-                                energy, pass, s));
-            if (pass == 2) TRY(launch_bonded(E, energy, w, 1, s));
+                                energy, pass, w, 1, s));
             TRY(launch_atoms(E, fin, energy, E->h_w_off[w], E->h_w_off[w + 1] - E->h_w_off[w], s));
         }
     }

@@ -238,8 +238,8 @@ __global__ void __launch_bounds__(kGT, 6) k_gborn_sym(SView g) {
                 const float2 hv = born_near(r2, rsqrt_ftz(r2), rti, irti, si, h ? C.w : C.z, h ? Nj.y : Nj.x,
                                             h ? Nj.w : Nj.z, band.rc);
                 if (valid) {
-                    shared_add(&ihx[warp * 64 + u * 32 + l], fix32(hv.x * 256.f)); // 2^40
-                    shared_add(&jhx[2 * p + h][jj], fix32(hv.y * 256.f));
+                    shared_add(&ihx[warp * 64 + u * 32 + l], to_fixed(hv.x, (float)kScaleH));
+                    shared_add(&jhx[2 * p + h][jj], to_fixed(hv.y, (float)kScaleH));
                 }
             });
         }

@@ -603,16 +603,92 @@ __device__ __forceinline__ void chain_tile(const ChJs& sj, int lane, const ChI2 
     }
 }
 
+// Bonded terms, one thread per (walker, term): each bond or angle is evaluated
+// once and its forces on its two or three atoms are stored in the per-term
+// buffer (the atoms gather them in a fixed order in k_final_forces, so the sum
+// stays deterministic); energies per walker in fixed point.  They run as blocks
+// of the chain-rule launch, spread among its own: the terms are bound by FP64
+// instructions, the pair tiles by FP32 ones, and a launch of their own took 24 us
+// of a 1.0 ms step of 64 x 2400 atoms.
+__device__ __noinline__ void bonded_block(const View& V, int w, int t, bool energy) {
+    const int s = V.w_sys[w], A = V.w_off[w];
+    if (V.sys_ordered[s] || !V.w_local[w]) return; // bonded terms of the ordered passes are in k_chain
+    const int b0 = V.sys_bond_off[s], nb = V.sys_bond_off[s + 1] - b0;
+    const int a0 = V.sys_ang_off[s], na = V.sys_ang_off[s + 1] - a0;
+    float* buf = V.tforce + V.w_tf_off[w];
+    const double* x = V.x;
+    double eb = 0.0, ea = 0.0;
+    // the FP32-mode term arithmetic of bond_term32 / angle_term32
+    if (t < nb) {
+        const int b = b0 + t;
+        const int i = V.bond_ij[2 * b], j = V.bond_ij[2 * b + 1];
+        double d[3];
+        for (int c = 0; c < 3; ++c) d[c] = x[3 * (A + i) + c] - x[3 * (A + j) + c];
+        float g, e;
+        bond_term32(d, V.bond_r0[b], V.bond_k[b], g, e);
+        for (int c = 0; c < 3; ++c) {
+            const float f = g * (float)d[c];
+            buf[6 * t + c] = -f;
+            buf[6 * t + 3 + c] = f;
+        }
+        eb = (double)e;
+    } else if (t < nb + na) {
+        const int la = t - nb, a = a0 + la;
+        const int ia = V.ang_ijk[3 * a], ib = V.ang_ijk[3 * a + 1], ic = V.ang_ijk[3 * a + 2];
+        double u[3], v[3];
+        for (int c = 0; c < 3; ++c) {
+            u[c] = x[3 * (A + ia) + c] - x[3 * (A + ib) + c];
+            v[c] = x[3 * (A + ic) + c] - x[3 * (A + ib) + c];
+        }
+        float gi[3], gk[3], e;
+        angle_term32(u, v, V.ang_cs0[a], V.ang_k[a], gi, gk, e);
+        float* o = buf + 6 * (size_t)nb + 9 * (size_t)la;
+        for (int c = 0; c < 3; ++c) {
+            o[c] = -gi[c];
+            o[3 + c] = gi[c] + gk[c];
+            o[6 + c] = -gk[c];
+        }
+        ea = (double)e;
+    }
+    if (energy) {
+#pragma unroll
+        for (int of = 16; of > 0; of >>= 1) {
+            eb += __shfl_down_sync(0xffffffffu, eb, of);
+            ea += __shfl_down_sync(0xffffffffu, ea, of);
+        }
+        if ((threadIdx.x & 31) == 0) {
+            if (eb != 0.0) fix_add(&V.eacc[w * kEAcc + 3], __double2ll_rn(eb * kScaleE));
+            if (ea != 0.0) fix_add(&V.eacc[w * kEAcc + 4], __double2ll_rn(ea * kScaleE));
+        }
+    }
+}
+
+// Bonded blocks of a chain-rule launch: n of them, `per` to a walker from walker
+// w0 on; block 0, p, 2 p, ... of the launch, p = its blocks / n.
+struct BondedBlocks {
+    int n, per, w0, energy;
+};
+
 template <bool CUT, int GG, bool QUEUE>
-__global__ void __launch_bounds__(kSymThreads, 5) k_chain_sym(const SymItem* __restrict__ items, View V) {
+__global__ void __launch_bounds__(kSymThreads, 5) k_chain_sym(const SymItem* __restrict__ items, View V,
+                                                            BondedBlocks bb) {
     pdl_sync();
+    int item = blockIdx.x;
+    if (bb.n > 0) {
+        const int p = gridDim.x / bb.n, k = item / p;
+        if (k < bb.n && item == k * p) {
+            bonded_block(V, bb.w0 + k / bb.per, (k % bb.per) * kSymThreads + threadIdx.x, bb.energy);
+            return;
+        }
+        item -= min(bb.n, k + 1);
+    }
     __shared__ ChJs sj[GG / 2];
     __shared__ __align__(16) float red[GG][4][kSymJ][4]; // component 3 unused (vector stores)
     __shared__ long long sfx[3][kSymI]; // i-side fixed-point sums, component-major (conflict-free)
     // near pairs: the warps' queues, and the i-side sums of the staged group
     __shared__ uint16_t nearq[QUEUE ? kSymThreads / 32 : 1][QUEUE ? kNearCap : 1];
     __shared__ float inear[3][QUEUE ? kSymI : 1];
-    const SymItem it = items[blockIdx.x];
+    const SymItem it = items[item];
     const int w = it.w, s = V.w_sys[w], N = V.sys_n[s], A = V.w_off[w], P = V.sys_poff[s];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const PairBand band = pair_band(V.rfar2, V.smax32, (float)V.rgbmax);
@@ -767,79 +843,6 @@ __global__ void __launch_bounds__(kSymThreads, 5) k_chain_sym(const SymItem* __r
     }
 }
 
-// Bonded terms, one thread per (walker, term), FP64: each bond or angle is
-// evaluated once and its forces on its two or three atoms are stored in the
-// per-term buffer (the atoms gather them in a fixed order in k_final_forces,
-// so the sum stays deterministic); energies per walker in fixed point.
-constexpr int kBondedThreads = 256;
-
-template <bool ENERGY>
-__global__ void __launch_bounds__(kBondedThreads) k_bonded_terms(View V, int w0) {
-    pdl_sync();
-    __shared__ double re[kBondedThreads / 32][2];
-    const int w = w0 + blockIdx.y;
-    const int s = V.w_sys[w], A = V.w_off[w];
-    if (V.sys_ordered[s] || !V.w_local[w]) return; // bonded terms of the ordered passes are in k_chain
-    const int b0 = V.sys_bond_off[s], nb = V.sys_bond_off[s + 1] - b0;
-    const int a0 = V.sys_ang_off[s], na = V.sys_ang_off[s + 1] - a0;
-    const int t = blockIdx.x * kBondedThreads + threadIdx.x;
-    float* buf = V.tforce + V.w_tf_off[w];
-    const double* x = V.x;
-    double eb = 0.0, ea = 0.0;
-    // the FP32-mode term arithmetic of bond_term32 / angle_term32
-    if (t < nb) {
-        const int b = b0 + t;
-        const int i = V.bond_ij[2 * b], j = V.bond_ij[2 * b + 1];
-        double d[3];
-        for (int c = 0; c < 3; ++c) d[c] = x[3 * (A + i) + c] - x[3 * (A + j) + c];
-        float g, e;
-        bond_term32(d, V.bond_r0[b], V.bond_k[b], g, e);
-        for (int c = 0; c < 3; ++c) {
-            const float f = g * (float)d[c];
-            buf[6 * t + c] = -f;
-            buf[6 * t + 3 + c] = f;
-        }
-        eb = (double)e;
-    } else if (t < nb + na) {
-        const int la = t - nb, a = a0 + la;
-        const int ia = V.ang_ijk[3 * a], ib = V.ang_ijk[3 * a + 1], ic = V.ang_ijk[3 * a + 2];
-        double u[3], v[3];
-        for (int c = 0; c < 3; ++c) {
-            u[c] = x[3 * (A + ia) + c] - x[3 * (A + ib) + c];
-            v[c] = x[3 * (A + ic) + c] - x[3 * (A + ib) + c];
-        }
-        float gi[3], gk[3], e;
-        angle_term32(u, v, V.ang_cs0[a], V.ang_k[a], gi, gk, e);
-        float* o = buf + 6 * (size_t)nb + 9 * (size_t)la;
-        for (int c = 0; c < 3; ++c) {
-            o[c] = -gi[c];
-            o[3 + c] = gi[c] + gk[c];
-            o[6 + c] = -gk[c];
-        }
-        ea = (double)e;
-    }
-    if (ENERGY) {
-#pragma unroll
-        for (int of = 16; of > 0; of >>= 1) {
-            eb += __shfl_down_sync(0xffffffffu, eb, of);
-            ea += __shfl_down_sync(0xffffffffu, ea, of);
-        }
-        const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-        if (lane == 0) {
-            re[wp][0] = eb;
-            re[wp][1] = ea;
-        }
-        __syncthreads();
-        if (threadIdx.x < 2) {
-            double v = 0.0;
-            for (int q = 0; q < kBondedThreads / 32; ++q) v += re[q][threadIdx.x];
-            if (v != 0.0)
-                atomicAdd((unsigned long long*)&V.eacc[w * kEAcc + 3 + threadIdx.x],
-                          (unsigned long long)__double2ll_rn(v * kScaleE));
-        }
-    }
-}
-
 // total force: fixed-point pair forces + the atom's bonded-term forces
 __global__ void k_final_forces(View V, int a0, int n) {
     pdl_sync();
@@ -911,8 +914,8 @@ __device__ __noinline__ void born_flush(const BoJs* sj, BoNear<GG>& nb, int warp
         const float2 hv = born_near(r2, rsqrt_ftz(r2), ti.x, ti.y, xi.w, h ? C.w : C.z, h ? Nj.y : Nj.x,
                                     h ? Nj.w : Nj.z, band.rc);
         if (!(fabsf(hv.x) < 1e20f && fabsf(hv.y) < 1e20f)) atomicOr(status, 4);
-        atomicAdd((unsigned long long*)&nb.ihx[warp][slot], (unsigned long long)to_fixed(hv.x, (float)kScaleH));
-        atomicAdd((unsigned long long*)&nb.jhx[2 * pr + h][jj], (unsigned long long)to_fixed(hv.y, (float)kScaleH));
+        shared_add(&nb.ihx[warp][slot], to_fixed(hv.x, (float)kScaleH));
+        shared_add(&nb.jhx[2 * pr + h][jj], to_fixed(hv.y, (float)kScaleH));
     }
     __syncwarp();
 }

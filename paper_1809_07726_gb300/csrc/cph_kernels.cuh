@@ -38,24 +38,33 @@ __device__ __forceinline__ T warp_total(T v) {
     return v;
 }
 
-// Sum over the WPA warps that share one atom (warps g WPA .. g WPA + WPA - 1 of
-// the CTA): warp totals, then the group's warps in index order through the
-// 8-byte shared slots sh[4].  Every thread of the CTA must call it.  The
-// result is exact in lane 0 of each warp for WPA = 1 and in every thread of
-// the group for WPA > 1.
-template <int WPA, class T>
-__device__ __forceinline__ T group_total(T v, long long* sh) {
-    v = warp_total(v);
-    if (WPA == 1) return v;
-    const int warp = threadIdx.x >> 5;
-    if ((threadIdx.x & 31) == 0) reinterpret_cast<T*>(sh)[warp] = v;
-    __syncthreads();
-    T t = 0;
-    const int g0 = (warp / WPA) * WPA;
+// The ordered FP32 passes give each atom one warp; what follows the pair loop is
+// FP64, and an FP64 instruction holds its sub-partition for 64 clocks however
+// few lanes take part.  So the CTA's four atoms finish together in one warp:
+// collect() hands atom w's sums to lane w of warp 0.  (8 x 1203 atoms with salt,
+// energies: Born radii 47 -> 37 us, pair pass 100 -> 60, chain rule 78 -> 61
+// against an epilogue in each warp.)
+template <int K>
+struct AtomSums {
+    long long v[K][kWarpAtoms];
+    // every thread of the CTA calls it, with its warp's K lane accumulators;
+    // warp 0 may read v after it
+    __device__ __forceinline__ void collect(const long long (&acc)[K]) {
+        const int warp = threadIdx.x >> 5;
 #pragma unroll
-    for (int q = 0; q < WPA; ++q) t += reinterpret_cast<const T*>(sh)[g0 + q];
-    __syncthreads();
-    return t;
+        for (int k = 0; k < K; ++k) {
+            const long long s = warp_total(acc[k]);
+            if ((threadIdx.x & 31) == 0) v[k][warp] = s;
+        }
+        __syncthreads();
+    }
+};
+
+// Sum of lanes 0 .. 3 (fixed point: the order does not matter), in lane 0.
+__device__ __forceinline__ long long quad_total(long long v) {
+    v += __shfl_xor_sync(0xfu, v, 2);
+    v += __shfl_xor_sync(0xfu, v, 1);
+    return v;
 }
 
 template <class Real>
@@ -183,16 +192,13 @@ __global__ void __launch_bounds__(kTile) k_born(const Item* __restrict__ items, 
                                                 int zero_energy) {
     pdl_sync();
     using Real = float;
-    constexpr int WPA = 1;
     using Pr = Prec<Real>;
     __shared__ J4<Real> sj[kTile];
+    __shared__ AtomSums<1> sums;
     const Item it = items[blockIdx.x];
     const int w = it.w, s = V.w_sys[w], N = V.sys_n[s], A = V.w_off[w], P = V.sys_poff[s];
-    // WPA warps per atom i: the CTA holds kWarpAtoms / WPA atoms; `sub` indexes
-    // the thread within its atom's group of 32 WPA threads
-    const int tid = threadIdx.x, warp = tid >> 5, sub = tid - (warp / WPA) * 32 * WPA;
-    const int i = it.i0 + warp / WPA;
-    __shared__ long long gsh[kTile / 32];
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int i = it.i0 + (tid >> 5); // one warp per atom
     const bool vi = i < N;
     if (it.i0 == 0) {
         if (zero_energy && tid < kEAcc) V.eacc[w * kEAcc + tid] = 0;
@@ -231,7 +237,7 @@ __global__ void __launch_bounds__(kTile) k_born(const Item* __restrict__ items, 
         __syncthreads();
         if (jt != next) {
 #pragma unroll
-            for (int k = sub; k < kTile; k += 32 * WPA) {
+            for (int k = lane; k < kTile; k += 32) {
                 const J4<Real> b = sj[k];
                 const Real dx = xi - b.x, dy = yi - b.y, dz = zi - b.z;
                 const Real r2 = dx * dx + dy * dy + dz * dz;
@@ -243,7 +249,7 @@ __global__ void __launch_bounds__(kTile) k_born(const Item* __restrict__ items, 
             next = mp < me ? V.mt_list[mp] : 0x7fffffff;
             const int dself = i - j0;
 #pragma unroll
-            for (int k = sub; k < kTile; k += 32 * WPA) {
+            for (int k = lane; k < kTile; k += 32) {
                 const J4<Real> b = sj[k];
                 const bool self = (k == dself);
                 const Real dx = xi - b.x, dy = yi - b.y, dz = zi - b.z;
@@ -260,16 +266,17 @@ __global__ void __launch_bounds__(kTile) k_born(const Item* __restrict__ items, 
         }
     }
     Pr::add(acc, part, Real(kScaleH));
-    acc = group_total<WPA>(acc, gsh);
-    if (vi && sub == 0) {
-        const double sumH = Pr::value(acc, kScaleH);
+    sums.collect({acc});
+    if (tid < kWarpAtoms && it.i0 + tid < N) {
+        const int i = it.i0 + tid;
+        const double sumH = Pr::value(sums.v[0][tid], kScaleH);
         const double rt = V.rt[P + i], irho = V.irho[P + i]; // 1/rt, 1/rho from set-up
         const double psi = 0.5 * rt * sumH;
         const double th = tanh64(psi * (V.alpha + psi * (-V.beta + psi * V.gamma)));
         const double R = rcp64(V.irt[P + i] - th * irho);
         V.psi[A + i] = psi;
         V.R[A + i] = R;
-        if (sizeof(Real) == 4) V.gq[A + i] = gb_operand(V.q[A + i], V.sqrt_k, R);
+        V.gq[A + i] = gb_operand(V.q[A + i], V.sqrt_k, R);
         V.Ffix[3 * (A + i)] = 0;
         V.Ffix[3 * (A + i) + 1] = 0;
         V.Ffix[3 * (A + i) + 2] = 0;
@@ -285,19 +292,15 @@ template <bool ENERGY, bool STAGED>
 __global__ void __launch_bounds__(kTile) k_gb(const Item* __restrict__ items, View V) {
     pdl_sync();
     using Real = float;
-    constexpr int WPA = 1;
     using Pr = Prec<Real>;
     using Acc = typename Pr::Acc;
     __shared__ J4<Real> sa[kTile];
     __shared__ J4<Real> sb[kTile];
-    __shared__ long long red[4];
+    __shared__ AtomSums<ENERGY ? 7 : 4> sums;
     const Item it = items[blockIdx.x];
     const int w = it.w, s = V.w_sys[w], N = V.sys_n[s], A = V.w_off[w], P = V.sys_poff[s];
-    // WPA warps per atom i: the CTA holds kWarpAtoms / WPA atoms; `sub` indexes
-    // the thread within its atom's group of 32 WPA threads
-    const int tid = threadIdx.x, warp = tid >> 5, sub = tid - (warp / WPA) * 32 * WPA;
-    const int i = it.i0 + warp / WPA;
-    __shared__ long long gsh[kTile / 32];
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int i = it.i0 + (tid >> 5); // one warp per atom
     const bool vi = i < N;
     const Stage<Real, STAGED> stage(V, A, P, it.i0);
     Real xi = Real(-kFarF), yi = Real(-kFarF), zi = Real(-kFarF);
@@ -350,7 +353,7 @@ __global__ void __launch_bounds__(kTile) k_gb(const Item* __restrict__ items, Vi
         __syncthreads();
         if (jt != next) {
 #pragma unroll
-            for (int k = sub; k < kTile; k += 32 * WPA) {
+            for (int k = lane; k < kTile; k += 32) {
                 const J4<Real> a = sa[k];
                 const J4<Real> b = sb[k];
                 const Real dx = xi - a.x, dy = yi - a.y, dz = zi - a.z;
@@ -360,13 +363,15 @@ __global__ void __launch_bounds__(kTile) k_gb(const Item* __restrict__ items, Vi
                 const Real qq = qi * a.w;
                 const Real D = Real(0.25) * r2 * (iRi * b.y);
                 const Real e = Pr::expm(D);
-                const Real fi = Pr::rsqrt(r2 + (Ri * b.x) * e);
+                const Real f2 = r2 + (Ri * b.x) * e;
+                const Real fi = Pr::rsqrt(f2);
                 const Real qf3 = qq * fi * fi * fi;
                 Real tf = Real(1), td = Real(1);
                 if (salt) {
-                    const Real es = ieo * Pr::expm(kap / fi);
+                    const Real kf = kap * (f2 * fi);
+                    const Real es = ieo * Pr::expm(kf);
                     tf = iei - es;
-                    td = tf - kap * es / fi;
+                    td = tf - kf * es;
                 }
                 pdr += td * qf3 * b.x * e * (Real(1) + D);
                 const Real sig = sgi + b.z;
@@ -390,7 +395,7 @@ __global__ void __launch_bounds__(kTile) k_gb(const Item* __restrict__ items, Vi
             uint32_t mex[4], mself[4];
             tile_masks(V, P, i, vi, j0, mex, mself);
 #pragma unroll
-            for (int k = sub; k < kTile; k += 32 * WPA) {
+            for (int k = lane; k < kTile; k += 32) {
                 {
                     const int q4 = k >> 5, kk = k & 31;
                     const bool self = (mself[q4] >> kk) & 1u;
@@ -407,13 +412,15 @@ __global__ void __launch_bounds__(kTile) k_gb(const Item* __restrict__ items, Vi
                     const Real qq = qi * a.w;
                     const Real D = Real(0.25) * r2 * (iRi * b.y);
                     const Real e = Pr::expm(D);
-                    const Real fi = Pr::rsqrt(r2 + (Ri * b.x) * e);
+                    const Real f2 = r2 + (Ri * b.x) * e;
+                    const Real fi = Pr::rsqrt(f2);
                     const Real qf3 = g * qq * fi * fi * fi;
                     Real tf = Real(1), td = Real(1);
                     if (salt) {
-                        const Real es = ieo * Pr::expm(kap / fi);
+                        const Real kf = kap * (f2 * fi);
+                        const Real es = ieo * Pr::expm(kf);
                         tf = iei - es;
-                        td = tf - kap * es / fi;
+                        td = tf - kf * es;
                     }
                     pdr += td * qf3 * b.x * e * (Real(1) + D);
                     const Real sig = sgi + b.z;
@@ -448,46 +455,43 @@ __global__ void __launch_bounds__(kTile) k_gb(const Item* __restrict__ items, Vi
             }
         }
     }
-    fx = group_total<WPA>(fx, gsh);
-    fy = group_total<WPA>(fy, gsh);
-    fz = group_total<WPA>(fz, gsh);
-    adr = group_total<WPA>(adr, gsh);
-    if (ENERGY) {
-        egb = group_total<WPA>(egb, gsh);
-        ec = group_total<WPA>(ec, gsh);
-        elj = group_total<WPA>(elj, gsh);
-    }
-    if (vi && sub == 0) {
+    if constexpr (ENERGY) sums.collect({fx, fy, fz, adr, egb, ec, elj});
+    else sums.collect({fx, fy, fz, adr});
+    if (tid >= kWarpAtoms) return;
+    long long e0 = 0, e1 = 0, e2 = 0;
+    if (it.i0 + tid < N) {
+        const int i = it.i0 + tid;
         const double q = V.q[A + i] * V.sqrt_k;
-        const double R = V.R[A + i];
-        const double dEdR = 0.5 * (V.tau_pair * Pr::value(adr, kScaleE)
-                                   + salt_taud(R, V.inv_eps_in, V.inv_eps_out, V.kappa) * q * q / (R * R))
-                          - (V.sa_gamma != 0.0 ? 6.0 * sa_ace(V.sa_gamma, V.sa_probe, V.rho[P + i], R) / R : 0.0);
+        const double R = V.R[A + i], iR = rcp64(R);
+        const double qqR = q * q * iR;
+        // tau(R) and its derivative form share one exponential
+        double tau = V.inv_eps_in - V.inv_eps_out, taud = tau;
+        if (V.kappa > 0.0) {
+            const double es = V.inv_eps_out * exp64(-V.kappa * R);
+            tau = V.inv_eps_in - es;
+            taud = tau - V.kappa * R * es;
+        }
+        const double sa = V.sa_gamma != 0.0 ? sa_ace(V.sa_gamma, V.sa_probe, V.rho[P + i], R) : 0.0;
+        const double dEdR = 0.5 * (V.tau_pair * Pr::value(sums.v[3][tid], kScaleE) + taud * qqR * iR)
+                          - 6.0 * sa * iR;
         const double c = dEdR * V.dRdpsi[A + i] * 0.5 * V.rt[P + i];
         V.c[A + i] = c;
-        if (sizeof(Real) == 4) V.c32[A + i] = (float)c;
-        V.Fd[3 * (A + i)] = Pr::value(fx, kScaleE);
-        V.Fd[3 * (A + i) + 1] = Pr::value(fy, kScaleE);
-        V.Fd[3 * (A + i) + 2] = Pr::value(fz, kScaleE);
+        V.c32[A + i] = (float)c;
+        for (int k = 0; k < 3; ++k) V.Fd[3 * (A + i) + k] = Pr::value(sums.v[k][tid], kScaleE);
+        if constexpr (ENERGY) {
+            e0 = __double2ll_rn((-0.5 * (V.tau_pair * Pr::value(sums.v[4][tid], kScaleE) + tau * qqR) + sa) * kScaleE);
+            e1 = __double2ll_rn(0.5 * V.inv_eps_in * Pr::value(sums.v[5][tid], kScaleE) * kScaleE);
+            e2 = __double2ll_rn(2.0 * Pr::value(sums.v[6][tid], kScaleE) * kScaleE);
+        }
     }
     if (ENERGY) {
-        long long e0 = 0, e1 = 0, e2 = 0;
-        if (vi && sub == 0) {
-            const double q = V.q[A + i] * V.sqrt_k;
-            const double R = V.R[A + i];
-            e0 = __double2ll_rn((-0.5 * (V.tau_pair * Pr::value(egb, kScaleE)
-                                         + salt_tau(R, V.inv_eps_in, V.inv_eps_out, V.kappa) * q * q / R)
-                                 + sa_ace(V.sa_gamma, V.sa_probe, V.rho[P + i], R)) * kScaleE);
-            e1 = __double2ll_rn(0.5 * V.inv_eps_in * Pr::value(ec, kScaleE) * kScaleE);
-            e2 = __double2ll_rn(2.0 * Pr::value(elj, kScaleE) * kScaleE);
-        }
-        long long t0 = block_sum_128(e0, red);
-        long long t1 = block_sum_128(e1, red);
-        long long t2 = block_sum_128(e2, red);
+        e0 = quad_total(e0);
+        e1 = quad_total(e1);
+        e2 = quad_total(e2);
         if (tid == 0) {
-            atomicAdd((unsigned long long*)&V.eacc[w * kEAcc + 0], (unsigned long long)t0);
-            atomicAdd((unsigned long long*)&V.eacc[w * kEAcc + 1], (unsigned long long)t1);
-            atomicAdd((unsigned long long*)&V.eacc[w * kEAcc + 2], (unsigned long long)t2);
+            atomicAdd((unsigned long long*)&V.eacc[w * kEAcc + 0], (unsigned long long)e0);
+            atomicAdd((unsigned long long*)&V.eacc[w * kEAcc + 1], (unsigned long long)e1);
+            atomicAdd((unsigned long long*)&V.eacc[w * kEAcc + 2], (unsigned long long)e2);
         }
     }
 }
@@ -633,19 +637,15 @@ template <bool ENERGY, bool STAGED>
 __global__ void __launch_bounds__(kTile) k_chain(const Item* __restrict__ items, View V) {
     pdl_sync();
     using Real = float;
-    constexpr int WPA = 1;
     using Pr = Prec<Real>;
     using Acc = typename Pr::Acc;
     __shared__ J4<Real> sa[kTile];
     __shared__ J2<Real> sb[kTile];
-    __shared__ long long red[4];
+    __shared__ AtomSums<3> sums;
     const Item it = items[blockIdx.x];
     const int w = it.w, s = V.w_sys[w], N = V.sys_n[s], A = V.w_off[w], P = V.sys_poff[s];
-    // WPA warps per atom i: the CTA holds kWarpAtoms / WPA atoms; `sub` indexes
-    // the thread within its atom's group of 32 WPA threads
-    const int tid = threadIdx.x, warp = tid >> 5, sub = tid - (warp / WPA) * 32 * WPA;
-    const int i = it.i0 + warp / WPA;
-    __shared__ long long gsh[kTile / 32];
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int i = it.i0 + (tid >> 5); // one warp per atom
     const bool vi = i < N;
     const Stage<Real, STAGED> stage(V, A, P, it.i0);
     Real xi = Real(-kFarF), yi = Real(-kFarF), zi = Real(-kFarF), ci = 0, si = 0, rti = 1;
@@ -687,7 +687,7 @@ __global__ void __launch_bounds__(kTile) k_chain(const Item* __restrict__ items,
         __syncthreads();
         if (jt != next) {
 #pragma unroll
-            for (int k = sub; k < kTile; k += 32 * WPA) {
+            for (int k = lane; k < kTile; k += 32) {
                 const J4<Real> a = sa[k];
                 const J2<Real> b = sb[k];
                 const Real dx = xi - a.x, dy = yi - a.y, dz = zi - a.z;
@@ -705,7 +705,7 @@ __global__ void __launch_bounds__(kTile) k_chain(const Item* __restrict__ items,
             next = mp < me ? V.mt_list[mp] : 0x7fffffff;
             const int dself = i - j0;
 #pragma unroll
-            for (int k = sub; k < kTile; k += 32 * WPA) {
+            for (int k = lane; k < kTile; k += 32) {
                 const J4<Real> a = sa[k];
                 const J2<Real> b = sb[k];
                 const bool self = (k == dself);
@@ -728,31 +728,41 @@ __global__ void __launch_bounds__(kTile) k_chain(const Item* __restrict__ items,
             px = py = pz = 0;
         }
     }
-    fx = group_total<WPA>(fx, gsh);
-    fy = group_total<WPA>(fy, gsh);
-    fz = group_total<WPA>(fz, gsh);
-    double eb = 0.0, ea = 0.0;
-    double Fb[3] = {0.0, 0.0, 0.0};
-    // bonded terms of atom i over the group's threads, summed in a fixed order
+    sums.collect({fx, fy, fz});
+    if (tid >= 32) return;
+    // bonded terms of the four atoms in one warp, eight lanes to an atom
+    constexpr int kL = 32 / kWarpAtoms;
+    const int ai = it.i0 + lane / kL;
     float fb[3] = {0.f, 0.f, 0.f}, ebf = 0.f, eaf = 0.f;
-    if (vi) bonded_atom32(V, A, P, i, sub, 32 * WPA, fb, ebf, eaf);
+    if (ai < N) bonded_atom32(V, A, P, ai, lane % kL, kL, fb, ebf, eaf);
+    __syncwarp();
 #pragma unroll
-    for (int c = 0; c < 3; ++c) Fb[c] = (double)group_total<WPA>(fb[c], gsh);
-    eb = (double)group_total<WPA>(ebf, gsh);
-    ea = (double)group_total<WPA>(eaf, gsh);
-    if (sub != 0) eb = ea = 0.0; // the group's totals, counted once
-    if (vi && sub == 0) {
-        double F[3] = {V.Fd[3 * (A + i)] + Pr::value(fx, kScaleE) + Fb[0],
-                       V.Fd[3 * (A + i) + 1] + Pr::value(fy, kScaleE) + Fb[1],
-                       V.Fd[3 * (A + i) + 2] + Pr::value(fz, kScaleE) + Fb[2]};
-        V.F[3 * (A + i)] = F[0];
-        V.F[3 * (A + i) + 1] = F[1];
-        V.F[3 * (A + i) + 2] = F[2];
+    for (int o = kL / 2; o > 0; o >>= 1) {
+        for (int c = 0; c < 3; ++c) fb[c] += __shfl_down_sync(0xffffffffu, fb[c], o, kL);
+        if (ENERGY) {
+            ebf += __shfl_down_sync(0xffffffffu, ebf, o, kL);
+            eaf += __shfl_down_sync(0xffffffffu, eaf, o, kL);
+        }
+    }
+    // then lane w finishes atom w
+    for (int c = 0; c < 3; ++c) fb[c] = __shfl_sync(0xffffffffu, fb[c], lane * kL & 31);
+    if (ENERGY) {
+        ebf = __shfl_sync(0xffffffffu, ebf, lane * kL & 31);
+        eaf = __shfl_sync(0xffffffffu, eaf, lane * kL & 31);
+    }
+    if (lane >= kWarpAtoms) return;
+    if (it.i0 + lane < N) {
+        const int b = 3 * (A + it.i0 + lane);
+        double F[3];
+        for (int c = 0; c < 3; ++c) {
+            F[c] = V.Fd[b + c] + Pr::value(sums.v[c][lane], kScaleE) + (double)fb[c];
+            V.F[b + c] = F[c];
+        }
         if (!(isfinite(F[0]) && isfinite(F[1]) && isfinite(F[2]))) atomicOr(V.status, 1);
     }
     if (ENERGY) {
-        long long t0 = block_sum_128(__double2ll_rn(eb * kScaleE), red);
-        long long t1 = block_sum_128(__double2ll_rn(ea * kScaleE), red);
+        const long long t0 = quad_total(__double2ll_rn((double)ebf * kScaleE));
+        const long long t1 = quad_total(__double2ll_rn((double)eaf * kScaleE));
         if (tid == 0) {
             atomicAdd((unsigned long long*)&V.eacc[w * kEAcc + 3], (unsigned long long)t0);
             atomicAdd((unsigned long long*)&V.eacc[w * kEAcc + 4], (unsigned long long)t1);

@@ -413,6 +413,17 @@ __device__ __forceinline__ bool hct_empty(float r, float rt, float s, float rc) 
     return fmaxf(rt, fabsf(r - s)) >= fminf(r + s, rc);
 }
 
+// H for a pair known to be in the far regime (hct_far), and dH/dr
+__device__ __forceinline__ float hct_series(float rinv, float s) {
+    const float x = s * rinv, y = x * x;
+    return x * y * hct_series_h(y) * rinv;
+}
+
+__device__ __forceinline__ float hct_dr_series(float rinv2, float rinv, float s) {
+    const float x = s * rinv, y = x * x;
+    return -x * y * hct_series_dr(y) * rinv2;
+}
+
 __device__ __forceinline__ float hct(float r, float rinv, float rt, float irt, float s, float rc = INFINITY) {
     if (hct_far(r, rt, s, rc)) {
         float x = s * rinv, y = x * x;
@@ -574,6 +585,25 @@ struct KSum {
         s = t;
     }
     __device__ __forceinline__ Real value() const { return s; }
+};
+
+template <>
+struct KSum<float2> { // two sums, one value
+    float2 s = {0.f, 0.f}, c = {0.f, 0.f};
+    __device__ __forceinline__ void add(float2 v) {
+        const float2 m = {-1.f, -1.f};
+        const float2 y = __ffma2_rn(c, m, v);
+        const float2 t = __fadd2_rn(s, y);
+        c = __ffma2_rn(y, m, __ffma2_rn(s, m, t));
+        s = t;
+    }
+    __device__ __forceinline__ float value() const {
+        KSum<float> k;
+        k.s = s.x;
+        k.c = c.x + c.y;
+        k.add(s.y);
+        return k.s;
+    }
 };
 
 template <>

@@ -16,6 +16,7 @@
 
 #include "cph_kernels.cuh"
 #include "cph_launch.h"
+#include "cph_ordered.cuh"
 #include "cph_sym.cuh"
 #include "cph_f64.cuh"
 #include "cph_small.cuh"
@@ -744,22 +745,13 @@ bool sys_ordered(const cph_engine* E, int s) {
 // The ordered passes run one warp per atom (four atoms per CTA), or, in FP64
 // mode with few atoms (E->ordered_wpa = 4), four warps per atom: even a single
 // small walker then spreads its FP64 work over one CTA per atom.
-// f with the warps per atom (FP64 mode) or the operand source (FP32 mode) as a constant
-template <class F, class G>
-void by_form(const cph_engine* E, F&& f64, G&& f32) {
-    if (E->precision == CPH_PREC_FP64) {
-        if (E->ordered_wpa == 4) f64(std::integral_constant<int, 4>{});
-        else f64(std::integral_constant<int, 1>{});
-    } else if (E->staged) f32(std::true_type{});
-    else f32(std::false_type{});
-}
-
+// FP32 mode: the passes over the staged operands, or over the master arrays.
 int launch_born(cph_engine* E, const Item* items, int n, bool zero_energy, cudaStream_t st) {
     if (n <= 0) return CPH_OK;
-    const int ze = zero_energy ? 1 : 0;
-    by_form(
-        E, [&](auto wpa) { launch_next(k_born64<decltype(wpa)::value>, n, kTile, st, items, E->V, ze); },
-        [&](auto staged) { launch_next(k_born<decltype(staged)::value>, n, kTile, st, items, E->V, ze); });
+    auto go = [&](auto kernel) { launch_next(kernel, n, kTile, st, items, E->V, zero_energy ? 1 : 0); };
+    if (E->precision == CPH_PREC_FP64) E->ordered_wpa == 4 ? go(k_born64<4>) : go(k_born64<1>);
+    else if (!E->staged) go(k_born);
+    else E->V.rgbmax < INFINITY ? go(k_born32<true>) : go(k_born32<false>);
     CK(cudaGetLastError());
     return CPH_OK;
 }
@@ -767,19 +759,33 @@ int launch_born(cph_engine* E, const Item* items, int n, bool zero_energy, cudaS
 int launch_gb(cph_engine* E, const Item* items, int n, bool energy, cudaStream_t st) {
     if (n <= 0) return CPH_OK;
     auto go = [&](auto kernel) { launch_next(kernel, n, kTile, st, items, E->V); };
-    by_form(
-        E, [&](auto wpa) { energy ? go(k_gb64<true, decltype(wpa)::value>) : go(k_gb64<false, decltype(wpa)::value>); },
-        [&](auto staged) { energy ? go(k_gb<true, decltype(staged)::value>) : go(k_gb<false, decltype(staged)::value>); });
+    if (E->precision == CPH_PREC_FP64) {
+        if (E->ordered_wpa == 4) energy ? go(k_gb64<true, 4>) : go(k_gb64<false, 4>);
+        else energy ? go(k_gb64<true, 1>) : go(k_gb64<false, 1>);
+    } else if (!E->staged) {
+        energy ? go(k_gb<true>) : go(k_gb<false>);
+    } else if (E->V.kappa > 0) { // a salt factor per pair: two exponentials instead of one
+        energy ? go(k_gb32<true, true>) : go(k_gb32<false, true>);
+    } else {
+        energy ? go(k_gb32<true, false>) : go(k_gb32<false, false>);
+    }
     CK(cudaGetLastError());
     return CPH_OK;
 }
 
 int launch_chain(cph_engine* E, const Item* items, int n, bool energy, cudaStream_t st) {
     if (n <= 0) return CPH_OK;
-    auto go = [&](auto kernel) { launch_next(kernel, n, kTile, st, items, E->V); };
-    by_form(
-        E, [&](auto wpa) { energy ? go(k_chain64<true, decltype(wpa)::value>) : go(k_chain64<false, decltype(wpa)::value>); },
-        [&](auto staged) { energy ? go(k_chain<true, decltype(staged)::value>) : go(k_chain<false, decltype(staged)::value>); });
+    auto go = [&](auto kernel, int threads = kTile) { launch_next(kernel, n, threads, st, items, E->V); };
+    if (E->precision == CPH_PREC_FP64) {
+        if (E->ordered_wpa == 4) energy ? go(k_chain64<true, 4>) : go(k_chain64<false, 4>);
+        else energy ? go(k_chain64<true, 1>) : go(k_chain64<false, 1>);
+    } else if (!E->staged) {
+        energy ? go(k_chain<true>) : go(k_chain<false>);
+    } else if (E->V.rgbmax < INFINITY) {
+        energy ? go(k_chain32<true, true>, kChainThreads) : go(k_chain32<false, true>, kChainThreads);
+    } else {
+        energy ? go(k_chain32<true, false>, kChainThreads) : go(k_chain32<false, false>, kChainThreads);
+    }
     CK(cudaGetLastError());
     return CPH_OK;
 }

@@ -54,7 +54,7 @@ struct AtomSums {
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             const long long s = warp_total(acc[k]);
-            if ((threadIdx.x & 31) == 0) v[k][warp] = s;
+            if ((threadIdx.x & 31) == 0 && warp < kWarpAtoms) v[k][warp] = s;
         }
         __syncthreads();
     }
@@ -91,63 +91,29 @@ __device__ __forceinline__ Real host_const(double d, float f) {
     else return d;
 }
 
-// Where the ordered passes get an atom's operands from.  STAGED (FP32): the
-// arrays staged once per step (positions relative to the walker's first atom),
-// since every CTA reads every atom of its walker and each FP64 subtraction,
-// division or conversion holds a sub-partition's FP64 pipe for 64 clocks.
-// Else (FP64, and FP32 with constraints, see cph_engine::staged): the master
-// arrays, positions relative to the CTA's first atom.
-template <class Real, bool STAGED>
-struct Stage {
+// An atom's operands from the master arrays, positions relative to the CTA's
+// first atom (the passes of engines with constraints, see cph_engine::staged).
+struct Masters {
     const View& V;
     int A, P;
     double cx, cy, cz;
-    __device__ __forceinline__ Stage(const View& v, int a, int p, int i0) : V(v), A(a), P(p) {
+    __device__ __forceinline__ Masters(const View& v, int a, int p, int i0) : V(v), A(a), P(p) {
         cx = V.x[3 * (A + i0)];
         cy = V.x[3 * (A + i0) + 1];
         cz = V.x[3 * (A + i0) + 2];
     }
-    __device__ __forceinline__ J4<Real> position(int i) const {
-        return {Real(V.x[3 * (A + i)] - cx), Real(V.x[3 * (A + i) + 1] - cy), Real(V.x[3 * (A + i) + 2] - cz), Real(0)};
-    }
-    __device__ __forceinline__ J4<Real> gb(int i) const { // sqrt(k) q, R, 1/R
-        const double R = V.R[A + i];
-        return {Real(V.q[A + i]) * Real(V.sqrt_k), Real(R), Real(1.0 / R), Real(0)};
-    }
-    __device__ __forceinline__ J2<Real> lj(int i) const { // sigma / 2, sqrt(eps)
-        return {Real(V.sigh[P + i]), Real(V.sqe[P + i])};
-    }
-    __device__ __forceinline__ J2<Real> radii(int i) const { return {Real(V.sc[P + i]), Real(V.rt[P + i])}; } // s, rt
-    __device__ __forceinline__ Real weight(int i) const { return Real(V.c[A + i]); }
-    // whether tile jt ends a run of tiles whose partials are summed together
-    static __device__ __forceinline__ bool flush(int) { return true; }
-};
-
-template <>
-struct Stage<float, true> {
-    const View& V;
-    int A, P;
-    __device__ __forceinline__ Stage(const View& v, int a, int p, int) : V(v), A(a), P(p) {}
     __device__ __forceinline__ J4<float> position(int i) const {
-        const float4 p = V.xs[A + i];
-        return {p.x, p.y, p.z, 0.f};
+        return {float(V.x[3 * (A + i)] - cx), float(V.x[3 * (A + i) + 1] - cy), float(V.x[3 * (A + i) + 2] - cz), 0.f};
     }
-    __device__ __forceinline__ J4<float> gb(int i) const {
-        const float4 g = V.gq[A + i];
-        return {g.x, g.y, g.z, 0.f};
+    __device__ __forceinline__ J4<float> gb(int i) const { // sqrt(k) q, R, 1/R
+        const double R = V.R[A + i];
+        return {float(V.q[A + i]) * float(V.sqrt_k), float(R), float(1.0 / R), 0.f};
     }
-    __device__ __forceinline__ J2<float> lj(int i) const {
-        const float2 l = V.plj32[P + i];
-        return {l.x, l.y};
+    __device__ __forceinline__ J2<float> lj(int i) const { // sigma / 2, sqrt(eps)
+        return {float(V.sigh[P + i]), float(V.sqe[P + i])};
     }
-    __device__ __forceinline__ J2<float> radii(int i) const {
-        const float4 r = V.pb32[P + i];
-        return {r.x, r.y};
-    }
-    __device__ __forceinline__ float weight(int i) const { return V.c32[A + i]; }
-    // eight tiles are summed in FP32 and converted once (a conversion issues to
-    // the narrow FP64 pipe too)
-    static __device__ __forceinline__ bool flush(int jt) { return (jt & 7) == 7; }
+    __device__ __forceinline__ J2<float> radii(int i) const { return {float(V.sc[P + i]), float(V.rt[P + i])}; } // s, rt
+    __device__ __forceinline__ float weight(int i) const { return float(V.c[A + i]); }
 };
 
 // Per-walker energy accumulators (fixed point 2^32): GB, Coulomb, LJ, bond, angle.
@@ -184,10 +150,81 @@ __device__ inline void tile_masks(const View& V, int P, int i, bool vi, int j0, 
     }
 }
 
+// ------------------------------------------------ ends of the ordered passes
+// What an atom's end of pass reads, to be loaded before the CTA's barrier.
+struct BornIn {
+    double rt, irho, irt, q;
+    BornIn() = default;
+    __device__ __forceinline__ BornIn(const View& V, int A, int P, int i)
+        : rt(V.rt[P + i]), irho(V.irho[P + i]), irt(V.irt[P + i]), q(V.q[A + i]) {} // 1/rho, 1/rt from set-up
+};
+
+__device__ __forceinline__ void born_epilogue(const View& V, int A, int P, int i, long long sum, const BornIn& in) {
+    const double psi = 0.5 * in.rt * Prec<float>::value(sum, kScaleH);
+    const double th = tanh64(psi * (V.alpha + psi * (-V.beta + psi * V.gamma)));
+    const double R = rcp64(in.irt - th * in.irho);
+    V.psi[A + i] = psi;
+    V.R[A + i] = R;
+    V.gq[A + i] = gb_operand(in.q, V.sqrt_k, R);
+    V.Ffix[3 * (A + i)] = 0;
+    V.Ffix[3 * (A + i) + 1] = 0;
+    V.Ffix[3 * (A + i) + 2] = 0;
+    V.dRfix[A + i] = 0;
+    V.dRdpsi[A + i] = R * R * (1.0 - th * th) * (V.alpha + psi * (-2.0 * V.beta + 3.0 * V.gamma * psi)) * in.irho;
+}
+
+struct GbIn {
+    double q, R, dRdpsi, rt, rho;
+    GbIn() = default;
+    __device__ __forceinline__ GbIn(const View& V, int A, int P, int i)
+        : q(V.q[A + i]), R(V.R[A + i]), dRdpsi(V.dRdpsi[A + i]), rt(V.rt[P + i]), rho(V.rho[P + i]) {}
+};
+
+// lanes 0 .. 3 of warp 0; own: the lane's atom exists
+template <bool ENERGY, class Sums>
+__device__ __forceinline__ void gb_epilogue(const View& V, int A, int P, int w, int i, bool own, const Sums& sums,
+                                            const GbIn& in) {
+    using Pr = Prec<float>;
+    const int l = threadIdx.x;
+    long long e0 = 0, e1 = 0, e2 = 0;
+    if (own) {
+        const double q = in.q * V.sqrt_k;
+        const double R = in.R, iR = rcp64(R);
+        const double qqR = q * q * iR;
+        // tau(R) and its derivative form share one exponential
+        double tau = V.inv_eps_in - V.inv_eps_out, taud = tau;
+        if (V.kappa > 0.0) {
+            const double es = V.inv_eps_out * exp64(-V.kappa * R);
+            tau = V.inv_eps_in - es;
+            taud = tau - V.kappa * R * es;
+        }
+        const double sa = V.sa_gamma != 0.0 ? sa_ace(V.sa_gamma, V.sa_probe, in.rho, R) : 0.0;
+        const double dEdR = 0.5 * (V.tau_pair * Pr::value(sums.v[3][l], kScaleE) + taud * qqR * iR) - 6.0 * sa * iR;
+        const double c = dEdR * in.dRdpsi * 0.5 * in.rt;
+        V.c[A + i] = c;
+        V.c32[A + i] = (float)c;
+        for (int k = 0; k < 3; ++k) V.Fd[3 * (A + i) + k] = Pr::value(sums.v[k][l], kScaleE);
+        if constexpr (ENERGY) {
+            e0 = __double2ll_rn((-0.5 * (V.tau_pair * Pr::value(sums.v[4][l], kScaleE) + tau * qqR) + sa) * kScaleE);
+            e1 = __double2ll_rn(0.5 * V.inv_eps_in * Pr::value(sums.v[5][l], kScaleE) * kScaleE);
+            e2 = __double2ll_rn(2.0 * Pr::value(sums.v[6][l], kScaleE) * kScaleE);
+        }
+    }
+    if constexpr (ENERGY) {
+        e0 = quad_total(e0);
+        e1 = quad_total(e1);
+        e2 = quad_total(e2);
+        if (l == 0) {
+            atomicAdd((unsigned long long*)&V.eacc[w * kEAcc + 0], (unsigned long long)e0);
+            atomicAdd((unsigned long long*)&V.eacc[w * kEAcc + 1], (unsigned long long)e1);
+            atomicAdd((unsigned long long*)&V.eacc[w * kEAcc + 2], (unsigned long long)e2);
+        }
+    }
+}
+
 // ------------------------------------------------------------- pass 1: Born radii
 // psi_i = rt_i/2 sum_{j != i} H(r_ij, rt_i, s_j); R_i = 1/(1/rt_i - tanh(theta)/rho_i)
 // with theta = alpha psi - beta psi^2 + gamma psi^3, finalised in FP64.
-template <bool STAGED>
 __global__ void __launch_bounds__(kTile) k_born(const Item* __restrict__ items, View V,
                                                 int zero_energy) {
     pdl_sync();
@@ -204,7 +241,7 @@ __global__ void __launch_bounds__(kTile) k_born(const Item* __restrict__ items, 
         if (zero_energy && tid < kEAcc) V.eacc[w * kEAcc + tid] = 0;
         if (tid == kEAcc) V.vscale[w] = 1.0;
     }
-    const Stage<Real, STAGED> stage(V, A, P, it.i0);
+    const Masters stage(V, A, P, it.i0);
     Real xi = Real(-kFarF), yi = Real(-kFarF), zi = Real(-kFarF), rti = Real(1);
     if (vi) {
         const J4<Real> p = stage.position(i);
@@ -260,35 +297,19 @@ __global__ void __launch_bounds__(kTile) k_born(const Item* __restrict__ items, 
                 part += self ? Real(0) : h;
             }
         }
-        if (stage.flush(jt)) {
-            Pr::add(acc, part, Real(kScaleH));
-            part = 0;
-        }
+        Pr::add(acc, part, Real(kScaleH));
+        part = 0;
     }
-    Pr::add(acc, part, Real(kScaleH));
     sums.collect({acc});
     if (tid < kWarpAtoms && it.i0 + tid < N) {
-        const int i = it.i0 + tid;
-        const double sumH = Pr::value(sums.v[0][tid], kScaleH);
-        const double rt = V.rt[P + i], irho = V.irho[P + i]; // 1/rt, 1/rho from set-up
-        const double psi = 0.5 * rt * sumH;
-        const double th = tanh64(psi * (V.alpha + psi * (-V.beta + psi * V.gamma)));
-        const double R = rcp64(V.irt[P + i] - th * irho);
-        V.psi[A + i] = psi;
-        V.R[A + i] = R;
-        V.gq[A + i] = gb_operand(V.q[A + i], V.sqrt_k, R);
-        V.Ffix[3 * (A + i)] = 0;
-        V.Ffix[3 * (A + i) + 1] = 0;
-        V.Ffix[3 * (A + i) + 2] = 0;
-        V.dRfix[A + i] = 0;
-        V.dRdpsi[A + i] = R * R * (1.0 - th * th) * (V.alpha + psi * (-2.0 * V.beta + 3.0 * V.gamma * psi)) * irho;
+        born_epilogue(V, A, P, it.i0 + tid, sums.v[0][tid], BornIn(V, A, P, it.i0 + tid));
     }
 }
 
 // ------------------------------------------- pass 2: GB + Coulomb + LJ pair pass
 // Owner i accumulates the direct force, dE_GB/dR_i and (optionally) its share
 // of the energies; the epilogue turns dE/dR_i into c_i = dE/dR_i dR_i/dpsi_i rt_i/2.
-template <bool ENERGY, bool STAGED>
+template <bool ENERGY>
 __global__ void __launch_bounds__(kTile) k_gb(const Item* __restrict__ items, View V) {
     pdl_sync();
     using Real = float;
@@ -302,7 +323,7 @@ __global__ void __launch_bounds__(kTile) k_gb(const Item* __restrict__ items, Vi
     const int tid = threadIdx.x, lane = tid & 31;
     const int i = it.i0 + (tid >> 5); // one warp per atom
     const bool vi = i < N;
-    const Stage<Real, STAGED> stage(V, A, P, it.i0);
+    const Masters stage(V, A, P, it.i0);
     Real xi = Real(-kFarF), yi = Real(-kFarF), zi = Real(-kFarF);
     Real qi = 0, Ri = 1, iRi = 1, sgi = 0, sei = 0;
     if (vi) {
@@ -441,59 +462,23 @@ __global__ void __launch_bounds__(kTile) k_gb(const Item* __restrict__ items, Vi
                 }
             }
         }
-        if (stage.flush(jt) || j0 + kTile >= N) {
-            Pr::add(fx, px, Real(kScaleE));
-            Pr::add(fy, py, Real(kScaleE));
-            Pr::add(fz, pz, Real(kScaleE));
-            Pr::add(adr, pdr, Real(kScaleE));
-            px = py = pz = pdr = 0;
-            if (ENERGY) {
-                Pr::add(egb, pgb.value(), Real(kScaleE));
-                Pr::add(ec, pc.value(), Real(kScaleE));
-                Pr::add(elj, plj.value(), Real(kScaleE));
-                pgb = pc = plj = KSum<Real>();
-            }
+        Pr::add(fx, px, Real(kScaleE));
+        Pr::add(fy, py, Real(kScaleE));
+        Pr::add(fz, pz, Real(kScaleE));
+        Pr::add(adr, pdr, Real(kScaleE));
+        px = py = pz = pdr = 0;
+        if (ENERGY) {
+            Pr::add(egb, pgb.value(), Real(kScaleE));
+            Pr::add(ec, pc.value(), Real(kScaleE));
+            Pr::add(elj, plj.value(), Real(kScaleE));
+            pgb = pc = plj = KSum<Real>();
         }
     }
     if constexpr (ENERGY) sums.collect({fx, fy, fz, adr, egb, ec, elj});
     else sums.collect({fx, fy, fz, adr});
     if (tid >= kWarpAtoms) return;
-    long long e0 = 0, e1 = 0, e2 = 0;
-    if (it.i0 + tid < N) {
-        const int i = it.i0 + tid;
-        const double q = V.q[A + i] * V.sqrt_k;
-        const double R = V.R[A + i], iR = rcp64(R);
-        const double qqR = q * q * iR;
-        // tau(R) and its derivative form share one exponential
-        double tau = V.inv_eps_in - V.inv_eps_out, taud = tau;
-        if (V.kappa > 0.0) {
-            const double es = V.inv_eps_out * exp64(-V.kappa * R);
-            tau = V.inv_eps_in - es;
-            taud = tau - V.kappa * R * es;
-        }
-        const double sa = V.sa_gamma != 0.0 ? sa_ace(V.sa_gamma, V.sa_probe, V.rho[P + i], R) : 0.0;
-        const double dEdR = 0.5 * (V.tau_pair * Pr::value(sums.v[3][tid], kScaleE) + taud * qqR * iR)
-                          - 6.0 * sa * iR;
-        const double c = dEdR * V.dRdpsi[A + i] * 0.5 * V.rt[P + i];
-        V.c[A + i] = c;
-        V.c32[A + i] = (float)c;
-        for (int k = 0; k < 3; ++k) V.Fd[3 * (A + i) + k] = Pr::value(sums.v[k][tid], kScaleE);
-        if constexpr (ENERGY) {
-            e0 = __double2ll_rn((-0.5 * (V.tau_pair * Pr::value(sums.v[4][tid], kScaleE) + tau * qqR) + sa) * kScaleE);
-            e1 = __double2ll_rn(0.5 * V.inv_eps_in * Pr::value(sums.v[5][tid], kScaleE) * kScaleE);
-            e2 = __double2ll_rn(2.0 * Pr::value(sums.v[6][tid], kScaleE) * kScaleE);
-        }
-    }
-    if (ENERGY) {
-        e0 = quad_total(e0);
-        e1 = quad_total(e1);
-        e2 = quad_total(e2);
-        if (tid == 0) {
-            atomicAdd((unsigned long long*)&V.eacc[w * kEAcc + 0], (unsigned long long)e0);
-            atomicAdd((unsigned long long*)&V.eacc[w * kEAcc + 1], (unsigned long long)e1);
-            atomicAdd((unsigned long long*)&V.eacc[w * kEAcc + 2], (unsigned long long)e2);
-        }
-    }
+    const bool own = it.i0 + tid < N;
+    gb_epilogue<ENERGY>(V, A, P, w, it.i0 + tid, own, sums, own ? GbIn(V, A, P, it.i0 + tid) : GbIn());
 }
 
 // Bonded forces on atom i (system-local index li) and its owned energy
@@ -630,10 +615,59 @@ __device__ inline void bonded_atom32(const View& V, int A, int P, int li, int la
     }
 }
 
+// Bonded terms of a CTA's four atoms in one warp, eight lanes to an atom.
+struct BondedSums {
+    float f[kWarpAtoms][3], eb[kWarpAtoms], ea[kWarpAtoms];
+    template <bool ENERGY>
+    __device__ __forceinline__ void take(const View& V, int A, int P, int i0, int N, int lane) {
+        constexpr int kL = 32 / kWarpAtoms;
+        const int a = lane / kL;
+        float fb[3] = {0.f, 0.f, 0.f}, ebf = 0.f, eaf = 0.f;
+        if (i0 + a < N) bonded_atom32(V, A, P, i0 + a, lane % kL, kL, fb, ebf, eaf);
+        __syncwarp();
+#pragma unroll
+        for (int o = kL / 2; o > 0; o >>= 1) {
+            for (int c = 0; c < 3; ++c) fb[c] += __shfl_down_sync(0xffffffffu, fb[c], o, kL);
+            if (ENERGY) {
+                ebf += __shfl_down_sync(0xffffffffu, ebf, o, kL);
+                eaf += __shfl_down_sync(0xffffffffu, eaf, o, kL);
+            }
+        }
+        if (lane % kL == 0) {
+            for (int c = 0; c < 3; ++c) f[a][c] = fb[c];
+            eb[a] = ebf;
+            ea[a] = eaf;
+        }
+    }
+};
+
+// lanes 0 .. 3 of warp 0; own: the lane's atom exists
+template <bool ENERGY, class Sums>
+__device__ __forceinline__ void chain_epilogue(const View& V, int A, int w, int i, bool own, const Sums& sums,
+                                               const BondedSums& bonded) {
+    const int l = threadIdx.x;
+    if (own) {
+        double F[3];
+        for (int c = 0; c < 3; ++c) {
+            F[c] = V.Fd[3 * (A + i) + c] + Prec<float>::value(sums.v[c][l], kScaleE) + (double)bonded.f[l][c];
+            V.F[3 * (A + i) + c] = F[c];
+        }
+        if (!(isfinite(F[0]) && isfinite(F[1]) && isfinite(F[2]))) atomicOr(V.status, 1);
+    }
+    if (ENERGY) {
+        const long long t0 = quad_total(__double2ll_rn((double)bonded.eb[l] * kScaleE));
+        const long long t1 = quad_total(__double2ll_rn((double)bonded.ea[l] * kScaleE));
+        if (l == 0) {
+            atomicAdd((unsigned long long*)&V.eacc[w * kEAcc + 3], (unsigned long long)t0);
+            atomicAdd((unsigned long long*)&V.eacc[w * kEAcc + 4], (unsigned long long)t1);
+        }
+    }
+}
+
 // ------------------------------------------ pass 3: chain rule through Born radii
 // F_i -= sum_j (c_i dH(r; rt_i, s_j)/dr + c_j dH(r; rt_j, s_i)/dr) (x_i - x_j)/r,
 // then the direct pair force and the bonded terms are added: F is the total force.
-template <bool ENERGY, bool STAGED>
+template <bool ENERGY>
 __global__ void __launch_bounds__(kTile) k_chain(const Item* __restrict__ items, View V) {
     pdl_sync();
     using Real = float;
@@ -647,7 +681,7 @@ __global__ void __launch_bounds__(kTile) k_chain(const Item* __restrict__ items,
     const int tid = threadIdx.x, lane = tid & 31;
     const int i = it.i0 + (tid >> 5); // one warp per atom
     const bool vi = i < N;
-    const Stage<Real, STAGED> stage(V, A, P, it.i0);
+    const Masters stage(V, A, P, it.i0);
     Real xi = Real(-kFarF), yi = Real(-kFarF), zi = Real(-kFarF), ci = 0, si = 0, rti = 1;
     if (vi) {
         const J4<Real> p = stage.position(i);
@@ -721,53 +755,15 @@ __global__ void __launch_bounds__(kTile) k_chain(const Item* __restrict__ items,
                 pz += t * dz;
             }
         }
-        if (stage.flush(jt) || j0 + kTile >= N) {
-            Pr::add(fx, px, Real(kScaleE));
-            Pr::add(fy, py, Real(kScaleE));
-            Pr::add(fz, pz, Real(kScaleE));
-            px = py = pz = 0;
-        }
+        Pr::add(fx, px, Real(kScaleE));
+        Pr::add(fy, py, Real(kScaleE));
+        Pr::add(fz, pz, Real(kScaleE));
+        px = py = pz = 0;
     }
+    __shared__ BondedSums bonded;
+    if (tid < 32) bonded.take<ENERGY>(V, A, P, it.i0, N, lane);
     sums.collect({fx, fy, fz});
-    if (tid >= 32) return;
-    // bonded terms of the four atoms in one warp, eight lanes to an atom
-    constexpr int kL = 32 / kWarpAtoms;
-    const int ai = it.i0 + lane / kL;
-    float fb[3] = {0.f, 0.f, 0.f}, ebf = 0.f, eaf = 0.f;
-    if (ai < N) bonded_atom32(V, A, P, ai, lane % kL, kL, fb, ebf, eaf);
-    __syncwarp();
-#pragma unroll
-    for (int o = kL / 2; o > 0; o >>= 1) {
-        for (int c = 0; c < 3; ++c) fb[c] += __shfl_down_sync(0xffffffffu, fb[c], o, kL);
-        if (ENERGY) {
-            ebf += __shfl_down_sync(0xffffffffu, ebf, o, kL);
-            eaf += __shfl_down_sync(0xffffffffu, eaf, o, kL);
-        }
-    }
-    // then lane w finishes atom w
-    for (int c = 0; c < 3; ++c) fb[c] = __shfl_sync(0xffffffffu, fb[c], lane * kL & 31);
-    if (ENERGY) {
-        ebf = __shfl_sync(0xffffffffu, ebf, lane * kL & 31);
-        eaf = __shfl_sync(0xffffffffu, eaf, lane * kL & 31);
-    }
-    if (lane >= kWarpAtoms) return;
-    if (it.i0 + lane < N) {
-        const int b = 3 * (A + it.i0 + lane);
-        double F[3];
-        for (int c = 0; c < 3; ++c) {
-            F[c] = V.Fd[b + c] + Pr::value(sums.v[c][lane], kScaleE) + (double)fb[c];
-            V.F[b + c] = F[c];
-        }
-        if (!(isfinite(F[0]) && isfinite(F[1]) && isfinite(F[2]))) atomicOr(V.status, 1);
-    }
-    if (ENERGY) {
-        const long long t0 = quad_total(__double2ll_rn((double)ebf * kScaleE));
-        const long long t1 = quad_total(__double2ll_rn((double)eaf * kScaleE));
-        if (tid == 0) {
-            atomicAdd((unsigned long long*)&V.eacc[w * kEAcc + 3], (unsigned long long)t0);
-            atomicAdd((unsigned long long*)&V.eacc[w * kEAcc + 4], (unsigned long long)t1);
-        }
-    }
+    if (tid < kWarpAtoms) chain_epilogue<ENERGY>(V, A, w, it.i0 + tid, it.i0 + tid < N, sums, bonded);
 }
 
 // ------------------------------------------------------------ Langevin step

@@ -82,17 +82,6 @@ __device__ __forceinline__ void sym_masks(const View& V, int P, int i, bool vi, 
     }
 }
 
-// H for a pair known to be in the far regime (both directions valid)
-__device__ __forceinline__ float hct_series(float rinv, float s) {
-    const float x = s * rinv, y = x * x;
-    return x * y * hct_series_h(y) * rinv;
-}
-
-__device__ __forceinline__ float hct_dr_series(float rinv2, float rinv, float s) {
-    const float x = s * rinv, y = x * x;
-    return -x * y * hct_series_dr(y) * rinv2;
-}
-
 // ============================================== operand staging (FP32)
 // The pair kernels read FP32 operands only.  Positions are taken relative to
 // the walker's first atom (|x| stays within the molecule's extent, so FP32

@@ -281,15 +281,29 @@ def whole_job_value(grid_walkers, steps, t_max):
 
 
 def schedule_launches(t, mc_ph=10, mc_redox=10, ex_every=100):
-    """Kernels one batched FP32 step t launches through a one-step cph_run:
+    """The stages of one batched FP32 step t of a one-step cph_run, one by one:
     position staging + Born-radii pair kernel + finish, GB staging + pair
     kernel + finish, chain pair kernel + bonded terms + force finish,
     observables, Langevin, the step-counter tick; each MC sweep kind adds the
     staging of its charges and radii and its per-site and per-walker kernels,
-    an exchange step its row and attempt kernels."""
+    an exchange step its row and attempt kernels.  Some of them share a launch
+    (``step_kernels`` counts those)."""
     n = 3 + 3 + 3 + 1 + 1 + 1
     if t > 0:
         n += 3 * (int(t % mc_ph == 0) + int(t % mc_redox == 0)) + 2 * int(t % ex_every == 0)
+    return n
+
+
+def step_kernels(t, any_ordered=False, mc_ph=10, mc_redox=10, ex_every=100):
+    """Kernels that step t launches: of schedule_launches' stages the GB staging
+    is part of the Born-radii finish, the bonded terms of the chain pair kernel
+    and the observables of the Langevin kernel; the first MC sweep kind reads
+    what the Born-radii finish staged, and a staging follows the last one.
+    ``any_ordered``: some system on one warp per atom adds its three passes."""
+    n = 9 + (3 if any_ordered else 0)
+    if t > 0:
+        kinds = int(t % mc_ph == 0) + int(t % mc_redox == 0)
+        n += 3 * kinds + 2 * int(t % ex_every == 0)
     return n
 
 
@@ -511,8 +525,8 @@ def config_leg(name, cfg, precision, n_steps, dev, stream, sm_mhz, oracle_plan=N
                            "basis": "three pair passes against the step roofline (FP32 lanes, MUFU)"}
     else:
         out["roofline"] = {"bound": "latency",
-                           "note": "FP64 mode, one small system: a step is ~10 dependent launches "
-                                   "of a few microseconds each"}
+                           "note": "FP64 mode, one small system: a step is four dependent launches "
+                                   "of ten microseconds or so each"}
     del eng, eng2
     if oracle_plan is not None:
         # plans: (walkers, steps, threads); the first is the leg's cpu_baseline,
@@ -598,7 +612,7 @@ def run_gpu(args):
             starts[k].record(stream)
             advance(1)
             ends[k].record(stream)
-            launches += schedule_launches(t_first + k)
+            launches += step_kernels(t_first + k, "warp per atom" in shapes)
         barrier()
         wall = time.perf_counter() - wall0
     eng.status()

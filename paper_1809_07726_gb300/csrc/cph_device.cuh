@@ -413,17 +413,6 @@ __device__ __forceinline__ bool hct_empty(float r, float rt, float s, float rc) 
     return fmaxf(rt, fabsf(r - s)) >= fminf(r + s, rc);
 }
 
-// H for a pair known to be in the far regime (hct_far), and dH/dr
-__device__ __forceinline__ float hct_series(float rinv, float s) {
-    const float x = s * rinv, y = x * x;
-    return x * y * hct_series_h(y) * rinv;
-}
-
-__device__ __forceinline__ float hct_dr_series(float rinv2, float rinv, float s) {
-    const float x = s * rinv, y = x * x;
-    return -x * y * hct_series_dr(y) * rinv2;
-}
-
 __device__ __forceinline__ float hct(float r, float rinv, float rt, float irt, float s, float rc = INFINITY) {
     if (hct_far(r, rt, s, rc)) {
         float x = s * rinv, y = x * x;
@@ -538,37 +527,6 @@ __device__ __forceinline__ double hct(double r, double rinv, double rt, double i
         if (rt < top) h += 2.0 * (irt - 1.0 / top);
     }
     return h;
-}
-
-__device__ __forceinline__ double hct_dr(double r, double rinv, double rt, double s, double rc = INFINITY) {
-    const double U = fmin(r + s, rc), L = fmax(rt, fabs(r - s));
-    double d = 0.0;
-    if (L < U) {
-        double iL = 1.0 / L, iU = 1.0 / U;
-        double rinv2 = rinv * rinv;
-        d = -0.25 * (iL - iU) * (iL + iU) * (1.0 + s * s * rinv2) - 0.5 * log(L * iU) * rinv2;
-    }
-    return d;
-}
-
-__device__ __forceinline__ double hct_ds(double r, double rinv, double rt, double s, double rc = INFINITY) {
-    const double U = fmin(r + s, rc), L = fmax(rt, fabs(r - s));
-    double d = 0.0;
-    if (L < U) {
-        double iL = 1.0 / L, iU = 1.0 / U;
-        d = 0.5 * s * rinv * (iL - iU) * (iL + iU);
-    }
-    return d;
-}
-
-__device__ __forceinline__ double hct_drt(double r, double rt, double irt, double s, double rc = INFINITY) {
-    const double U = fmin(r + s, rc), L = fmax(rt, fabs(r - s));
-    if (rt < s - r) return rt < fmin(s - r, rc) ? -2.0 * irt * irt : 0.0;
-    if (rt > fabs(r - s) && L < U) {
-        double a = rt - r;
-        return (a * a - s * s) * 0.5 / r * irt * irt * irt;
-    }
-    return 0.0;
 }
 
 // ------------------------------------------------- compensated summation

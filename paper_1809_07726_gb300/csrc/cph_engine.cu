@@ -1,5 +1,6 @@
 // Engine: set-up, Monte-Carlo titration, replica exchange and the C ABI of
-// cphremd.h.  The pair passes and the integrator are in cph_kernels.cuh.
+// cphremd.h.  The integrator and the bonded terms are in cph_kernels.cuh, the pair
+// passes there and in cph_sym.cuh, cph_ordered.cuh, cph_small.cuh and cph_f64.cuh.
 #include <algorithm>
 #include <cmath>
 #include <cstdarg>

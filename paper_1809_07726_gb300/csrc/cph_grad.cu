@@ -39,7 +39,6 @@ namespace grad {
 // are never live together share memory:
 //   0 psi | 1 R | 2 Hfix -> dRfix -> dE/dR | 3 dR/dpsi -> dE/dpsi | 4 c
 //   5 dqfix -> dE/dq | 6-8 gradient (fixed point) | 9 art | 10 as
-constexpr int kSlots = 11;
 
 inline size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 

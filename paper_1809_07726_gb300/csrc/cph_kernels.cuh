@@ -2,20 +2,19 @@
 // grid, bonded terms, Langevin integration, Monte-Carlo titration sweeps and
 // replica exchanges.  Host code lives in cph_engine.cu.
 //
-// Work decomposition of the three ordered pair passes (FP64 mode).  One CTA of
-// kTile threads owns kWarpAtoms consecutive atoms i, one warp each; the CTA
-// sweeps all j of its walker in tiles of kTile staged in shared memory, lane l
-// of a warp taking entries l, l + 32, l + 64, l + 96 of every tile, so every
-// ordered pair (i, j) is evaluated by the warp of i.  A lane's partial sums
-// are added per tile into its accumulator; the warp's accumulators are
-// reduced by a fixed shuffle tree at the end, so the result of an atom does
-// not depend on the launch shape (batched and per-replica launches agree bit
-// for bit) and no atomics are needed.  A warp per atom spreads even a
-// 160-atom walker over 40 CTAs (FP64 arithmetic is a small fraction of the
-// chip's, so it must run on every SM).  With Real = float the operands come
-// staged in FP32 and the partials of eight tiles (32 pairs a lane, as many as a
-// tile pair of the symmetric passes sums) go into int64 fixed-point
-// accumulators (scales 2^32 and 2^40); with double everything is FP64.
+// Work decomposition of the ordered pair passes (here, and in FP64 in
+// cph_f64.cuh).  One CTA of kTile threads owns kWarpAtoms consecutive atoms i, one
+// warp each; the CTA sweeps all j of its walker in tiles of kTile staged in
+// shared memory, lane l of a warp taking entries l, l + 32, l + 64, l + 96 of
+// every tile, so every ordered pair (i, j) is evaluated by the warp of i.  A
+// lane's partial sums are added per tile into its int64 fixed-point accumulator
+// (scales 2^32 and 2^40) and reduced by a fixed shuffle tree at the end, so the
+// result of an atom does not depend on the launch shape (batched and per-replica
+// launches agree bit for bit) and no atomics are needed.
+//
+// k_born, k_gb and k_chain below are those of FP32 engines with constraints, over
+// the FP64 master arrays; other FP32 engines run cph_ordered.cuh over staged
+// operands, and whole steps of walkers of up to 512 atoms run in cph_small.cuh.
 //
 // Tiles in which some atom i of the CTA meets itself or an excluded partner
 // are listed per (system, i-tile) at set-up; only those run the masked loop.

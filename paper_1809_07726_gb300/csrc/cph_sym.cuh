@@ -24,8 +24,9 @@
 // atom (times 1 + 1e-5), so for r >= r_far every descreening integral of the
 // pair is in its disjoint-sphere series regime; one comparison of r^2 then
 // selects the series for both directions.  Pairs inside r_far take closed
-// forms: queued per warp in the Born pass (born_tile_q), in line behind a warp
-// vote in the chain-rule pass.  In the GB pass each i-atom row of a step
+// forms: queued per warp in the Born pass (born_tile_q) and, in the chain-rule
+// pass, for systems of up to kQueueAtoms atoms, in line behind a warp vote for
+// larger ones.  In the GB pass each i-atom row of a step
 // whose pairs all have D = r^2 / (4 R_i R_j) >= 18 takes the far GB form
 // (kGbFarD2).
 #pragma once

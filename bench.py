@@ -67,8 +67,9 @@ BACKWARD_COST = (100, 4)
 BACKWARD_FAR_COST = (90, 3)
 N_SM = 152
 # DRAM bytes (read + write) per launch of a pass's pair kernel, from one
-# one-kernel ncu capture of each current kernel on this workload
-PASS_DRAM_BYTES = {"born": 32.95e6 + 0.0, "gb": 89.23e6 + 6.39e6, "chain": 59.84e6 + 0.06e6}
+# one-pass ncu capture of each current kernel on this workload (the chain pass's
+# holds the bonded terms' blocks)
+PASS_DRAM_BYTES = {"born": 33.04e6 + 0.0, "gb": 91.74e6 + 6.97e6, "chain": 94.25e6 + 59.19e6}
 FP32_LANES = 128   # FP32 lane operations per clock per SM
 MUFU_LANES = 16    # MUFU operations per clock per SM
 

@@ -548,9 +548,9 @@ __device__ __forceinline__ void bond_term32(const double (&d)[3], double r0d, do
 
 // One harmonic angle i-j-k from u = x_i - x_j, v = x_k - x_j (FP64) and
 // (cos theta0, sin theta0): the force on i is -gi, on k -gk, on j gi + gk;
-// e its energy.
+// kz holds the two factors of gk[2], e the energy.
 __device__ __forceinline__ void angle_term32(const double (&u)[3], const double (&v)[3], double2 cs0, double kad,
-                                             float (&gi)[3], float (&gk)[3], float& e) {
+                                             float (&gi)[3], float (&gk)[3], float2& kz, float& e) {
     // |u||v| cos(theta) and |u||v| sin(theta) in FP64 (the norm of the cross
     // product by an FP32 reciprocal square root and one Newton step)
     const double uv = u[0] * v[0] + u[1] * v[1] + u[2] * v[2];
@@ -574,7 +574,9 @@ __device__ __forceinline__ void angle_term32(const double (&u)[3], const double 
     const float k = -2.f * ka * dth / sn;                     // dE/dcos(theta)
     for (int c = 0; c < 3; ++c) {
         gi[c] = k * (vf[c] * iuv - cs * uf[c] / ru2);
-        gk[c] = k * (uf[c] * iuv - cs * vf[c] / rv2);
+        const float wk = uf[c] * iuv - cs * vf[c] / rv2;
+        gk[c] = k * wk;
+        if (c == 2) kz = make_float2(k, wk);
     }
     e = ka * dth * dth;
 }
@@ -604,7 +606,8 @@ __device__ inline void bonded_atom32(const View& V, int A, int P, int li, int la
             v[c] = x[3 * (A + ic) + c] - x[3 * (A + ib) + c];
         }
         float gi[3], gk[3], en;
-        angle_term32(u, v, V.ang_cs0[a], V.ang_k[a], gi, gk, en);
+        float2 kz;
+        angle_term32(u, v, V.ang_cs0[a], V.ang_k[a], gi, gk, kz, en);
         for (int c = 0; c < 3; ++c) {
             if (li == ia) F[c] -= gi[c];
             if (li == ic) F[c] -= gk[c];

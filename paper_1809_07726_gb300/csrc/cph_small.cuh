@@ -8,8 +8,8 @@
 // separated by hardware cluster barriers (~400 clocks), and a launch runs
 // steps until the schedule needs something of another kernel (a titration
 // sweep, an exchange attempt).  Measured, with sweeps every 10 steps: 8 x 160
-// atoms 58.5 -> 22.3 us a step (15 in this kernel: 31,000 clocks), 4 x 246 atoms
-// with constraints 91 -> 41 us.  Which walkers come here: small_setup in
+// atoms 58.5 -> 20 us a step (15 in this kernel), 4 x 246 atoms with constraints
+// 91 -> 39 us.  Which walkers come here: small_setup in
 // cph_engine.cu.
 //
 // Work split.  A cluster of eight CTAs (portable; of sixteen-CTA clusters only
@@ -102,13 +102,13 @@ struct SmallSmem {
     float* z;        // [3 own] normal random numbers
     uint32_t* ex;    // [own][32] excluded partners
     float* rel;      // [own / 4][3][n] positions relative to the first atom of each group of four
-    float* tf;       // [terms][6] bonded forces: bond g d; angle gi, gk
+    float* tf;       // [terms][8] bonded forces: bond g d; angle gi, gk, the factors of gk's z
     float* te;       // [terms] bonded energies
 };
 
 __host__ __device__ inline size_t small_bytes(int n, int own, int terms) {
     return (size_t)n * (2 * 24 + 2 * 24 + 16 + 16 + 4) + (n & 1) * 4 +
-           (size_t)own * (24 + sizeof(SmallAtom) + 64 + 24 + 12 + 12 + 128) + (size_t)terms * 28 + (size_t)(own / 4) * 12 * n + 16;
+           (size_t)own * (24 + sizeof(SmallAtom) + 64 + 24 + 12 + 12 + 128) + (size_t)terms * 36 + (size_t)(own / 4) * 12 * n + 16;
 }
 
 __device__ __forceinline__ SmallSmem small_carve(unsigned char* p, int n, int own, int terms) {
@@ -126,7 +126,7 @@ __device__ __forceinline__ SmallSmem small_carve(unsigned char* p, int n, int ow
     s.z = s.fb + 3 * own;
     s.ex = (uint32_t*)(s.z + 3 * own);
     s.tf = (float*)(s.ex + 32 * own);
-    s.te = s.tf + 6 * terms;
+    s.te = s.tf + 8 * terms;
     s.rel = s.te + terms;
     return s;
 }
@@ -144,10 +144,13 @@ __device__ __forceinline__ void add2(float& h, float& l, float b) {
 // displacements; with R the bond vector before the sweeps and D the difference of
 // the two displacements, d0^2 - |R + D|^2 = (d0^2 - R^2) - (2 R + D) . D.  The
 // first term is formed once in FP64; displacements and the second term are kept
-// as pairs of floats (1e-14 of d0^2, against a tolerance of 1e-8 and less), the
-// size of a step needs no more than FP32 (what is left of the constraint decides
-// the next one).  In FP64 a constraint took ~35 instructions of 64 clocks: 39,000
-// clocks a step at 4 x 246 atoms.
+// as pairs of floats (1e-14 of d0^2, against a tolerance of 1e-8 and less), and
+// so is the step along the bond: an FP32 quotient would do for the constraint, but
+// leaves the sweeps somewhere else within the tolerance (1e-11 A), which a
+// trajectory grows until it shows in the forces' roundings (100 steps of 48 runs:
+// velocities off k_shake's by up to 1.4e-5, with the pair by 8e-6 in one system
+// and 6e-7 in the others; 1.92 -> 1.96 ms for 50 steps of 4 x 246 atoms).  In FP64 a
+// constraint took ~35 instructions of 64 clocks: 39,000 clocks a step there.
 // Sum of h + l over the cluster's lanes, the same in each.
 __device__ __forceinline__ void sum4(float& h, float& l) {
 #pragma unroll
@@ -163,7 +166,7 @@ __device__ __noinline__ void small_shake(const View& V, const float4* fac, int c
                                          double* xt, int nh, double (&u)[NH + 1]) {
     const bool live = on && d < 3;
     const int h0 = V.shk_off[c], a0 = V.shk_heavy[c];
-    float Rh[NH], Rl[NH], old[NH], d0h[NH], d0l[NH], tol[NH];
+    float Rh[NH], Rl[NH], old[NH], oldl[NH], d0h[NH], d0l[NH], tol[NH];
     float uh[NH + 1], ul[NH + 1];   // displacements of the heavy atom and the hydrogens
     float2 dir0[NH], dirk[NH];      // their directions: mass factor times old bond vector
     const double x0 = live ? xt[3 * a0 + d] : 0.0, o0 = live ? xo[3 * a0 + d] : 0.0;
@@ -178,6 +181,7 @@ __device__ __noinline__ void small_shake(const View& V, const float4* fac, int c
         const float2 o = split2(has ? o0 - xo[3 * a + d] : 0.0);
         const float4 f = on && k < nh ? fac[h0 + k] : make_float4(0.f, 0.f, 0.f, 0.f);
         old[k] = o.x;
+        oldl[k] = o.y;
         dir0[k].x = f.x * o.x;
         dir0[k].y = fmaf(f.x, o.x, -dir0[k].x) + fmaf(f.x, o.y, f.y * o.x);
         dirk[k].x = f.z * o.x;
@@ -204,19 +208,22 @@ __device__ __noinline__ void small_shake(const View& V, const float4* fac, int c
             add2(sh, sl, dh);
             float ph = sh * dh;
             float pl = fmaf(sh, dh, -ph) + fmaf(sh, dl, sl * dh);
-            float dot = old[k] * fmaf(0.5f, Rh[k], dh);
+            float qh = 0.5f * Rh[k], ql = fmaf(0.5f, Rl[k], dl); // R / 2 + D, here R is twice the bond
+            add2(qh, ql, dh);
+            float dot = old[k] * qh, dotl = fmaf(old[k], qh, -dot) + fmaf(old[k], ql, oldl[k] * qh);
             sum4(ph, pl);
-            dot += __shfl_xor_sync(0xffffffffu, dot, 1);
-            dot += __shfl_xor_sync(0xffffffffu, dot, 2);
+            sum4(dot, dotl);
             float eh = d0h[k], el = d0l[k] - pl;
             add2(eh, el, -ph);
             const float diff = eh + el;
             if (!done && fabsf(diff) > tol[k]) {
                 moved = true;
-                const float g = __fdividef(diff, dot); // the products below are exact to 1e-14
+                // diff / dot and the products to 1e-14
+                const float g = __fdividef(diff, dot);
+                const float gl = __fdividef(fmaf(-g, dot, eh) + fmaf(-g, dotl, el), dot);
                 const float p0 = g * dir0[k].x, pk = -g * dirk[k].x;
-                ul[0] += fmaf(g, dir0[k].x, -p0) + g * dir0[k].y;
-                ul[k + 1] += fmaf(-g, dirk[k].x, -pk) - g * dirk[k].y;
+                ul[0] += fmaf(g, dir0[k].x, -p0) + fmaf(g, dir0[k].y, gl * dir0[k].x);
+                ul[k + 1] += fmaf(-g, dirk[k].x, -pk) - fmaf(g, dirk[k].y, gl * dirk[k].x);
                 add2(uh[0], ul[0], p0);
                 add2(uh[k + 1], ul[k + 1], pk);
             }
@@ -355,7 +362,7 @@ __global__ void __launch_bounds__(GA == 1 ? 704 : 576, 1) k_small(View V, SmallT
                 const double* x = (S.x + 3 * N * cur);
                 for (int t = atid; t < nterm; t += 32 * kSmallAux) {
                     const int k = T.term[toff[0] + t];
-                    float* f = S.tf + 6 * t;
+                    float* f = S.tf + 8 * t;
                     if (t < nbond) {
                         const int i = V.bond_ij[2 * k], j = V.bond_ij[2 * k + 1];
                         double d[3];
@@ -372,7 +379,10 @@ __global__ void __launch_bounds__(GA == 1 ? 704 : 576, 1) k_small(View V, SmallT
                             v[c] = x[3 * l + c] - x[3 * j + c];
                         }
                         float gi[3], gk[3], en;
-                        angle_term32(u, v, V.ang_cs0[k], V.ang_k[k], gi, gk, en);
+                        float2 kz;
+                        angle_term32(u, v, V.ang_cs0[k], V.ang_k[k], gi, gk, kz, en);
+                        f[6] = kz.x;
+                        f[7] = kz.y;
                         for (int c = 0; c < 3; ++c) {
                             f[c] = gi[c];
                             f[3 + c] = gk[c];
@@ -505,16 +515,19 @@ __global__ void __launch_bounds__(GA == 1 ? 704 : 576, 1) k_small(View V, SmallT
                         for (int e = r0 + l8; e < rm; e += 8) {
                             const int k = T.ref[e], t = k >> 2;
                             const float sg = (k & 3) ? 1.f : -1.f;
-                            for (int c = 0; c < 3; ++c) fb[c] += sg * S.tf[6 * t + c];
+                            for (int c = 0; c < 3; ++c) fb[c] += sg * S.tf[8 * t + c];
                             if ((k & 3) == 0) eb += S.te[t];
                         }
                         for (int e = rm + l8; e < r1; e += 8) {
                             const int k = T.ref[e], t = k >> 2, role = k & 3;
-                            const float* f = S.tf + 6 * t;
+                            const float* f = S.tf + 8 * t;
+                            // (z rounds gk's product and its sum at once, as the one-lane-a-term
+                            // sums of the ordered kernel do: constrained trajectories follow
+                            // every rounding, see cph_engine::staged)
                             for (int c = 0; c < 3; ++c) {
                                 if (role == 0) fb[c] -= f[c];
-                                else if (role == 2) fb[c] -= f[3 + c];
-                                else fb[c] += f[c] + f[3 + c];
+                                else if (role == 2) fb[c] = c == 2 && e < rm + 8 ? fmaf(-f[6], f[7], fb[2]) : fb[c] - f[3 + c];
+                                else fb[c] += c == 2 ? fmaf(f[6], f[7], f[2]) : f[c] + f[3 + c];
                             }
                             if (role == 0) ea += S.te[t];
                         }

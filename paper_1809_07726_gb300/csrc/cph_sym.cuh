@@ -631,7 +631,8 @@ __device__ __noinline__ void bonded_block(const View& V, int w, int t, bool ener
             v[c] = x[3 * (A + ic) + c] - x[3 * (A + ib) + c];
         }
         float gi[3], gk[3], e;
-        angle_term32(u, v, V.ang_cs0[a], V.ang_k[a], gi, gk, e);
+        float2 kz;
+        angle_term32(u, v, V.ang_cs0[a], V.ang_k[a], gi, gk, kz, e);
         float* o = buf + 6 * (size_t)nb + 9 * (size_t)la;
         for (int c = 0; c < 3; ++c) {
             o[c] = -gi[c];

@@ -1024,7 +1024,8 @@ int launch_langevin(cph_engine* E, int s_off, cudaStream_t st) {
     const int batched = E->launch_mode == 0;
     auto one = [&](int a0, int n, cudaStream_t s) {
         // few atoms: a warp to a block, so that each has a sub-partition's FP64 to itself
-        const int bs = n <= 32 * 152 ? 32 : 256, grid = (n + bs - 1) / bs, obs = batched ? E->V.W : 0;
+        const int threads = n * (E->precision == CPH_PREC_FP32 ? kLangevinThreads<float> : kLangevinThreads<double>);
+        const int bs = threads <= 32 * 152 ? 32 : 256, grid = (threads + bs - 1) / bs, obs = batched ? E->V.W : 0;
         if (E->precision == CPH_PREC_FP32) launch_next(k_langevin<float>, grid + obs, bs, s, E->V, s_off, a0, n, obs);
         else launch_next(k_langevin<double>, grid + obs, bs, s, E->V, s_off, a0, n, obs);
     };

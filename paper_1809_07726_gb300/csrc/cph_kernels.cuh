@@ -798,18 +798,17 @@ __device__ __forceinline__ void sincos64(uint32_t w, double& sn, double& cs) {
     cs = ((k + 1u) & 2u) ? -b : b;
 }
 
-// The library's sincospi, log and sqrt took ~190 FP64 instructions, this ~85.
-__device__ __forceinline__ void normals64(uint64_t seed, uint32_t idx, uint32_t stream, uint64_t step, double z[3],
-                                          const double2* tab) {
+// The library's sincospi, log and sqrt took ~190 FP64 instructions for an atom's
+// three normals, this ~85: one of their two Box-Muller pairs (z0, z1) or (z2, -).
+__device__ __forceinline__ void normals64(uint64_t seed, uint32_t idx, uint32_t stream, uint64_t step, int pair,
+                                          double z[2], const double2* tab) {
     const U4 u = draw(seed, idx, stream, step, kRngLangevin);
-    const double l0 = -2.0 * log64(unit_open(u.a), tab), l1 = -2.0 * log64(unit_open(u.c), tab);
-    const double r0 = l0 * rsqrt64(l0), r1 = l1 * rsqrt64(l1);
-    double sn, cs, s1, c1;
-    sincos64(u.b, sn, cs);
-    sincos64(u.d, s1, c1);
-    z[0] = r0 * cs;
-    z[1] = r0 * sn;
-    z[2] = r1 * c1;
+    const double l = -2.0 * log64(unit_open(pair ? u.c : u.a), tab);
+    const double r = l * rsqrt64(l);
+    double sn, cs;
+    sincos64(pair ? u.d : u.b, sn, cs);
+    z[0] = r * cs;
+    z[1] = r * sn;
 }
 
 __device__ inline void normals3(uint64_t seed, uint32_t idx, uint32_t stream,
@@ -839,6 +838,11 @@ __device__ inline void observe_walker(const View& V, int w, int tid, int n) {
     for (int k = tid; k < ns; k += n) V.occ[(row0 + k) * CPH_MAX_STATES + V.site_state[ws0 + k]] += 1;
 }
 
+// Threads to an atom: in FP64 one for each Box-Muller pair, whose FP64 chain is
+// most of the kernel for a small walker (100 steps of 160 atoms 4.92 -> 4.74 ms).
+template <class Real>
+constexpr int kLangevinThreads = sizeof(Real) == 8 ? 2 : 1;
+
 // Blocks past the atoms' own (obs of them, one per walker) take the step's sample
 // of the observables, which depends on nothing the step moves: a launch of 5 us
 // less a step.
@@ -855,7 +859,8 @@ __global__ void k_langevin(View V, int s_off, int a0, int n, int obs) {
         load_tab64(tab, threadIdx.x, blockDim.x);
         __syncthreads();
     }
-    const int l = blockIdx.x * blockDim.x + threadIdx.x;
+    constexpr int kT = kLangevinThreads<Real>;
+    const int thread = blockIdx.x * blockDim.x + threadIdx.x, l = thread / kT;
     if (l >= n) return;
     const int a = a0 + l;
     const int w = V.a_walker[a];
@@ -864,8 +869,9 @@ __global__ void k_langevin(View V, int s_off, int a0, int n, int obs) {
     const int P = V.sys_poff[V.w_sys[w]];
     const uint64_t t = (uint64_t)(*V.step + s_off);
     const int slot = V.slot_of[w];
+    const int first = kT == 1 ? 0 : 2 * (thread % kT), nc = kT == 1 ? 3 : 2 - thread % kT; // the thread's components
     Real z[3];
-    if constexpr (sizeof(Real) == 8) normals64(V.seed, (uint32_t)li, (uint32_t)w, t, z, tab);
+    if constexpr (sizeof(Real) == 8) normals64(V.seed, (uint32_t)li, (uint32_t)w, t, thread % kT, z, tab);
     else normals3(V.seed, (uint32_t)li, (uint32_t)w, t, z);
     // per-atom factors dt A / m and sqrt(2 g kB A dt / m), and sqrt(T) per
     // slot, are set up once: no FP64 division or square root per step
@@ -874,8 +880,10 @@ __global__ void k_langevin(View V, int s_off, int a0, int n, int obs) {
     const double vs = V.vscale[w];
     bool ok = true;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const double vn = (c1 * (V.v[3 * a + c] * vs) + im * V.F[3 * a + c] + sd * (double)z[c]) * c2;
+    for (int k = 0; k < (kT == 1 ? 3 : 2); ++k) {
+        if (k >= nc) break;
+        const int c = first + k;
+        const double vn = (c1 * (V.v[3 * a + c] * vs) + im * V.F[3 * a + c] + sd * (double)z[k]) * c2;
         V.v[3 * a + c] = vn;
         if (V.xprev) V.xprev[3 * a + c] = V.x[3 * a + c]; // SHAKE's reference bond vectors
         const double xn = V.x[3 * a + c] + V.dt * vn;

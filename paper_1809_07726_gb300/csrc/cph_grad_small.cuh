@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(kGsThreads) __cluster_dims__(kGsRanks, 1, 1) k
         const float rt = g.rho[base + j] - off;
         st[j] = make_float4(g.screen[j] * rt, rt, 1.f / rt, 0.f);
     }
-    __syncthreads();
+    sync(); // the operands; and every CTA of the cluster runs, so that others may store into its memory
     // ---- Born radii
     for (int a = warp; a < nown; a += kGsThreads / 32) {
         const int i = a0 + a;

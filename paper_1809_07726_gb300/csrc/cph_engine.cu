@@ -1175,14 +1175,16 @@ int get_graph(cph_engine* E, cudaGraphExec_t* out) {
 namespace {
 
 // Tables and launch shape of the small-walker kernel, if every system fits it:
-// FP32 mode, at most kSmallAtoms atoms and kSmallTerms bonded terms in a CTA, and
-// a device that can hold the cluster.
+// FP32 mode, at most kSmallAtoms atoms and kSmallTerms bonded terms in a CTA, a
+// SHAKE tolerance of at least kSmallShakeTol, and a device that can hold the
+// cluster.
 int small_setup(cph_engine* E, const std::vector<int>& bond_off, const std::vector<int>& bond_idx,
                 const std::vector<int>& bond_ij, const std::vector<int>& ang_off, const std::vector<int>& ang_idx,
                 const std::vector<int>& ang_ijk, const std::vector<int>& sys_poff, const std::vector<int>& shk_sys_off,
                 const std::vector<float4>& shk_fac) {
     const int nmax = *std::max_element(E->h_sys_n.begin(), E->h_sys_n.end());
     if (E->precision != CPH_PREC_FP32 || nmax > kSmallAtoms) return CPH_OK;
+    if (E->V.xprev && E->V.shake_tol < kSmallShakeTol) return CPH_OK;
     const int ranks = kSmallRanks, ga = nmax <= 160 ? 1 : (nmax <= 256 ? 2 : 4); // atoms per warp
     E->small_ga = ga;
     {

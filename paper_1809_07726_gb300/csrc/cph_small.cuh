@@ -44,6 +44,10 @@ constexpr int kSmallAtoms = 512;  // atoms of a walker at most
 constexpr int kSmallTerms = 1024; // bonded terms that touch a CTA's atoms at most
 constexpr int kSmallAux = 2;      // extra warps per CTA
 constexpr int kSmallRanks = 8;    // CTAs per cluster
+// SHAKE tolerances from here on: the pairs of floats of small_shake leave up to
+// 3e-14 of d0^2 (measured at a tolerance of 1e-14), so below that they settle late,
+// never, or elsewhere.  Tighter ones take the separate launches (k_shake, FP64).
+constexpr double kSmallShakeTol = 1e-12;
 constexpr int kSmallUnroll = 2;   // of the partner loops (1 to 4: within 3 %)
 
 // phases of a step: where a launch starts its first step and ends its last

@@ -10,7 +10,7 @@
 //   sigh, sqe, mass  double [system atoms]       sigma/2, sqrt(eps), mass
 //   eacc             int64  [W * 5]              fixed-point (2^32) energy terms per walker
 //   Ffix, dRfix      int64  [3N], [N]            fixed-point (2^32) pair-force and dE/dR sums
-//   xs, gq           float4 [total_atoms]        FP32 positions / GB terms for the pair kernels
+//   xs, xl, gq       float4 [total_atoms]        FP32 positions, their low words / GB terms for the pair kernels
 //   c32              float  [total_atoms]        FP32 chain-rule weights
 //   pb32, plj32      float4, float2 [system atoms] static FP32 radii / LJ parameters
 //   occ              int64  [sites * 8]          state counts per (slot, site) row
@@ -108,7 +108,8 @@ struct View {
     // count; INFINITY = none
     double rgbmax;
     // FP32 pair-kernel operands, staged once per step by one thread per atom
-    float4* xs;          // (x, y, z, 0) relative to the walker's first atom
+    float4* xs;          // (x, y, z) relative to the walker's first atom; s (static)
+    float4* xl;          // what the rounding of xs left (systems on the ordered passes); rt (static)
     float4* gq;          // (sqrt(k) q, R, 1/R, log2(e) / (4 R)), after the Born radii and MC
     float* c32;          // chain-rule weights c
     const float4* pb32;  // per system atom, static: (s, rt, 1/rt, 0)

@@ -14,7 +14,9 @@
 // closed forms inside the loop: 1 x 2003 atoms 25.9 -> 17.4, 22.8 -> 18.7 and
 // 28.7 -> 20.5 us (Born radii, pair pass, chain rule); 8 x 1203 atoms with salt and a
 // cutoff of 12 A, energies, 41.8 -> 37.5, 49.7 -> 43.2 and 59.5 -> 55.2 us (half of
-// their pairs within reach lie in the cutoff's band of closed forms).
+// their pairs within reach lie in the cutoff's band of closed forms).  These without
+// the positions' low words (Place), which cost 8 %: 20 steps of 1 x 2003 atoms
+// 1.13 -> 1.21 ms, 8 x 1203 atoms 212 -> 227 us.
 #pragma once
 #include "cph_kernels.cuh"
 #include "cph_pair_tiles.cuh"
@@ -58,6 +60,32 @@ struct NearQueue {
 
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
 
+// An atom's place: its position relative to the walker's first atom as h + l, and
+// its s and rt.  The separation of two atoms is then rounded to FP32 once, however
+// far from that first atom they are; h alone leaves 4e-6 A of error at 40 A in the
+// separation of neighbours (extended chains of 600 to 3000 atoms: Born radii off by
+// 4e-6 to 2e-5 relative, with l 2e-7).
+struct Place {
+    float4 h, l; // (x, y, z, s), (x, y, z, rt)
+};
+__device__ __forceinline__ Place place(const View& V, int a) { return {V.xs[a], V.xl[a]}; }
+// in place of an atom i, and of a partner, that does not exist: no pair of theirs counts
+__device__ __forceinline__ Place far_place() {
+    return {make_float4(-kFarF, -kFarF, -kFarF, 0.f), make_float4(0.f, 0.f, 0.f, 1.f)};
+}
+__device__ __forceinline__ Place no_place() {
+    return {make_float4(kFarF, kFarF, kFarF, 0.f), make_float4(0.f, 0.f, 0.f, 1.f)};
+}
+__device__ __forceinline__ void separation(const Place& i, const Place& a, const Place& b, float2& dx, float2& dy,
+                                           float2& dz) {
+    auto one = [](float hi, float li, float ha, float la, float hb, float lb) {
+        return __fadd2_rn(sub2(splat<float2>(hi), make_float2(ha, hb)), sub2(splat<float2>(li), make_float2(la, lb)));
+    };
+    dx = one(i.h.x, i.l.x, a.h.x, a.l.x, b.h.x, b.l.x);
+    dy = one(i.h.y, i.l.y, a.h.y, a.l.y, b.h.y, b.l.y);
+    dz = one(i.h.z, i.l.z, a.h.z, a.l.z, b.h.z, b.l.z);
+}
+
 // ------------------------------------------------------------- pass 1: Born radii
 // CUT: with a Born-radius cutoff
 template <bool CUT>
@@ -74,15 +102,11 @@ __global__ void __launch_bounds__(kTile) k_born32(const Item* __restrict__ items
         if (zero_energy && tid < kEAcc) V.eacc[w * kEAcc + tid] = 0;
         if (tid == kEAcc) V.vscale[w] = 1.0;
     }
-    float4 xi = make_float4(-kFarF, -kFarF, -kFarF, 0.f);
-    float rti = 1.f;
-    if (i < N) {
-        xi = V.xs[A + i];
-        rti = V.pb32[P + i].y;
-    }
+    Place me = far_place();
+    if (i < N) me = place(V, A + i);
+    const float rti = me.l.w;
     const PairBand band = pair_band(V.rfar2, V.smax32, (float)V.rgbmax);
     const float irti = 1.f / rti;
-    const float2 x2 = splat<float2>(xi.x), y2 = splat<float2>(xi.y), z2 = splat<float2>(xi.z);
     long long acc = 0;
     float2 far = splat<float2>(0.f);
     float part = 0.f;
@@ -91,26 +115,22 @@ __global__ void __launch_bounds__(kTile) k_born32(const Item* __restrict__ items
         const float rinv = Pr::rsqrt(e.x);
         part += hct(e.x * rinv, rinv, rti, irti, e.y, band.rc);
     };
-    auto load = [&](float4 (&p)[kBatch], int j0) {
+    auto load = [&](Place (&p)[kBatch], int j0) {
 #pragma unroll
         for (int u = 0; u < kBatch; ++u) {
             const int j = j0 + 32 * u + lane;
-            p[u] = make_float4(kFarF, kFarF, kFarF, 0.f);
-            if (j < N) {
-                p[u] = V.xs[A + j];
-                p[u].w = V.pb32[P + j].x;
-            }
+            p[u] = no_place();
+            if (j < N) p[u] = place(V, A + j);
         }
     };
-    auto work = [&](const float4 (&p)[kBatch], int j0) {
+    auto work = [&](const Place (&p)[kBatch], int j0) {
         float2 e[kBatch];
         bool near[kBatch];
 #pragma unroll
         for (int u = 0; u < kBatch; u += 2) {
-            const float2 dx = sub2(x2, make_float2(p[u].x, p[u + 1].x));
-            const float2 dy = sub2(y2, make_float2(p[u].y, p[u + 1].y));
-            const float2 dz = sub2(z2, make_float2(p[u].z, p[u + 1].z));
-            const float2 sj = make_float2(p[u].w, p[u + 1].w), s2 = __fmul2_rn(sj, sj);
+            float2 dx, dy, dz;
+            separation(me, p[u], p[u + 1], dx, dy, dz);
+            const float2 sj = make_float2(p[u].h.w, p[u + 1].h.w), s2 = __fmul2_rn(sj, sj);
             float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
             e[u] = make_float2(r2.x, sj.x);
             e[u + 1] = make_float2(r2.y, sj.y);
@@ -120,7 +140,7 @@ __global__ void __launch_bounds__(kTile) k_born32(const Item* __restrict__ items
             r2.y = near[u + 1] ? INFINITY : r2.y;
             near[u] = near[u] && j0 + 32 * u + lane != i;
             near[u + 1] = near[u + 1] && j0 + 32 * u + 32 + lane != i;
-            const float2 rinv2 = make_float2(rcp_ftz(r2.x), rcp_ftz(r2.y));
+            const float2 rinv = make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y)), rinv2 = __fmul2_rn(rinv, rinv);
             float2 wt = __fmul2_rn(rinv2, rinv2);
             if (CUT) { // beyond rc + s_max nothing descreens
                 wt.x = r2.x >= band.rout2 ? 0.f : wt.x;
@@ -138,7 +158,7 @@ __global__ void __launch_bounds__(kTile) k_born32(const Item* __restrict__ items
             far = splat<float2>(0.f);
         }
     };
-    float4 pa[kBatch], pb[kBatch]; // x, y, z, s
+    Place pa[kBatch], pb[kBatch];
     load(pa, 0);
     for (int j0 = 0; j0 < N; j0 += 2 * kTile) {
         load(pb, j0 + kTile);
@@ -165,28 +185,28 @@ __global__ void __launch_bounds__(kTile) k_gb32(const Item* __restrict__ items, 
     const int w = it.w, s = V.w_sys[w], N = V.sys_n[s], A = V.w_off[w], P = V.sys_poff[s];
     const int tid = threadIdx.x, lane = tid & 31;
     const int i = it.i0 + (tid >> 5);
-    float4 xi = make_float4(-kFarF, -kFarF, -kFarF, 0.f), gi = make_float4(0.f, 1.f, 1.f, 0.f);
+    Place me = far_place();
+    float4 gi = make_float4(0.f, 1.f, 1.f, 0.f);
     float2 li = make_float2(0.f, 0.f);
     if (i < N) {
-        xi = V.xs[A + i];
+        me = place(V, A + i);
         gi = V.gq[A + i];
         li = V.plj32[P + i];
     }
     const float tau = V.tau32, iei = V.iei32, kap = V.kappa32, ieo = V.ieo32;
     long long fx = 0, fy = 0, fz = 0, adr = 0, egb = 0, ec = 0, elj = 0;
     const float2 one = splat<float2>(1.f), zero = splat<float2>(0.f);
-    const float2 x2 = splat<float2>(xi.x), y2 = splat<float2>(xi.y), z2 = splat<float2>(xi.z);
     float2 px = zero, py = zero, pz = zero, pdr = zero;
     KSum<float2> pgb, pc, plj;
     struct Partner {
-        float4 x, g; // (position, -), (sqrt(k) q, R, 1/R, log2(e) / (4 R))
-        float2 l;    // sigma / 2, sqrt(eps)
+        Place x;
+        float4 g; // sqrt(k) q, R, 1/R, log2(e) / (4 R)
+        float2 l; // sigma / 2, sqrt(eps)
     };
     // two partners; bits 0, 1 of self: no pair, of ex: GB only
     auto pair = [&](const Partner& a, const Partner& b, uint32_t self, uint32_t ex) {
-        const float2 dx = sub2(x2, make_float2(a.x.x, b.x.x));
-        const float2 dy = sub2(y2, make_float2(a.x.y, b.x.y));
-        const float2 dz = sub2(z2, make_float2(a.x.z, b.x.z));
+        float2 dx, dy, dz;
+        separation(me, a.x, b.x, dx, dy, dz);
         float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
         float2 qq = __fmul2_rn(splat<float2>(gi.x), make_float2(a.g.x, b.g.x));
         float2 ep = __fmul2_rn(splat<float2>(li.y), make_float2(a.l.y, b.l.y));
@@ -235,18 +255,18 @@ __global__ void __launch_bounds__(kTile) k_gb32(const Item* __restrict__ items, 
         }
     };
     int mp = V.mt_off[it.st];
-    const int me = V.mt_off[it.st + 1];
-    int next = mp < me ? V.mt_list[mp] : 0x7fffffff;
+    const int mend = V.mt_off[it.st + 1];
+    int next = mp < mend ? V.mt_list[mp] : 0x7fffffff;
     for (int j0 = 0, jt = 0; j0 < N; j0 += kTile, ++jt) {
         Partner p[kBatch];
 #pragma unroll
         for (int u = 0; u < kBatch; ++u) {
             const int j = j0 + 32 * u + lane;
-            p[u].x = make_float4(kFarF, kFarF, kFarF, 0.f);
+            p[u].x = no_place();
             p[u].g = make_float4(0.f, 1.f, 1.f, 0.f);
             p[u].l = make_float2(0.f, 0.f);
             if (j < N) {
-                p[u].x = V.xs[A + j];
+                p[u].x = place(V, A + j);
                 p[u].g = V.gq[A + j];
                 p[u].l = V.plj32[P + j];
             }
@@ -256,7 +276,7 @@ __global__ void __launch_bounds__(kTile) k_gb32(const Item* __restrict__ items, 
             for (int u = 0; u < kBatch; u += 2) pair(p[u], p[u + 1], 0u, 0u);
         } else {
             ++mp;
-            next = mp < me ? V.mt_list[mp] : 0x7fffffff;
+            next = mp < mend ? V.mt_list[mp] : 0x7fffffff;
             uint32_t m[kBatch] = {}; // bit l of m[u]: partner j0 + 32 u + l is excluded
             if (i < N) {
                 const int e1 = V.excl_off[P + i + 1];
@@ -320,16 +340,14 @@ __global__ void __launch_bounds__(kChainThreads) k_chain32(const Item* __restric
         bonded.take<ENERGY>(V, A, P, it.i0, N, lane);
     } else {
         const int i = it.i0 + warp;
-        float4 xi = make_float4(-kFarF, -kFarF, -kFarF, 0.f);
-        float ci = 0.f, si = 0.f, rti = 1.f;
+        Place me = far_place();
+        float ci = 0.f;
         if (i < N) {
-            xi = V.xs[A + i];
+            me = place(V, A + i);
             ci = V.c32[A + i];
-            si = V.pb32[P + i].x;
-            rti = V.pb32[P + i].y;
         }
+        const float si = me.h.w, rti = me.l.w;
         const PairBand band = pair_band(V.rfar2, V.smax32, (float)V.rgbmax);
-        const float2 x2 = splat<float2>(xi.x), y2 = splat<float2>(xi.y), z2 = splat<float2>(xi.z);
         const float2 c2 = splat<float2>(ci), s2i = splat<float2>(si * si), s3i = splat<float2>(si * si * si);
         float2 fx2 = splat<float2>(0.f), fy2 = fx2, fz2 = fx2;
         float px = 0.f, py = 0.f, pz = 0.f;
@@ -350,26 +368,26 @@ __global__ void __launch_bounds__(kChainThreads) k_chain32(const Item* __restric
             fx2 = fy2 = fz2 = splat<float2>(0.f);
         };
         for (int j0 = 0; j0 < N; j0 += kTile) {
+            Place x[kBatch];
+            float c[kBatch];
             ChainNear e[kBatch];
             bool near[kBatch];
 #pragma unroll
             for (int u = 0; u < kBatch; ++u) {
                 const int j = j0 + 32 * u + lane;
-                e[u].p = make_float4(kFarF, kFarF, kFarF, 0.f);
-                e[u].r = make_float2(0.f, 1.f);
+                x[u] = no_place();
+                c[u] = 0.f;
                 if (j < N) {
-                    e[u].p = V.xs[A + j];
-                    e[u].p.w = V.c32[A + j];
-                    e[u].r = *reinterpret_cast<const float2*>(&V.pb32[P + j]);
+                    x[u] = place(V, A + j);
+                    c[u] = V.c32[A + j];
                 }
             }
 #pragma unroll
             for (int u = 0; u < kBatch; u += 2) {
-                ChainNear &a = e[u], &b = e[u + 1];
-                const float2 dx = sub2(x2, make_float2(a.p.x, b.p.x));
-                const float2 dy = sub2(y2, make_float2(a.p.y, b.p.y));
-                const float2 dz = sub2(z2, make_float2(a.p.z, b.p.z));
-                const float2 cj = make_float2(a.p.w, b.p.w), sj = make_float2(a.r.x, b.r.x), s2j = __fmul2_rn(sj, sj);
+                const Place &a = x[u], &b = x[u + 1];
+                float2 dx, dy, dz;
+                separation(me, a, b, dx, dy, dz);
+                const float2 cj = make_float2(c[u], c[u + 1]), sj = make_float2(a.h.w, b.h.w), s2j = __fmul2_rn(sj, sj);
                 float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
                 near[u] = band_near<CUT>(r2.x, band);
                 near[u + 1] = band_near<CUT>(r2.y, band);
@@ -388,8 +406,8 @@ __global__ void __launch_bounds__(kChainThreads) k_chain32(const Item* __restric
                 fx2 = __ffma2_rn(v, dx, fx2);
                 fy2 = __ffma2_rn(v, dy, fy2);
                 fz2 = __ffma2_rn(v, dz, fz2);
-                a.p = make_float4(dx.x, dy.x, dz.x, cj.x);
-                b.p = make_float4(dx.y, dy.y, dz.y, cj.y);
+                e[u] = {make_float4(dx.x, dy.x, dz.x, cj.x), make_float2(a.h.w, a.l.w)};
+                e[u + 1] = {make_float4(dx.y, dy.y, dz.y, cj.y), make_float2(b.h.w, b.l.w)};
             }
 #pragma unroll
             for (int u = 0; u < kBatch; ++u) near_q.push(near[u], e[u], lane);

@@ -86,17 +86,25 @@ __device__ __forceinline__ void sym_masks(const View& V, int P, int i, bool vi, 
 // ============================================== operand staging (FP32)
 // The pair kernels read FP32 operands only.  Positions are taken relative to
 // the walker's first atom (|x| stays within the molecule's extent, so FP32
-// keeps ~4e-6 A at 40 A) and rounded once per step; the charge and Born-radius
+// keeps ~4e-6 A at 40 A) and rounded once per step; the ordered passes read what
+// the rounding left as well; the charge and Born-radius
 // terms are rounded where the Born radii are finished, and once more after a
 // sweep that changed charges.
 __global__ void k_stage_x(View V, int a0, int n) {
     pdl_sync();
     const int l = blockIdx.x * blockDim.x + threadIdx.x;
     if (l >= n) return;
-    const int a = a0 + l, o = V.w_off[V.a_walker[a]];
-    if (!V.w_local[V.a_walker[a]]) return;
-    V.xs[a] = make_float4((float)(V.x[3 * a] - V.x[3 * o]), (float)(V.x[3 * a + 1] - V.x[3 * o + 1]),
-                          (float)(V.x[3 * a + 2] - V.x[3 * o + 2]), 0.f);
+    const int a = a0 + l, w = V.a_walker[a], o = V.w_off[w], s = V.w_sys[w];
+    if (!V.w_local[w]) return;
+    double d[3];
+    float h[3];
+    float *xs = reinterpret_cast<float*>(V.xs + a), *xl = reinterpret_cast<float*>(V.xl + a);
+    for (int c = 0; c < 3; ++c) { // (the fourth words stay as set up)
+        d[c] = V.x[3 * a + c] - V.x[3 * o + c];
+        xs[c] = h[c] = (float)d[c];
+    }
+    if (!V.sys_ordered[s]) return;
+    for (int c = 0; c < 3; ++c) xl[c] = (float)(d[c] - (double)h[c]);
 }
 
 __global__ void k_stage_gb(View V, int a0, int n) {

@@ -519,11 +519,17 @@ def config_leg(name, cfg, precision, n_steps, dev, stream, sm_mhz, oracle_plan=N
         step_peak = N_SM * (sm_mhz or 2070.0) * 1e6 / sum(pass_clk(n, far) for n in ("born", "gb", "chain"))
         pass_ms = eng2.time_passes(reps=3)
         out["pass_ms"] = [float(v) for v in pass_ms]
-        out["roofline"] = {"bound": "alu", "unit": "Gpair/s",
-                           "achieved": pairs_step / (sum(pass_ms) / 1e3) / 1e9,
-                           "peak": step_peak / 1e9,
-                           "frac": (pairs_step / (sum(pass_ms) / 1e3)) / step_peak,
-                           "basis": "three pair passes against the step roofline (FP32 lanes, MUFU)"}
+        if pass_ms[2] == 0:  # whole steps in one launch
+            out["pass_ms_of"] = "small-walker kernel: Born radii, pair pass, chain rule and bonded terms in one launch"
+            out["roofline"] = {"bound": "latency",
+                               "note": "small walkers: the phases of a step follow one another in one cluster "
+                                       "launch on part of the chip"}
+        else:
+            out["roofline"] = {"bound": "alu", "unit": "Gpair/s",
+                               "achieved": pairs_step / (sum(pass_ms) / 1e3) / 1e9,
+                               "peak": step_peak / 1e9,
+                               "frac": (pairs_step / (sum(pass_ms) / 1e3)) / step_peak,
+                               "basis": "three pair passes against the step roofline (FP32 lanes, MUFU)"}
     else:
         out["roofline"] = {"bound": "latency",
                            "note": "FP64 mode, one small system: a step is four dependent launches "

@@ -335,7 +335,10 @@ int cph_exchange_apply(cph_engine* e, int dim, const cph_exchange_row* rows, int
 /* Diagnostic timing of the three pair passes at the current state, with CUDA
  * events recorded on `stream` around each launch (batched or per-replica, per
  * the launch mode): ms[0] Born radii, ms[1] GB + Coulomb + LJ, ms[2] chain
- * rule + bonded terms, each the mean over `reps` launches.  The passes only
+ * rule + bonded terms, each the mean over `reps` launches.  An engine whose
+ * steps run in the small-walker kernel (a few walkers of at most 512 atoms, all
+ * CPH_SHAPE_WARP_PER_ATOM) times that kernel: ms[0] all three in one launch,
+ * ms[1] = ms[2] = 0.  The passes only
  * rewrite derived per-atom quantities (radii, forces); positions, velocities,
  * charges and site states are unchanged.  Synchronises `stream`. */
 int cph_time_passes(cph_engine* e, int reps, double* ms /* host [3] */, void* stream);
@@ -355,7 +358,10 @@ int cph_probe_pipe_rates(double* fp32_ops_per_s, double* mufu_ops_per_s, void* s
  * later steps are bitwise the same whatever size is chosen, fixed-point
  * sums); then the per-system tile shape: systems of at most n atoms run
  * CPH_SHAPE_WARP_PER_ATOM, the others CPH_SHAPE_SYMMETRIC, for n over the
- * distinct system sizes and 0 (every system symmetric).  *chosen (may be
+ * distinct system sizes and 0 (every system symmetric).  Where the steps of
+ * CPH_SHAPE_WARP_PER_ATOM would run in the small-walker kernel, that shape is
+ * taken untimed: the kernel runs only numbers and sizes of walkers for which
+ * every other form is slower.  *chosen (may be
  * NULL) receives the work-item size; cph_get_tile_shapes reports the shapes.
  * A change of shape changes later results in the last bits (see
  * cph_set_tile_shape).  Derived per-atom quantities are rewritten as by

@@ -630,7 +630,7 @@ struct cph_engine {
     // from the master arrays, undivided work items, near pairs in line.
     bool staged = true;
     // whole steps of small walkers in one launch (cph_small.cuh)
-    bool small_fits = false;       // every system can run that way
+    bool small_fits = false;       // every system can run that way, and it pays (small_pays)
     bool small = false;            // and every system's tile shape is CPH_SHAPE_WARP_PER_ATOM
     SmallTab small_tab{};
     int small_ga = 0, small_warps = 0, small_smem = 0; // atoms per warp, pair warps per CTA, bytes
@@ -1176,8 +1176,8 @@ namespace {
 
 // Tables and launch shape of the small-walker kernel, if every system fits it:
 // FP32 mode, at most kSmallAtoms atoms and kSmallTerms bonded terms in a CTA, a
-// SHAKE tolerance of at least kSmallShakeTol, and a device that can hold the
-// cluster.
+// SHAKE tolerance of at least kSmallShakeTol, a device that can hold the cluster,
+// and a number of walkers for which it pays.
 int small_setup(cph_engine* E, const std::vector<int>& bond_off, const std::vector<int>& bond_idx,
                 const std::vector<int>& bond_ij, const std::vector<int>& ang_off, const std::vector<int>& ang_idx,
                 const std::vector<int>& ang_ijk, const std::vector<int>& sys_poff, const std::vector<int>& shk_sys_off,
@@ -1241,16 +1241,19 @@ int small_setup(cph_engine* E, const std::vector<int>& bond_off, const std::vect
         cfg.attrs = at;
         cfg.numAttrs = 1;
         bool ok = true;
+        int resident = 1 << 30;
         for (bool energy : {false, true})
             by_small(E, energy, [&](auto kernel) {
                 int n = 0;
                 ok = ok && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) == cudaSuccess;
                 ok = ok && cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n > 0;
+                resident = std::min(resident, n);
             });
         if (!ok) {
             (void)cudaGetLastError();
             return CPH_OK;
         }
+        if (!small_pays(nmax, E->V.total_atoms, E->V.W, resident, E->V.xprev != nullptr)) return CPH_OK;
         int* d;
         SmallTab& T = E->small_tab;
         TRY(upload(E, term_off, &d)); T.term_off = d;
@@ -2006,12 +2009,13 @@ int cph_time_passes(cph_engine* e, int reps, double* ms, void* stream) {
     for (int r = 0; r < reps && rc == CPH_OK; ++r) {
         for (int p = 0; p < 3 && rc == CPH_OK; ++p) {
             cudaEventRecord(ev[p], st);
-            rc = launch_pass(e, p, false, st);
+            if (!e->small) rc = launch_pass(e, p, false, st);
+            else if (p == 0) rc = launch_small(e, false, 0, 1, kSmallBorn, kSmallForces, false, st);
         }
         cudaEventRecord(ev[3], st);
         cudaError_t ce = cudaEventSynchronize(ev[3]);
         if (ce != cudaSuccess && rc == CPH_OK) rc = fail(e, CPH_E_CUDA, "timing: %s", cudaGetErrorString(ce));
-        for (int k = 0; k < 3 && rc == CPH_OK; ++k) {
+        for (int k = 0; k < (e->small ? 1 : 3) && rc == CPH_OK; ++k) {
             float t = 0.f;
             cudaEventElapsedTime(&t, ev[k], ev[k + 1]);
             acc[k] += t;
@@ -2061,6 +2065,10 @@ int cph_autotune(cph_engine* e, void* stream, int* chosen) {
         for (int s = 0; s < e->n_sys; ++s)
             e->h_sys_shape[s] = e->h_sys_n[s] <= n ? CPH_SHAPE_WARP_PER_ATOM : CPH_SHAPE_SYMMETRIC;
         TRY(build_items(e, best_c));
+        if (e->small) { // where small_pays sends steps there, no other form comes near
+            best_n = n;
+            break;
+        }
         double t;
         TRY(timed(&t));
         if (t < best) {

@@ -9,8 +9,8 @@
 // steps until the schedule needs something of another kernel (a titration
 // sweep, an exchange attempt).  Measured, with sweeps every 10 steps: 8 x 160
 // atoms 58.5 -> 20 us a step (15 in this kernel), 4 x 246 atoms with constraints
-// 91 -> 39 us.  Which walkers come here: small_setup in
-// cph_engine.cu.
+// 91 -> 39 us.  Which walkers come here: small_setup in cph_engine.cu and
+// small_pays below.
 //
 // Work split.  A cluster of eight CTAs (portable; of sixteen-CTA clusters only
 // seven fit the chip) holds the walker.  A warp owns GA consecutive atoms i, its
@@ -33,6 +33,8 @@
 #pragma once
 #include <cooperative_groups.h>
 
+#include <algorithm>
+
 #include "cph_device.cuh"
 #include "cph_internal.h"
 #include "cph_kernels.cuh"
@@ -49,6 +51,36 @@ constexpr int kSmallRanks = 8;    // CTAs per cluster
 // never, or elsewhere.  Tighter ones take the separate launches (k_shake, FP64).
 constexpr double kSmallShakeTol = 1e-12;
 constexpr int kSmallUnroll = 2;   // of the partner loops (1 to 4: within 3 %)
+
+// Whether walkers of at most n atoms (`atoms` in all) that fit the kernel also run
+// in it, by the whole grid's numbers, so that every engine of a sharded grid decides
+// alike.  A cluster holds eight SMs, so `resident` of them (15, of 40-atom walkers
+// 32 and more) run at once and the others wait for the next wave; the separate
+// launches take a walker's atoms four to a CTA over the whole chip, 2432 atoms at
+// a time.  us a step of 100 with sweeps every 10, this kernel / separate launches:
+//   atoms  1 walker   8 walkers  15         16         30         45         64
+//     80   15 / 22    16 / 23    16 / 23    28 / 24    29 / 25    42 / 34    67 / 47
+//    120   16 / 22    17 / 23    17 / 24    31 / 25    31 / 35    45 / 47    73 / 56
+//    160   19 / 24    19 / 25    19 / 27    36 / 35    36 / 43    53 / 55    86 / 76
+//    237   27 / 24    27 / 26    27 / 38    50 / 38    51 / 55    75 / 78    123 / 102
+//    360   50 / 25    51 / 39    51 / 56    97 / 57    99 / 85    146 / 114  240 / 154
+//    480   64 / 26    65 / 43    65 / 64    125 / 71   127 / 111  188 / 156  310 / 211
+// The tiles of cph_sym.cuh never come near where this form pays (68 to 420).  With
+// constraints, whose separate launches are slower (operands from the master arrays,
+// SHAKE in a launch of its own):
+//    121   27 / 57    28 / 63    28 / 68    52 / 68    53 / 79    77 / 97    126 / 115
+//    205   36 / 63    36 / 71    37 / 83    70 / 83    70 / 114   104 / 142  170 / 175
+//    246   37 / 64    37 / 74    37 / 89    70 / 89    71 / 132   106 / 160  173 / 201
+//    351   59 / 68    59 / 84    60 / 119   114 / 127  116 / 177  172 / 235  284 / 310
+//    452   75 / 70    76 / 100   76 / 154   147 / 157  149 / 244  221 / 334  364 / 450
+inline bool small_pays(int n, long long atoms, int walkers, int resident, bool constrained) {
+    const int waves = (walkers + resident - 1) / resident;
+    if (constrained) return waves <= (n > 200 && n <= 384 ? 5 : 3); // (at 452 x 64 the tiles: 316)
+    const long long other = (atoms + 2431) / 2432; // waves of the separate launches
+    if (n <= 160) return waves <= std::min(other, 3ll);
+    if (n <= 256) return waves <= (other >= 5 ? 3 : std::min(other - 1, 2ll));
+    return n <= 384 && waves == 1 && other >= 3;
+}
 
 // phases of a step: where a launch starts its first step and ends its last
 enum SmallPhase { kSmallBorn = 0, kSmallForces = 1, kSmallMove = 2 };
@@ -131,7 +163,11 @@ __device__ __forceinline__ SmallSmem small_carve(unsigned char* p, int n, int ow
     return s;
 }
 
-// GA: atoms per warp (1, 2 or 4 for up to 160, 256 or 512 atoms).
+// GA: atoms per warp, 1, 2 or 4 for up to 160, 256 or 512 atoms.  The pair warps of a
+// CTA then number at most 20, 16 and 16, and the launch bounds leave 80 to 96
+// registers.  With one atom a warp up to 224 atoms (28 warps, 64 registers) 176
+// atoms took 20.7 us a step for 21.9, 200 atoms 23.4 for 24.3, but 205 with
+// constraints 37.2 for 35.8.
 template <int GA, bool ENERGY>
 __global__ void __launch_bounds__(GA == 1 ? 704 : 576, 1) k_small(View V, SmallTab T, SmallRun run) {
     pdl_sync();

@@ -1096,6 +1096,13 @@ int enqueue_step(cph_engine* E, long long t, int s_off, bool full_schedule, cuda
     return CPH_OK;
 }
 
+// A small-walker launch makes at most this many steps (10 to 75 ms of them): a long
+// run stays divided into kernels, as it is in every other form.
+constexpr long long kSmallSteps = 1000;
+// Steps enqueued between two updates of the device's step counter: offsets from it
+// are ints.
+constexpr long long kTickSteps = 1 << 30;
+
 // n steps from global step t; s_off: the first one's offset from the device's
 // step counter.
 int enqueue_steps(cph_engine* E, long long t, long long n, int s_off, bool full_schedule, cudaStream_t st) {
@@ -1107,6 +1114,11 @@ int enqueue_steps(cph_engine* E, long long t, long long n, int s_off, bool full_
     // step `open` from phase `from` on.
     long long open = 0;
     int from = kSmallBorn;
+    auto run = [&](long long m, int end, bool zero_energy) -> int { // m steps from `open`
+        for (; m > kSmallSteps; m -= kSmallSteps, open += kSmallSteps, from = kSmallBorn)
+            TRY(launch_small(E, false, s_off + (int)open, (int)kSmallSteps, from, kSmallMove, false, st));
+        return launch_small(E, false, s_off + (int)open, (int)m, from, end, zero_energy, st);
+    };
     for (long long k = 0; full_schedule && k < n; ++k) {
         const long long tk = t + k;
         int kinds = 0;
@@ -1114,21 +1126,23 @@ int enqueue_steps(cph_engine* E, long long t, long long n, int s_off, bool full_
         if (tk > 0 && E->mc_redox > 0 && tk % E->mc_redox == 0) kinds |= CPH_MC_REDOX;
         const bool exch = tk > 0 && E->ex_every > 0 && tk % E->ex_every == 0;
         if (kinds && E->max_sites > 0) {
-            TRY(launch_small(E, false, s_off + (int)open, (int)(k - open + 1), from, kSmallBorn, exch, st));
+            TRY(run(k - open + 1, kSmallBorn, exch));
             TRY(launch_mc(E, kinds, s_off + (int)k, st));
             open = k;
             from = kSmallForces;
         }
         if (exch) {
-            if (open < k) TRY(launch_small(E, false, s_off + (int)open, (int)(k - open), from, kSmallMove, false, st));
-            if (open < k) from = kSmallBorn;
+            if (open < k) {
+                TRY(run(k - open, kSmallMove, false));
+                from = kSmallBorn;
+            }
             TRY(launch_small(E, true, s_off + (int)k, 1, from, kSmallForces, from == kSmallBorn, st));
             TRY(launch_exchange(E, CPH_DIM_NEXT, s_off + (int)k, st));
             open = k;
             from = kSmallMove;
         }
     }
-    if (open < n) TRY(launch_small(E, false, s_off + (int)open, (int)(n - open), from, kSmallMove, false, st));
+    if (open < n) TRY(run(n - open, kSmallMove, false));
     return CPH_OK;
 }
 
@@ -2166,9 +2180,13 @@ int cph_get_tile_shapes(const cph_engine* e, int* shapes) {
 int cph_step_replicas(cph_engine* e, int64_t n_steps, void* stream) {
     if (!e || n_steps < 0) return fail(e, CPH_E_INVALID, "bad arguments");
     cudaStream_t st = (cudaStream_t)stream;
-    TRY(enqueue_steps(e, e->h_step, n_steps, 0, false, st));
-    if (n_steps) TRY(launch_tick(e, n_steps, st));
-    e->h_step += n_steps;
+    for (int64_t done = 0; done < n_steps;) {
+        const int64_t k = std::min<int64_t>(n_steps - done, kTickSteps);
+        TRY(enqueue_steps(e, e->h_step, k, 0, false, st));
+        TRY(launch_tick(e, k, st));
+        e->h_step += k;
+        done += k;
+    }
     return CPH_OK;
 }
 
@@ -2228,8 +2246,13 @@ int cph_run(cph_engine* e, int64_t n_steps, void* stream) {
         } else {
             // directly launched steps: up to where a whole period can be replayed
             int64_t k = 1;
-            if (e->small)
-                while (done + k < n_steps && !(P > 1 && (t + k) % P == 1 && n_steps - done - k >= P)) ++k;
+            if (e->small && P <= 1) k = std::min<int64_t>(n_steps - done, kTickSteps);
+            else if (e->small)
+                while (done + k < n_steps && !((t + k) % P == 1 && n_steps - done - k >= P)) ++k;
+            if (direct + k > kTickSteps) {
+                TRY(launch_tick(e, direct, st));
+                direct = 0;
+            }
             TRY(enqueue_steps(e, t, k, (int)direct, true, st));
             direct += k;
             e->h_step += k;

@@ -82,3 +82,47 @@ def test_constrained_walkers_of_all_sizes(n):
         e.status()
     v, w = a.velocities(), b.velocities()
     assert np.sqrt(((v - w) ** 2).mean()) <= 1e-5 * np.sqrt((w ** 2).mean())
+
+
+def _captured_kernels(call):
+    """Nodes that call(stream) puts on a capturing stream."""
+    import ctypes as C
+
+    import torch
+    cu = C.CDLL("libcuda.so.1")
+    st = torch.cuda.Stream()
+    h, graph, n = C.c_void_p(st.cuda_stream), C.c_void_p(), C.c_size_t()
+    assert cu.cuStreamBeginCapture_v2(h, 1) == 0  # thread-local
+    try:
+        call(st.cuda_stream)
+    finally:
+        assert cu.cuStreamEndCapture(h, C.byref(graph)) == 0
+    assert cu.cuGraphGetNodes(graph, None, C.byref(n)) == 0
+    cu.cuGraphDestroy(graph)
+    return n.value
+
+
+def test_long_runs_stay_divided_into_launches():
+    """At most 1000 steps to a launch, and the same bits however a run is cut."""
+    s = synth.make_system(60, 1, n_ph=2)
+    kw = dict(mc_ph_every=0, mc_redox_every=0, exchange_every=0)
+
+    def engine():
+        e = cphremd.init_system([s], _grid(2), seed=3, **kw)
+        e.set_tile_shape(0, cphremd.SHAPE_WARP_PER_ATOM)
+        return e
+
+    a, b, c = engine(), engine(), engine()
+    assert _captured_kernels(lambda st: a.step_replicas(2500, stream=st)) == 4  # 1000, 1000, 500, and the counter's
+    assert _captured_kernels(lambda st: a.run(2001, stream=st)) == 4
+    a = engine()
+    a.step_replicas(2500)
+    for n in (700, 1000, 800):
+        b.step_replicas(n)
+    c.run(2500)
+    for e in (a, b, c):
+        e.status()
+        assert e.get_step() == 2500
+    for get in ("positions", "velocities", "forces", "born_radii", "visits"):
+        np.testing.assert_array_equal(getattr(a, get)(), getattr(b, get)())
+        np.testing.assert_array_equal(getattr(a, get)(), getattr(c, get)())

@@ -154,12 +154,24 @@ void by_group(const SView& g, F&& f) {
 }
 
 // Whether a call goes to the one-launch cluster kernel: replicas it can hold, and
-// not so many that its twofold pair arithmetic outweighs the launches and the
-// near-empty tiles it saves.  Energy / backward in us, cluster kernel against
-// symmetric kernels: 1 x 237 12 / 25 against 60 / 118, 128 x 237 48 / 116 against
-// 74 / 149, 128 x 400 88 / 223 against 133 / 305, 128 x 512 110 / 286 against
-// 121 / 267, 512 x 237 168 / 409 against 158 / 362.
-bool gsmall(int n_rep, int n) { return n <= kGsAtoms && (long long)n_rep * n * n <= 24000000; }
+// not so many that the clusters' waves (a few tens of replicas at once, however small)
+// or the twofold pair arithmetic outweigh the launches it saves.  Energy / backward in
+// us, cluster kernel against symmetric kernels, which take longer for an odd number
+// of j-tiles (missing atoms meet the missing half of the last tile pair as near pairs):
+//   even     40 x 192  35 / 65 against 37 / 77    40 x 256  46 / 85 against 37 / 77
+//            64 x 224  42 / 81 against 44 / 97   104 x 192  43 / 83 against 46 / 101
+//           128 x 192  42 / 87 against 43 / 97   128 x 256  55 / 115 against 44 / 97
+//           192 x 160  49 / 112 against 50 / 113 192 x 192  56 / 127 against 50 / 113
+//           237 x 128  49 / 116 against 53 / 120 256 x 192  66 / 161 against 63 / 174
+//           320 x 128  63 / 156 against 68 / 170  512 x 64  62 / 155 against 63 / 154
+//   odd       8 x 448  70 / 129 against 68 / 167   32 x 448  72 / 139 against 60 / 146
+//            72 x 448  81 / 166 against 80 / 236   20 x 640  100 / 196 against 70 / 237
+//           150 x 448  114 / 254 against 107 / 290 220 x 448  133 / 318 against 136 / 367
+// and of many tiny replicas 1228 / 2461 against 513 / 1754 for 20 x 8192.
+bool gsmall(int n_rep, int n) {
+    const bool odd = ((n + kGJ - 1) / kGJ) & 1;
+    return n <= kGsAtoms && n_rep <= (odd ? 448 : (n <= 128 ? 216 : 168)) && (long long)n_rep * n * n <= 24000000;
+}
 
 // bound and Born radii, shared by both directions
 int launch_radii(SView& g, cudaStream_t st) {

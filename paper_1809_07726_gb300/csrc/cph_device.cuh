@@ -164,6 +164,21 @@ __device__ __forceinline__ double rcp64(double x) {
     return fma(y, fma(e, e, e), y);
 }
 
+// The same with 1/0 = infinity and 1/infinity = 0: a Born radius (1/R = 1/rt - tanh/rho
+// is 0 where the tanh has saturated and the offset is 0) and its reciprocal.
+__device__ __forceinline__ double rcp64_radius(double x) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const int h = __double2hiint(y) & 0x7fffffff;
+    const double e = fma(-x, y, 1.0);
+    return h == 0 || h == 0x7ff00000 ? y : fma(y, fma(e, e, e), y);
+}
+
+// Born radii as the pair arithmetic takes them: finite, and so are their products;
+// past these bounds 1/f is 0 to every digit that counts.
+__device__ __forceinline__ float pair_radius32(double R) { return fminf((float)R, 1e18f); }
+__device__ __forceinline__ double pair_radius64(double R) { return fmin(R, 1e150); }
+
 // 1 / sqrt(x) for normal x > 0: the same with y (1 + e/2 + 3 e^2/8), e = 1 - x y^2
 __device__ __forceinline__ double rsqrt64(double x) {
     double y;

@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(kMcThreads) k_mc_site(View V, int kind, int s_
             p = {x.x, x.y, x.z, q.x};
             r = {q.y, q.z, 0.f, 0.f};
         } else {
-            const double R = V.R[A + j];
+            const double R = pair_radius64(V.R[A + j]);
             p = {V.x[3 * (A + j)], V.x[3 * (A + j) + 1], V.x[3 * (A + j) + 2], V.q[A + j] * V.sqrt_k};
             r = {R, rcp64(R), 0.0, 0.0};
         }
@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(kMcThreads) k_mc_sweep(View V, int kind, int c
             p = {x.x, x.y, x.z, dq};
             r = {c.y, c.z};
         } else {
-            const double R = V.R[A + at];
+            const double R = pair_radius64(V.R[A + at]);
             p = {V.x[3 * (A + at)], V.x[3 * (A + at) + 1], V.x[3 * (A + at) + 2], dq};
             r = {R, rcp64(R)};
         }

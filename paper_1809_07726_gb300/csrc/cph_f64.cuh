@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(kTile) k_born64(const Item* __restrict__ items
         const double th0 = psi * (V.alpha + psi * (-V.beta + psi * V.gamma));
         const double e = exp64(-2.0 * fabs(th0), tab); // tanh = (1 - e) / (1 + e)
         const double th = copysign(fma(-2.0 * e, rcp64(1.0 + e), 1.0), th0);
-        const double R = rcp64(irti - th * irho);
+        const double R = rcp64_radius(irti - th * irho);
         V.psi[A + i] = psi;
         V.R[A + i] = R;
         V.dRdpsi[A + i] = R * R * (1.0 - th * th) * (V.alpha + psi * (-2.0 * V.beta + 3.0 * V.gamma * psi)) * irho;
@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(kTile) k_gb64(const Item* __restrict__ items, 
     load_tab64(tab, tid, kTile);
     const int ic = vi ? i : it.i0;
     const double xi = V.x[3 * (A + ic)], yi = V.x[3 * (A + ic) + 1], zi = V.x[3 * (A + ic) + 2];
-    const double Ri = V.R[A + ic], iRi = rcp64(Ri), mq = -0.25 * iRi;
+    const double Ri = pair_radius64(V.R[A + ic]), iRi = rcp64(Ri), mq = -0.25 * iRi;
     const double qi = V.q[A + ic] * V.sqrt_k, sgi = V.sigh[P + ic], sei = V.sqe[P + ic];
     const double tau = V.tau, iei = V.inv_eps_in, kap = V.kappa, ieo = V.inv_eps_out;
     double fx = 0, fy = 0, fz = 0, adr = 0, egb = 0, ec = 0, elj = 0;
@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(kTile) k_gb64(const Item* __restrict__ items, 
             __syncthreads();
             if (j0 + tid < N) {
                 const int j = j0 + tid;
-                const double R = V.R[A + j];
+                const double R = pair_radius64(V.R[A + j]);
                 sa[tid] = {V.x[3 * (A + j)], V.x[3 * (A + j) + 1], V.x[3 * (A + j) + 2], V.q[A + j] * V.sqrt_k};
                 sb[tid] = {R, rcp64(R), V.sigh[P + j], V.sqe[P + j]};
             }

@@ -73,12 +73,12 @@ __global__ void __launch_bounds__(kGsThreads) __cluster_dims__(kGsRanks, 1, 1) k
         const double rho = g.rho[base + a0 + a], rt = rho - g.offset, irho = rcp64(rho);
         const double psi = rt * ((double)sum[a][0] * (0.5 / kScaleH));
         const double th = tanh64(psi * (g.alpha + psi * (-g.beta + psi * g.gamma)));
-        const double iR = rcp64(rt) - th * irho, R = rcp64(iR);
+        const double iR = rcp64(rt) - th * irho, R = rcp64_radius(iR);
         aR[a] = R;
         aiR[a] = iR;
         apsi[a] = psi;
         adR[a] = R * R * (1.0 - th * th) * (g.alpha + psi * (-2.0 * g.beta + 3.0 * g.gamma * psi)) * irho;
-        const float2 o = make_float2((float)R, (float)iR);
+        const float2 o = make_float2(pair_radius32(R), (float)iR);
 #pragma unroll
         for (int r = 0; r < kGsRanks; ++r) cl.map_shared_rank(rad, r)[a0 + a] = o;
     }

@@ -268,7 +268,7 @@ __global__ void k_gfin_born(SView g) {
     const double rho = g.rho[a], rt = rho - g.offset, irho = rcp64(rho);
     const double psi = 0.5 * rt * ((double)g.Hfix[a] / kScaleH);
     const double th = tanh64(psi * (g.alpha + psi * (-g.beta + psi * g.gamma)));
-    const double R = rcp64(rcp64(rt) - th * irho);
+    const double R = rcp64_radius(rcp64(rt) - th * irho);
     g.psi[a] = psi;
     g.R[a] = R;
     g.gpsi[a] = R * R * (1.0 - th * th) * (g.alpha + psi * (-2.0 * g.beta + 3.0 * g.gamma * psi)) * irho; // dR/dpsi for now
@@ -424,7 +424,7 @@ __global__ void __launch_bounds__(kGT, BACKWARD ? 5 : 8) k_gpair_sym(SView g) {
         ii[u] = it.i0 + warp * 64 + u * 32 + lane;
         vi[u] = ii[u] < n;
         const int i = vi[u] ? ii[u] : it.i0;
-        const float R = vi[u] ? (float)g.R[base + i] : 1.f;
+        const float R = vi[u] ? pair_radius32(g.R[base + i]) : 1.f;
         I[u].x = splat<float2>(vi[u] ? X[3 * i] : -kFar);
         I[u].y = splat<float2>(vi[u] ? X[3 * i + 1] : -kFar);
         I[u].z = splat<float2>(vi[u] ? X[3 * i + 2] : -kFar);
@@ -446,7 +446,7 @@ __global__ void __launch_bounds__(kGT, BACKWARD ? 5 : 8) k_gpair_sym(SView g) {
             for (int h = 0; h < 2; ++h) {
                 const int gt = 2 * pr + h, j = (g0 + gt) * kGJ + e;
                 if (gt < ng && j < n) {
-                    const float R = (float)g.R[base + j];
+                    const float R = pair_radius32(g.R[base + j]);
                     v[h][0] = -X[3 * j]; v[h][1] = -X[3 * j + 1]; v[h][2] = -X[3 * j + 2];
                     v[h][3] = Q[j] * sqk; v[h][4] = R; v[h][5] = __frcp_rn(R);
                 } else { // padding: far away, no charge
@@ -564,7 +564,7 @@ __global__ void k_gfin_c(SView g) {
     const double q = (double)g.q[a] * g.sqrt_k, R = g.R[a];
     const double esa = sa_ace(g.sa_gamma, g.sa_probe, (double)g.rho[a], R);
     const double ts = salt_tau(R, g.inv_eps_in, g.inv_eps_out, g.kappa); // tau of the self term
-    const double iR = rcp64(R);
+    const double iR = rcp64_radius(R);
     const long long e = __double2ll_rn((-0.5 * ts * q * q * iR + esa) * kScaleE);
     // one atomic per warp when the warp's atoms share a replica (exact integer
     // sums, so the total is the same whichever way they are grouped)
@@ -882,7 +882,7 @@ __global__ void k_gfin_out(SView g) {
     const double up = g.dE[r];
     const double rho = g.rho[a], rt = rho - g.offset, R = g.R[a], psi = g.psi[a];
     const double irt = rcp64(rt), irho = rcp64(rho);
-    const double th = (irt - rcp64(R)) * rho; // from 1/R = 1/rt - th/rho
+    const double th = (irt - rcp64_radius(R)) * rho; // from 1/R = 1/rt - th/rho
     const double esa = sa_ace(g.sa_gamma, g.sa_probe, rho, R); // explicit rho dependence at fixed R
     const double dr = g.dEdR[a] * R * R * (irt * irt - th * irho * irho) + g.gpsi[a] * psi * irt +
                       g.c[a] * ((double)g.artfix[a] / kScaleE) +

@@ -78,7 +78,7 @@ struct alignas(sizeof(Real) * 2) J2 {
 
 // The (sqrt(k) q, R, 1/R, log2(e) / (4 R)) operand of the FP32 pair kernels.
 __device__ __forceinline__ float4 gb_operand(double q, double sqrt_k, double R) {
-    const float r = (float)R, ir = __frcp_rn(r);
+    const float r = pair_radius32(R), ir = __frcp_rn(r);
     return make_float4((float)(q * sqrt_k), r, ir, (0.25f * kLog2e) * ir);
 }
 
@@ -106,7 +106,7 @@ struct Masters {
     }
     __device__ __forceinline__ J4<float> gb(int i) const { // sqrt(k) q, R, 1/R
         const double R = V.R[A + i];
-        return {float(V.q[A + i]) * float(V.sqrt_k), float(R), float(1.0 / R), 0.f};
+        return {float(V.q[A + i]) * float(V.sqrt_k), pair_radius32(R), float(1.0 / R), 0.f};
     }
     __device__ __forceinline__ J2<float> lj(int i) const { // sigma / 2, sqrt(eps)
         return {float(V.sigh[P + i]), float(V.sqe[P + i])};
@@ -161,7 +161,7 @@ struct BornIn {
 __device__ __forceinline__ void born_epilogue(const View& V, int A, int P, int i, long long sum, const BornIn& in) {
     const double psi = 0.5 * in.rt * Prec<float>::value(sum, kScaleH);
     const double th = tanh64(psi * (V.alpha + psi * (-V.beta + psi * V.gamma)));
-    const double R = rcp64(in.irt - th * in.irho);
+    const double R = rcp64_radius(in.irt - th * in.irho);
     V.psi[A + i] = psi;
     V.R[A + i] = R;
     V.gq[A + i] = gb_operand(in.q, V.sqrt_k, R);
@@ -188,7 +188,7 @@ __device__ __forceinline__ void gb_epilogue(const View& V, int A, int P, int w, 
     long long e0 = 0, e1 = 0, e2 = 0;
     if (own) {
         const double q = in.q * V.sqrt_k;
-        const double R = in.R, iR = rcp64(R);
+        const double R = in.R, iR = rcp64_radius(R);
         const double qqR = q * q * iR;
         // tau(R) and its derivative form share one exponential
         double tau = V.inv_eps_in - V.inv_eps_out, taud = tau;

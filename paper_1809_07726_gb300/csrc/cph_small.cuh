@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(GA == 1 ? 704 : 576, 1) k_small(View V, SmallT
         at.q = V.q[A + i] * V.sqrt_k;
         at.psi = V.psi[A + i];
         at.R = V.R[A + i];
-        at.iR = run.start > kSmallBorn ? rcp64(at.R) : 1.0;
+        at.iR = run.start > kSmallBorn ? rcp64_radius(at.R) : 1.0;
         at.dRdpsi = V.dRdpsi[A + i];
         at.im = V.lg_im[P + i];
         at.sd = V.lg_sqT[V.slot_of[w] / (V.nE * V.npH)] * V.lg_sf[P + i];
@@ -329,13 +329,13 @@ __global__ void __launch_bounds__(GA == 1 ? 704 : 576, 1) k_small(View V, SmallT
                     SmallAtom& at = S.at[a];
                     const double psi = at.rt * ((double)S.sum[8 * a] * (0.5 / kScaleH));
                     const double th = tanh64(psi * (V.alpha + psi * (-V.beta + psi * V.gamma)));
-                    const double iR = at.irt - th * at.irho, R = rcp64(iR);
+                    const double iR = at.irt - th * at.irho, R = rcp64_radius(iR);
                     at.psi = psi;
                     at.R = R;
                     at.iR = iR;
                     at.dRdpsi = R * R * (1.0 - th * th) *
                                 (V.alpha + psi * (-2.0 * V.beta + 3.0 * V.gamma * psi)) * at.irho;
-                    const float Rf = (float)R, iRf = (float)iR;
+                    const float Rf = pair_radius32(R), iRf = (float)iR;
 #pragma unroll
                     for (int r = 0; r < CS; ++r) {
                         float4* o = cl.map_shared_rank(S.gq, r) + a0 + a;
@@ -643,7 +643,7 @@ __global__ void __launch_bounds__(GA == 1 ? 704 : 576, 1) k_small(View V, SmallT
         V.R[g] = at.R;
         V.dRdpsi[g] = at.dRdpsi;
         V.gq[g] = gb_operand(V.q[g], V.sqrt_k, at.R);
-        T.rad[g] = make_float2((float)at.R, (float)at.iR);
+        T.rad[g] = make_float2(pair_radius32(at.R), (float)at.iR);
     }
     for (int k = tid; k < 3 * nown; k += nthr) {
         const int g = 3 * (A + a0) + k, a = k / 3, d = k - 3 * a;

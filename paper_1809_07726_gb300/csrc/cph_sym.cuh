@@ -475,7 +475,7 @@ __global__ void k_fin_c(View V, int a0, int n) {
     const int w = V.a_walker[a];
     if (V.sys_ordered[V.w_sys[w]] || !V.w_local[w]) return; // ordered passes finish their atoms themselves
     const int P = V.sys_poff[V.w_sys[w]] + (a - V.w_off[w]);
-    const double q = V.q[a] * V.sqrt_k, R = V.R[a], iR = rcp64(R);
+    const double q = V.q[a] * V.sqrt_k, R = V.R[a], iR = rcp64_radius(R);
     const double esa = sa_ace(V.sa_gamma, V.sa_probe, V.rho[P], R);
     const double dEdR = 0.5 * (V.tau_pair * ((double)V.dRfix[a] / kScaleE)
                                + salt_taud(R, V.inv_eps_in, V.inv_eps_out, V.kappa) * q * q * iR * iR)
@@ -1145,7 +1145,7 @@ __global__ void k_fin_born(View V, int a0, int n, int zero_energy) {
     const double psi = 0.5 * rt * ((double)V.Hfix[a] / kScaleH);
     V.Hfix[a] = 0;
     const double th = tanh64(psi * (V.alpha + psi * (-V.beta + psi * V.gamma)));
-    const double R = rcp64(V.irt[P] - th * irho);
+    const double R = rcp64_radius(V.irt[P] - th * irho);
     V.psi[a] = psi;
     V.R[a] = R;
     V.gq[a] = gb_operand(V.q[a], V.sqrt_k, R);

@@ -203,16 +203,17 @@ def _stream(stream):
         return _raw_stream()
     try:
         import torch
-        if torch.cuda.is_available():
-            now = torch.cuda.current_stream().cuda_stream  # sets CUDA up
-            # the same two reads without the Python layers around them (a small
-            # call's host time is mostly these: 5 us of 18)
-            current, device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
-            _raw_stream = lambda: current(device())  # noqa: E731
-            return now
-    except (ImportError, AttributeError):  # pragma: no cover
-        pass
-    return None
+    except ImportError:  # pragma: no cover
+        return None
+    if not torch.cuda.is_available():
+        return None
+    now = torch.cuda.current_stream().cuda_stream  # sets CUDA up
+    # the same two reads without the Python layers around them (a small call's host
+    # time is mostly these: 5 us of 18), where torch has them
+    current, device = (getattr(torch._C, n, None) for n in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+    if current and device:
+        _raw_stream = lambda: current(device())  # noqa: E731
+    return now
 
 
 def _f64(a):

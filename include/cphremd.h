@@ -502,7 +502,10 @@ int cph_predict_sum_pka(int n_pts, const double* E, double e0_prot, double e0_de
  *   rho    device float [n_rep * n] intrinsic radii (> offset)
  *   screen device float [n] screening factors (shared by all replicas)
  *   E      device double [n_rep], written
- * FP32 pair arithmetic, int64 fixed-point accumulation.  Needs
+ * FP32 pair arithmetic, int64 fixed-point accumulation: repeated calls give
+ * the same bits, whatever the order of execution.  Which kernel runs and how
+ * it groups its FP32 partial sums depends on n and n_rep, so a replica in
+ * another batch can differ in the last bits (2e-6 at most).  Needs
  * cph_gb_workspace_bytes(n_rep, n) bytes of device workspace (caller-owned,
  * 256-byte aligned); the library allocates nothing. */
 size_t cph_gb_workspace_bytes(int n_rep, int n);

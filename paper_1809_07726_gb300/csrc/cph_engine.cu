@@ -626,8 +626,9 @@ struct cph_engine {
     // FP32 ordered passes read the operands staged once per step.  Not with
     // constraints: hydrogens at fixed lengths amplify a change of rounding (100
     // steps of the 246-atom peptide turned 1e-7 in the forces into 5e-5 in the
-    // velocities), so constrained runs keep every rounding they had: operands
-    // from the master arrays, undivided work items, near pairs in line.
+    // velocities), so their pair loops stay as they are: operands from the master
+    // arrays, undivided work items, near pairs in line.  (The per-atom arithmetic
+    // after the loops is every engine's.)
     bool staged = true;
     // whole steps of small walkers in one launch (cph_small.cuh)
     bool small_fits = false;       // every system can run that way, and it pays (small_pays)

@@ -24,7 +24,9 @@
 namespace cph {
 
 constexpr int kBatch = 4;            // partners of a lane at a time, in float2 pairs
-constexpr int kOrdFlush = 8 * kTile; // partners summed in FP32 before a conversion to fixed point
+// partners summed in FP32 before a conversion to fixed point (with 128: forces of 2003
+// atoms 4.70e-7 instead of 4.72e-7 from FP64's, radii the same, 20 steps 1.21 -> 1.30 ms)
+constexpr int kOrdFlush = 8 * kTile;
 
 // Near pairs.  A warp step that meets one would run
 // the closed forms for all its lanes, in the middle of the pair loop, and 20 to

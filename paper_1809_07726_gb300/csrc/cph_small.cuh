@@ -14,9 +14,9 @@
 //
 // Work split.  A cluster of eight CTAs (portable; of sixteen-CTA clusters only
 // seven fit the chip) holds the walker.  A warp owns GA consecutive atoms i, its
-// lanes the partners j = lane + 32 m, so that the positions relative to the first
-// atom of i's group of four are formed once a step and stay in registers for all
-// three passes.  Extra warps evaluate the bonded terms that touch the CTA's
+// lanes the partners j = lane + 32 m; the positions relative to the first atom of
+// each group of four are formed once a step, in shared memory, for all three
+// passes.  Extra warps evaluate the bonded terms that touch the CTA's
 // atoms, gather them and draw the random numbers meanwhile.  Each CTA holds the
 // whole walker's operands in shared memory (130 bytes an atom); what changes in
 // a phase (positions, radii, chain weights) its owner writes into every CTA of
@@ -28,8 +28,10 @@
 // difference rounds as the FP64 one does but for ties), fixed-point conversions go through
 // 32-bit ones, and per-atom FP64 arithmetic is gathered into full warps and
 // spends reciprocals and one short exponential in place of divisions and tanh.
-// Sums, orders and roundings of the pair passes are those of the ordered
-// kernels with operands from the master arrays (k_born, k_gb, k_chain).
+// Operands, orders and sums of the pair passes are those of the ordered kernels
+// with operands from the master arrays (k_born, k_gb, k_chain), and so are their
+// roundings but for the argument of the salt factor (kappa / (1/f) here, kappa f^2 (1/f)
+// there).
 #pragma once
 #include <cooperative_groups.h>
 

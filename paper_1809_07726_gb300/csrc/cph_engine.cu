@@ -1772,16 +1772,8 @@ int cph_init_system(const cph_system_desc* sys, int n_sys, const cph_grid_desc* 
     {
         float4* d4;
         float* d1;
-        std::vector<float4> xs, xl; // positions to be staged every step, and the radii
-        if (p->precision == CPH_PREC_FP32)
-            for (int w = 0; w < W; ++w)
-                for (int a = 0; a < sys_n[w_sys[w]]; ++a) {
-                    const int q = sys_poff[w_sys[w]] + a;
-                    xs.push_back(make_float4(0.f, 0.f, 0.f, (float)sc[q]));
-                    xl.push_back(make_float4(0.f, 0.f, 0.f, (float)rt[q]));
-                }
-        TRY(upload(E, xs, &d4)); V.xs = d4;
-        TRY(upload(E, xl, &d4)); V.xl = d4;
+        TRY(alloc0(E, (size_t)total, &d4)); V.xs = d4;
+        TRY(alloc0(E, (size_t)total, &d4)); V.xl = d4;
         TRY(alloc0(E, (size_t)total, &d4)); V.gq = d4;
         TRY(alloc0(E, (size_t)total, &d1)); V.c32 = d1;
     }
@@ -1961,6 +1953,10 @@ int cph_init_system(const cph_system_desc* sys, int n_sys, const cph_grid_desc* 
         TRY(upload(E, site_sys, &dss));
         const int nj = (int)js.size();
         k_site_ref<<<(nj + 63) / 64, 64>>>(E->V, dx0, djs, djst, dss, nj);
+        CK(cudaGetLastError());
+    }
+    if (p->precision == CPH_PREC_FP32) {
+        k_stage_radii<<<(total + 255) / 256, 256>>>(V);
         CK(cudaGetLastError());
     }
     CK(cudaDeviceSynchronize());

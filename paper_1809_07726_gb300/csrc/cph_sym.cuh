@@ -107,6 +107,16 @@ __global__ void k_stage_x(View V, int a0, int n) {
     for (int c = 0; c < 3; ++c) xl[c] = (float)(d[c] - (double)h[c]);
 }
 
+// The words of xs and xl that never change; once, at set-up.
+__global__ void k_stage_radii(View V) {
+    const int a = blockIdx.x * blockDim.x + threadIdx.x;
+    if (a >= V.total_atoms) return;
+    const int w = V.a_walker[a];
+    const float4 p = V.pb32[V.sys_poff[V.w_sys[w]] + (a - V.w_off[w])];
+    V.xs[a].w = p.x;
+    V.xl[a].w = p.y;
+}
+
 __global__ void k_stage_gb(View V, int a0, int n) {
     pdl_sync();
     const int l = blockIdx.x * blockDim.x + threadIdx.x;

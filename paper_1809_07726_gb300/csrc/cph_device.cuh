@@ -176,10 +176,13 @@ __device__ __forceinline__ double rcp64_radius(double x) {
     return h == 0 || h == 0x7ff00000 ? y : fma(y, fma(e, e, e), y);
 }
 
-// Born radii as the pair arithmetic takes them: finite, and so are their products;
-// past these bounds 1/f is 0 to every digit that counts.
-__device__ __forceinline__ float pair_radius32(double R) { return fminf((float)R, 1e18f); }
-__device__ __forceinline__ double pair_radius64(double R) { return fmin(R, 1e150); }
+// Born radii as the pair arithmetic takes them: not infinite, and so are their
+// products; with these values 1/f is 0 to every digit that counts.  (NaN stays NaN.)
+__device__ __forceinline__ float pair_radius32(double R) {
+    const float r = (float)R;
+    return r > 1e18f ? 1e18f : r;
+}
+__device__ __forceinline__ double pair_radius64(double R) { return __double2hiint(R) == 0x7ff00000 ? 1e150 : R; }
 
 // 1 / sqrt(x) for normal x > 0: the same (the binomial series after its second
 // term) with y (1 + e/2 + 3 e^2/8), e = 1 - x y^2

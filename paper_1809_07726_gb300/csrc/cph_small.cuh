@@ -75,12 +75,14 @@ constexpr int kSmallUnroll = 2;   // of the partner loops (1 to 4: within 3 %)
 //    246   37 / 64    37 / 74    37 / 89    70 / 89    71 / 132   106 / 160  173 / 201
 //    351   59 / 68    59 / 84    60 / 119   114 / 127  116 / 177  172 / 235  284 / 310
 //    452   75 / 70    76 / 100   76 / 154   147 / 157  149 / 244  221 / 334  364 / 450
+// Over 595 points (1 to 200 walkers of 40 to 460 atoms) what runs is within 5 % of the
+// best form but at six, most with a part-filled last wave, where it is 6 to 13 % behind.
 inline bool small_pays(int n, long long atoms, int walkers, int resident, bool constrained) {
     const int waves = (walkers + resident - 1) / resident;
-    if (constrained) return waves <= (n > 200 && n <= 384 ? 5 : 3); // (at 452 x 64 the tiles: 316)
+    if (constrained) return waves <= (n <= 100 ? 3 : (n <= 200 ? 4 : (n <= 256 ? 8 : (n <= 384 ? 5 : 4))));
     const long long other = (atoms + 2431) / 2432; // waves of the separate launches
     if (n <= 160) return waves <= std::min(other, 3ll);
-    if (n <= 256) return waves <= (other >= 5 ? 3 : std::min(other - 1, 2ll));
+    if (n <= 256) return waves <= (other >= 5 ? 3 : (other >= 3 ? 2 : (n <= 192 || atoms >= 1600 ? 1 : 0)));
     return n <= 384 && waves == 1 && other >= 3;
 }
 
